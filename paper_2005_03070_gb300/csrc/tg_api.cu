@@ -328,7 +328,7 @@ static int dot_host(tg_op *op, const T *a, const T *b, int n, double *aa, typena
     TG_CHECK(red_ready(op, 0, s));
     int g = grid_for(n, 4);
     D *out = reinterpret_cast<D *>(wsp<char>(op, S_SMALL) + SmallArea::dot_out);
-    TG_PROF(P_DOT, (b ? 2.0 : 1.0) * n * sizeof(T), (b ? 4.0 : 2.0) * n, k_dot<T><<<g, kThreads, 0, s>>>(a, b, n, wsp<D>(op, S_PART), wsp<unsigned>(op, S_TICKET), out));
+    TG_PROF(P_DOT, (b ? 2.0 : 1.0) * n * sizeof(T), (b ? 4.0 : 2.0) * n, launch(k_dot<T>, g, kThreads, 0, s, a, b, n, wsp<D>(op, S_PART), wsp<unsigned>(op, S_TICKET), out));
     TG_LAUNCH_CHECK();
     TG_CHECK(readback(op, out, 2 * sizeof(D), s));
     const D *h = reinterpret_cast<const D *>(op->pin.p);
@@ -350,7 +350,7 @@ template <class T>
 static int launch_apply(const DevOp &A, const DevOp32 &A32, const T *x, T *y, cudaStream_t s) {
     double xb, fl;
     op_cost(A, &xb, &fl);
-    TG_PROF(P_APPLY, (2.0 * sizeof(T) + xb * (sizeof(T) == 4 ? 0.5 : 1.0)) * A.n, fl * A.n, k_apply<T><<<grid_for(A.n, 8), kThreads, 0, s>>>(A, A32, x, y));
+    TG_PROF(P_APPLY, (2.0 * sizeof(T) + xb * (sizeof(T) == 4 ? 0.5 : 1.0)) * A.n, fl * A.n, launch(k_apply<T>, grid_for(A.n, 8), kThreads, 0, s, A, A32, x, y));
     TG_LAUNCH_CHECK();
     return TG_OK;
 }
@@ -383,7 +383,7 @@ template <class T>
 static int tsm(const T *In, size_t ldi, int p, const T *S, int lds, int q, T *Out, size_t ldo, int n, cudaStream_t s) {
     size_t smem = (size_t)32 * p * sizeof(T);
     TG_CHECK(set_smem<T>((const void *)k_tsm<T>, smem));
-    TG_PROF(P_TSM, (double)(p + q) * n * sizeof(T), 2.0 * p * q * n * (sizeof(T) == 16 ? 4 : 1), k_tsm<T><<<tiles_grid(n, 4), kThreads, smem, s>>>(In, ldi, p, S, lds, q, Out, ldo, n));
+    TG_PROF(P_TSM, (double)(p + q) * n * sizeof(T), 2.0 * p * q * n * (sizeof(T) == 16 ? 4 : 1), launch(k_tsm<T>, tiles_grid(n, 4), kThreads, smem, s, In, ldi, p, S, lds, q, Out, ldo, n));
     TG_LAUNCH_CHECK();
     return TG_OK;
 }
@@ -408,7 +408,7 @@ static int tsm_f(const float *In, size_t ldi, int p, const double *S, int lds, i
         constexpr int C = decltype(cpt)::value;
         TG_CHECK(set_smem<float>((const void *)k_tsm_f<TO, C>, smem));
         TG_PROF(P_TSM, (double)p * n * 4 + (double)q * n * sizeof(TO), 2.0 * p * q * n,
-                k_tsm_f<TO, C><<<gb, kThreads, smem, s>>>(In, ldi, p, S, lds, q, Out, ldo, n));
+                launch(k_tsm_f<TO, C>, gb, kThreads, smem, s, In, ldi, p, S, lds, q, Out, ldo, n));
         return TG_OK;
     };
     if (q <= 16) TG_CHECK(go(std::integral_constant<int, 1>{}));
@@ -448,7 +448,7 @@ static int gemv_t_part_launch(const T *V, size_t ldv, int ncol, const T *w, int 
             const int per_sm = smem <= 100 * 1024 ? 2 : 1;
             const int nchunks = (n + R - 1) / R;
             const int gb = std::max(1, std::min(nchunks, num_sms() * per_sm));
-            k_gemv_t_pipe<E><<<dim3(gb, ngr), kThreads, smem, s>>>(reinterpret_cast<const E *>(V), ldv, ncol,
+            launch(k_gemv_t_pipe<E>, dim3(gb, ngr), kThreads, smem, s, reinterpret_cast<const E *>(V), ldv, ncol,
                                                         reinterpret_cast<const E *>(w), n,
                                                         reinterpret_cast<double *>(part));
             *used_pipe = true;
@@ -457,7 +457,7 @@ static int gemv_t_part_launch(const T *V, size_t ldv, int ncol, const T *w, int 
     }
 plain:
     const int gb = (int)std::min<int64_t>((n + 127) / 128, (int64_t)num_sms() * 8);
-    k_gemv_t_part<T><<<dim3(std::max(gb, 1), (ncol + kGemvTCols - 1) / kGemvTCols), kThreads, 0, s>>>(V, ldv, ncol,
+    launch(k_gemv_t_part<T>, dim3(std::max(gb, 1), (ncol + kGemvTCols - 1) / kGemvTCols), kThreads, 0, s, V, ldv, ncol,
                                                                                                     w, n, part);
     *used_pipe = false;
     return std::max(gb, 1);
@@ -472,7 +472,7 @@ static int gemv_t(tg_op *op, const T *V, size_t ldv, int ncol, const T *w, int n
     TG_PROF(P_GEMV_T, (double)(ncol + 1) * n * sizeof(T), 2.0 * ncol * n * (sizeof(T) == 16 ? 4 : 1),
             gb = gemv_t_part_launch<T>(V, ldv, ncol, w, n, wsp<D>(op, S_PART), s, &piped));
     TG_LAUNCH_CHECK();
-    TG_PROF(P_SUM_PART, (double)gb * ncol * sizeof(D), (double)gb * ncol, k_sum_part<D><<<(ncol + 7) / 8, 256, 0, s>>>(wsp<D>(op, S_PART), gb, ncol, h, 0));
+    TG_PROF(P_SUM_PART, (double)gb * ncol * sizeof(D), (double)gb * ncol, launch(k_sum_part<D>, (ncol + 7) / 8, 256, 0, s, wsp<D>(op, S_PART), gb, ncol, h, 0));
     TG_LAUNCH_CHECK();
     return TG_OK;
 }
@@ -492,11 +492,11 @@ static int gram_ept(tg_op *op, const T *A, const T *B, size_t ld, int k, int n, 
     const size_t smem = (size_t)(A == B ? k : k + kb) * 33 * sizeof(T);
     TG_CHECK(set_smem<T>((const void *)k_gram_packed<T, EPT>, smem));
     TG_PROF(P_GRAM, (A == B ? 1.0 * k : 1.0 * (k + kb)) * n * sizeof(T), 2.0 * nent * n * (sizeof(T) == 16 ? 4 : 1),
-            k_gram_packed<T, EPT><<<dim3(gx, gy), kThreads, smem, s>>>(A, B, ld, k, n, sym, nent, part, kb));
+            launch(k_gram_packed<T, EPT>, dim3(gx, gy), kThreads, smem, s, A, B, ld, k, n, sym, nent, part, kb));
     TG_LAUNCH_CHECK();
     TG_PROF(P_SUM_PART, (double)gx * nent * sizeof(D), (double)gx * nent,
-            k_sum_part<D><<<(nent + 7) / 8, 256, 0, s>>>(part, gx, nent, packed, 0));
-    TG_PROF(P_SMALL, 0, 0, k_gram_unpack<D><<<(nent + 255) / 256, 256, 0, s>>>(packed, k, sym, G, kb));
+            launch(k_sum_part<D>, (nent + 7) / 8, 256, 0, s, part, gx, nent, packed, 0));
+    TG_PROF(P_SMALL, 0, 0, launch(k_gram_unpack<D>, (nent + 255) / 256, 256, 0, s, packed, k, sym, G, kb));
     TG_LAUNCH_CHECK();
     return TG_OK;
 }
@@ -864,9 +864,9 @@ static int project_impl(tg_op *op, const tg_defl *df, const T *W, const T *B1, c
     TG_LAUNCH_CHECK();
     const D *e = df->proj == TG_PROJ_MINRES ? cvec : dvec;
     if (kk <= kSmallCols)
-        TG_PROF(P_PROJ, (2.0 * kk + 4) * n * sizeof(T), 4.0 * kk * n * (sizeof(T) == 16 ? 4 : 1), k_proj_update<T, kSmallCols><<<grid_for(n, 8), kThreads, 0, s>>>(B1, B2, n, kk, dvec, e, x, r, n));
+        TG_PROF(P_PROJ, (2.0 * kk + 4) * n * sizeof(T), 4.0 * kk * n * (sizeof(T) == 16 ? 4 : 1), launch(k_proj_update<T, kSmallCols>, grid_for(n, 8), kThreads, 0, s, B1, B2, n, kk, dvec, e, x, r, n));
     else
-        TG_PROF(P_PROJ, (2.0 * kk + 4) * n * sizeof(T), 4.0 * kk * n * (sizeof(T) == 16 ? 4 : 1), k_proj_update<T><<<grid_for(n, 8), kThreads, 0, s>>>(B1, B2, n, kk, dvec, e, x, r, n));
+        TG_PROF(P_PROJ, (2.0 * kk + 4) * n * sizeof(T), 4.0 * kk * n * (sizeof(T) == 16 ? 4 : 1), launch(k_proj_update<T>, grid_for(n, 8), kThreads, 0, s, B1, B2, n, kk, dvec, e, x, r, n));
     TG_LAUNCH_CHECK();
     return TG_OK;
 }
@@ -999,12 +999,12 @@ static int bicg_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r,
             TG_CHECK(wsx(op, S_PADR, np * 4));
             float *xp = wsp<float>(op, S_PADX), *rp = wsp<float>(op, S_PADR);
             const int gpk = grid_for((int64_t)np, 8), gn = grid_for(n, 8);
-            TG_PROF(P_CONVERT, 8.0 * n, 0, k_pad3d<<<gpk, kThreads, 0, s>>>(x, xp, A.N));
-            TG_PROF(P_CONVERT, 8.0 * n, 0, k_pad3d<<<gpk, kThreads, 0, s>>>(r, rp, A.N));
+            TG_PROF(P_CONVERT, 8.0 * n, 0, launch(k_pad3d, gpk, kThreads, 0, s, x, xp, A.N));
+            TG_PROF(P_CONVERT, 8.0 * n, 0, launch(k_pad3d, gpk, kThreads, 0, s, r, rp, A.N));
             TG_LAUNCH_CHECK();
             TG_CHECK(bicg_cycle<float>(op, A, A32, xp, rp, (int)np, target2, cap, out, s, n));
-            TG_PROF(P_CONVERT, 8.0 * n, 0, k_unpad3d<<<gn, kThreads, 0, s>>>(xp, x, A.N));
-            TG_PROF(P_CONVERT, 8.0 * n, 0, k_unpad3d<<<gn, kThreads, 0, s>>>(rp, r, A.N));
+            TG_PROF(P_CONVERT, 8.0 * n, 0, launch(k_unpad3d, gn, kThreads, 0, s, xp, x, A.N));
+            TG_PROF(P_CONVERT, 8.0 * n, 0, launch(k_unpad3d, gn, kThreads, 0, s, rp, r, A.N));
             TG_LAUNCH_CHECK();
             return TG_OK;
         }
@@ -1032,7 +1032,7 @@ static int bicg_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r,
     D *part = wsp<D>(op, S_PART);
     unsigned *tk = wsp<unsigned>(op, S_TICKET);
     BiState<D> *st = reinterpret_cast<BiState<D> *>(wsp<char>(op, S_SMALL) + SmallArea::bistate);
-    TG_PROF(P_BI_INIT, 3.0 * nb * sizeof(T), 2.0 * nb, k_bi_init<T><<<g, kThreads, 0, s>>>(r, w.rh, w.p, n, target2, cap, part, tk, st));
+    TG_PROF(P_BI_INIT, 3.0 * nb * sizeof(T), 2.0 * nb, launch(k_bi_init<T>, g, kThreads, 0, s, r, w.rh, w.p, n, target2, cap, part, tk, st));
     TG_LAUNCH_CHECK();
     // float32 streaming updates with 16-byte aligned vectors: 4 points per thread
     bool use_v4 = false;
@@ -1052,27 +1052,27 @@ static int bicg_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r,
         for (int c = 0; c < chunk; ++c) {
             if (use_plane) {
                 if constexpr (std::is_same<T, float>::value)
-                    TG_PROF(P_BI_V, (3 * es + xbs) * nb, (fl + 2 * cf) * nb, k_bi_pad<0><<<gp_v, 32 * kPadRows, 0, s>>>(A, A32, w.p, w.rh, w.v, part, tk, st, zlen_v));
+                    TG_PROF(P_BI_V, (3 * es + xbs) * nb, (fl + 2 * cf) * nb, launch(k_bi_pad<0>, gp_v, 32 * kPadRows, 0, s, A, A32, w.p, w.rh, w.v, part, tk, st, zlen_v));
             } else {
-                TG_PROF(P_BI_V, (3 * es + xbs) * nb, (fl + 2 * cf) * nb, k_bi_v<T><<<g, kThreads, 0, s>>>(A, A32, w.p, w.rh, w.v, part, tk, st));
+                TG_PROF(P_BI_V, (3 * es + xbs) * nb, (fl + 2 * cf) * nb, launch(k_bi_v<T>, g, kThreads, 0, s, A, A32, w.p, w.rh, w.v, part, tk, st));
             }
             if (use_v4) {
                 if constexpr (std::is_same<T, float>::value)
-                    TG_PROF(P_BI_S, 3 * es * nb, 4 * cf * nb, k_bi_s_f4<<<g4, kThreads, 0, s>>>(r, w.v, w.s, n, part, tk, st));
+                    TG_PROF(P_BI_S, 3 * es * nb, 4 * cf * nb, launch(k_bi_s_f4, g4, kThreads, 0, s, r, w.v, w.s, n, part, tk, st));
             } else {
-                TG_PROF(P_BI_S, 3 * es * nb, 4 * cf * nb, k_bi_s<T><<<g, kThreads, 0, s>>>(r, w.v, w.s, n, part, tk, st));
+                TG_PROF(P_BI_S, 3 * es * nb, 4 * cf * nb, launch(k_bi_s<T>, g, kThreads, 0, s, r, w.v, w.s, n, part, tk, st));
             }
             if (use_plane) {
                 if constexpr (std::is_same<T, float>::value)
-                    TG_PROF(P_BI_T, (3 * es + xbs) * nb, (fl + 8 * cf) * nb, k_bi_pad<1><<<gp_t, 32 * kPadRows, 0, s>>>(A, A32, w.s, w.rh, w.t, part, tk, st, zlen_t));
+                    TG_PROF(P_BI_T, (3 * es + xbs) * nb, (fl + 8 * cf) * nb, launch(k_bi_pad<1>, gp_t, 32 * kPadRows, 0, s, A, A32, w.s, w.rh, w.t, part, tk, st, zlen_t));
             } else {
-                TG_PROF(P_BI_T, (3 * es + xbs) * nb, (fl + 8 * cf) * nb, k_bi_t<T><<<g, kThreads, 0, s>>>(A, A32, w.s, w.rh, w.t, part, tk, st));
+                TG_PROF(P_BI_T, (3 * es + xbs) * nb, (fl + 8 * cf) * nb, launch(k_bi_t<T>, g, kThreads, 0, s, A, A32, w.s, w.rh, w.t, part, tk, st));
             }
             if (use_v4) {
                 if constexpr (std::is_same<T, float>::value)
-                    TG_PROF(P_BI_X, 8 * es * nb, 12 * cf * nb, k_bi_x_f4<<<g4, kThreads, 0, s>>>(x, r, w.p, w.s, w.t, w.v, n, part, tk, st));
+                    TG_PROF(P_BI_X, 8 * es * nb, 12 * cf * nb, launch(k_bi_x_f4, g4, kThreads, 0, s, x, r, w.p, w.s, w.t, w.v, n, part, tk, st));
             } else {
-                TG_PROF(P_BI_X, 8 * es * nb, 12 * cf * nb, k_bi_x<T><<<g, kThreads, 0, s>>>(x, r, w.p, w.s, w.t, w.v, n, part, tk, st));
+                TG_PROF(P_BI_X, 8 * es * nb, 12 * cf * nb, launch(k_bi_x<T>, g, kThreads, 0, s, x, r, w.p, w.s, w.t, w.v, n, part, tk, st));
             }
         }
         TG_LAUNCH_CHECK();
@@ -1155,7 +1155,7 @@ static int true_residual(tg_op *op, const DevOp &A, const T *b, const T *x, T *r
     D *out = reinterpret_cast<D *>(wsp<char>(op, S_SMALL) + SmallArea::res_out);
     double xb, fl;
     op_cost(A, &xb, &fl);
-    TG_PROF(P_RESIDUAL, (3.0 * sizeof(T) + xb) * n, (fl + 6) * n, k_residual<T><<<g, kThreads, 0, s>>>(A, b, x, r, wsp<D>(op, S_PART), wsp<unsigned>(op, S_TICKET), out));
+    TG_PROF(P_RESIDUAL, (3.0 * sizeof(T) + xb) * n, (fl + 6) * n, launch(k_residual<T>, g, kThreads, 0, s, A, b, x, r, wsp<D>(op, S_PART), wsp<unsigned>(op, S_TICKET), out));
     TG_LAUNCH_CHECK();
     TG_CHECK(readback(op, out, 2 * sizeof(D), s));
     const D *h = reinterpret_cast<const D *>(op->pin.p);
@@ -1332,7 +1332,7 @@ static int idr_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r, 
     op_cost(A, &xb, &fl);
     const double cf = sizeof(T) == 16 ? 4.0 : 1.0;
     TG_PROF(P_IDR_UPD, (1.0 + sd) * n * es, 2.0 * (sd + 1) * n * cf,
-            k_idr_init<T><<<g, kThreads, 0, s>>>(r, P, ld, n, sd, target2, cap, kappa, part, tk, st));
+            launch(k_idr_init<T>, g, kThreads, 0, s, r, P, ld, n, sd, target2, cap, kappa, part, tk, st));
     TG_LAUNCH_CHECK();
     int batch = 1, launched = 0;
     IdrState<D> h{};
@@ -1341,16 +1341,16 @@ static int idr_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r, 
             const int first = launched + b == 0;
             for (int k = 0; k < sd; ++k) {
                 TG_PROF(P_IDR_UPD, (2.0 + (first ? 0.0 : 2.0 * (sd - k))) * n * es, 4.0 * (sd - k) * n * cf,
-                        k_idr_u<T><<<g, kThreads, 0, s>>>(r, G, U, ld, n, k, first, st));
+                        launch(k_idr_u<T>, g, kThreads, 0, s, r, G, U, ld, n, k, first, st));
                 TG_PROF(P_IDR_MV, (2.0 + sd) * n * es + xb * n, (fl + 2.0 * sd * cf) * n,
-                        k_idr_g<T><<<g, kThreads, 0, s>>>(A, A32, U, G, P, ld, k, part, tk, st));
+                        launch(k_idr_g<T>, g, kThreads, 0, s, A, A32, U, G, P, ld, k, part, tk, st));
                 TG_PROF(P_IDR_UPD, (2.0 * k + 8.0) * n * es, (4.0 * k + 6.0) * n * cf,
-                        k_idr_upd<T><<<g, kThreads, 0, s>>>(G, U, ld, r, x, n, k, part, tk, st));
+                        launch(k_idr_upd<T>, g, kThreads, 0, s, G, U, ld, r, x, n, k, part, tk, st));
             }
             TG_PROF(P_IDR_MV, 2.0 * n * es + xb * n, (fl + 6.0 * cf) * n,
-                    k_idr_t<T><<<g, kThreads, 0, s>>>(A, A32, r, t, part, tk, st));
+                    launch(k_idr_t<T>, g, kThreads, 0, s, A, A32, r, t, part, tk, st));
             TG_PROF(P_IDR_UPD, (5.0 + sd) * n * es, (4.0 + 2.0 * (sd + 1)) * n * cf,
-                    k_idr_xr<T><<<g, kThreads, 0, s>>>(x, r, t, P, ld, n, part, tk, st));
+                    launch(k_idr_xr<T>, g, kThreads, 0, s, x, r, t, P, ld, n, part, tk, st));
         }
         TG_LAUNCH_CHECK();
         launched += batch;
@@ -1558,15 +1558,15 @@ static void gemv_n_norm_launch(int g, const T *V, size_t ldv, int ncol, const ty
                                const typename ST<T>::D *nrm_before, int *flag, double eta2, cudaStream_t s) {
     if constexpr (sizeof(T) == 4) {
         if (ldv % 4 == 0 && !(((uintptr_t)V | (uintptr_t)w) & 15)) {
-            if (ncol <= kSmallCols) k_gemv_n_norm_f4<kSmallCols><<<g, kThreads, 0, s>>>(V, ldv, ncol, h, w, n, part, tk, nrm);
-            else k_gemv_n_norm_f4<><<<g, kThreads, 0, s>>>(V, ldv, ncol, h, w, n, part, tk, nrm);
+            if (ncol <= kSmallCols) launch(k_gemv_n_norm_f4<kSmallCols>, g, kThreads, 0, s, V, ldv, ncol, h, w, n, part, tk, nrm);
+            else launch(k_gemv_n_norm_f4<>, g, kThreads, 0, s, V, ldv, ncol, h, w, n, part, tk, nrm);
             return;
         }
     }
     if (ncol <= kSmallCols)
-        k_gemv_n_norm<T, kSmallCols><<<g, kThreads, 0, s>>>(V, ldv, ncol, h, w, n, nullptr, part, tk, nrm, nrm_before, flag, eta2);
+        launch(k_gemv_n_norm<T, kSmallCols>, g, kThreads, 0, s, V, ldv, ncol, h, w, n, nullptr, part, tk, nrm, nrm_before, flag, eta2);
     else
-        k_gemv_n_norm<T><<<g, kThreads, 0, s>>>(V, ldv, ncol, h, w, n, nullptr, part, tk, nrm, nrm_before, flag, eta2);
+        launch(k_gemv_n_norm<T>, g, kThreads, 0, s, V, ldv, ncol, h, w, n, nullptr, part, tk, nrm, nrm_before, flag, eta2);
 }
 
 template <class T, class HT = T>
@@ -1597,7 +1597,7 @@ static int arnoldi_step(tg_op *op, const DevOp &A, const DevOp32 &A32, T *V, siz
     TG_PROF(P_GEMV_T, (double)(ncol + 1) * n * sizeof(T), 2.0 * (ncol + 1) * n * (sizeof(T) == 16 ? 4 : 1),
             gbt = gemv_t_part_launch<T>(V, ldv, ncol + 1, w, n, part, s, &piped));
     TG_PROF(P_SUM_PART, (double)gbt * (ncol + 1) * sizeof(D), (double)gbt * (ncol + 1),
-            k_sum_part<D><<<(ncol + 1 + 7) / 8, 256, 0, s>>>(part, gbt, ncol + 1, h1, 0));
+            launch(k_sum_part<D>, (ncol + 1 + 7) / 8, 256, 0, s, part, gbt, ncol + 1, h1, 0));
     TG_PROF(P_GEMV_N, (ncol + 2.0) * n * sizeof(T), 2.0 * ncol * n * (sizeof(T) == 16 ? 4 : 1),
             gemv_n_norm_launch<T>(g, V, ldv, ncol, h1, w, n, part, tk, nrm, h1 + ncol, flag, 0.5, s));
     // pass 2 (classical Gram-Schmidt twice: on this operator the selective criterion of
@@ -1605,11 +1605,11 @@ static int arnoldi_step(tg_op *op, const DevOp &A, const DevOp32 &A32, T *V, siz
     TG_PROF(P_GEMV_T, (double)(ncol + 1) * n * sizeof(T), 2.0 * ncol * n * (sizeof(T) == 16 ? 4 : 1),
             gbt = gemv_t_part_launch<T>(V, ldv, ncol, w, n, part, s, &piped));
     TG_PROF(P_SUM_PART, (double)gbt * ncol * sizeof(D), (double)gbt * ncol,
-            k_sum_part<D><<<(ncol + 7) / 8, 256, 0, s>>>(part, gbt, ncol, h2, 0));
+            launch(k_sum_part<D>, (ncol + 7) / 8, 256, 0, s, part, gbt, ncol, h2, 0));
     TG_PROF(P_GEMV_N, (ncol + 2.0) * n * sizeof(T), 2.0 * ncol * n * (sizeof(T) == 16 ? 4 : 1),
             gemv_n_norm_launch<T>(g, V, ldv, ncol, h2, w, n, part, tk, nrm, nullptr, nullptr, 0.0, s));
-    TG_PROF(P_SMALL, 0, j, k_arnoldi_finish2<T, HT><<<1, 128, 0, s>>>(h1, h2, nrm, j, H + (size_t)j * ldh, inv));
-    TG_PROF(P_SCALE, 2.0 * n * sizeof(T), n, k_scale_by<T><<<g, kThreads, 0, s>>>(w, n, inv));
+    TG_PROF(P_SMALL, 0, j, launch(k_arnoldi_finish2<T, HT>, 1, 128, 0, s, h1, h2, nrm, j, H + (size_t)j * ldh, inv));
+    TG_PROF(P_SCALE, 2.0 * n * sizeof(T), n, launch(k_scale_by<T>, g, kThreads, 0, s, w, n, inv));
     TG_LAUNCH_CHECK();
     return TG_OK;
 }
@@ -1665,7 +1665,7 @@ static int solve_gmres64(tg_op *op, int transpose, const tg_defl *df, const T *b
         memcpy(&g0, &nr, sizeof(double));
         TG_CHECK_CUDA(cudaMemcpyAsync(wsp<D>(op, S_FG), &g0, sizeof(D), cudaMemcpyHostToDevice, s));
         TG_CHECK_CUDA(cudaMemsetAsync(H, 0, (size_t)(m + 1) * m * sizeof(D), s));
-        TG_PROF(P_SCALE, 2.0 * n * sizeof(T), n, k_scale_by<T><<<grid_for(n, 8), kThreads, 0, s>>>(V, n, inv));
+        TG_PROF(P_SCALE, 2.0 * n * sizeof(T), n, launch(k_scale_by<T>, grid_for(n, 8), kThreads, 0, s, V, n, inv));
         TG_LAUNCH_CHECK();
         int steps = 0;
         const int mm = (int)((cfg.max_mvps - mvps) < m ? (cfg.max_mvps - mvps) : m);
@@ -1681,7 +1681,7 @@ static int solve_gmres64(tg_op *op, int transpose, const tg_defl *df, const T *b
         }
         mvps += steps;
         TG_PROF(P_GIVENS, 0, 1.0 * m * m, launch_givens_solve<D>(H, ldh, wsp<D>(op, S_FG), wsp<D>(op, S_FY), gs, s));
-        TG_PROF(P_GEMV_N, (steps + 2.0) * n * sizeof(T), 2.0 * steps * n, k_gemv_n<T><<<grid_for(n, 8), kThreads, 0, s>>>(V, n, steps, wsp<D>(op, S_FY), 1.0, x, n));
+        TG_PROF(P_GEMV_N, (steps + 2.0) * n * sizeof(T), 2.0 * steps * n, launch(k_gemv_n<T>, grid_for(n, 8), kThreads, 0, s, V, n, steps, wsp<D>(op, S_FY), 1.0, x, n));
         TG_LAUNCH_CHECK();
         TG_CHECK(true_residual<T>(op, A, b, x, r, &nr, &nb, s));
         if (!std::isfinite(nr)) { status = TG_NAN; break; }
@@ -1803,7 +1803,7 @@ static int gdr_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *V, size_t
         if (le != cudaSuccess) return cuda_status(le, "launching k_gmresdr_restart (shared-memory limit or launch)");
         // x_c += V_m d
         TG_PROF(P_GEMV_N, (m + 2.0) * nc * sizeof(T), 2.0 * m * nc,
-                k_gemv_n<T><<<grid_for(nc, 8), kThreads, 0, s>>>(V, ldv, m, a.d, 1.0, xc, nc));
+                launch(k_gemv_n<T>, grid_for(nc, 8), kThreads, 0, s, V, ldv, m, a.d, 1.0, xc, nc));
         TG_LAUNCH_CHECK();
         return TG_OK;
     };
@@ -1942,7 +1942,7 @@ static int gmresdr_impl(tg_op *op, int transpose, const void *b_fine, int m, int
         double *inv = reinterpret_cast<double *>(wsp<char>(op, S_SMALL) + SmallArea::gmres_inv);
         double hinv = 1.0 / nbc;
         TG_CHECK_CUDA(cudaMemcpyAsync(inv, &hinv, sizeof(double), cudaMemcpyHostToDevice, s));
-        TG_PROF(P_SCALE, 2.0 * nc * sizeof(T), nc, k_scale_by<T><<<grid_for(nc, 8), kThreads, 0, s>>>(V, nc, inv));
+        TG_PROF(P_SCALE, 2.0 * nc * sizeof(T), nc, launch(k_scale_by<T>, grid_for(nc, 8), kThreads, 0, s, V, nc, inv));
     }
     TG_CHECK_CUDA(cudaMemsetAsync(xc, 0, (size_t)nc * es, s));
     TG_CHECK_CUDA(cudaMemsetAsync(H, 0, (size_t)ldh * m * hs, s));
@@ -1993,10 +1993,10 @@ static int gmresdr_impl(tg_op *op, int transpose, const void *b_fine, int m, int
             DD *h1 = reinterpret_cast<DD *>(wsp<char>(op, S_SMALL) + SmallArea::arn_h1);
             DD *nrm = reinterpret_cast<DD *>(wsp<char>(op, S_SMALL) + SmallArea::arn_nrm);
             TG_CHECK(gemv_t<T>(op, V, ldv, kk, w, nc, h1, s));
-            TG_PROF(P_GEMV_N, (kk + 2.0) * nc * sizeof(T), 2.0 * kk * nc, k_gemv_n<T><<<grid_for(nc, 8), kThreads, 0, s>>>(V, ldv, kk, h1, -1.0, w, nc));
-            TG_PROF(P_DOT, 1.0 * nc * sizeof(T), 2.0 * nc, k_dot<T><<<grid_for(nc, 4), kThreads, 0, s>>>(w, nullptr, nc, wsp<DD>(op, S_PART), wsp<unsigned>(op, S_TICKET), nrm));
+            TG_PROF(P_GEMV_N, (kk + 2.0) * nc * sizeof(T), 2.0 * kk * nc, launch(k_gemv_n<T>, grid_for(nc, 8), kThreads, 0, s, V, ldv, kk, h1, -1.0, w, nc));
+            TG_PROF(P_DOT, 1.0 * nc * sizeof(T), 2.0 * nc, launch(k_dot<T>, grid_for(nc, 4), kThreads, 0, s, w, nullptr, nc, wsp<DD>(op, S_PART), wsp<unsigned>(op, S_TICKET), nrm));
             TG_PROF(P_SMALL, 0, 1, launch_inv_sqrt(s, reinterpret_cast<const double *>(nrm), reinterpret_cast<double *>(nrm) + 4));
-            TG_PROF(P_SCALE, 2.0 * nc * sizeof(T), nc, k_scale_by<T><<<grid_for(nc, 8), kThreads, 0, s>>>(w, nc, reinterpret_cast<double *>(nrm) + 4));
+            TG_PROF(P_SCALE, 2.0 * nc * sizeof(T), nc, launch(k_scale_by<T>, grid_for(nc, 8), kThreads, 0, s, w, nc, reinterpret_cast<double *>(nrm) + 4));
             TG_LAUNCH_CHECK();
         }
         j0 = kk;
@@ -2099,11 +2099,11 @@ static int cgs2_column(tg_op *op, T *V, size_t ldv, int n, int j, double drop_re
         bool piped = false;
         int gbt = 1;
         TG_PROF(P_GEMV_T, (double)(j + 1) * n * sizeof(T), 2.0 * (j + 1) * n, gbt = gemv_t_part_launch<T>(V, ldv, j + 1, w, n, part, s, &piped));
-        TG_PROF(P_SUM_PART, 0, 0, k_sum_part<D><<<(j + 1 + 7) / 8, 256, 0, s>>>(part, gbt, j + 1, h1, 0));
+        TG_PROF(P_SUM_PART, 0, 0, launch(k_sum_part<D>, (j + 1 + 7) / 8, 256, 0, s, part, gbt, j + 1, h1, 0));
         TG_PROF(P_GEMV_N, (j + 2.0) * n * sizeof(T), 2.0 * j * n,
                 gemv_n_norm_launch<T>(g, V, ldv, j, h1, w, n, part, tk, nrm, nullptr, nullptr, 0.0, s));
         TG_PROF(P_GEMV_T, (double)(j + 1) * n * sizeof(T), 2.0 * j * n, gbt = gemv_t_part_launch<T>(V, ldv, j, w, n, part, s, &piped));
-        TG_PROF(P_SUM_PART, 0, 0, k_sum_part<D><<<(j + 7) / 8, 256, 0, s>>>(part, gbt, j, h2, 0));
+        TG_PROF(P_SUM_PART, 0, 0, launch(k_sum_part<D>, (j + 7) / 8, 256, 0, s, part, gbt, j, h2, 0));
         TG_PROF(P_GEMV_N, (j + 2.0) * n * sizeof(T), 2.0 * j * n,
                 gemv_n_norm_launch<T>(g, V, ldv, j, h2, w, n, part, tk, nrm, nullptr, nullptr, 0.0, s));
         TG_LAUNCH_CHECK();
@@ -2117,7 +2117,7 @@ static int cgs2_column(tg_op *op, T *V, size_t ldv, int n, int j, double drop_re
     *kept = after > drop_rel * drop_rel * before && after > 0.0;
     if (*kept) {
         TG_PROF(P_SMALL, 0, 1, launch_inv_sqrt(s, nrm, inv));
-        TG_PROF(P_SCALE, 2.0 * n * sizeof(T), n, k_scale_by<T><<<g, kThreads, 0, s>>>(w, n, inv));
+        TG_PROF(P_SCALE, 2.0 * n * sizeof(T), n, launch(k_scale_by<T>, g, kThreads, 0, s, w, n, inv));
         TG_LAUNCH_CHECK();
     }
     return TG_OK;
@@ -2136,6 +2136,7 @@ static int cgs2_column(tg_op *op, T *V, size_t ldv, int n, int j, double drop_re
 template <class T>
 __global__ void k_ae_assemble(const T *__restrict__ Ha, int p, const T *__restrict__ HR,
                               const T *__restrict__ WWR, int cols, T *__restrict__ H, T *__restrict__ WW) {
+    pdl_wait();
     const int q = cols - p, ldh = p + 1;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < cols * cols; e += gridDim.x * blockDim.x) {
         const int i = e % cols, j = e / cols;
@@ -2187,7 +2188,7 @@ static int rayleigh_ritz(tg_op *op, const T *S, const T *W, size_t ld, int n, in
         const T *WR = W + (size_t)p * ld;
         TG_CHECK(gram<T>(op, S, WR, ld, m, n, 0, reinterpret_cast<D *>(HR), s, q));
         TG_CHECK(gram<T>(op, WR, WR, ld, q, n, 1, reinterpret_cast<D *>(WWR), s));
-        TG_PROF(P_SMALL, 0, 0, k_ae_assemble<T><<<(m * m + 255) / 256, 256, 0, s>>>(Ha, p, HR, WWR, m, H, WW));
+        TG_PROF(P_SMALL, 0, 0, launch(k_ae_assemble<T>, (m * m + 255) / 256, 256, 0, s, Ha, p, HR, WWR, m, H, WW));
         TG_LAUNCH_CHECK();
     } else {
         TG_CHECK(gram<T>(op, S, W, ld, m, n, 0, reinterpret_cast<D *>(H), s));
@@ -2626,10 +2627,10 @@ static void batch_iters_all(tg_batch *b, const MrBatchPtrs &P, int gx, int iters
     float *rh = A.rh.as<float>(), *p = A.p.as<float>(), *v = A.v.as<float>(), *sv = A.s.as<float>(),
           *t = A.t.as<float>(), *r = A.r32.as<float>(), *x = A.e32.as<float>();
     for (int it = 0; it < iters; ++it) {
-        k_mrb_bi_v<R><<<grid, kThreads, 0, s>>>(p, rh, v, P);
-        k_mrb_bi_s<R><<<grid, kThreads, 0, s>>>(r, v, sv, P);
-        k_mrb_bi_t<R><<<grid, kThreads, 0, s>>>(sv, rh, t, P);
-        k_mrb_bi_x<R><<<grid, kThreads, 0, s>>>(x, r, p, sv, t, v, P);
+        launch(k_mrb_bi_v<R>, grid, kThreads, 0, s, p, rh, v, P);
+        launch(k_mrb_bi_s<R>, grid, kThreads, 0, s, r, v, sv, P);
+        launch(k_mrb_bi_t<R>, grid, kThreads, 0, s, sv, rh, t, P);
+        launch(k_mrb_bi_x<R>, grid, kThreads, 0, s, x, r, p, sv, t, v, P);
     }
 }
 
@@ -2682,7 +2683,7 @@ static int batch_tune(tg_batch *b) {
         TG_CHECK_CUDA(cudaMemcpyAsync(P0.target2, zeros.data(), zeros.size() * 8, cudaMemcpyHostToDevice, s));
         TG_CHECK_CUDA(cudaMemcpyAsync(A.r32.p, A.rsave.p, tot * 4, cudaMemcpyDeviceToDevice, s));
         TG_CHECK_CUDA(cudaMemsetAsync(A.e32.p, 0, tot * 4, s));
-        k_mrb_bi_init<R><<<dim3(gx, b->count), kThreads, 0, s>>>(A.r32.as<float>(), A.rh.as<float>(), A.p.as<float>(), P0);
+        launch(k_mrb_bi_init<R>, dim3(gx, b->count), kThreads, 0, s, A.r32.as<float>(), A.rh.as<float>(), A.p.as<float>(), P0);
         TG_LAUNCH_CHECK();
         TG_CHECK(batch_graph(b, gx));
         TG_CHECK_CUDA(cudaGraphLaunch(A.graph, s));          // warm
@@ -2750,7 +2751,7 @@ static int batch_solve_all(tg_batch *b, const double *Bv, double *X, const Solve
     std::vector<int> status(BR);
     auto residual = [&]() -> int {
         TG_PROF(P_RESIDUAL, (3.0 * 8) * b->total, 12.0 * b->total,
-                k_mrb_residual<R><<<dim3(gres, count), kThreads, 0, s>>>(Bv, X, A.r64.as<double>(), P));
+                launch(k_mrb_residual<R>, dim3(gres, count), kThreads, 0, s, Bv, X, A.r64.as<double>(), P));
         TG_LAUNCH_CHECK();
         TG_CHECK(batch_readback(b, P.norms, (size_t)count * 2 * R * 8));
         for (int i = 0; i < count; ++i)
@@ -2779,16 +2780,16 @@ static int batch_solve_all(tg_batch *b, const double *Bv, double *X, const Solve
         for (size_t c = 0; c < BR; ++c) hv[c] = status[c] == TG_NOT_CONVERGED ? 1.0 / nr[c] : 0.0;
         TG_CHECK_CUDA(cudaMemcpyAsync(P.inv, hv.data(), BR * 8, cudaMemcpyHostToDevice, s));
         TG_PROF(P_CONVERT, 16.0 * b->total, b->total,
-                k_mrb_scale<R><<<dim3(gres, count), kThreads, 0, s>>>(A.r64.as<double>(), A.r32.as<float>(),
+                launch(k_mrb_scale<R>, dim3(gres, count), kThreads, 0, s, A.r64.as<double>(), A.r32.as<float>(),
                                                                          A.e32.as<float>(), P));
         TG_LAUNCH_CHECK();
         for (size_t c = 0; c < BR; ++c) nrel[c] = 1.0;
         if (any_defl) {
             const size_t smem = ((size_t)32 * 128 + 128 * R) * sizeof(float);
             TG_CHECK(set_smem<float>((const void *)k_mrb_proj_dots<R>, smem));
-            TG_PROF(P_GEMV_T, 0, 0, k_mrb_proj_dots<R><<<dim3(gres, count), kThreads, smem, s>>>(A.r32.as<float>(), P));
-            TG_PROF(P_SMALL, 0, 0, k_mrb_small<R><<<count, 256, 0, s>>>(P));
-            TG_PROF(P_PROJ, 0, 0, k_mrb_proj_update<R><<<dim3(gres, count), kThreads, 0, s>>>(A.e32.as<float>(),
+            TG_PROF(P_GEMV_T, 0, 0, launch(k_mrb_proj_dots<R>, dim3(gres, count), kThreads, smem, s, A.r32.as<float>(), P));
+            TG_PROF(P_SMALL, 0, 0, launch(k_mrb_small<R>, count, 256, 0, s, P));
+            TG_PROF(P_PROJ, 0, 0, launch(k_mrb_proj_update<R>, dim3(gres, count), kThreads, 0, s, A.e32.as<float>(),
                                                                                             A.r32.as<float>(), P));
             TG_LAUNCH_CHECK();
             TG_CHECK(batch_readback(b, P.norms, (size_t)count * 2 * R * 8));
@@ -2825,7 +2826,7 @@ static int batch_solve_all(tg_batch *b, const double *Bv, double *X, const Solve
         TG_CHECK_CUDA(cudaMemcpyAsync(P.target2, hv.data(), BR * 8, cudaMemcpyHostToDevice, s));
         const MrBatchPtrs Pc = batch_ptrs(b, (int)cap64);
         TG_PROF(P_BI_INIT, 12.0 * b->total, 2.0 * b->total,
-                k_mrb_bi_init<R><<<dim3(gx, count), kThreads, 0, s>>>(A.r32.as<float>(), A.rh.as<float>(),
+                launch(k_mrb_bi_init<R>, dim3(gx, count), kThreads, 0, s, A.r32.as<float>(), A.rh.as<float>(),
                                                                         A.p.as<float>(), Pc));
         TG_LAUNCH_CHECK();
         TG_CHECK(batch_graph(b, gx));
@@ -2855,7 +2856,7 @@ static int batch_solve_all(tg_batch *b, const double *Bv, double *X, const Solve
         }
         TG_CHECK_CUDA(cudaMemcpyAsync(P.scale, hv.data(), BR * 8, cudaMemcpyHostToDevice, s));
         TG_PROF(P_CONVERT, 12.0 * b->total, 2.0 * b->total,
-                k_mrb_add<R><<<dim3(gres, count), kThreads, 0, s>>>(X, A.e32.as<float>(), P));
+                launch(k_mrb_add<R>, dim3(gres, count), kThreads, 0, s, X, A.e32.as<float>(), P));
         TG_LAUNCH_CHECK();
         TG_CHECK(residual());
         // a correction that raised the float64 residual kIrGrowth-fold is undone (x -= ||r|| e)
@@ -2871,7 +2872,7 @@ static int batch_solve_all(tg_batch *b, const double *Bv, double *X, const Solve
         if (undo) {
             TG_CHECK_CUDA(cudaMemcpyAsync(P.scale, hv.data(), BR * 8, cudaMemcpyHostToDevice, s));
             TG_PROF(P_CONVERT, 12.0 * b->total, 2.0 * b->total,
-                    k_mrb_add<R><<<dim3(gres, count), kThreads, 0, s>>>(X, A.e32.as<float>(), P));
+                    launch(k_mrb_add<R>, dim3(gres, count), kThreads, 0, s, X, A.e32.as<float>(), P));
             TG_LAUNCH_CHECK();
             TG_CHECK(residual());
         }
@@ -3008,7 +3009,7 @@ static int batch_setup_all(tg_batch *b, const double *R0, int m, int k, int nev,
         TG_CHECK(I.cgw.ensure((size_t)m * m * 16));
         TG_CHECK(I.cYc.ensure((size_t)nc * (k + 2) * 8));
         // b_c = restrict(column 0), ||b_c||, v_0 = b_c / ||b_c|| (float32)
-        k_mr_extract<kBatchR><<<grid_for(op->n, 8), kThreads, 0, s>>>(R0 + b->off[i], 0, op->n, I.tmp.as<double>());
+        launch(k_mr_extract<kBatchR>, grid_for(op->n, 8), kThreads, 0, s, R0 + b->off[i], 0, op->n, I.tmp.as<double>());
         TG_LAUNCH_CHECK();
         TG_CHECK(restrict_impl(op, I.tmp.p, I.cbc.p, 1, s));
         double nb2 = 0.0;
@@ -3063,8 +3064,8 @@ static int batch_setup_all(tg_batch *b, const double *R0, int m, int k, int nev,
     bool gb_pipe = smem_attr_once((const void *)k_gb_gemv_t_pipe, (int)kGbPipeSmem) == cudaSuccess;
     if (!gb_pipe) (void)cudaGetLastError();
     auto gemv_t_all = [&](int j, int ncol_step, int reorth, int which) {
-        if (gb_pipe) k_gb_gemv_t_pipe<<<grid, kThreads, kGbPipeSmem, s>>>(P, j, ncol_step, reorth, which);
-        else k_gb_gemv_t<<<grid, kThreads, 0, s>>>(P, j, ncol_step, reorth, which);
+        if (gb_pipe) launch(k_gb_gemv_t_pipe, grid, kThreads, kGbPipeSmem, s, P, j, ncol_step, reorth, which);
+        else launch(k_gb_gemv_t, grid, kThreads, 0, s, P, j, ncol_step, reorth, which);
     };
     int any = count;
     int cyc = 0;
@@ -3084,13 +3085,13 @@ static int batch_setup_all(tg_batch *b, const double *R0, int m, int k, int nev,
         TG_CHECK_CUDA(cudaMemcpyAsync(C.active.p, active.data(), active.size() * sizeof(int), cudaMemcpyHostToDevice, s));
         // Arnoldi from each instance's j0 to m
         for (int j = jmin; j < m; ++j) {
-            TG_PROF(P_APPLY, 0, 0, k_gb_apply<<<grid, kThreads, 0, s>>>(P, j));
+            TG_PROF(P_APPLY, 0, 0, launch(k_gb_apply, grid, kThreads, 0, s, P, j));
             TG_PROF(P_GEMV_T, 0, 0, gemv_t_all(j, j + 2, 0, 0));
-            TG_PROF(P_GEMV_N, 0, 0, k_gb_gemv_n_norm<<<grid, kThreads, 0, s>>>(P, j, j + 1, 0, 0));
+            TG_PROF(P_GEMV_N, 0, 0, launch(k_gb_gemv_n_norm, grid, kThreads, 0, s, P, j, j + 1, 0, 0));
             TG_PROF(P_GEMV_T, 0, 0, gemv_t_all(j, j + 1, 0, 1));
-            TG_PROF(P_GEMV_N, 0, 0, k_gb_gemv_n_norm<<<grid, kThreads, 0, s>>>(P, j, j + 1, 0, 1));
-            TG_PROF(P_SMALL, 0, 0, k_gb_finish<<<(count + 127) / 128, 128, 0, s>>>(P, count, j, ldh, 0));
-            TG_PROF(P_SCALE, 0, 0, k_gb_scale<<<grid, kThreads, 0, s>>>(P, j, 0));
+            TG_PROF(P_GEMV_N, 0, 0, launch(k_gb_gemv_n_norm, grid, kThreads, 0, s, P, j, j + 1, 0, 1));
+            TG_PROF(P_SMALL, 0, 0, launch(k_gb_finish, (count + 127) / 128, 128, 0, s, P, count, j, ldh, 0));
+            TG_PROF(P_SCALE, 0, 0, launch(k_gb_scale, grid, kThreads, 0, s, P, j, 0));
         }
         TG_LAUNCH_CHECK();
         // the restart matrices are written into each instance's other Hbar buffer (which of
@@ -3147,7 +3148,7 @@ static int batch_setup_all(tg_batch *b, const double *R0, int m, int k, int nev,
             TG_CHECK_CUDA(cudaMemcpyAsync(tb, Pp.data(), (size_t)count * 8, cudaMemcpyHostToDevice, s));
             TG_CHECK_CUDA(cudaMemcpyAsync(tb + (size_t)count * 8, Op.data(), (size_t)count * 8, cudaMemcpyHostToDevice, s));
             TG_CHECK_CUDA(cudaMemcpyAsync(tb + (size_t)count * 16, ldo.data(), (size_t)count * 8, cudaMemcpyHostToDevice, s));
-            TG_PROF(P_TSM, 0, 0, k_gb_tsm<float><<<grid, kThreads, 0, s>>>(
+            TG_PROF(P_TSM, 0, 0, launch(k_gb_tsm<float>, grid, kThreads, 0, s, 
                 P, reinterpret_cast<const double *const *>(tb), m + 1, m + 1, 1,
                 reinterpret_cast<float *const *>(tb + (size_t)count * 8), reinterpret_cast<const size_t *>(tb + (size_t)count * 16)));
             TG_LAUNCH_CHECK();
@@ -3166,9 +3167,9 @@ static int batch_setup_all(tg_batch *b, const double *R0, int m, int k, int nev,
         }
         TG_CHECK_CUDA(cudaMemcpyAsync(C.seg.p, seg.data(), seg.size() * sizeof(GdrSeg), cudaMemcpyHostToDevice, s));
         TG_PROF(P_REORTH, 0, 0, gemv_t_all(0, 0, 1, 0));
-        TG_PROF(P_REORTH, 0, 0, k_gb_gemv_n_norm<<<grid, kThreads, 0, s>>>(P, 0, 0, 1, 0));
-        TG_PROF(P_SMALL, 0, 0, k_gb_finish<<<(count + 127) / 128, 128, 0, s>>>(P, count, 0, ldh, 1));
-        TG_PROF(P_SCALE, 0, 0, k_gb_scale<<<grid, kThreads, 0, s>>>(P, 0, 1));
+        TG_PROF(P_REORTH, 0, 0, launch(k_gb_gemv_n_norm, grid, kThreads, 0, s, P, 0, 0, 1, 0));
+        TG_PROF(P_SMALL, 0, 0, launch(k_gb_finish, (count + 127) / 128, 128, 0, s, P, count, 0, ldh, 1));
+        TG_PROF(P_SCALE, 0, 0, launch(k_gb_scale, grid, kThreads, 0, s, P, 0, 1));
         TG_LAUNCH_CHECK();
         for (int i = 0; i < count; ++i) active[i] = cont[i];
     }
@@ -3188,7 +3189,7 @@ static int batch_setup_all(tg_batch *b, const double *R0, int m, int k, int nev,
         TG_CHECK_CUDA(cudaMemcpyAsync(tb, Pp.data(), (size_t)count * 8, cudaMemcpyHostToDevice, s));
         TG_CHECK_CUDA(cudaMemcpyAsync(tb + (size_t)count * 8, Op.data(), (size_t)count * 8, cudaMemcpyHostToDevice, s));
         TG_CHECK_CUDA(cudaMemcpyAsync(tb + (size_t)count * 16, ldo.data(), (size_t)count * 8, cudaMemcpyHostToDevice, s));
-        TG_PROF(P_TSM, 0, 0, k_gb_tsm<double><<<grid, kThreads, 0, s>>>(
+        TG_PROF(P_TSM, 0, 0, launch(k_gb_tsm<double>, grid, kThreads, 0, s, 
             P, reinterpret_cast<const double *const *>(tb), m + 1, m, 0,
             reinterpret_cast<double *const *>(tb + (size_t)count * 8), reinterpret_cast<const size_t *>(tb + (size_t)count * 16)));
         TG_LAUNCH_CHECK();
@@ -3296,7 +3297,7 @@ extern "C" int tg_batch_setup(tg_batch *b, const void *rhs, int m, int k, int ne
         BatchInst &I = *b->inst[i];
         tg_op *op = b->ops[i];
         TG_CHECK(I.tmp.ensure((size_t)op->n * 8));
-        k_mr_extract<kBatchR><<<grid_for(op->n, 8), kThreads, 0, I.stream>>>(R0 + b->off[i], 0, op->n, I.tmp.as<double>());
+        launch(k_mr_extract<kBatchR>, grid_for(op->n, 8), kThreads, 0, I.stream, R0 + b->off[i], 0, op->n, I.tmp.as<double>());
         TG_LAUNCH_CHECK();
         tg_stats st{};
         tg_defl *d = nullptr;

@@ -86,6 +86,7 @@ __device__ __forceinline__ void mrb_final(const double *slice, int partw, double
 template <int R>
 __global__ void __launch_bounds__(kThreads) k_mrb_bi_init(const float *__restrict__ r, float *__restrict__ rh,
                                                            float *__restrict__ p, MrBatchPtrs P) {
+    pdl_wait();
     const int b = blockIdx.y;
     const MrSeg &S = P.seg[b];
     const int n = S.op.n;
@@ -132,6 +133,7 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_init(const float *__restric
 template <int R>
 __global__ void __launch_bounds__(kThreads) k_mrb_bi_v(const float *__restrict__ p, const float *__restrict__ rh,
                                                         float *__restrict__ v, MrBatchPtrs P) {
+    pdl_wait();
     const int b = blockIdx.y;
     if (P.ctl[b].active == 0) return;
     const MrSeg &S = P.seg[b];
@@ -180,6 +182,7 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_v(const float *__restrict__
 template <int R>
 __global__ void __launch_bounds__(kThreads) k_mrb_bi_s(const float *__restrict__ r, const float *__restrict__ v,
                                                         float *__restrict__ s, MrBatchPtrs P) {
+    pdl_wait();
     const int b = blockIdx.y;
     if (P.ctl[b].active == 0) return;
     const MrSeg &S = P.seg[b];
@@ -229,6 +232,7 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_s(const float *__restrict__
 template <int R>
 __global__ void __launch_bounds__(kThreads) k_mrb_bi_t(const float *__restrict__ s, const float *__restrict__ rh,
                                                         float *__restrict__ t, MrBatchPtrs P) {
+    pdl_wait();
     const int b = blockIdx.y;
     if (P.ctl[b].active == 0) return;
     const MrSeg &S = P.seg[b];
@@ -289,6 +293,7 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_x(float *__restrict__ x, fl
                                                         float *__restrict__ p, const float *__restrict__ s,
                                                         const float *__restrict__ t, const float *__restrict__ v,
                                                         MrBatchPtrs P) {
+    pdl_wait();
     const int b = blockIdx.y;
     if (P.ctl[b].active == 0) return;
     const MrSeg &S = P.seg[b];
@@ -377,6 +382,7 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_x(float *__restrict__ x, fl
 template <int R>
 __global__ void __launch_bounds__(kThreads) k_mrb_residual(const double *__restrict__ B, const double *__restrict__ X,
                                                             double *__restrict__ r64, MrBatchPtrs P) {
+    pdl_wait();
     const int b = blockIdx.y;
     const MrSeg &S = P.seg[b];
     const DevOp op = S.op;
@@ -423,6 +429,7 @@ __global__ void __launch_bounds__(kThreads) k_mrb_residual(const double *__restr
 template <int R>
 __global__ void k_mrb_scale(const double *__restrict__ r64, float *__restrict__ r32, float *__restrict__ e32,
                             MrBatchPtrs P) {
+    pdl_wait();
     const int b = blockIdx.y;
     const MrSeg &S = P.seg[b];
     const size_t tot = (size_t)S.op.n * R;
@@ -437,6 +444,7 @@ __global__ void k_mrb_scale(const double *__restrict__ r64, float *__restrict__ 
 // x64 += scale[q] e32 (columns with scale != 0).
 template <int R>
 __global__ void k_mrb_add(double *__restrict__ X, const float *__restrict__ e32, MrBatchPtrs P) {
+    pdl_wait();
     const int b = blockIdx.y;
     const MrSeg &S = P.seg[b];
     const size_t tot = (size_t)S.op.n * R;
@@ -453,6 +461,7 @@ __global__ void k_mrb_add(double *__restrict__ X, const float *__restrict__ e32,
 // the last of the instance's blocks reduces in block order.
 template <int R>
 __global__ void __launch_bounds__(kThreads) k_mrb_proj_dots(const float *__restrict__ r, MrBatchPtrs P) {
+    pdl_wait();
     constexpr int kChunk = 128;
     const int b = blockIdx.y;
     const MrSeg &S = P.seg[b];
@@ -501,6 +510,7 @@ __global__ void __launch_bounds__(kThreads) k_mrb_proj_dots(const float *__restr
 // dvec[b] = M cvec[b] (one block per instance).
 template <int R>
 __global__ void k_mrb_small(MrBatchPtrs P) {
+    pdl_wait();
     const int b = blockIdx.x;
     const MrSeg &S = P.seg[b];
     const int k = S.kk;
@@ -518,6 +528,7 @@ __global__ void k_mrb_small(MrBatchPtrs P) {
 template <int R>
 __global__ void __launch_bounds__(kThreads) k_mrb_proj_update(float *__restrict__ e, float *__restrict__ r,
                                                                MrBatchPtrs P) {
+    pdl_wait();
     const int b = blockIdx.y;
     const MrSeg &S = P.seg[b];
     const int k = S.kk, n = S.op.n;
@@ -591,6 +602,7 @@ __device__ __forceinline__ bool gdr_takes(const GdrSeg &S, int j) { return S.act
 
 // w = A v_j (float32) for the instances taking part in step j
 __global__ void __launch_bounds__(kThreads) k_gb_apply(GdrBatchPtrs P, int j) {
+    pdl_wait();
     const GdrSeg &S = P.seg[blockIdx.y];
     if (!gdr_takes(S, j)) return;
     const DevOp op = S.op;
@@ -606,6 +618,7 @@ __global__ void __launch_bounds__(kThreads) k_gb_apply(GdrBatchPtrs P, int j) {
 // Warp w owns columns w, w + 8, ...; 4 rows per lane per pass (as k_gemv_t_part).
 __global__ void __launch_bounds__(kThreads) k_gb_gemv_t(GdrBatchPtrs P, int j, int ncol_step, int reorth,
                                                          int which) {
+    pdl_wait();
     constexpr int kMaxPerWarp = 17;
     constexpr int kU = 4;
     const int b = blockIdx.y;
@@ -671,6 +684,7 @@ constexpr int kGbPipeCols = 64;
 constexpr size_t kGbPipeSmem = (size_t)3 * (kGbPipeCols + 1) * 128 * sizeof(float);
 __global__ void __launch_bounds__(kThreads, 2) k_gb_gemv_t_pipe(GdrBatchPtrs P, int j, int ncol_step, int reorth,
                                                               int which) {
+    pdl_wait();
     constexpr int R = 128, PE = 4, U = R / 32, kStages = 3, kMaxPerWarp = kGbPipeCols / 8;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float *buf = reinterpret_cast<float *>(smem_raw);
@@ -755,6 +769,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_gb_gemv_t_pipe(GdrBatchPtrs P, 
 // nrm[0] (per instance, deterministic).
 __global__ void __launch_bounds__(kThreads) k_gb_gemv_n_norm(GdrBatchPtrs P, int j, int ncol_step, int reorth,
                                                               int which) {
+    pdl_wait();
     const int b = blockIdx.y;
     const GdrSeg &S = P.seg[b];
     const bool on = reorth ? (S.active != 0) : gdr_takes(S, j);
@@ -831,6 +846,7 @@ __global__ void __launch_bounds__(kThreads) k_gb_gemv_n_norm(GdrBatchPtrs P, int
 // Hbar column j = h1 + h2 (rows 0..j), H[j+1, j] = ||w||, nrm[4] = 1 / ||w|| (one thread per
 // instance); reorth = 1: only nrm[4] (the re-orthogonalised v_kk is normalised).
 __global__ void k_gb_finish(GdrBatchPtrs P, int count, int j, int ldh, int reorth) {
+    pdl_wait();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= count) return;
     const GdrSeg &S = P.seg[b];
@@ -846,6 +862,7 @@ __global__ void k_gb_finish(GdrBatchPtrs P, int count, int j, int ldh, int reort
 
 // v *= 1 / ||w|| for column j + 1 (or kk when reorth)
 __global__ void k_gb_scale(GdrBatchPtrs P, int j, int reorth) {
+    pdl_wait();
     const GdrSeg &S = P.seg[blockIdx.y];
     const bool on = reorth ? (S.active != 0) : gdr_takes(S, j);
     if (!on) return;
@@ -856,6 +873,7 @@ __global__ void k_gb_scale(GdrBatchPtrs P, int j, int reorth) {
 
 // x_c += V[:, 0..m-1] d (coefficients of the restart step's least-squares solution)
 __global__ void __launch_bounds__(kThreads) k_gb_xc(GdrBatchPtrs P, int m) {
+    pdl_wait();
     const GdrSeg &S = P.seg[blockIdx.y];
     if (!S.active) return;
     __shared__ float ds[kSmallCols];
@@ -874,6 +892,7 @@ __global__ void __launch_bounds__(kThreads) k_gb_xc(GdrBatchPtrs P, int m) {
 template <class TO>
 __global__ void __launch_bounds__(kThreads) k_gb_tsm(GdrBatchPtrs P, const double *const *Pm, int ldp, int p,
                                                       int plus_one, TO *const *Out, const size_t *ldo) {
+    pdl_wait();
     const int b = blockIdx.y;
     const GdrSeg &S = P.seg[b];
     if (!S.active) return;

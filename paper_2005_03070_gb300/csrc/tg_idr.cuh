@@ -52,6 +52,7 @@ __global__ void __launch_bounds__(kThreads) k_idr_init(const T *__restrict__ r, 
                                                         int n, int s, double target2, int cap, double kappa,
                                                         typename ST<T>::D *part, unsigned *ticket,
                                                         IdrState<typename ST<T>::D> *st) {
+    pdl_wait();
     using D = typename ST<T>::D;
     __shared__ D red[(kThreads / 32) * (kIdrMaxS + 1)];
     __shared__ D tot[kIdrMaxS + 1];
@@ -100,6 +101,7 @@ template <class T>
 __global__ void __launch_bounds__(kThreads) k_idr_u(const T *__restrict__ r, const T *__restrict__ G, T *__restrict__ U,
                                                      size_t ld, int n, int k, int first,
                                                      const IdrState<typename ST<T>::D> *st) {
+    pdl_wait();
     using D = typename ST<T>::D;
     if (st->status != 0) return;
     __shared__ T cs[kIdrMaxS];
@@ -138,6 +140,7 @@ __global__ void __launch_bounds__(kThreads) k_idr_g(DevOp op, DevOp32 o32, const
                                                      const T *__restrict__ P, size_t ld, int k,
                                                      typename ST<T>::D *part, unsigned *ticket,
                                                      IdrState<typename ST<T>::D> *st) {
+    pdl_wait();
     using D = typename ST<T>::D;
     if (st->status != 0) return;
     __shared__ D red[(kThreads / 32) * kIdrMaxS];
@@ -192,6 +195,7 @@ template <class T>
 __global__ void __launch_bounds__(kThreads) k_idr_upd(T *__restrict__ G, T *__restrict__ U, size_t ld, T *__restrict__ r,
                                                        T *__restrict__ x, int n, int k, typename ST<T>::D *part,
                                                        unsigned *ticket, IdrState<typename ST<T>::D> *st) {
+    pdl_wait();
     using D = typename ST<T>::D;
     if (st->status != 0) return;
     __shared__ T al_s[kIdrMaxS];
@@ -236,6 +240,7 @@ template <class T>
 __global__ void __launch_bounds__(kThreads) k_idr_t(DevOp op, DevOp32 o32, const T *__restrict__ r, T *__restrict__ t,
                                                      typename ST<T>::D *part, unsigned *ticket,
                                                      IdrState<typename ST<T>::D> *st) {
+    pdl_wait();
     using D = typename ST<T>::D;
     if (st->status != 0) return;
     __shared__ D red[(kThreads / 32) * 3];
@@ -277,6 +282,7 @@ __global__ void __launch_bounds__(kThreads) k_idr_xr(T *__restrict__ x, T *__res
                                                       const T *__restrict__ P, size_t ld, int n,
                                                       typename ST<T>::D *part, unsigned *ticket,
                                                       IdrState<typename ST<T>::D> *st) {
+    pdl_wait();
     using D = typename ST<T>::D;
     if (st->status != 0) return;
     __shared__ D red[(kThreads / 32) * (kIdrMaxS + 1)];

@@ -51,6 +51,7 @@ template <> struct Part<float> { using P = float; };
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_apply(DevOp op, DevOp32 o32, const T *__restrict__ x,
                                                      T *__restrict__ y) {
+    pdl_wait();
     const int n = op.n;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
         y[i] = Apply<T>::at(op, o32, i, [&](int j) { return x[j]; });
@@ -62,6 +63,7 @@ template <class T>
 __global__ void __launch_bounds__(kThreads) k_dot(const T *__restrict__ a, const T *__restrict__ b, int n,
                                                    typename ST<T>::D *part, unsigned *ticket,
                                                    typename ST<T>::D *out) {
+    pdl_wait();
     using D = typename ST<T>::D;
     using P = typename Part<T>::P;
     __shared__ D red[(kThreads / 32) * 2];
@@ -88,6 +90,7 @@ template <class T>
 __global__ void __launch_bounds__(kThreads) k_residual(DevOp op, const T *__restrict__ b, const T *__restrict__ x,
                                                         T *__restrict__ r, typename ST<T>::D *part,
                                                         unsigned *ticket, typename ST<T>::D *out) {
+    pdl_wait();
     using D = typename ST<T>::D;
     __shared__ D red[(kThreads / 32) * 2];
     __shared__ D tot[2];
@@ -141,6 +144,7 @@ __global__ void __launch_bounds__(kThreads) k_bi_init(const T *__restrict__ r, T
                                                        T *__restrict__ p, int n, double target2, int cap,
                                                        typename ST<T>::D *part, unsigned *ticket,
                                                        BiState<typename ST<T>::D> *st) {
+    pdl_wait();
     using D = typename ST<T>::D;
     using P = typename Part<T>::P;
     __shared__ D red[(kThreads / 32)];
@@ -184,6 +188,7 @@ __global__ void __launch_bounds__(kThreads) k_bi_v(DevOp op, DevOp32 o32, const 
                                                     const T *__restrict__ rh, T *__restrict__ v,
                                                     typename ST<T>::D *part, unsigned *ticket,
                                                     BiState<typename ST<T>::D> *st) {
+    pdl_wait();
     using D = typename ST<T>::D;
     using P = typename Part<T>::P;
     if (st->status != 0) return;
@@ -214,6 +219,7 @@ template <class T>
 __global__ void __launch_bounds__(kThreads) k_bi_s(const T *__restrict__ r, const T *__restrict__ v,
                                                     T *__restrict__ s, int n, typename ST<T>::D *part,
                                                     unsigned *ticket, BiState<typename ST<T>::D> *st) {
+    pdl_wait();
     using D = typename ST<T>::D;
     using P = typename Part<T>::P;
     if (st->status != 0) return;
@@ -247,6 +253,7 @@ __global__ void __launch_bounds__(kThreads) k_bi_t(DevOp op, DevOp32 o32, const 
                                                     const T *__restrict__ rh, T *__restrict__ t,
                                                     typename ST<T>::D *part, unsigned *ticket,
                                                     BiState<typename ST<T>::D> *st) {
+    pdl_wait();
     using D = typename ST<T>::D;
     using P = typename Part<T>::P;
     if (st->status != 0 || st->half) return;
@@ -293,6 +300,7 @@ __global__ void __launch_bounds__(kThreads) k_bi_x(T *__restrict__ x, T *__restr
                                                     const T *__restrict__ s, const T *__restrict__ t,
                                                     const T *__restrict__ v, int n, typename ST<T>::D *part,
                                                     unsigned *ticket, BiState<typename ST<T>::D> *st) {
+    pdl_wait();
     using D = typename ST<T>::D;
     using P = typename Part<T>::P;
     if (st->status != 0) return;
@@ -358,6 +366,7 @@ __device__ __forceinline__ float4 ld4(const float *__restrict__ p, int a) {
 __global__ void __launch_bounds__(kThreads) k_bi_s_f4(const float *__restrict__ r, const float *__restrict__ v,
                                                        float *__restrict__ s, int n, double *part,
                                                        unsigned *ticket, BiState<double> *st) {
+    pdl_wait();
     if (st->status != 0) return;
     __shared__ double red[(kThreads / 32)];
     __shared__ double tot[1];
@@ -402,6 +411,7 @@ __global__ void __launch_bounds__(kThreads) k_bi_x_f4(float *__restrict__ x, flo
                                                        float *__restrict__ p, const float *__restrict__ s,
                                                        const float *__restrict__ t, const float *__restrict__ v,
                                                        int n, double *part, unsigned *ticket, BiState<double> *st) {
+    pdl_wait();
     if (st->status != 0) return;
     __shared__ double red[(kThreads / 32)];
     __shared__ double tot[1];
@@ -475,9 +485,9 @@ constexpr int kGemvTCols = 136;          // 8 warps x 17 columns
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_gemv_t_part(const T *__restrict__ V, size_t ldv, int ncol,
                                                            const T *__restrict__ w, int n,
-                                                           typename ST<T>::D *part, const int *cond = nullptr) {
+                                                           typename ST<T>::D *part) {
+    pdl_wait();
     using P = typename Part<T>::P;
-    if (cond && !*cond) return;     // a skipped re-orthogonalisation pass
     constexpr int kMaxPerWarp = kGemvTCols / 8;
     constexpr int kU = 4;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -542,6 +552,7 @@ template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile(
 template <class E>
 __global__ void __launch_bounds__(kThreads, 2) k_gemv_t_pipe(const E *__restrict__ V, size_t ldv, int ncol,
                                                            const E *__restrict__ w, int n, double *part) {
+    pdl_wait();
     constexpr int kMaxPerWarp = kPipeCols / 8;
     constexpr int R = PipeRows<E>::value;
     constexpr int PE = 16 / sizeof(E);           // elements per 16-byte piece
@@ -613,15 +624,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_gemv_t_pipe(const E *__restrict
 // out[e] (mode 0: =, mode 1: +=) sum_b part[b * nent + e].  One warp per entry: lane l
 // adds blocks l, l + 32, ... in order, then the fixed shuffle tree (deterministic).
 template <class D>
-__global__ void k_sum_part(const D *__restrict__ part, int nblk, int nent, D *out, int mode,
-                           const int *cond = nullptr) {
+__global__ void k_sum_part(const D *__restrict__ part, int nblk, int nent, D *out, int mode) {
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (e >= nent) return;
-    if (cond && !*cond) {           // skipped pass: its coefficients are zero
-        if (lane == 0 && !mode) out[e] = D{};
-        return;
-    }
     D s = D{};
     for (int b = lane; b < nblk; b += 32) s = dadd(s, part[(size_t)b * nent + e]);
     s = warp_sum(s);
@@ -636,6 +643,7 @@ template <class T, int MC = kMaxCols>
 __global__ void __launch_bounds__(kThreads) k_gemv_n(const T *__restrict__ V, size_t ldv, int ncol,
                                                       const typename ST<T>::D *__restrict__ h, double sign,
                                                       T *__restrict__ w, int n) {
+    pdl_wait();
     // coefficients converted to the vector type once per block (a per-element float64 ->
     // float32 conversion would run on the float64 pipe)
     __shared__ T hs[MC];
@@ -661,6 +669,7 @@ __global__ void __launch_bounds__(kThreads) k_gemv_n_norm(const T *__restrict__ 
                                                            double *nrm2_out,
                                                            const typename ST<T>::D *nrm2_before,
                                                            int *flag_out, double eta2) {
+    pdl_wait();
     using D = typename ST<T>::D;
     using P = typename Part<T>::P;
     if (cond && !*cond) return;
@@ -696,6 +705,7 @@ __global__ void __launch_bounds__(kThreads) k_gemv_n_norm_f4(const float *__rest
                                                               const double *__restrict__ h, float *__restrict__ w,
                                                               int n, double *part, unsigned *ticket,
                                                               double *nrm2_out) {
+    pdl_wait();
     __shared__ float hs[MC];
     __shared__ double red[(kThreads / 32)];
     __shared__ double tot[1];
@@ -740,6 +750,7 @@ template <class TO, int CPT>
 __global__ void __launch_bounds__(kThreads) k_tsm_f(const float *__restrict__ In, size_t ldi, int p,
                                                      const double *__restrict__ S, int lds, int q,
                                                      TO *__restrict__ Out, size_t ldo, int n) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float *tiles = reinterpret_cast<float *>(smem_raw);         // 2 x [p][64]
     float *Ss = tiles + (size_t)2 * p * 64;                     // [q][p]
@@ -812,6 +823,7 @@ __global__ void __launch_bounds__(kThreads) k_tsm_f(const float *__restrict__ In
 template <class T, class HT = T>
 __global__ void k_arnoldi_finish2(const typename ST<T>::D *h1, const typename ST<T>::D *h2, const double *nrm2,
                                   int j, HT *Hcol, double *inv) {
+    pdl_wait();
     for (int i = threadIdx.x; i <= j; i += blockDim.x) Hcol[i] = dadd(h1[i], h2[i]);
     if (threadIdx.x == 0) {
         const double nn = sqrt(nrm2[0]);
@@ -829,6 +841,7 @@ __global__ void __launch_bounds__(kThreads) k_proj_update(const T *__restrict__ 
                                                            const typename ST<T>::D *__restrict__ d,
                                                            const typename ST<T>::D *__restrict__ e,
                                                            T *__restrict__ x, T *__restrict__ r, int n) {
+    pdl_wait();
     __shared__ T ds[MC], es[MC];   // in the vector type, converted once per block
     for (int c = threadIdx.x; c < k; c += blockDim.x) {
         ds[c] = KS<T>::of(d[c]);
@@ -852,6 +865,7 @@ template <class T>
 __global__ void __launch_bounds__(kThreads) k_tsm(const T *__restrict__ In, size_t ldi, int p,
                                                    const T *__restrict__ S, int lds, int q,
                                                    T *__restrict__ Out, size_t ldo, int n) {
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *tile = reinterpret_cast<T *>(smem_raw);
     for (int row0 = blockIdx.x * 32; row0 < n; row0 += gridDim.x * 32) {
@@ -885,6 +899,7 @@ template <class T, int EPT>
 __global__ void __launch_bounds__(kThreads) k_gram_packed(const T *__restrict__ A, const T *__restrict__ B,
                                                            size_t ld, int k, int n, int sym, int nent,
                                                            typename ST<T>::D *part, int kb) {
+    pdl_wait();
     using D = typename ST<T>::D;
     constexpr int kS = 33;                   // staged row stride (elements)
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -949,6 +964,7 @@ __device__ __forceinline__ double dconj(double a) { return a; }
 __device__ __forceinline__ cplx dconj(cplx a) { return conj(a); }
 template <class D>
 __global__ void k_gram_unpack(const D *__restrict__ packed, int k, int sym, D *G, int kb) {
+    pdl_wait();
     const int nent = sym ? k * (k + 1) / 2 : k * kb;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nent; e += gridDim.x * blockDim.x) {
         int i, j;
@@ -974,6 +990,7 @@ __device__ __forceinline__ cplx scal(double s, cplx a) { return s * a; }
 
 template <class T>
 __global__ void k_scale_by(T *__restrict__ w, int n, const double *__restrict__ inv) {
+    pdl_wait();
     // w *= inv[0]
     const double s = inv[0];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) w[i] = scal(s, w[i]);
@@ -984,6 +1001,7 @@ __global__ void k_scale_by(T *__restrict__ w, int n, const double *__restrict__ 
 template <class T>
 __global__ void k_arnoldi_finish(const typename ST<T>::D *h1, const typename ST<T>::D *h2,
                                  const typename ST<T>::D *nrm2, int j, T *Hcol, double *inv) {
+    pdl_wait();
     for (int i = threadIdx.x; i <= j; i += blockDim.x) Hcol[i] = dadd(h1[i], h2[i]);
     if (threadIdx.x == 0) {
         const double nn = sqrt(dreal(nrm2[0]));
@@ -1024,6 +1042,7 @@ __host__ __device__ __forceinline__ int pad_tiles(int N) {
 
 // in (N^3, x fastest) -> outp (padded, zero padding)
 __global__ void k_pad3d(const float *__restrict__ in, float *__restrict__ outp, int N) {
+    pdl_wait();
     const unsigned P = (unsigned)pad_pitch(N), n = P * (unsigned)N * (unsigned)N;
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const unsigned x = i % P, row = i / P;
@@ -1033,6 +1052,7 @@ __global__ void k_pad3d(const float *__restrict__ in, float *__restrict__ outp, 
 
 // inp (padded) -> out (N^3)
 __global__ void k_unpad3d(const float *__restrict__ inp, float *__restrict__ out, int N) {
+    pdl_wait();
     const unsigned P = (unsigned)pad_pitch(N), n = (unsigned)N * (unsigned)N * (unsigned)N;
     for (unsigned j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
         const unsigned x = j % (unsigned)N, row = j / (unsigned)N;
@@ -1062,6 +1082,7 @@ __global__ void __launch_bounds__(32 * kPadRows, 2) k_bi_pad(DevOp op, DevOp32 o
                                                              const float *__restrict__ rh, float *__restrict__ out,
                                                              double *part, unsigned *ticket, BiState<double> *st,
                                                              int zlen) {
+    pdl_wait();
     if (st->status != 0) return;
     if (MODE == 1 && st->half) return;
     constexpr int ND = MODE == 0 ? 1 : 4;

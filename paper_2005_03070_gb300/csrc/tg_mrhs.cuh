@@ -87,6 +87,7 @@ struct MrCtl {
 // column q of an interleaved n x R float64 block, as a plain vector
 template <int R>
 __global__ void k_mr_extract(const double *__restrict__ src, int q, int n, double *__restrict__ dst) {
+    pdl_wait();
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) dst[j] = src[(size_t)j * R + q];
 }
 

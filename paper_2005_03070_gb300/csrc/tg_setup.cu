@@ -17,6 +17,7 @@ namespace tg {
 // coef[5][n] for A (sgn = +1) or A^T (sgn = -1): diag, west, east, south, north.
 __global__ void k_vark_coefs(const double *__restrict__ kappa, int N, double beta, int sgn,
                              double *__restrict__ coef, float *__restrict__ coef32) {
+    pdl_wait();
     const int n = N * N;
     const double h = 1.0 / (N + 1);
     const double s = 0.5 / (h * h);
@@ -44,6 +45,7 @@ __global__ void k_vark_coefs(const double *__restrict__ kappa, int N, double bet
 // flips (A = D_a L + C with L symmetric and C antisymmetric, so A^T = L D_a - C).
 __global__ void k_exp2d_coefs(int N, double bx, double by, double gamma, double shift, int transpose,
                               double *__restrict__ coef, float *__restrict__ coef32) {
+    pdl_wait();
     const int n = N * N;
     const double h = 1.0 / (N + 1);
     const double ih2 = 1.0 / (h * h);
@@ -74,6 +76,7 @@ __global__ void k_exp2d_coefs(int N, double bx, double by, double gamma, double 
 
 // kappa_c(I, J) = kappa(2I, 2J) on the coarse (Nc+2)^2 node grid.
 __global__ void k_inject_kappa(const double *__restrict__ kappa, int N, double *__restrict__ kc) {
+    pdl_wait();
     const int Nc = (N - 1) / 2;
     const int NPc = Nc + 2, NP = N + 2;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < NPc * NPc; e += gridDim.x * blockDim.x) {
@@ -91,6 +94,7 @@ __device__ __forceinline__ cplx cmul_nofma(cplx a, cplx b) {
 // pw[x] = (1/4) conj(W(x)), W(x) the product of links along the path from the block
 // corner 2X to x, one step in each mu = 0, 1, 2, 3 with delta_mu = 1.
 __global__ void k_lattice_weights(const cplx *__restrict__ links, int L, cplx *__restrict__ pw) {
+    pdl_wait();
     const int V = L * L * L * L;
     for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < V; x += gridDim.x * blockDim.x) {
         int c[4] = {x % L, (x / L) % L, (x / (L * L)) % L, x / (L * L * L)};
@@ -113,6 +117,7 @@ __device__ __forceinline__ int site_of(const int c[4], int L) { return c[0] + L 
 // cst[5+mu][X] = A_c[X, X-mu].  Sums over the 16 block sites in order delta = 0..15.
 __global__ void k_lattice_coarse(const cplx *__restrict__ links, const cplx *__restrict__ pw, int L,
                                  double mdiag, cplx *__restrict__ cst) {
+    pdl_wait();
     const int Lc = L / 2;
     const int V = L * L * L * L, Vc = Lc * Lc * Lc * Lc;
     for (int X = blockIdx.x * blockDim.x + threadIdx.x; X < Vc; X += gridDim.x * blockDim.x) {
@@ -152,6 +157,7 @@ __device__ __forceinline__ double cval2(const double *uc, int Nc, int I, int J) 
 
 // Bilinear prolongation of one column (fine 1-based (i, j); coarse I, J).
 __global__ void k_prolong2d(const double *__restrict__ uc, int Nc, double *__restrict__ uf) {
+    pdl_wait();
     const int N = 2 * Nc + 1;
     const int n = N * N;
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x) {
@@ -176,6 +182,7 @@ __device__ __forceinline__ double cval3(const double *uc, int Nc, int I, int J, 
 
 // Trilinear prolongation: pairs along x, then y, then z; weight 2^-(px+py+pz) last.
 __global__ void k_prolong3d(const double *__restrict__ uc, int Nc, double *__restrict__ uf) {
+    pdl_wait();
     const int N = 2 * Nc + 1;
     const int n = N * N * N;
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x) {
@@ -241,6 +248,7 @@ __device__ __forceinline__ double cub_sum(const double (&v)[4]) {
 __device__ __forceinline__ double cub_term(double sgn, double u) { return sgn == 0.0 ? 0.0 : (sgn < 0.0 ? -u : u); }
 
 __global__ void k_prolong2d_cubic(const double *__restrict__ uc, int Nc, double *__restrict__ uf) {
+    pdl_wait();
     const int N = 2 * Nc + 1;
     const int n = N * N;
     for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < n; idx += gridDim.x * blockDim.x) {
@@ -270,6 +278,7 @@ __global__ void k_prolong2d_cubic(const double *__restrict__ uc, int Nc, double 
 }
 
 __global__ void k_prolong3d_cubic(const double *__restrict__ uc, int Nc, double *__restrict__ uf) {
+    pdl_wait();
     const int N = 2 * Nc + 1;
     const int64_t n = (int64_t)N * N * N;
     for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < n; idx += (int64_t)gridDim.x * blockDim.x) {
@@ -304,6 +313,7 @@ __global__ void k_prolong3d_cubic(const double *__restrict__ uc, int Nc, double 
 
 // Full weighting: uc(I, J) = (1/4) sum_f P[f, (I,J)] uf(f) (weights 1, 1/2, 1/4).
 __global__ void k_restrict2d(const double *__restrict__ uf, int N, double *__restrict__ uc) {
+    pdl_wait();
     const int Nc = (N - 1) / 2;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < Nc * Nc; e += gridDim.x * blockDim.x) {
         const int I = e % Nc + 1, J = e / Nc + 1;
@@ -319,6 +329,7 @@ __global__ void k_restrict2d(const double *__restrict__ uf, int N, double *__res
 }
 
 __global__ void k_restrict3d(const double *__restrict__ uf, int N, double *__restrict__ uc) {
+    pdl_wait();
     const int Nc = (N - 1) / 2;
     const int nc = Nc * Nc * Nc;
     for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nc; e += gridDim.x * blockDim.x) {
@@ -337,6 +348,7 @@ __global__ void k_restrict3d(const double *__restrict__ uf, int N, double *__res
 
 __global__ void k_prolong_lattice(const cplx *__restrict__ uc, const cplx *__restrict__ pw, int L,
                                   cplx *__restrict__ uf) {
+    pdl_wait();
     const int V = L * L * L * L, Lc = L / 2;
     for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < V; x += gridDim.x * blockDim.x) {
         const int c0 = x % L, c1 = (x / L) % L, c2 = (x / (L * L)) % L, c3 = x / (L * L * L);
@@ -347,6 +359,7 @@ __global__ void k_prolong_lattice(const cplx *__restrict__ uc, const cplx *__res
 
 __global__ void k_restrict_lattice(const cplx *__restrict__ uf, const cplx *__restrict__ pw, int L,
                                    cplx *__restrict__ uc) {
+    pdl_wait();
     const int Lc = L / 2, Vc = Lc * Lc * Lc * Lc;
     for (int X = blockIdx.x * blockDim.x + threadIdx.x; X < Vc; X += gridDim.x * blockDim.x) {
         const int C[4] = {X % Lc, (X / Lc) % Lc, (X / (Lc * Lc)) % Lc, X / (Lc * Lc * Lc)};
@@ -366,6 +379,7 @@ __global__ void k_restrict_lattice(const cplx *__restrict__ uf, const cplx *__re
 // (lam = x = 0 on boundary nodes; faces with both nodes on the boundary contribute 0).
 __global__ void k_kappa_grad(const double *__restrict__ x, const double *__restrict__ lam, int N,
                              double *__restrict__ g) {
+    pdl_wait();
     const int NP = N + 2;
     const double h = 1.0 / (N + 1);
     const double s = -0.5 / (h * h);
@@ -387,24 +401,29 @@ __global__ void k_kappa_grad(const double *__restrict__ x, const double *__restr
 }
 
 __global__ void k_inv_sqrt(const double *in, double *out) {
+    pdl_wait();
     if (threadIdx.x == 0 && blockIdx.x == 0) out[0] = in[0] > 0 ? 1.0 / sqrt(in[0]) : 0.0;
 }
 
 // ----------------------------------------------------------------------------- conversions
 __global__ void k_d2f_scaled(const double *__restrict__ a, float *__restrict__ b, int n, double s) {
+    pdl_wait();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) b[i] = (float)(a[i] * s);
 }
 __global__ void k_add_f2d_scaled(double *__restrict__ x, const float *__restrict__ e, int n, double s) {
+    pdl_wait();
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) x[i] = fma(s, (double)e[i], x[i]);
 }
 __global__ void k_d2f(const double *__restrict__ a, float *__restrict__ b, size_t n) {
+    pdl_wait();
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
         b[i] = (float)a[i];
 }
 
 // ----------------------------------------------------------------------------- launchers
+#define TG_ARGS(...) __VA_ARGS__
 #define TG_L(name, params, args) \
-    void launch_##name params { k_##name<<<grid, kThreads, 0, s>>> args; }
+    void launch_##name params { launch(k_##name, grid, kThreads, 0, s, TG_ARGS args); }
 TG_L(vark_coefs, (int grid, cudaStream_t s, const double *kappa, int N, double beta, int sgn, double *coef, float *coef32),
      (kappa, N, beta, sgn, coef, coef32))
 TG_L(exp2d_coefs, (int grid, cudaStream_t s, int N, double bx, double by, double gamma, double shift, int transpose,
@@ -426,6 +445,7 @@ TG_L(d2f_scaled, (int grid, cudaStream_t s, const double *a, float *b, int n, do
 TG_L(add_f2d_scaled, (int grid, cudaStream_t s, double *x, const float *e, int n, double sc), (x, e, n, sc))
 TG_L(d2f, (int grid, cudaStream_t s, const double *a, float *b, size_t n), (a, b, n))
 #undef TG_L
-void launch_inv_sqrt(cudaStream_t s, const double *in, double *out) { k_inv_sqrt<<<1, 1, 0, s>>>(in, out); }
+#undef TG_ARGS
+void launch_inv_sqrt(cudaStream_t s, const double *in, double *out) { launch(k_inv_sqrt, 1, 1, 0, s, in, out); }
 
 }  // namespace tg

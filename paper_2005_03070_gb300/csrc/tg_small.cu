@@ -812,6 +812,7 @@ __device__ bool ritz_less_m(double ma, double ar, double ai, double mb, double b
 // Rinv = R^{-1}.  info[0] = 0 on success, j+1 if the j-th pivot is not positive.
 template <class D>
 __global__ void k_chol_inv(const D *G, int k, D *R, D *Rinv, int *info) {
+    pdl_wait();
     __shared__ int bad;
     if (threadIdx.x == 0) bad = 0;
     for (int e = threadIdx.x; e < k * k; e += blockDim.x) {
@@ -852,6 +853,7 @@ __global__ void k_chol_inv(const D *G, int k, D *R, D *Rinv, int *info) {
 // 2 k^2).  info[0] = 0, or j+1 for a zero pivot.
 template <class D>
 __global__ void k_inverse(const D *H, int k, D *Hinv, D *W, int *info) {
+    pdl_wait();
     __shared__ int p_s, bad;
     D *A = W;
     D *B = W + (size_t)k * k;
@@ -905,6 +907,7 @@ __global__ void k_inverse(const D *H, int k, D *Hinv, D *W, int *info) {
 // out = M c (k x k times k), one thread per row.
 template <class D>
 __global__ void k_small_gemv(const D *M, int k, const D *c, D *out) {
+    pdl_wait();
     for (int i = threadIdx.x; i < k; i += blockDim.x) {
         D s = Cx<D>::zero();
         for (int j = 0; j < k; ++j) s = add(s, Cx<D>::mul(M[i + (size_t)j * k], c[j]));
@@ -1302,6 +1305,7 @@ __device__ __forceinline__ void gmresdr_restart_body(const GdrArgs<T> &a) {
 
 template <class T>
 __global__ void __launch_bounds__(kGdrThreads) k_gmresdr_restart(GdrArgs<T> a) {
+    pdl_wait();
     gmresdr_restart_body<T>(a);
 }
 
@@ -1309,6 +1313,7 @@ __global__ void __launch_bounds__(kGdrThreads) k_gmresdr_restart(GdrArgs<T> a) {
 // args[b] when active[b] is set
 template <class T>
 __global__ void __launch_bounds__(kGdrThreads) k_gmresdr_restart_batch(const GdrArgs<T> *args, const int *active) {
+    pdl_wait();
     if (!active[blockIdx.x]) return;
     const GdrArgs<T> a = args[blockIdx.x];
     gmresdr_restart_body<T>(a);
@@ -1320,6 +1325,7 @@ __global__ void __launch_bounds__(kGdrThreads) k_gmresdr_restart_batch(const Gdr
 // updated; state->resid = |g[j+1]|; state->done = 1 when resid <= target or h[j,j] = 0.
 template <class D>
 __global__ void k_givens_step(D *H, int ldh, int j, D *cs, D *sn, D *g, GivensState *state) {
+    pdl_wait();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     if (state->done) return;
     D *h = H + (size_t)j * ldh;
@@ -1350,6 +1356,7 @@ __global__ void k_givens_step(D *H, int ldh, int j, D *cs, D *sn, D *g, GivensSt
 // y = R^{-1} g[0..kj-1] for the rotated (upper triangular) Hessenberg.
 template <class D>
 __global__ void k_givens_solve(const D *H, int ldh, const D *g, D *y, const GivensState *state) {
+    pdl_wait();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     const int kj = state->steps;
     for (int i = kj - 1; i >= 0; --i) {
@@ -1363,15 +1370,15 @@ __global__ void k_givens_solve(const D *H, int ldh, const D *g, D *y, const Give
 // ----------------------------------------------------------------------------- launchers
 template <class D>
 void launch_chol_inv(const D *G, int k, D *R, D *Rinv, int *info, cudaStream_t s) {
-    k_chol_inv<D><<<1, kSmallThreads, 0, s>>>(G, k, R, Rinv, info);
+    launch(k_chol_inv<D>, 1, kSmallThreads, 0, s, G, k, R, Rinv, info);
 }
 template <class D>
 void launch_inverse(const D *H, int k, D *Hinv, D *W, int *info, cudaStream_t s) {
-    k_inverse<D><<<1, kSmallThreads, 0, s>>>(H, k, Hinv, W, info);
+    launch(k_inverse<D>, 1, kSmallThreads, 0, s, H, k, Hinv, W, info);
 }
 template <class D>
 void launch_small_gemv(const D *M, int k, const D *c, D *out, cudaStream_t s) {
-    k_small_gemv<D><<<1, kSmallThreads, 0, s>>>(M, k, c, out);
+    launch(k_small_gemv<D>, 1, kSmallThreads, 0, s, M, k, c, out);
 }
 template <class T>
 cudaError_t launch_gmresdr_restart(const GdrArgs<T> &a_in, cudaStream_t s) {
@@ -1391,7 +1398,7 @@ cudaError_t launch_gmresdr_restart(const GdrArgs<T> &a_in, cudaStream_t s) {
         const cudaError_t e = smem_attr_once((const void *)k_gmresdr_restart<T>, (int)kGdrSmemMax);
         if (e != cudaSuccess) return e;
     }
-    k_gmresdr_restart<T><<<1, kGdrThreads, smem, s>>>(a);
+    launch(k_gmresdr_restart<T>, 1, kGdrThreads, smem, s, a);
     return cudaGetLastError();
 }
 template <class T>
@@ -1414,16 +1421,16 @@ cudaError_t launch_gmresdr_restart_batch(const GdrArgs<T> *args, const int *acti
         const cudaError_t e = smem_attr_once((const void *)k_gmresdr_restart_batch<T>, (int)kGdrSmemMax);
         if (e != cudaSuccess) return e;
     }
-    k_gmresdr_restart_batch<T><<<count, kGdrThreads, smem, s>>>(args, active);
+    launch(k_gmresdr_restart_batch<T>, count, kGdrThreads, smem, s, args, active);
     return cudaGetLastError();
 }
 template <class D>
 void launch_givens_step(D *H, int ldh, int j, D *cs, D *sn, D *g, GivensState *state, cudaStream_t s) {
-    k_givens_step<D><<<1, 1, 0, s>>>(H, ldh, j, cs, sn, g, state);
+    launch(k_givens_step<D>, 1, 1, 0, s, H, ldh, j, cs, sn, g, state);
 }
 template <class D>
 void launch_givens_solve(const D *H, int ldh, const D *g, D *y, const GivensState *state, cudaStream_t s) {
-    k_givens_solve<D><<<1, 1, 0, s>>>(H, ldh, g, y, state);
+    launch(k_givens_solve<D>, 1, 1, 0, s, H, ldh, g, y, state);
 }
 
 #define TG_INST(D)                                                                                   \
