@@ -19,6 +19,7 @@
 #include "tg_idr.cuh"
 #include "tg_kernels.cuh"
 #include "tg_mrhs.cuh"
+#include "tg_split.cuh"
 #include "tg_batch.cuh"
 #include "tg_setup.cuh"
 #include "tg_small.cuh"
@@ -366,9 +367,9 @@ static int max_dyn_smem() {
 }
 
 template <class T>
-static int set_smem(const void *fn, size_t bytes) {
+static int set_smem(const void *fn, size_t bytes, int less = 0) {      // less: room for static shared memory
     if (bytes > 48 * 1024) {
-        const int mx = max_dyn_smem();
+        const int mx = max_dyn_smem() + less;
         if ((int)bytes > mx) {
             set_error("a launch needs %zu bytes of shared memory, more than the %d available", bytes, mx);
             return TG_BAD_ARG;
@@ -378,9 +379,63 @@ static int set_smem(const void *fn, size_t bytes) {
     return TG_OK;
 }
 
+// The tensor-core split serves products over at least this many rows: below, a launch is a few
+// microseconds either way and the plain kernels, which convert nothing, are not slower.
+constexpr int kSplitMinRows = 4096;
+
+// The launch shape of k_tsm_split for Out (n x q) = In (n x p) S, or wr = 0 when it does not fit.
+// Of the row / column warp splits and buffer counts whose tile and digits of S fit in shared
+// memory, the one with the fewest 16-column passes per row; in place needs all columns in one
+// block.
+template <class T>
+static TsmSplitCfg tsm_split_cfg(int p, int q, bool in_place) {
+    const int f = sizeof(T) == 16 ? 2 : 1, KT = split_kt(f * p), CT = (f * q + 7) / 8;
+    const int64_t room = max_dyn_smem() - 2048;      // the kernel's static shared memory
+    TsmSplitCfg best{0, 0, 0, 0};
+    double cost = 1e300;
+    for (int wr : {8, 4, 2})
+        for (int nbuf : {2, 1}) {
+            const int64_t tile = (int64_t)nbuf * split_pc<T>(p) * (16 * wr + 2) * sizeof(T), per = (int64_t)KT * kSplitDigits * 256;
+            const int ctb = (int)std::min<int64_t>(std::min(CT, 32), (room - tile) / per);
+            if (room < tile || ctb < 1 || (in_place && ctb < CT)) continue;
+            const int wc = kTsmWarps / wr, gy = (CT + ctb - 1) / ctb;
+            const int passes = ((ctb + kTsmCt - 1) / kTsmCt + wc - 1) / wc;
+            const double c = (double)gy * passes / wr * (nbuf == 2 ? 1.0 : 1.3);
+            if (c < cost) {
+                cost = c;
+                best = TsmSplitCfg{wr, nbuf, ctb, (size_t)(tile + ctb * per)};
+            }
+        }
+    return best;
+}
+
+template <class T, int WR>
+static int tsm_split(const TsmSplitCfg &c, const T *In, size_t ldi, int p, const T *S, int lds, int q, T *Out,
+                     size_t ldo, int n, cudaStream_t s) {
+    TG_CHECK(set_smem<T>((const void *)k_tsm_split<T, WR>, c.smem, -2048));
+    const int f = sizeof(T) == 16 ? 2 : 1, CT = (f * q + 7) / 8;
+    const int gy = (CT + c.ctb - 1) / c.ctb, tiles = (n + 16 * WR - 1) / (16 * WR);
+    const int gx = std::max(1, std::min(tiles, std::max(1, num_sms() / gy)));
+    launch(k_tsm_split<T, WR>, dim3(gx, gy), kTsmThreads, c.smem, s, In, ldi, p, S, lds, q, Out, ldo, n, c.ctb, c.nbuf);
+    return TG_OK;
+}
+
 // Out (n x q) = In (n x p) S (p x q)
 template <class T>
 static int tsm(const T *In, size_t ldi, int p, const T *S, int lds, int q, T *Out, size_t ldo, int n, cudaStream_t s) {
+    if (n >= kSplitMinRows && q >= 4) {
+        const TsmSplitCfg c = tsm_split_cfg<T>(p, q, In == Out);
+        if (c.wr) {
+            int rc = TG_OK;
+            TG_PROF(P_TSM, (double)(p + q) * n * sizeof(T), 2.0 * p * q * n * (sizeof(T) == 16 ? 4 : 1),
+                    rc = c.wr == 8   ? tsm_split<T, 8>(c, In, ldi, p, S, lds, q, Out, ldo, n, s)
+                         : c.wr == 4 ? tsm_split<T, 4>(c, In, ldi, p, S, lds, q, Out, ldo, n, s)
+                                     : tsm_split<T, 2>(c, In, ldi, p, S, lds, q, Out, ldo, n, s));
+            TG_CHECK(rc);
+            TG_LAUNCH_CHECK();
+            return TG_OK;
+        }
+    }
     size_t smem = (size_t)32 * p * sizeof(T);
     TG_CHECK(set_smem<T>((const void *)k_tsm<T>, smem));
     TG_PROF(P_TSM, (double)(p + q) * n * sizeof(T), 2.0 * p * q * n * (sizeof(T) == 16 ? 4 : 1), launch(k_tsm<T>, tiles_grid(n, 4), kThreads, smem, s, In, ldi, p, S, lds, q, Out, ldo, n));
@@ -501,12 +556,41 @@ static int gram_ept(tg_op *op, const T *A, const T *B, size_t ld, int k, int n, 
     return TG_OK;
 }
 
+// The same on the tensor cores (k_gram_split): panels of 32 real columns, one panel pair per
+// grid y.
+template <class T>
+static int gram_split(tg_op *op, const T *A, const T *B, size_t ld, int k, int n, int sym, typename ST<T>::D *G,
+                      cudaStream_t s, int kb) {
+    using D = typename ST<T>::D;
+    const int f = sizeof(T) == 16 ? 2 : 1;
+    const int nent = sym ? k * (k + 1) / 2 : k * kb;
+    const int npi = (f * k + kGramPanel - 1) / kGramPanel, npj = (f * kb + kGramPanel - 1) / kGramPanel;
+    const int gy = sym ? npi * (npi + 1) / 2 : npi * npj;
+    const bool one = A == B && npi == 1 && npj == 1;
+    const size_t smem = (size_t)(one ? 1 : 2) * kSplitDigits * kGramPanel * kGramStride * 2;
+    const int pieces = (n + kGramRows - 1) / kGramRows;
+    const int gx = std::max(1, std::min(pieces, num_sms() * (one ? 2 : 1) / gy));
+    TG_CHECK(red_ready(op, (size_t)gx * nent * sizeof(D) + (size_t)nent * sizeof(D), s));
+    D *part = wsp<D>(op, S_PART);
+    D *packed = part + (size_t)gx * nent;
+    TG_CHECK(set_smem<T>((const void *)k_gram_split<T>, smem, -2048));
+    TG_PROF(P_GRAM, (A == B ? 1.0 * k : 1.0 * (k + kb)) * n * sizeof(T), 2.0 * nent * n * (sizeof(T) == 16 ? 4 : 1),
+            launch(k_gram_split<T>, dim3(gx, gy), kThreads, smem, s, A, B, ld, k, kb, n, sym, npi, nent, part));
+    TG_LAUNCH_CHECK();
+    TG_PROF(P_SUM_PART, (double)gx * nent * sizeof(D), (double)gx * nent,
+            launch(k_sum_part<D>, (nent + 7) / 8, 256, 0, s, part, gx, nent, packed, 0));
+    TG_PROF(P_SMALL, 0, 0, launch(k_gram_unpack<D>, (nent + 255) / 256, 256, 0, s, packed, k, sym, G, kb));
+    TG_LAUNCH_CHECK();
+    return TG_OK;
+}
+
 // G = A^H B: A has k columns, B has kb columns (kb < 0: kb = k); sym requires B = A.
 template <class T>
 static int gram(tg_op *op, const T *A, const T *B, size_t ld, int k, int n, int sym, typename ST<T>::D *G,
                 cudaStream_t s, int kb = -1) {
     if (kb < 0) kb = k;
     const int nent = sym ? k * (k + 1) / 2 : k * kb;
+    if (n >= kSplitMinRows && nent >= 16) return gram_split<T>(op, A, B, ld, k, n, sym, G, s, kb);
     if (nent <= kThreads) return gram_ept<T, 1>(op, A, B, ld, k, n, sym, G, s, kb);
     if (nent <= 2 * kThreads) return gram_ept<T, 2>(op, A, B, ld, k, n, sym, G, s, kb);
     if (nent <= 4 * kThreads) return gram_ept<T, 4>(op, A, B, ld, k, n, sym, G, s, kb);
