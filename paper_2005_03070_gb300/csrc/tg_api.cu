@@ -16,6 +16,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "tg_arnoldi.cuh"
 #include "tg_idr.cuh"
 #include "tg_kernels.cuh"
 #include "tg_mrhs.cuh"
@@ -291,10 +292,11 @@ struct SmallArea {
     static constexpr size_t idr = 4096;         // IdrState
     static constexpr size_t proj_c = 8192;      // projection coefficients c
     static constexpr size_t proj_d = 16384;     // projection coefficients d
-    static constexpr size_t arn_h1 = 24576;     // Arnoldi: V^H w, first pass (and ||w||^2)
-    static constexpr size_t arn_h2 = 32768;     // Arnoldi: second pass
-    static constexpr size_t arn_nrm = 40960;    // ||w||^2, 1 / ||w|| (+ 32), re-orthogonalisation flag (+ 64)
+    static constexpr size_t arn_h1 = 24576;     // V^H w, first pass; Arnoldi: s
+    static constexpr size_t arn_h2 = 32768;     // second pass; Arnoldi: z
+    static constexpr size_t arn_nrm = 40960;    // ||w||^2, 1 / ||w|| (+ 32); Arnoldi: beta, 1 / beta, t (+ 64)
     static constexpr size_t gmres_inv = 41984;  // 1 / ||r|| of a GMRES cycle
+    static constexpr size_t arn_c = 49152;      // Arnoldi: first-pass coefficients h1
     static constexpr size_t bytes = 1 << 16;
 };
 static_assert(kMaxCols * 16 <= 8192, "coefficient vectors must fit their slots");
@@ -305,8 +307,8 @@ static_assert(kMaxCols * 16 <= 8192, "coefficient vectors must fit their slots")
 static int red_ready(tg_op *op, size_t part_bytes, cudaStream_t s) {
     TG_CHECK(wsx(op, S_PART, part_bytes < (4 << 20) ? (4 << 20) : part_bytes));
     if (!op->ws[S_TICKET].p) {
-        TG_CHECK(wsx(op, S_TICKET, 64));
-        TG_CHECK_CUDA(cudaMemsetAsync(op->ws[S_TICKET].p, 0, 64, s));
+        TG_CHECK(wsx(op, S_TICKET, kArnTickets * sizeof(unsigned)));
+        TG_CHECK_CUDA(cudaMemsetAsync(op->ws[S_TICKET].p, 0, kArnTickets * sizeof(unsigned), s));
     }
     TG_CHECK(wsx(op, S_SMALL, SmallArea::bytes));
     TG_CHECK(op->pin.ensure(1 << 16));
@@ -1631,71 +1633,113 @@ static int solve_idr_ir(tg_op *op, const tg_defl *df, const double *b, double *x
     return status;
 }
 
-// ----------------------------------------------------------------------------- Arnoldi (CGS2)
-// Extends V (ld ldv, columns 0..j orthonormal) by column j+1 = A v_j orthogonalised; writes
-// Hbar column j (ld ldh).  Two classical Gram-Schmidt passes as tall-skinny products.
-// w -= V h and ||w||^2 (k_gemv_n_norm), with the float4 kernel for an aligned float32 basis
-// (its rows in groups of 4; no re-orthogonalisation flag, which no caller reads there)
+// ----------------------------------------------------------------------------- Arnoldi
+// w -= V h and ||w||^2 (k_gemv_n_norm)
 template <class T>
 static void gemv_n_norm_launch(int g, const T *V, size_t ldv, int ncol, const typename ST<T>::D *h, T *w, int n,
-                               typename ST<T>::D *part, unsigned *tk, double *nrm,
-                               const typename ST<T>::D *nrm_before, int *flag, double eta2, cudaStream_t s) {
-    if constexpr (sizeof(T) == 4) {
-        if (ldv % 4 == 0 && !(((uintptr_t)V | (uintptr_t)w) & 15)) {
-            if (ncol <= kSmallCols) launch(k_gemv_n_norm_f4<kSmallCols>, g, kThreads, 0, s, V, ldv, ncol, h, w, n, part, tk, nrm);
-            else launch(k_gemv_n_norm_f4<>, g, kThreads, 0, s, V, ldv, ncol, h, w, n, part, tk, nrm);
-            return;
-        }
-    }
+                               typename ST<T>::D *part, unsigned *tk, double *nrm, cudaStream_t s) {
     if (ncol <= kSmallCols)
-        launch(k_gemv_n_norm<T, kSmallCols>, g, kThreads, 0, s, V, ldv, ncol, h, w, n, nullptr, part, tk, nrm, nrm_before, flag, eta2);
+        launch(k_gemv_n_norm<T, kSmallCols>, g, kThreads, 0, s, V, ldv, ncol, h, w, n, part, tk, nrm);
     else
-        launch(k_gemv_n_norm<T>, g, kThreads, 0, s, V, ldv, ncol, h, w, n, nullptr, part, tk, nrm, nrm_before, flag, eta2);
+        launch(k_gemv_n_norm<T>, g, kThreads, 0, s, V, ldv, ncol, h, w, n, part, tk, nrm);
 }
 
+// The dots and update sweeps of Arnoldi step j (tg_arnoldi.cuh); last: column j is finished
+// without a product.  j0: the column the run started from (its Hbar columns before j0 stand).
 template <class T, class HT = T>
-static int arnoldi_step(tg_op *op, const DevOp &A, const DevOp32 &A32, T *V, size_t ldv, int n, int j, HT *H, int ldh,
-                        cudaStream_t s) {
+static int arnoldi_sweeps(tg_op *op, T *V, size_t ldv, int n, int j, int last, int j0, HT *H, int ldh,
+                          cudaStream_t s, const int *skip = nullptr) {
     using D = typename ST<T>::D;
-    // w = A v_j, then two classical Gram-Schmidt passes, each a tall-skinny V^H w and a
-    // fused update + norm
-    T *w = V + (size_t)(j + 1) * ldv;
-    TG_CHECK(launch_apply<T>(A, A32, V + (size_t)j * ldv, w, s));
-    TG_CHECK(red_ready(op, 0, s));
+    const int sms = num_sms(), nv = last ? 1 : 2, ncol = j + 1, nent = nv * ncol;
+    const double cf = sizeof(T) == 16 ? 4.0 : 1.0, es = sizeof(T);
+    const T *u = V + (size_t)j * ldv;
+    constexpr bool kReal = sizeof(T) != 16;
+    bool piped = kReal && pipe_ok<T>(V, ldv, u, n, ncol);
+    size_t smem = 0;
+    int gx = 1, gy = 1;
+    if constexpr (kReal) {
+        if (piped) {
+            using E = typename std::conditional<sizeof(T) == 8, double, float>::type;
+            constexpr int R = PipeRows<E>::value;
+            smem = (size_t)kPipeStages * (std::min(ncol, kPipeCols) + nv) * R * sizeof(E);
+            piped = smem_attr_once((const void *)k_arn_dots_pipe<E>, max_dyn_smem() - 8192) == cudaSuccess;
+            if (!piped) (void)cudaGetLastError();
+            const int chunks = (n + R - 1) / R;
+            gy = (ncol + kPipeCols - 1) / kPipeCols;
+            // few chunks: two groups' worth of blocks, one level of reduction
+            gx = chunks <= 4 * kArnGroup ? std::min(chunks, 2 * kArnGroup)
+                                         : std::min(chunks, std::max(1, sms * (smem <= 100 * 1024 ? 2 : 1) / gy));
+        }
+    }
+    if (!piped) {
+        const int64_t passes = ((int64_t)n + 63) / 64;
+        gy = (ncol + kArnCols - 1) / kArnCols;
+        gx = passes <= 4 * kArnGroup ? (int)std::min<int64_t>(passes, 2 * kArnGroup)
+                                     : (int)std::min<int64_t>(passes, std::max(1, sms * 2 / gy));
+    }
+    TG_CHECK(red_ready(op, (size_t)(gx + gx / kArnGroup + 1) * nent * sizeof(D), s));
     char *sm = wsp<char>(op, S_SMALL);
-    D *h1 = reinterpret_cast<D *>(sm + SmallArea::arn_h1);   // j+2 entries: V_j^H w and ||w||^2
-    D *h2 = reinterpret_cast<D *>(sm + SmallArea::arn_h2);
-    double *nrm = reinterpret_cast<double *>(sm + SmallArea::arn_nrm);
-    double *inv = nrm + 4;
-    int *flag = reinterpret_cast<int *>(sm + SmallArea::arn_nrm + 64);
-    const int g = grid_for(n, 8);
-    const int gb = (int)std::min<int64_t>((n + 127) / 128, (int64_t)num_sms() * 8);
-    const int ncol = j + 1;
-    D *part = wsp<D>(op, S_PART);
-    unsigned *tk = wsp<unsigned>(op, S_TICKET);
-    TG_CHECK(red_ready(op, (size_t)gb * (ncol + 1) * sizeof(D), s));
-    part = wsp<D>(op, S_PART);
-    // pass 1: h1 = [V_j, w]^H w
-    bool piped = false;
-    int gbt = gb;
-    TG_PROF(P_GEMV_T, (double)(ncol + 1) * n * sizeof(T), 2.0 * (ncol + 1) * n * (sizeof(T) == 16 ? 4 : 1),
-            gbt = gemv_t_part_launch<T>(V, ldv, ncol + 1, w, n, part, s, &piped));
-    TG_PROF(P_SUM_PART, (double)gbt * (ncol + 1) * sizeof(D), (double)gbt * (ncol + 1),
-            launch(k_sum_part<D>, (ncol + 1 + 7) / 8, 256, 0, s, part, gbt, ncol + 1, h1, 0));
-    TG_PROF(P_GEMV_N, (ncol + 2.0) * n * sizeof(T), 2.0 * ncol * n * (sizeof(T) == 16 ? 4 : 1),
-            gemv_n_norm_launch<T>(g, V, ldv, ncol, h1, w, n, part, tk, nrm, h1 + ncol, flag, 0.5, s));
-    // pass 2 (classical Gram-Schmidt twice: on this operator the selective criterion of
-    // Daniel, Gragg, Kaufman and Stewart asked for the second pass on nearly every step)
-    TG_PROF(P_GEMV_T, (double)(ncol + 1) * n * sizeof(T), 2.0 * ncol * n * (sizeof(T) == 16 ? 4 : 1),
-            gbt = gemv_t_part_launch<T>(V, ldv, ncol, w, n, part, s, &piped));
-    TG_PROF(P_SUM_PART, (double)gbt * ncol * sizeof(D), (double)gbt * ncol,
-            launch(k_sum_part<D>, (ncol + 7) / 8, 256, 0, s, part, gbt, ncol, h2, 0));
-    TG_PROF(P_GEMV_N, (ncol + 2.0) * n * sizeof(T), 2.0 * ncol * n * (sizeof(T) == 16 ? 4 : 1),
-            gemv_n_norm_launch<T>(g, V, ldv, ncol, h2, w, n, part, tk, nrm, nullptr, nullptr, 0.0, s));
-    TG_PROF(P_SMALL, 0, j, launch(k_arnoldi_finish2<T, HT>, 1, 128, 0, s, h1, h2, nrm, j, H + (size_t)j * ldh, inv));
-    TG_PROF(P_SCALE, 2.0 * n * sizeof(T), n, launch(k_scale_by<T>, g, kThreads, 0, s, w, n, inv));
+    ArnState<D> a;
+    a.s = reinterpret_cast<D *>(sm + SmallArea::arn_h1);
+    a.z = reinterpret_cast<D *>(sm + SmallArea::arn_h2);
+    a.h1 = reinterpret_cast<D *>(sm + SmallArea::arn_c);
+    a.beta = reinterpret_cast<double *>(sm + SmallArea::arn_nrm);
+    a.t = reinterpret_cast<D *>(sm + SmallArea::arn_nrm + 64);
+    a.part = wsp<D>(op, S_PART);
+    a.ticket = wsp<unsigned>(op, S_TICKET);
+    a.skip = skip;
+    const int ev = prof_begin(s);
+    if (piped) {
+        if constexpr (kReal) {
+            using E = typename std::conditional<sizeof(T) == 8, double, float>::type;
+            launch(k_arn_dots_pipe<E>, dim3(gx, gy), kThreads, smem, s, reinterpret_cast<const E *>(V), ldv, j, n, last, a);
+        }
+    } else {
+        launch(k_arn_dots<T>, dim3(gx, gy), kThreads, 0, s, V, ldv, j, n, last, a);
+    }
+    prof_end(ev, P_GEMV_T, (ncol + nv - 1.0) * n * es, 2.0 * nent * n * cf, s);
+    TG_LAUNCH_CHECK();
+    auto update = [&](auto f4, auto cs, auto mc) {
+        constexpr bool F4 = decltype(f4)::value;
+        constexpr int CS = decltype(cs)::value, MC = decltype(mc)::value;
+        const int64_t rows = F4 ? ((int64_t)n + 3) / 4 : n, per = kThreads / CS;
+        const int nb = (int)std::min<int64_t>((rows + per - 1) / per, (int64_t)sms * 8);
+        TG_PROF(P_GEMV_N, (j + 2.0 * nv) * n * es, 2.0 * nv * j * n * cf,
+                launch(k_arn_update<T, HT, F4, CS, MC>, nb + 1, kThreads, 0, s, V, ldv, j, n, last, H, ldh, j0, a));
+    };
+    auto pick = [&](auto f4) {
+        // fewer rows than two threads each per SM slot of 256: four threads share a row
+        const int64_t rows = decltype(f4)::value ? n / 4 : n;
+        const bool few = rows < (int64_t)sms * 2 * kThreads, small = j <= kSmallCols;
+        using C1 = std::integral_constant<int, 1>;
+        using C4 = std::integral_constant<int, 4>;
+        using MS = std::integral_constant<int, kSmallCols>;
+        using ML = std::integral_constant<int, kMaxCols>;
+        if (few && small) update(f4, C4{}, MS{});
+        else if (few) update(f4, C4{}, ML{});
+        else if (small) update(f4, C1{}, MS{});
+        else update(f4, C1{}, ML{});
+    };
+    if constexpr (sizeof(T) == 4) {
+        if (ldv % 4 == 0 && !((uintptr_t)V & 15) && ldv >= (size_t)((n + 3) / 4 * 4)) pick(std::true_type{});
+        else pick(std::false_type{});
+    } else {
+        pick(std::false_type{});
+    }
     TG_LAUNCH_CHECK();
     return TG_OK;
+}
+
+// Extends V from column j0 (not yet orthogonalised against the columns before it, which are
+// orthonormal) to column m; Hbar columns j0..m-1 (leading dimension ldh).
+template <class T, class HT = T>
+static int arnoldi_run(tg_op *op, const DevOp &A, const DevOp32 &A32, T *V, size_t ldv, int n, int j0, int m, HT *H,
+                       int ldh, cudaStream_t s) {
+    for (int j = j0; j < m; ++j) {
+        TG_CHECK(launch_apply<T>(A, A32, V + (size_t)j * ldv, V + (size_t)(j + 1) * ldv, s));
+        TG_CHECK((arnoldi_sweeps<T, HT>(op, V, ldv, n, j, 0, j0, H, ldh, s)));
+    }
+    return arnoldi_sweeps<T, HT>(op, V, ldv, n, m, 1, j0, H, ldh, s);
 }
 
 // GMRES(m)-Proj(k) (Section 2.2) in float64 / complex128.
@@ -1707,9 +1751,10 @@ static int solve_gmres64(tg_op *op, int transpose, const tg_defl *df, const T *b
     const DevOp32 &A32 = pick32(op, TG_FINE, transpose);
     const int n = op->n, m = cfg.m3;
     const int ldh = m + 1;
+    const size_t ldv = ((size_t)n + 63) / 64 * 64;       // whole pipeline chunks, as in the coarse phase
     TG_CHECK(wsx(op, S_R64, (size_t)n * sizeof(T)));
-    TG_CHECK(wsx(op, S_FV, (size_t)n * (m + 1) * sizeof(T)));
-    TG_CHECK(wsx(op, S_FH, (size_t)(m + 1) * m * sizeof(T)));
+    TG_CHECK(wsx(op, S_FV, ldv * (m + 1) * sizeof(T)));
+    TG_CHECK(wsx(op, S_FH, (size_t)2 * (m + 1) * m * sizeof(T)));
     TG_CHECK(wsx(op, S_FCS, (size_t)(m + 1) * sizeof(D)));
     TG_CHECK(wsx(op, S_FSN, (size_t)(m + 1) * sizeof(D)));
     TG_CHECK(wsx(op, S_FG, (size_t)(m + 1) * sizeof(D)));
@@ -1717,7 +1762,7 @@ static int solve_gmres64(tg_op *op, int transpose, const tg_defl *df, const T *b
     TG_CHECK(wsx(op, S_FSTATE, sizeof(GivensState)));
     T *r = wsp<T>(op, S_R64);
     T *V = wsp<T>(op, S_FV);
-    D *H = wsp<D>(op, S_FH);
+    D *Hb = wsp<D>(op, S_FH), *H = Hb + (size_t)(m + 1) * m;     // Hbar, and its rotated copy
     GivensState *gs = wsp<GivensState>(op, S_FSTATE);
     double nr, nb;
     TG_CHECK(true_residual<T>(op, A, b, x, r, &nr, &nb, s));
@@ -1748,24 +1793,30 @@ static int solve_gmres64(tg_op *op, int transpose, const tg_defl *df, const T *b
         D g0{};
         memcpy(&g0, &nr, sizeof(double));
         TG_CHECK_CUDA(cudaMemcpyAsync(wsp<D>(op, S_FG), &g0, sizeof(D), cudaMemcpyHostToDevice, s));
-        TG_CHECK_CUDA(cudaMemsetAsync(H, 0, (size_t)(m + 1) * m * sizeof(D), s));
+        TG_CHECK_CUDA(cudaMemsetAsync(Hb, 0, (size_t)2 * (m + 1) * m * sizeof(D), s));
         TG_PROF(P_SCALE, 2.0 * n * sizeof(T), n, launch(k_scale_by<T>, grid_for(n, 8), kThreads, 0, s, V, n, inv));
         TG_LAUNCH_CHECK();
-        int steps = 0;
         const int mm = (int)((cfg.max_mvps - mvps) < m ? (cfg.max_mvps - mvps) : m);
-        for (int j = 0; j < mm; ++j) {
-            TG_CHECK(arnoldi_step<T>(op, A, A32, V, n, n, j, reinterpret_cast<T *>(H), ldh, s));
-            TG_PROF(P_GIVENS, 0, 6.0 * j, launch_givens_step<D>(H, ldh, j, wsp<D>(op, S_FCS), wsp<D>(op, S_FSN), wsp<D>(op, S_FG), gs, s));
-            TG_LAUNCH_CHECK();
-            TG_CHECK(readback(op, gs, sizeof(GivensState), s));
-            GivensState hg;
-            memcpy(&hg, op->pin.p, sizeof(hg));
-            steps = hg.steps;
-            if (hg.done) break;
+        // the sweeps of step j finish Hbar column j - 1; once a column meets the target (done) the
+        // launches after it return at once, so the host looks only every kGmresLook steps
+        constexpr int kGmresLook = 16;
+        GivensState hg{};
+        for (int j = 0; j <= mm && !hg.done; ++j) {
+            if (j < mm) TG_CHECK(launch_apply<T>(A, A32, V + (size_t)j * ldv, V + (size_t)(j + 1) * ldv, s));
+            TG_CHECK(arnoldi_sweeps<T>(op, V, ldv, n, j, j == mm, 0, reinterpret_cast<T *>(Hb), ldh, s, &gs->done));
+            if (j > 0) {
+                TG_PROF(P_GIVENS, 0, 6.0 * j, launch_givens_step<D>(Hb, H, ldh, j - 1, wsp<D>(op, S_FCS), wsp<D>(op, S_FSN), wsp<D>(op, S_FG), gs, s));
+                TG_LAUNCH_CHECK();
+            }
+            if (j == mm || (j % kGmresLook == 0 && j > 0)) {
+                TG_CHECK(readback(op, gs, sizeof(GivensState), s));
+                memcpy(&hg, op->pin.p, sizeof(hg));
+            }
         }
-        mvps += steps;
+        const int steps = hg.steps;
+        mvps += steps + (hg.done && steps < mm ? 1 : 0);     // a column ends one product after its own
         TG_PROF(P_GIVENS, 0, 1.0 * m * m, launch_givens_solve<D>(H, ldh, wsp<D>(op, S_FG), wsp<D>(op, S_FY), gs, s));
-        TG_PROF(P_GEMV_N, (steps + 2.0) * n * sizeof(T), 2.0 * steps * n, launch(k_gemv_n<T>, grid_for(n, 8), kThreads, 0, s, V, n, steps, wsp<D>(op, S_FY), 1.0, x, n));
+        TG_PROF(P_GEMV_N, (steps + 2.0) * n * sizeof(T), 2.0 * steps * n, launch(k_gemv_n<T>, grid_for(n, 8), kThreads, 0, s, V, ldv, steps, wsp<D>(op, S_FY), 1.0, x, n));
         TG_LAUNCH_CHECK();
         TG_CHECK(true_residual<T>(op, A, b, x, r, &nr, &nb, s));
         if (!std::isfinite(nr)) { status = TG_NAN; break; }
@@ -1880,7 +1931,7 @@ static int gdr_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *V, size_t
     const cudaStream_t s_caller = s;
     // the cycle's launches, queued on stream s (the caller's, or the capture stream)
     auto body = [&](cudaStream_t s) -> int {
-        for (int j = j0; j < m; ++j) TG_CHECK((arnoldi_step<T, HT>(op, A, A32, V, ldv, nc, j, H, ldh, s)));
+        TG_CHECK((arnoldi_run<T, HT>(op, A, A32, V, ldv, nc, j0, m, H, ldh, s)));
         TG_CHECK_CUDA(cudaMemsetAsync(H2, 0, (size_t)ldh * m * sizeof(HT), s));
         cudaError_t le = cudaSuccess;
         TG_PROF(P_GDR_RESTART, 0, 30.0 * m * m * m, le = launch_gmresdr_restart<HT>(a, s));
@@ -1894,8 +1945,7 @@ static int gdr_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *V, size_t
     if (g_prof.on) return body(s_caller);
     // the reduction scratch the Arnoldi steps use, at its largest, before any capture: a
     // capture may not allocate
-    const int gb = (int)std::min<int64_t>((nc + 127) / 128, (int64_t)num_sms() * 8);
-    TG_CHECK(red_ready(op, (size_t)std::max(gb, 1) * (m + 2) * sizeof(D), s));
+    TG_CHECK(red_ready(op, (size_t)num_sms() * 3 * 2 * (m + 2) * sizeof(D), s));
     // entries of older workspace generations refer to freed buffers: drop them
     for (auto &g : op->graphs)
         if (g.gen != op->ws_gen && g.exec) {
@@ -2070,19 +2120,7 @@ static int gmresdr_impl(tg_op *op, int transpose, const void *b_fine, int m, int
         std::swap(H, H2);
         TG_CHECK_CUDA(cudaMemsetAsync(c, 0, (size_t)(m + 1) * hs, s));
         TG_CHECK_CUDA(cudaMemcpyAsync(c, a.cnew, (size_t)(kk + 1) * hs, cudaMemcpyDeviceToDevice, s));
-        // re-orthogonalise v_{k+1} against V_k and normalise
-        {
-            using DD = typename ST<T>::D;
-            T *w = V + (size_t)kk * ldv;
-            DD *h1 = reinterpret_cast<DD *>(wsp<char>(op, S_SMALL) + SmallArea::arn_h1);
-            DD *nrm = reinterpret_cast<DD *>(wsp<char>(op, S_SMALL) + SmallArea::arn_nrm);
-            TG_CHECK(gemv_t<T>(op, V, ldv, kk, w, nc, h1, s));
-            TG_PROF(P_GEMV_N, (kk + 2.0) * nc * sizeof(T), 2.0 * kk * nc, launch(k_gemv_n<T>, grid_for(nc, 8), kThreads, 0, s, V, ldv, kk, h1, -1.0, w, nc));
-            TG_PROF(P_DOT, 1.0 * nc * sizeof(T), 2.0 * nc, launch(k_dot<T>, grid_for(nc, 4), kThreads, 0, s, w, nullptr, nc, wsp<DD>(op, S_PART), wsp<unsigned>(op, S_TICKET), nrm));
-            TG_PROF(P_SMALL, 0, 1, launch_inv_sqrt(s, reinterpret_cast<const double *>(nrm), reinterpret_cast<double *>(nrm) + 4));
-            TG_PROF(P_SCALE, 2.0 * nc * sizeof(T), nc, launch(k_scale_by<T>, grid_for(nc, 8), kThreads, 0, s, w, nc, reinterpret_cast<double *>(nrm) + 4));
-            TG_LAUNCH_CHECK();
-        }
+        // v_{k+1} is orthogonalised again and normalised by the first sweeps of the next cycle
         j0 = kk;
     }
     // the V_m P_k basis of the final cycle, prolonged; x_c out
@@ -2185,11 +2223,11 @@ static int cgs2_column(tg_op *op, T *V, size_t ldv, int n, int j, double drop_re
         TG_PROF(P_GEMV_T, (double)(j + 1) * n * sizeof(T), 2.0 * (j + 1) * n, gbt = gemv_t_part_launch<T>(V, ldv, j + 1, w, n, part, s, &piped));
         TG_PROF(P_SUM_PART, 0, 0, launch(k_sum_part<D>, (j + 1 + 7) / 8, 256, 0, s, part, gbt, j + 1, h1, 0));
         TG_PROF(P_GEMV_N, (j + 2.0) * n * sizeof(T), 2.0 * j * n,
-                gemv_n_norm_launch<T>(g, V, ldv, j, h1, w, n, part, tk, nrm, nullptr, nullptr, 0.0, s));
+                gemv_n_norm_launch<T>(g, V, ldv, j, h1, w, n, part, tk, nrm, s));
         TG_PROF(P_GEMV_T, (double)(j + 1) * n * sizeof(T), 2.0 * j * n, gbt = gemv_t_part_launch<T>(V, ldv, j, w, n, part, s, &piped));
         TG_PROF(P_SUM_PART, 0, 0, launch(k_sum_part<D>, (j + 7) / 8, 256, 0, s, part, gbt, j, h2, 0));
         TG_PROF(P_GEMV_N, (j + 2.0) * n * sizeof(T), 2.0 * j * n,
-                gemv_n_norm_launch<T>(g, V, ldv, j, h2, w, n, part, tk, nrm, nullptr, nullptr, 0.0, s));
+                gemv_n_norm_launch<T>(g, V, ldv, j, h2, w, n, part, tk, nrm, s));
         TG_LAUNCH_CHECK();
         TG_CHECK(readback(op, h1 + j, sizeof(D), s));
         D hb;
@@ -2341,7 +2379,7 @@ static int improve_impl(tg_op *op, tg_defl *d, int m, int cycles, int nstart, in
         TG_CHECK_CUDA(cudaMemcpyAsync(S, u, (size_t)n * sizeof(T), cudaMemcpyDeviceToDevice, s));
         bool kept = false;
         TG_CHECK(cgs2_column<T>(op, S, ld, n, 0, 0.0, &kept, s));
-        for (int j = 0; j < p; ++j) TG_CHECK((arnoldi_step<T, T>(op, A, A32, S, ld, n, j, Ha, p + 1, s)));
+        TG_CHECK(arnoldi_run<T>(op, A, A32, S, ld, n, 0, p, Ha, p + 1, s));
         mvps += p;
         cols = p + 1;
         // then the current approximate eigenvectors (u lies in their span: one drops out)

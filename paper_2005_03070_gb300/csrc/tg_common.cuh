@@ -113,6 +113,11 @@ __device__ __forceinline__ float shfl_down(float v, int o) { return __shfl_down_
 __device__ __forceinline__ cplx shfl_down(cplx v, int o) {
     return {__shfl_down_sync(0xffffffffu, v.re, o), __shfl_down_sync(0xffffffffu, v.im, o)};
 }
+__device__ __forceinline__ float shfl_xor(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
+__device__ __forceinline__ cplx shfl_xor(cplx v, int o) {
+    return {__shfl_xor_sync(0xffffffffu, v.re, o), __shfl_xor_sync(0xffffffffu, v.im, o)};
+}
 __device__ __forceinline__ double dadd(double a, double b) { return a + b; }
 __device__ __forceinline__ float dadd(float a, float b) { return a + b; }
 __device__ __forceinline__ cplx dadd(cplx a, cplx b) { return a + b; }

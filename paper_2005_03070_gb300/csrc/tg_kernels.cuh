@@ -660,23 +660,17 @@ __global__ void __launch_bounds__(kThreads) k_gemv_n(const T *__restrict__ V, si
     }
 }
 
-// Arnoldi orthogonalisation pass: w -= V h (ncol columns), then ||w||^2 (deterministic);
-// the last block writes nrm2_out[0] and, when flag_out is given, the selective
-// re-orthogonalisation decision (Daniel, Gragg, Kaufman and Stewart): a second pass is
-// needed when the pass cancelled more than half of ||w||^2, i.e. ||w_new||^2 < eta2 ||w||^2
-// with ||w||^2 = real(nrm2_before[0]).  cond: skip the whole kernel when *cond == 0.
+// Orthogonalisation pass: w -= V h (ncol columns), then ||w||^2 (deterministic); the last block
+// writes nrm2_out[0].
 template <class T, int MC = kMaxCols>
 __global__ void __launch_bounds__(kThreads) k_gemv_n_norm(const T *__restrict__ V, size_t ldv, int ncol,
                                                            const typename ST<T>::D *__restrict__ h,
-                                                           T *__restrict__ w, int n, const int *cond,
+                                                           T *__restrict__ w, int n,
                                                            typename ST<T>::D *part, unsigned *ticket,
-                                                           double *nrm2_out,
-                                                           const typename ST<T>::D *nrm2_before,
-                                                           int *flag_out, double eta2) {
+                                                           double *nrm2_out) {
     pdl_wait();
     using D = typename ST<T>::D;
     using P = typename Part<T>::P;
-    if (cond && !*cond) return;
     __shared__ T hs[MC];         // coefficients in the vector type, converted once per block
     __shared__ D red[(kThreads / 32)];
     __shared__ D tot[1];
@@ -694,52 +688,8 @@ __global__ void __launch_bounds__(kThreads) k_gemv_n_norm(const T *__restrict__ 
     if (last_block(ticket)) {
         final_sum<D, 1>(part, tot, ticket);
         if (threadIdx.x == 0) {
-            const double nn = dreal(tot[0]);
-            nrm2_out[0] = nn;
-            if (flag_out) flag_out[0] = (nn < eta2 * dreal(nrm2_before[0])) ? 1 : 0;
+            nrm2_out[0] = dreal(tot[0]);
         }
-    }
-}
-
-// k_gemv_n_norm for float32 V with 16-byte aligned columns (ldv a multiple of 4, V and w
-// 16-byte aligned): each thread takes 4 consecutive rows as float4 loads; the rows beyond
-// the last whole group of 4 are taken one by one by the first threads.
-template <int MC = kMaxCols>
-__global__ void __launch_bounds__(kThreads) k_gemv_n_norm_f4(const float *__restrict__ V, size_t ldv, int ncol,
-                                                              const double *__restrict__ h, float *__restrict__ w,
-                                                              int n, double *part, unsigned *ticket,
-                                                              double *nrm2_out) {
-    pdl_wait();
-    __shared__ float hs[MC];
-    __shared__ double red[(kThreads / 32)];
-    __shared__ double tot[1];
-    for (int c = threadIdx.x; c < ncol; c += blockDim.x) hs[c] = (float)h[c];
-    __syncthreads();
-    float acc[1] = {0.0f};
-    const int n4 = n >> 2;
-    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < n4; g += gridDim.x * blockDim.x) {
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
-        for (int c = 0; c < ncol; ++c) {
-            const float4 v = reinterpret_cast<const float4 *>(V + (size_t)c * ldv)[g];
-            const float hc = hs[c];
-            a.x = fmaf(hc, v.x, a.x); a.y = fmaf(hc, v.y, a.y); a.z = fmaf(hc, v.z, a.z); a.w = fmaf(hc, v.w, a.w);
-        }
-        float4 wv = reinterpret_cast<float4 *>(w)[g];
-        wv.x -= a.x; wv.y -= a.y; wv.z -= a.z; wv.w -= a.w;
-        reinterpret_cast<float4 *>(w)[g] = wv;
-        acc[0] = fmaf(wv.x, wv.x, fmaf(wv.y, wv.y, fmaf(wv.z, wv.z, fmaf(wv.w, wv.w, acc[0]))));
-    }
-    for (int row = 4 * n4 + blockIdx.x * blockDim.x + threadIdx.x; row < n; row += gridDim.x * blockDim.x) {
-        float a = 0.0f;
-        for (int c = 0; c < ncol; ++c) a = fmaf(hs[c], V[(size_t)c * ldv + row], a);
-        const float wv = w[row] - a;
-        w[row] = wv;
-        acc[0] = fmaf(wv, wv, acc[0]);
-    }
-    block_reduce_store<float, double, 1>(acc, part, red);
-    if (last_block(ticket)) {
-        final_sum<double, 1>(part, tot, ticket);
-        if (threadIdx.x == 0) nrm2_out[0] = tot[0];
     }
 }
 
@@ -820,22 +770,6 @@ __global__ void __launch_bounds__(kThreads) k_tsm_f(const float *__restrict__ In
         __syncthreads();                         // everyone is done with this buffer
     }
     cp_async_wait<0>();
-}
-
-// Hbar column j: H[i] = h1[i] + h2[i] (i <= j), H[j+1] = sqrt(nrm2[0]), inv[0] = 1/H[j+1].
-// HT is the Hessenberg type: the basis type, or float64 for a float32 basis.
-template <class T, class HT = T>
-__global__ void k_arnoldi_finish2(const typename ST<T>::D *h1, const typename ST<T>::D *h2, const double *nrm2,
-                                  int j, HT *Hcol, double *inv) {
-    pdl_wait();
-    for (int i = threadIdx.x; i <= j; i += blockDim.x) Hcol[i] = dadd(h1[i], h2[i]);
-    if (threadIdx.x == 0) {
-        const double nn = sqrt(nrm2[0]);
-        HT hv = ST<HT>::zero();
-        *reinterpret_cast<double *>(&hv) = nn;
-        Hcol[j + 1] = hv;
-        inv[0] = nn > 0 ? 1.0 / nn : 0.0;
-    }
 }
 
 // Projection update: x += B1 d; r -= B2 e.  (B1, B2: n x k; d, e: device D vectors.)
@@ -999,25 +933,6 @@ __global__ void k_scale_by(T *__restrict__ w, int n, const double *__restrict__ 
     const double s = inv[0];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) w[i] = scal(s, w[i]);
 }
-
-// Hbar column j of an Arnoldi step: H[i] = h1[i] + h2[i] (i <= j), H[j+1] = ||w||,
-// inv[0] = 1 / ||w|| (0 if w vanished: an invariant subspace was found).
-template <class T>
-__global__ void k_arnoldi_finish(const typename ST<T>::D *h1, const typename ST<T>::D *h2,
-                                 const typename ST<T>::D *nrm2, int j, T *Hcol, double *inv) {
-    pdl_wait();
-    for (int i = threadIdx.x; i <= j; i += blockDim.x) Hcol[i] = dadd(h1[i], h2[i]);
-    if (threadIdx.x == 0) {
-        const double nn = sqrt(dreal(nrm2[0]));
-        T hv = ST<T>::zero();
-        *reinterpret_cast<double *>(&hv) = nn;
-        Hcol[j + 1] = hv;
-        inv[0] = nn > 0 ? 1.0 / nn : 0.0;
-    }
-}
-
-
-
 
 // ----------------------------------------------------------------------------- float32 3D stencil, padded rows
 // Inside a float32 BiCGStab cycle on a 3D constant-coefficient grid the cycle's vectors are

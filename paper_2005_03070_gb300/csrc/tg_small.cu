@@ -1320,15 +1320,16 @@ __global__ void __launch_bounds__(kGdrThreads) k_gmresdr_restart_batch(const Gdr
 }
 
 // ----------------------------------------------------------------------------- GMRES(m) Givens step
-// Column j of the Arnoldi Hessenberg (h[0..j+1], ld = m+1) is rotated by the previous
-// rotations, a new rotation zeroes h[j+1]; g (the least-squares right-hand side) is
+// Column j of the Arnoldi Hessenberg Hbar (rows 0..j+1, ld = m+1) is copied to H and rotated by
+// the previous rotations, a new rotation zeroes h[j+1]; g (the least-squares right-hand side) is
 // updated; state->resid = |g[j+1]|; state->done = 1 when resid <= target or h[j,j] = 0.
 template <class D>
-__global__ void k_givens_step(D *H, int ldh, int j, D *cs, D *sn, D *g, GivensState *state) {
+__global__ void k_givens_step(const D *Hbar, D *H, int ldh, int j, D *cs, D *sn, D *g, GivensState *state) {
     pdl_wait();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     if (state->done) return;
     D *h = H + (size_t)j * ldh;
+    for (int i = 0; i <= j + 1; ++i) h[i] = Hbar[i + (size_t)j * ldh];
     for (int i = 0; i < j; ++i) {
         D a = h[i], b = h[i + 1];
         h[i] = add(Cx<D>::mul(Cx<D>::cj(cs[i]), a), Cx<D>::mul(Cx<D>::cj(sn[i]), b));
@@ -1425,8 +1426,8 @@ cudaError_t launch_gmresdr_restart_batch(const GdrArgs<T> *args, const int *acti
     return cudaGetLastError();
 }
 template <class D>
-void launch_givens_step(D *H, int ldh, int j, D *cs, D *sn, D *g, GivensState *state, cudaStream_t s) {
-    launch(k_givens_step<D>, 1, 1, 0, s, H, ldh, j, cs, sn, g, state);
+void launch_givens_step(const D *Hbar, D *H, int ldh, int j, D *cs, D *sn, D *g, GivensState *state, cudaStream_t s) {
+    launch(k_givens_step<D>, 1, 1, 0, s, Hbar, H, ldh, j, cs, sn, g, state);
 }
 template <class D>
 void launch_givens_solve(const D *H, int ldh, const D *g, D *y, const GivensState *state, cudaStream_t s) {
@@ -1440,7 +1441,7 @@ void launch_givens_solve(const D *H, int ldh, const D *g, D *y, const GivensStat
     template cudaError_t launch_gmresdr_restart<D>(const GdrArgs<D> &, cudaStream_t);                \
     template size_t gmresdr_restart_smem<D>(int, int *);                                              \
     template cudaError_t launch_gmresdr_restart_batch<D>(const GdrArgs<D> *, const int *, int, int, cudaStream_t); \
-    template void launch_givens_step<D>(D *, int, int, D *, D *, D *, GivensState *, cudaStream_t);  \
+    template void launch_givens_step<D>(const D *, D *, int, int, D *, D *, D *, GivensState *, cudaStream_t);  \
     template void launch_givens_solve<D>(const D *, int, const D *, D *, const GivensState *, cudaStream_t);
 TG_INST(double)
 TG_INST(cplx)

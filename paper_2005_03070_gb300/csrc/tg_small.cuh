@@ -76,7 +76,7 @@ template <class T> size_t gmresdr_restart_smem(int m, int *parts);
 template <class T>
 cudaError_t launch_gmresdr_restart_batch(const GdrArgs<T> *args, const int *active, int count, int m, cudaStream_t s);
 template <class D>
-void launch_givens_step(D *H, int ldh, int j, D *cs, D *sn, D *g, GivensState *state, cudaStream_t s);
+void launch_givens_step(const D *Hbar, D *H, int ldh, int j, D *cs, D *sn, D *g, GivensState *state, cudaStream_t s);
 template <class D>
 void launch_givens_solve(const D *H, int ldh, const D *g, D *y, const GivensState *state, cudaStream_t s);
 
