@@ -20,6 +20,7 @@
 #include "tg_idr.cuh"
 #include "tg_kernels.cuh"
 #include "tg_mrhs.cuh"
+#include "tg_persist.cuh"
 #include "tg_split.cuh"
 #include "tg_batch.cuh"
 #include "tg_setup.cuh"
@@ -81,12 +82,12 @@ static int tiles_grid(int64_t n, int per_sm) {
 enum ProfClass {
     P_APPLY, P_DOT, P_RESIDUAL, P_BI_INIT, P_BI_V, P_BI_S, P_BI_T, P_BI_X, P_GEMV_T, P_SUM_PART, P_GEMV_N,
     P_PROJ, P_TSM, P_GRAM, P_SMALL, P_GDR_RESTART, P_SCALE, P_TRANSFER, P_SETUP, P_CONVERT, P_GRAD, P_GIVENS,
-    P_NOOP, P_REORTH, P_IDR_MV, P_IDR_UPD, P_COUNT
+    P_NOOP, P_REORTH, P_IDR_MV, P_IDR_UPD, P_BI_CYCLE, P_IDR_CYCLE, P_COUNT
 };
 static const char *kProfName[P_COUNT] = {
     "apply", "dot", "residual", "bicg_init", "bicg_v", "bicg_s", "bicg_t", "bicg_x", "gemv_t", "sum_part",
     "gemv_n", "proj_update", "tsm", "gram", "small_dense", "gmresdr_restart", "scale", "transfer", "setup",
-    "convert", "kappa_grad", "givens", "bicg_noop", "reorth_pass", "idr_apply", "idr_update"};
+    "convert", "kappa_grad", "givens", "bicg_noop", "reorth_pass", "idr_apply", "idr_update", "bicg_cycle", "idr_cycle"};
 
 struct ProfRec {
     int cls;
@@ -207,6 +208,7 @@ enum Slot {
     S_IG, S_IU, S_IP, S_IPR, S_IPRI, S_IT, S_IINFO,
     S_AE_S, S_AE_W, S_AE_H, S_AE_WW, S_AE_HA, S_AE_Y, S_AE_U, S_AE_P, S_AE_Z, S_AE_TH, S_AE_WR, S_AE_WI,
     S_AE_ORD, S_AE_ERES, S_AE_WORK, S_AE_YW, S_AE_GW, S_AE_INFO, S_AE_DUM, S_PADX, S_PADR, S_AE_HR, S_AE_WWR, S_IP32,
+    S_P2, S_V2, S_BAR,
     S_COUNT
 };
 
@@ -957,11 +959,18 @@ static int project_impl(tg_op *op, const tg_defl *df, const T *W, const T *B1, c
     return TG_OK;
 }
 
+// The float64 / complex128 projection data: c = W^H r, x += B1 d, r -= B2 e.
+template <class T>
+static void proj_data64(const tg_defl *df, const T **W, const T **B1, const T **B2) {
+    *W = df ? df->Q.as<T>() : nullptr;
+    *B1 = !df ? nullptr : df->proj == TG_PROJ_MINRES ? df->Y.as<T>() : df->Q.as<T>();
+    *B2 = !df ? nullptr : df->proj == TG_PROJ_MINRES ? df->Q.as<T>() : df->AV.as<T>();
+}
+
 template <class T>
 static int project64(tg_op *op, const tg_defl *df, T *x, T *r, cudaStream_t s) {
-    const T *W = df->Q.as<T>();
-    const T *B1 = df->proj == TG_PROJ_MINRES ? df->Y.as<T>() : df->Q.as<T>();
-    const T *B2 = df->proj == TG_PROJ_MINRES ? df->Q.as<T>() : df->AV.as<T>();
+    const T *W, *B1, *B2;
+    proj_data64<T>(df, &W, &B1, &B2);
     return project_impl<T>(op, df, W, B1, B2, x, r, op->n, s);
 }
 
@@ -1069,6 +1078,97 @@ struct CycleOut {
     double rr = 0;
 };
 
+// Cycles on real grids of up to this many points run in one cooperative launch (tg_persist.cuh);
+// beyond, the neighbours' recomputed updates and one block per SM cost more than the launches.
+// us per product, one launch / chain of launches: BiCGStab float64 127^2 7.1 / 21 (plain launches),
+// 511^2 18.5 / 34, 767^2 36 / 40, 79^3 42 / 50, 95^3 67 / 58; float32 + refinement 127^2 6.0 / 20,
+// 639^2 15.9 / 17.8, 71^3 23.6 / 24.8, 79^3 29 / 27; IDR(4) 511^2 28 / 70, 767^2 55 / 79, 95^3 100 / 107,
+// 1023^2 126 / 103.
+template <class T> constexpr int pers_max_rows(bool idr) {
+    return sizeof(T) == 4 ? 6 << 16 : idr ? 13 << 16 : 9 << 16;
+}
+
+// Queues one cooperative launch of a cycle kernel over the whole GPU (fewer blocks than SMs for
+// fewer than 32 points each) and its zeroed barrier word.
+template <class K, class Args>
+static int persist_launch(K kernel, const DevOp &A, const DevOp32 &A32, const Args &a, cudaStream_t s) {
+    TG_CHECK_CUDA(cudaMemsetAsync(a.bar, 0, sizeof(unsigned), s));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(std::max(1, std::min(num_sms(), (A.n + 31) / 32)));
+    cfg.blockDim = dim3(kPersThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeCooperative;
+    at.val.cooperative = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    TG_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kernel, A, A32, a));
+    return TG_OK;
+}
+static int persist_ready(tg_op *op, cudaStream_t s) {
+    // two reduction buffers and the projection's partial sums
+    TG_CHECK(red_ready(op, (size_t)(2 * kPersPart + kPersCols) * num_sms() * sizeof(double), s));
+    return wsx(op, S_BAR, 64);
+}
+
+// Runs the cycle that `a` describes (first launch and continuations); res: the launch's report.
+template <class T>
+static int bicg_persist_run(tg_op *op, const DevOp &A, const DevOp32 &A32, BiPersArgs<T> &a, int n, BiPersOut *res,
+                            cudaStream_t s) {
+    BiVecs<T> w;
+    TG_CHECK(bicg_vecs<T>(op, n, &w));
+    TG_CHECK(wsx(op, S_P2, (size_t)n * sizeof(T)));
+    TG_CHECK(wsx(op, S_V2, (size_t)n * sizeof(T)));
+    TG_CHECK(persist_ready(op, s));
+    a.rh = w.rh; a.p[0] = w.p; a.p[1] = wsp<T>(op, S_P2); a.v[0] = w.v; a.v[1] = wsp<T>(op, S_V2);
+    a.s = w.s; a.t = w.t;
+    a.part = wsp<double>(op, S_PART);
+    a.bar = wsp<unsigned>(op, S_BAR);
+    a.out = reinterpret_cast<BiPersOut *>(wsp<char>(op, S_SMALL) + SmallArea::bistate);
+    a.max_iters = 1024;              // bounds one launch to some tens of milliseconds
+    static_assert(sizeof(BiPersOut) <= SmallArea::dot_out - SmallArea::bistate, "the report fits its slot");
+    *res = BiPersOut{};
+    double xb, fl;
+    op_cost(A, &xb, &fl);
+    auto look = [&]() -> int {
+        TG_CHECK(readback(op, a.out, sizeof(BiPersOut), s));
+        memcpy(res, op->pin.p, sizeof(BiPersOut));
+        return TG_OK;
+    };
+    for (a.first = 1;; a.first = 0) {
+        const int it0 = res->st.iters, ev = prof_begin(s);
+        TG_CHECK(persist_launch(k_bi_persist<T>, A, A32, a, s));
+        if (ev >= 0) TG_CHECK(look());           // the work of a profiled launch is counted by its iterations
+        const double its = res->st.iters - it0;
+        prof_end(ev, P_BI_CYCLE, its * n * (17.0 + 2 * xb / 8) * sizeof(T), its * n * (2 * fl + 26), s);
+        if (ev < 0) TG_CHECK(look());
+        if (res->st.status != 0) break;
+        if (res->st.iters > a.cap) {
+            set_error("BiCGStab cycle exceeded its product cap");
+            return TG_SYNC_TIMEOUT;
+        }
+    }
+    if (res->st.status == kStatusSync) {
+        set_error("a grid barrier of the BiCGStab cycle timed out");
+        return TG_SYNC_TIMEOUT;
+    }
+    return TG_OK;
+}
+
+template <class T>
+static int bicg_persist(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r, int n, double target2, int cap,
+                        CycleOut *out, cudaStream_t s) {
+    BiPersArgs<T> a{};
+    a.x = x; a.r = r; a.target2 = target2; a.cap = cap;
+    BiPersOut o;
+    TG_CHECK(bicg_persist_run<T>(op, A, A32, a, n, &o, s));
+    out->mvps = o.st.mvps;
+    out->iters = o.st.iters;
+    out->status = o.st.status;
+    out->rr = o.st.rr;
+    return TG_OK;
+}
+
 // One BiCGStab cycle on A e = r, updating x and r in place (device-resident scalars).
 // A float32 cycle on a 3D constant-coefficient grid runs in the padded layout of
 // k_bi_pad (rows of pitch P, a multiple of 4 above N, zero padding): x and r are copied in
@@ -1078,6 +1178,9 @@ template <class T>
 static int bicg_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r, int n, double target2, int cap,
                       CycleOut *out, cudaStream_t s, int padded = 0) {
     using D = typename ST<T>::D;
+    if constexpr (sizeof(T) != 16) {
+        if (n <= pers_max_rows<T>(false) && !padded) return bicg_persist<T>(op, A, A32, x, r, n, target2, cap, out, s);
+    }
     if constexpr (std::is_same<T, float>::value) {
         if (A.kind == DK_CD3D && !padded) {
             const size_t np = (size_t)pad_pitch(A.N) * A.N * A.N;
@@ -1231,6 +1334,43 @@ static void hist_push(tg_stats *st, double relres, double rt, int64_t mvps) {
     st->history_len += 1;
 }
 
+// Whether a solve's cycles run whole in one launch each: small real grids and a basis that the
+// launch's own projection takes.
+template <class T>
+static bool whole_cycles(const tg_op *op, const tg_defl *df) {
+    return !op->cplx_ && op->n <= pers_max_rows<T>(false) && (!df || df->kk <= kPersCols);
+}
+
+// One whole cycle (tg_persist.cuh): projection, tolerance, BiCGStab, and the float64 residual of
+// the updated x.  nr: in ||r||, out the norm after the projection; *nr_new, *nb: the residual's.
+template <class T>
+static int bicg_whole(tg_op *op, const DevOp &A, const DevOp32 &A32, const tg_defl *df, const double *b, double *x,
+                      double *r, T *xc, T *rc, double *xbak, const T *W, const T *B1, const T *B2, const SolveCfg &cfg,
+                      int cyc, double floor, int cap, double *nr, double *nb, double *rt, double *nr_new,
+                      CycleOut *co, cudaStream_t s) {
+    BiPersArgs<T> a{};
+    a.whole = 1;
+    a.x = xc; a.r = rc; a.b = b; a.x64 = x; a.r64 = r; a.xbak = xbak;
+    a.W = W; a.B1 = B1; a.B2 = B2;
+    a.kk = df ? df->kk : 0;
+    a.Mp = df ? df->M.as<double>() : nullptr;
+    a.minres = df && df->proj == TG_PROJ_MINRES;
+    a.sched = cfg.ncyc && cyc <= cfg.ncyc;
+    a.nr = *nr; a.nb = *nb; a.rtol = cfg.rtol; a.floor = floor; a.cap = cap;
+    if (a.sched) {
+        a.ex = 1.0 / (cfg.ncyc - cyc + 1);
+        a.pw = pow(cfg.rtol, (double)cyc / cfg.ncyc);
+    }
+    BiPersOut o;
+    TG_CHECK(bicg_persist_run<T>(op, A, A32, a, op->n, &o, s));
+    *co = CycleOut{o.st.mvps, o.st.iters, o.st.status, o.st.rr};
+    *nr = o.nr;
+    *rt = o.rt;
+    *nr_new = sqrt(o.rr);
+    *nb = sqrt(o.bb);
+    return TG_OK;
+}
+
 // r = b - A x (float64 / complex128); returns ||r||, ||b||.
 template <class T>
 static int true_residual(tg_op *op, const DevOp &A, const T *b, const T *x, T *r, double *nr, double *nb, cudaStream_t s) {
@@ -1266,25 +1406,41 @@ static int solve_bicg64(tg_op *op, int transpose, const tg_defl *df, const T *b,
     int status = TG_NOT_CONVERGED;
     if (!std::isfinite(nr)) status = TG_NAN;
     else if (nb == 0.0 || nr <= cfg.rtol * nb) status = TG_OK;
+    const bool whole = whole_cycles<double>(op, df);
     while (status == TG_NOT_CONVERGED) {
         ++cyc;
         const bool sched = cfg.ncyc && cyc <= cfg.ncyc;   // beyond ncyc: finish with rtol ||b|| / ||r||
-        if (df && df->kk > 0) {                                    // step a
-            TG_CHECK(project64<T>(op, df, x, r, s));
-            double rr;
-            TG_CHECK(dot_host<T>(op, r, nullptr, n, &rr, nullptr, s));
-            nr = sqrt(rr);
-        }
-        double rt = sched ? cycle_tol(cfg.rtol, nb, nr, cyc, cfg.ncyc) : cfg.rtol * nb / nr;   // step b
-        hist_push(st, nr / nb, rt, mvps);
         int64_t cap64 = cfg.max_mvps - mvps;
         if (cfg.restart_mvps > 0 && cap64 > cfg.restart_mvps) cap64 = cfg.restart_mvps;
         if (cap64 > INT_MAX / 2) cap64 = INT_MAX / 2;
         CycleOut co;
-        TG_CHECK(bicg_cycle<T>(op, A, A32, x, r, n, (rt * nr) * (rt * nr), (int)cap64, &co, s));   // step c
-        mvps += co.mvps;
-        if (co.status == 4) { status = TG_NAN; break; }
-        TG_CHECK(true_residual<T>(op, A, b, x, r, &nr, &nb, s));
+        if constexpr (std::is_same<T, double>::value) {
+            if (whole) {
+                double rt, nr_new, nb_old = nb;
+                const double *W, *B1, *B2;
+                proj_data64<double>(df, &W, &B1, &B2);
+                TG_CHECK(bicg_whole<double>(op, A, A32, df, b, x, r, x, r, nullptr, W, B1, B2, cfg, cyc, 0.0,
+                                            (int)cap64, &nr, &nb, &rt, &nr_new, &co, s));
+                hist_push(st, nr / nb_old, rt, mvps);
+                mvps += co.mvps;
+                if (co.status == 4) { nb = nb_old; status = TG_NAN; break; }
+                nr = nr_new;
+            }
+        }
+        if (!whole) {
+            if (df && df->kk > 0) {                                    // step a
+                TG_CHECK(project64<T>(op, df, x, r, s));
+                double rr;
+                TG_CHECK(dot_host<T>(op, r, nullptr, n, &rr, nullptr, s));
+                nr = sqrt(rr);
+            }
+            double rt = sched ? cycle_tol(cfg.rtol, nb, nr, cyc, cfg.ncyc) : cfg.rtol * nb / nr;   // step b
+            hist_push(st, nr / nb, rt, mvps);
+            TG_CHECK(bicg_cycle<T>(op, A, A32, x, r, n, (rt * nr) * (rt * nr), (int)cap64, &co, s));   // step c
+            mvps += co.mvps;
+            if (co.status == 4) { status = TG_NAN; break; }
+            TG_CHECK(true_residual<T>(op, A, b, x, r, &nr, &nb, s));
+        }
         if (!std::isfinite(nr)) { status = TG_NAN; break; }
         if (nr <= cfg.rtol * nb) { status = TG_OK; break; }        // step d
         if (mvps >= cfg.max_mvps) break;
@@ -1324,39 +1480,51 @@ static int solve_bicg_ir(tg_op *op, int transpose, const tg_defl *df, const doub
     if (!std::isfinite(nr)) status = TG_NAN;
     else if (nb == 0.0 || nr <= cfg.rtol * nb) status = TG_OK;
     const int g = grid_for(n, 8);
+    const bool whole = whole_cycles<float>(op, df);
     while (status == TG_NOT_CONVERGED) {
         ++cyc;
         const bool sched = cfg.ncyc && cyc <= cfg.ncyc;   // beyond ncyc: finish with rtol ||b|| / ||r||
-        // correction equation A e = r, scaled so that ||r32|| = 1
-        TG_PROF(P_CONVERT, 12.0 * n, n, launch_d2f_scaled(g, s, r, r32, n, 1.0 / nr));
-        TG_CHECK_CUDA(cudaMemsetAsync(e32, 0, (size_t)n * 4, s));
-        double scale = nr;
-        double nrel = 1.0;
-        if (df && df->kk > 0) {
-            TG_CHECK(project_impl<float>(op, df, df->W32.as<float>(), df->B1_32.as<float>(), df->B2_32.as<float>(), e32,
-                                         r32, n, s));
-            double rr;
-            TG_CHECK(dot_host<float>(op, r32, nullptr, n, &rr, nullptr, s));
-            nrel = sqrt(rr);
-        }
-        const double nrp = nrel * scale;    // residual norm after the projection
-        double rt = sched ? cycle_tol(cfg.rtol, nb, nrp, cyc, cfg.ncyc) : cfg.rtol * nb / nrp;
-        if (rt < 1e-6) rt = 1e-6;   // a float32 cycle cannot resolve more; refinement continues
-        hist_push(st, nrp / nb, rt, mvps);
         int64_t cap64 = cfg.max_mvps - mvps;
         // a float32 cycle that stagnates above its target ends after kIrCycleCap products
         const int64_t cyc_cap = cfg.restart_mvps > 0 ? cfg.restart_mvps : kIrCycleCap;
         if (cap64 > cyc_cap) cap64 = cyc_cap;
         if (cap64 > INT_MAX / 2) cap64 = INT_MAX / 2;
         CycleOut co;
-        TG_CHECK(bicg_cycle<float>(op, A, A32, e32, r32, n, (rt * nrel) * (rt * nrel), (int)cap64, &co, s));
-        mvps += co.mvps;
-        // keep x: a float32 correction that does not lower the float64 residual is undone
-        TG_CHECK_CUDA(cudaMemcpyAsync(xbak, x, (size_t)n * 8, cudaMemcpyDeviceToDevice, s));
         const double nr_before = nr;
-        TG_PROF(P_CONVERT, 20.0 * n, 2.0 * n, launch_add_f2d_scaled(g, s, x, e32, n, scale));
-        TG_LAUNCH_CHECK();
-        TG_CHECK(true_residual<double>(op, A, b, x, r, &nr, &nb, s));
+        if (whole) {
+            double rt, nr_new;
+            const double nb_old = nb;
+            TG_CHECK(bicg_whole<float>(op, A, A32, df, b, x, r, e32, r32, xbak, df ? df->W32.as<float>() : nullptr,
+                                       df ? df->B1_32.as<float>() : nullptr, df ? df->B2_32.as<float>() : nullptr, cfg,
+                                       cyc, 1e-6, (int)cap64, &nr, &nb, &rt, &nr_new, &co, s));
+            hist_push(st, nr / nb_old, rt, mvps);
+            mvps += co.mvps;
+            nr = nr_new;
+        } else {
+            // correction equation A e = r, scaled so that ||r32|| = 1
+            TG_PROF(P_CONVERT, 12.0 * n, n, launch_d2f_scaled(g, s, r, r32, n, 1.0 / nr));
+            TG_CHECK_CUDA(cudaMemsetAsync(e32, 0, (size_t)n * 4, s));
+            double scale = nr;
+            double nrel = 1.0;
+            if (df && df->kk > 0) {
+                TG_CHECK(project_impl<float>(op, df, df->W32.as<float>(), df->B1_32.as<float>(), df->B2_32.as<float>(),
+                                             e32, r32, n, s));
+                double rr;
+                TG_CHECK(dot_host<float>(op, r32, nullptr, n, &rr, nullptr, s));
+                nrel = sqrt(rr);
+            }
+            const double nrp = nrel * scale;    // residual norm after the projection
+            double rt = sched ? cycle_tol(cfg.rtol, nb, nrp, cyc, cfg.ncyc) : cfg.rtol * nb / nrp;
+            if (rt < 1e-6) rt = 1e-6;   // a float32 cycle cannot resolve more; refinement continues
+            hist_push(st, nrp / nb, rt, mvps);
+            TG_CHECK(bicg_cycle<float>(op, A, A32, e32, r32, n, (rt * nrel) * (rt * nrel), (int)cap64, &co, s));
+            mvps += co.mvps;
+            // keep x: a float32 correction that does not lower the float64 residual is undone
+            TG_CHECK_CUDA(cudaMemcpyAsync(xbak, x, (size_t)n * 8, cudaMemcpyDeviceToDevice, s));
+            TG_PROF(P_CONVERT, 20.0 * n, 2.0 * n, launch_add_f2d_scaled(g, s, x, e32, n, scale));
+            TG_LAUNCH_CHECK();
+            TG_CHECK(true_residual<double>(op, A, b, x, r, &nr, &nb, s));
+        }
         if (std::isfinite(nr) && nr <= cfg.rtol * nb) { status = TG_OK; break; }
         if (!std::isfinite(nr) || nr >= nr_before || co.status == 4 || co.status == 5) {
             // float32 cannot resolve this system (its rounding times the condition number is
@@ -1413,6 +1581,37 @@ static int idr_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r, 
     D *part = wsp<D>(op, S_PART);
     unsigned *tk = wsp<unsigned>(op, S_TICKET);
     IdrState<D> *st = reinterpret_cast<IdrState<D> *>(wsp<char>(op, S_SMALL) + SmallArea::idr);
+    if constexpr (sizeof(T) != 16) {
+        if (n <= pers_max_rows<T>(true)) {
+            TG_CHECK(persist_ready(op, s));
+            IdrPersArgs<T> a;
+            a.P = P; a.x = x; a.r = r; a.G = G; a.U = U; a.t = t; a.ld = ld;
+            a.part = wsp<double>(op, S_PART);
+            a.bar = wsp<unsigned>(op, S_BAR);
+            a.st = st; a.target2 = target2; a.kappa = kappa; a.s = sd; a.cap = cap;
+            a.max_rounds = 64;           // bounds one launch to a few milliseconds
+            IdrState<double> h{};
+            for (a.first = 1;; a.first = 0) {
+                TG_PROF(P_IDR_CYCLE, 0, 0, TG_CHECK(persist_launch(k_idr_persist<T>, A, A32, a, s)));
+                TG_CHECK(readback(op, st, sizeof(h), s));
+                memcpy(&h, op->pin.p, sizeof(h));
+                if (h.status != 0) break;
+                if ((int64_t)h.rounds * (sd + 1) > (int64_t)cap + 2 * (sd + 1)) {
+                    set_error("IDR cycle exceeded its product cap");
+                    return TG_SYNC_TIMEOUT;
+                }
+            }
+            if (h.status == kStatusSync) {
+                set_error("a grid barrier of the IDR cycle timed out");
+                return TG_SYNC_TIMEOUT;
+            }
+            out->mvps = h.mvps;
+            out->iters = h.rounds;
+            out->status = h.status;
+            out->rr = h.rr;
+            return TG_OK;
+        }
+    }
     const double es = sizeof(T);
     double xb, fl;
     op_cost(A, &xb, &fl);
