@@ -299,77 +299,113 @@ __device__ void hessenberg(T *A, int m, T *Z, T *v) {
 
 // ----------------------------------------------------------------------------- Schur form: shared pieces
 // Cost model of the QR sweeps on this GPU: every float64 warp instruction occupies its SM
-// sub-partition's float64 unit for tens of cycles whatever the number of active lanes, and
-// sqrt / division / hypot are long sequences of them.  So a bulge-chasing step is organised
-// as two phases between two barriers: (1) all warps apply the current transform to the rows
-// it touches (and to part of the Schur vector rows), (2) warp 0 updates the few entries that
-// define the next transform and computes it with one rsqrt (and, real case, one reciprocal),
-// lanes in parallel, while warps 1.. apply the column transform to the remaining rows and
-// Schur vector rows.  Bulge entries that the next transform annihilates are stored as exact
-// zeros, so no clean-up pass is needed.
+// sub-partition's float64 unit for 64 cycles whatever the number of active lanes, and a dependent
+// one waits as long; sqrt and division are sequences of six to seven of them.  So a bulge-chasing
+// step takes as long as the chain of operations from one transform to the next, if nothing else
+// shares that sub-partition's unit.  One step t of a sweep, between two block barriers:
+//   warp 0 (the chain) reads the 3 x 3 (complex 2 x 2) block of transform t and the entry below
+//     it, applies transform t to the one column that defines transform t + 1 (lanes in
+//     parallel), computes transform t + 1 and stores that column's final values;
+//   warp 1 (the window) applies transform t to the few columns and rows next to the diagonal that
+//     step t + 1 reads;
+//   the far warps (2, 3, 5, 6, 7: none shares the chain's sub-partition) apply it to the other
+//     columns, rows and Schur vector rows.
+// The three write disjoint entries; the chain and the window share reads at the start of the step,
+// which a two-warp barrier separates from the window's writes.  Real m = 60: 22 float64
+// operations in the chain, where row phase, column phase and reflector in turn took 2600 cycles a
+// step.
 constexpr unsigned kFull = 0xffffffffu;
+
+// Seeds good to about 2^-20 (rsqrt.approx.ftz.f64, rcp.approx.ftz.f64) and one cubic step each:
+// r (1 + e (1/2 + 3/8 e)) with e = 1 - x r^2 (Halley), r (1 + e + e^2) with e = 1 - x r.  The
+// remaining error is below 2^-58 for x in the normal range.
+__device__ __forceinline__ double rsqrt_seed(double x) {
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    return r;
+}
+__device__ __forceinline__ double rcp_fast(double x) {
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+// 2^-900 < x < 2^900, on the exponent bits
+__device__ __forceinline__ bool mid_range(double x) {
+    return (unsigned)((__double2hiint(x) >> 20) - 123) < 1800u;
+}
+__device__ __forceinline__ void bar_two_warps() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
+
+// lane's place among the far warps' lanes (2, 3, 5, 6, 7), and their number
+constexpr int kFarLanes = 5 * 32;
+__device__ __forceinline__ int far_index() {
+    const int w = threadIdx.x >> 5;
+    return w < 2 || w == 4 ? -1 : 32 * (w < 4 ? w - 2 : w - 3) + (threadIdx.x & 31);
+}
 
 // Complex Givens rotation G = [conj(a) conj(b); -b a] with G [x; y] = [r; 0], r = ||(x, y)||:
 // a = x / r, b = y / r.  Warp-wide call; lanes 0..3 hold x.re, x.im, y.re, y.im in v and
-// write a.re, a.im, b.re, b.im to rs[0..3].  (x, y) = 0 gives the identity.
-__device__ __forceinline__ void givens_warp(double v, double *rs) {
+// write a.re, a.im, b.re, b.im to rs[0..3].  (x, y) = 0 gives the identity.  Returns r.
+__device__ __forceinline__ double givens_warp(double v, double *rs) {
     const int lane = threadIdx.x & 31;
-    double s2 = v * v;
-    s2 += __shfl_xor_sync(kFull, s2, 1);
-    s2 += __shfl_xor_sync(kFull, s2, 2);
-    s2 = __shfl_sync(kFull, s2, 0);
-    double out;
-    if (s2 == 0.0) {
+    auto norm2 = [&](double u) {
+        double q = u * u;
+        q += __shfl_xor_sync(kFull, q, 1);
+        q += __shfl_xor_sync(kFull, q, 2);
+        return __shfl_sync(kFull, q, 0);
+    };
+    double s2 = norm2(v), out, r;
+    if (__double_as_longlong(s2) == 0) {
         out = lane == 0 ? 1.0 : 0.0;
-    } else if (s2 > 1e-280 && s2 < 1e280) {
-        out = v * rsqrt(s2);
+        r = 0.0;
     } else {
-        // scale by the largest component first (no overflow or underflow in the squares)
-        double mx = fabs(v);
-        mx = fmax(mx, __shfl_xor_sync(kFull, mx, 1));
-        mx = fmax(mx, __shfl_xor_sync(kFull, mx, 2));
-        mx = __shfl_sync(kFull, mx, 0);
-        const double w = v * (1.0 / mx);
-        double t2 = w * w;
-        t2 += __shfl_xor_sync(kFull, t2, 1);
-        t2 += __shfl_xor_sync(kFull, t2, 2);
-        t2 = __shfl_sync(kFull, t2, 0);
-        out = w * rsqrt(t2);
+        double u = v, mx = 1.0;
+        if (!mid_range(s2)) {       // scale by the largest component first
+            mx = fabs(v);
+            mx = fmax(mx, __shfl_xor_sync(kFull, mx, 1));
+            mx = fmax(mx, __shfl_xor_sync(kFull, mx, 2));
+            mx = __shfl_sync(kFull, mx, 0);
+            u = v * (1.0 / mx);
+            s2 = norm2(u);
+        }
+        const double r0 = rsqrt_seed(s2), e = fma(-(s2 * r0), r0, 1.0);
+        const double inv = fma(r0, e * fma(0.375, e, 0.5), r0);
+        out = u * inv;
+        r = s2 * inv * mx;
     }
     if (lane < 4) rs[lane] = out;
+    return r;
 }
 
-// Householder reflector (I - tau u u^T), u = (1, u1, u2), mapping (x, y, z) to (beta, 0, 0),
-// beta = -sign(x) ||(x, y, z)||: tau = (beta - x) / beta, u_i = (y, z) / (x - beta).
-// Warp-wide call; lanes 0..2 hold x, y, z in v (z = 0 for a 2-vector); writes tau, u1, u2
-// to hs[0..2].  y = z = 0 gives tau = 0 (the identity).
-__device__ __forceinline__ void house3_warp(double v, double *hs) {
+// Householder reflector I - g w w^T (g = 2 / w^T w) mapping (x, y, z) to (beta, 0, 0),
+// beta = -sign(x) ||(x, y, z)||: w = (x - beta, y, z) and g = 1 / (n2 + ||.|| |x|), n2 the square
+// norm.  Warp-wide, every lane with the same x, y, z; writes w and g w to hs[0..5] and returns
+// beta.  y = z = 0 gives the identity.
+__device__ __forceinline__ double reflect_warp(double x, double y, double z, double *hs) {
     const int lane = threadIdx.x & 31;
-    const double x = __shfl_sync(kFull, v, 0), y = __shfl_sync(kFull, v, 1), z = __shfl_sync(kFull, v, 2);
-    const double sn = y * y + z * z;
-    if (lane == 0) {
-        double tau = 0.0, u1 = 0.0, u2 = 0.0;
-        if (sn != 0.0) {
-            double n2 = x * x + sn;
-            double xs = x, ys = y, zs = z;
-            if (!(n2 > 1e-280 && n2 < 1e280)) {      // rescale (the reflector is scale invariant)
-                const double mx = fmax(fabs(x), fmax(fabs(y), fabs(z)));
-                const double r = 1.0 / mx;
-                xs = x * r; ys = y * r; zs = z * r;
-                n2 = xs * xs + (ys * ys + zs * zs);
-            }
-            const double inv = rsqrt(n2);                  // 1 / ||(x, y, z)||
-            const double beta = -copysign(n2 * inv, xs);
-            const double u0 = xs - beta;
-            const double ru0 = 1.0 / u0;
-            tau = u0 * copysign(inv, xs);                  // -u0 / beta
-            u1 = ys * ru0;
-            u2 = zs * ru0;
-        }
-        hs[0] = tau;
-        hs[1] = u1;
-        hs[2] = u2;
+    double w0 = 0.0, w1 = 0.0, w2 = 0.0, g = 0.0, beta = x, mx = 1.0;
+    double sn = fma(z, z, y * y), n2 = fma(x, x, sn);
+    if (!mid_range(n2)) {               // rescale (the reflector does not depend on the scale)
+        mx = fmax(fabs(x), fmax(fabs(y), fabs(z)));
+        const double r = mx > 0.0 ? 1.0 / mx : 0.0;
+        x *= r; y *= r; z *= r;
+        sn = fma(z, z, y * y);
+        n2 = fma(x, x, sn);
     }
+    if (__double_as_longlong(sn) != 0) {       // tests on the bits: a float64 compare is a link of the chain too
+        const double r0 = rsqrt_seed(n2), h = n2 * r0, e = fma(-h, r0, 1.0);
+        const double alpha = fma(h * e, fma(0.375, e, 0.5), h);
+        g = rcp_fast(fma(alpha, fabs(x), n2));
+        const double bs = -copysign(alpha, x);
+        w0 = x - bs;
+        w1 = y;
+        w2 = z;
+        beta = mx == 1.0 ? bs : bs * mx;
+    }
+    const int c = lane % 3;
+    const double v = c == 0 ? w0 : c == 1 ? w1 : w2, gv = v * g;
+    if (lane < 6) hs[lane] = lane < 3 ? v : gv;
+    return beta;
 }
 
 // ----------------------------------------------------------------------------- real Schur form
@@ -377,8 +413,8 @@ __device__ __forceinline__ void house3_warp(double v, double *hs) {
 // Returns 0 on success, 1 if an eigenvalue failed to converge in 40 m sweeps.
 __device__ int real_schur(double *H, int m, double *Z) {
     __shared__ int hi_s, l_s, status_s, act_s;
-    __shared__ double hs_s[3];
-    __shared__ double x_s, y_s, z_s;
+    __shared__ double hs_s[2][6];      // w and g w of the current and the next reflector
+    __shared__ double win_s[9];
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) { hi_s = m - 1; status_s = 0; }
     __syncthreads();
@@ -478,87 +514,113 @@ __device__ int real_schur(double *H, int m, double *Z) {
             __syncthreads();
             break;
         }
-        if (tid == 0) {
-            double s, t;
+        if (warp == 0) {
+            double sh, t;
             if (its % 10 == 0) {
                 // exceptional shift
                 double w = fabs(H[hi + (size_t)(hi - 1) * m]) + fabs(H[(hi - 1) + (size_t)(hi - 2 >= 0 ? hi - 2 : 0) * m]);
-                s = 1.5 * w + H[hi + (size_t)hi * m];
+                sh = 1.5 * w + H[hi + (size_t)hi * m];
                 t = w * w;
             } else {
                 double a = H[(hi - 1) + (size_t)(hi - 1) * m], b = H[(hi - 1) + (size_t)hi * m];
                 double c = H[hi + (size_t)(hi - 1) * m], d = H[hi + (size_t)hi * m];
-                s = a + d;
+                sh = a + d;
                 t = a * d - b * c;
             }
             // first column of (H - s1 I)(H - s2 I) = H^2 - s H + t I
-            double h00 = H[l + (size_t)l * m], h01 = H[l + (size_t)(l + 1) * m];
-            double h10 = H[(l + 1) + (size_t)l * m], h11 = H[(l + 1) + (size_t)(l + 1) * m];
-            x_s = h00 * h00 + h01 * h10 - s * h00 + t;
-            y_s = h10 * (h00 + h11 - s);
-            z_s = (l + 2 <= hi) ? h10 * H[(l + 2) + (size_t)(l + 1) * m] : 0.0;
+            const double h00 = H[l + (size_t)l * m], h01 = H[l + (size_t)(l + 1) * m];
+            const double h10 = H[(l + 1) + (size_t)l * m], h11 = H[(l + 1) + (size_t)(l + 1) * m];
+            reflect_warp(h00 * h00 + h01 * h10 - sh * h00 + t, h10 * (h00 + h11 - sh),
+                         (l + 2 <= hi) ? h10 * H[(l + 2) + (size_t)(l + 1) * m] : 0.0, hs_s[l & 1]);
         }
         __syncthreads();
-        if (warp == 0) house3_warp(lane == 0 ? x_s : lane == 1 ? y_s : lane == 2 ? z_s : 0.0, hs_s);
-        __syncthreads();
-        for (int kk = l; kk <= hi - 1; ++kk) {
-            const int nr = (kk <= hi - 2) ? 3 : 2;
-            const double tau = hs_s[0], v1 = hs_s[1], v2 = nr == 3 ? hs_s[2] : 0.0;
-            // phase 1: rows kk..kk+nr-1 over columns c0..m-1; Schur vector rows [0, zs)
-            const int c0 = kk > l ? kk - 1 : l;
-            const int ncol = m - c0;
-            const int zs = min(m, max(0, nt - ncol));
-            for (int t = tid; t < ncol + zs; t += nt) {
-                if (t < ncol) {
-                    const int c = c0 + t;
-                    const double h0 = H[kk + (size_t)c * m], h1 = H[kk + 1 + (size_t)c * m];
-                    const double h2 = nr == 3 ? H[kk + 2 + (size_t)c * m] : 0.0;
-                    const double s = tau * fma(v2, h2, fma(v1, h1, h0));
-                    const bool bulge = kk > l && c == kk - 1;     // entries the reflector annihilates
-                    H[kk + (size_t)c * m] = h0 - s;
-                    H[kk + 1 + (size_t)c * m] = bulge ? 0.0 : fma(-s, v1, h1);
-                    if (nr == 3) H[kk + 2 + (size_t)c * m] = bulge ? 0.0 : fma(-s, v2, h2);
-                } else {
-                    double *zr = Z + (t - ncol);
-                    const double h0 = zr[(size_t)kk * m], h1 = zr[(size_t)(kk + 1) * m];
-                    const double h2 = nr == 3 ? zr[(size_t)(kk + 2) * m] : 0.0;
-                    const double s = tau * fma(v2, h2, fma(v1, h1, h0));
-                    zr[(size_t)kk * m] = h0 - s;
-                    zr[(size_t)(kk + 1) * m] = fma(-s, v1, h1);
-                    if (nr == 3) zr[(size_t)(kk + 2) * m] = fma(-s, v2, h2);
-                }
-            }
-            __syncthreads();
-            // phase 2: columns kk..kk+nr-1 of rows 0..rmax and of Schur vector rows [zs, m)
-            const int rmax = (kk + 3 < hi) ? kk + 3 : hi;
+        const int far = far_index();
+        for (int k = l; k <= hi - 1; ++k) {
+            const double *hb = hs_s[k & 1];
+            const bool r3 = k <= hi - 2;               // the last reflector has two rows
+            const double w0 = hb[0], w1 = hb[1], w2 = r3 ? hb[2] : 0.0, g0 = hb[3], g1 = hb[4], g2 = r3 ? hb[5] : 0.0;
             if (warp == 0) {
-                // rows kk+1..rmax (at most 3, one per lane), then the next reflector from
-                // column kk of those rows
-                const int r = kk + 1 + lane;
-                double xv = 0.0;
-                if (lane < 3 && r <= rmax) {
-                    double *hr = H + r;
-                    const double h0 = hr[(size_t)kk * m], h1 = hr[(size_t)(kk + 1) * m];
-                    const double h2 = nr == 3 ? hr[(size_t)(kk + 2) * m] : 0.0;
-                    const double s = tau * fma(v2, h2, fma(v1, h1, h0));
-                    xv = h0 - s;
-                    hr[(size_t)kk * m] = xv;
-                    hr[(size_t)(kk + 1) * m] = fma(-s, v1, h1);
-                    if (nr == 3) hr[(size_t)(kk + 2) * m] = fma(-s, v2, h2);
+                // rows k+1..k+3 of column k after reflector k: lane 3 (r - 1) + j holds row k + r of
+                // column k + j after the row part, then the column part for column k
+                const int r = 1 + lane / 3, j = lane % 3;
+                const bool ok = lane < 9 && (j < 2 || r3);
+                const double *col = H + (size_t)(ok ? k + j : k) * m;
+                const double b0 = ok ? col[k] : 0.0, b1 = ok ? col[k + 1] : 0.0, b2 = ok && r3 ? col[k + 2] : 0.0;
+                const double b3 = ok && j == 2 && k + 3 <= hi ? col[k + 3] : 0.0;
+                bar_two_warps();
+                const double c = fma(g2, b2, fma(g1, b1, g0 * b0));
+                const double v = fma(r == 1 ? -w1 : r == 2 ? -w2 : 0.0, c, r == 1 ? b1 : r == 2 ? b2 : b3);
+                const int base = lane < 9 ? 3 * (lane / 3) : 0;
+                const double v0 = __shfl_sync(kFull, v, base), v1 = __shfl_sync(kFull, v, base + 1),
+                             v2 = __shfl_sync(kFull, v, base + 2);
+                const double xr = fma(-fma(v2, w2, fma(v1, w1, v0 * w0)), g0, v0);
+                const double x = __shfl_sync(kFull, xr, 0), y = __shfl_sync(kFull, xr, 3), z = __shfl_sync(kFull, xr, 6);
+                double *ck = H + (size_t)k * m;
+                if (k < hi - 1) {
+                    const double beta = reflect_warp(x, y, k + 3 <= hi ? z : 0.0, hs_s[(k + 1) & 1]);
+                    if (lane == 0) {
+                        ck[k + 1] = beta;
+                        ck[k + 2] = 0.0;
+                        if (k + 3 <= hi) ck[k + 3] = 0.0;
+                    }
+                } else if (lane == 0) {
+                    ck[hi] = x;
+                }
+            } else if (warp == 1) {
+                // columns k..k+4 of rows k..k+2, then columns k..k+2 of rows k..k+3 (column k below
+                // the diagonal is the chain's)
+                const int c = k + lane;
+                const bool oc = lane < 5 && c < m;
+                double *col = H + (size_t)(oc ? c : k) * m;
+                double h0 = 0.0, h1 = 0.0, h2 = 0.0;
+                if (oc) {
+                    h0 = col[k];
+                    h1 = col[k + 1];
+                    if (r3) h2 = col[k + 2];
+                }
+                const double below = k + 3 <= hi ? H[k + 3 + (size_t)(k + 2) * m] : 0.0;
+                bar_two_warps();
+                const double q = fma(g2, h2, fma(g1, h1, g0 * h0));
+                h0 = fma(-q, w0, h0);
+                h1 = fma(-q, w1, h1);
+                h2 = fma(-q, w2, h2);
+                if (lane < (r3 ? 3 : 2)) {
+                    win_s[lane] = h0;
+                    win_s[3 + lane] = h1;
+                    win_s[6 + lane] = h2;
+                } else if (oc) {
+                    col[k] = h0;
+                    col[k + 1] = h1;
+                    if (r3) col[k + 2] = h2;
                 }
                 __syncwarp();
-                if (kk < hi - 1) house3_warp(xv, hs_s);      // z = 0 when kk + 3 > hi
-            } else {
-                const int nh = kk + 1;            // rows 0..kk
-                const int nz = m - zs;
-                for (int t = tid - 32; t < nh + nz; t += nt - 32) {
-                    double *hr = t < nh ? H + t : Z + zs + (t - nh);
-                    const double h0 = hr[(size_t)kk * m], h1 = hr[(size_t)(kk + 1) * m];
-                    const double h2 = nr == 3 ? hr[(size_t)(kk + 2) * m] : 0.0;
-                    const double s = tau * fma(v2, h2, fma(v1, h1, h0));
-                    hr[(size_t)kk * m] = h0 - s;
-                    hr[(size_t)(kk + 1) * m] = fma(-s, v1, h1);
-                    if (nr == 3) hr[(size_t)(kk + 2) * m] = fma(-s, v2, h2);
+                const int r = lane;                    // row k + r
+                if (r < 4 && k + r <= hi) {
+                    const double m0 = r < 3 ? win_s[3 * r] : 0.0, m1 = r < 3 ? win_s[3 * r + 1] : 0.0;
+                    const double m2 = !r3 ? 0.0 : r < 3 ? win_s[3 * r + 2] : below;
+                    const double p = fma(m2, w2, fma(m1, w1, m0 * w0));
+                    if (r == 0) H[k + (size_t)k * m] = fma(-p, g0, m0);
+                    H[k + r + (size_t)(k + 1) * m] = fma(-p, g1, m1);
+                    if (r3) H[k + r + (size_t)(k + 2) * m] = fma(-p, g2, m2);
+                }
+            } else if (far >= 0) {
+                const int na = max(0, m - k - 5), total = na + k + m;
+                for (int t = far; t < total; t += kFarLanes) {
+                    if (t < na) {                      // row part, columns k+5..
+                        double *col = H + (size_t)(k + 5 + t) * m + k;
+                        const double h0 = col[0], h1 = col[1], h2 = r3 ? col[2] : 0.0;
+                        const double q = fma(g2, h2, fma(g1, h1, g0 * h0));
+                        col[0] = fma(-q, w0, h0);
+                        col[1] = fma(-q, w1, h1);
+                        if (r3) col[2] = fma(-q, w2, h2);
+                    } else {                           // column part, rows 0..k-1 and the Schur vectors
+                        double *row = (t < na + k ? H + (t - na) : Z + (t - na - k)) + (size_t)k * m;
+                        const double h0 = row[0], h1 = row[m], h2 = r3 ? row[2 * (size_t)m] : 0.0;
+                        const double q = fma(h2, w2, fma(h1, w1, h0 * w0));
+                        row[0] = fma(-q, g0, h0);
+                        row[m] = fma(-q, g1, h1);
+                        if (r3) row[2 * (size_t)m] = fma(-q, g2, h2);
+                    }
                 }
             }
             __syncthreads();
@@ -574,7 +636,8 @@ __device__ __forceinline__ double cabs1(cplx a) { return fabs(a.re) + fabs(a.im)
 
 __device__ int complex_schur(cplx *H, int m, cplx *Z) {
     __shared__ int hi_s, l_s, act_s, status_s;
-    __shared__ double rs_s[4];      // a.re, a.im, b.re, b.im of the current rotation
+    __shared__ double rs_s[2][4];   // a.re, a.im, b.re, b.im of the current and the next rotation
+    __shared__ cplx win_s[6];
     __shared__ cplx x_s, y_s;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) { hi_s = m - 1; status_s = 0; }
@@ -644,57 +707,73 @@ __device__ int complex_schur(cplx *H, int m, cplx *Z) {
             y_s = H[(l + 1) + (size_t)l * m];
         }
         __syncthreads();
-        if (warp == 0) givens_warp(lane == 0 ? x_s.re : lane == 1 ? x_s.im : lane == 2 ? y_s.re : y_s.im, rs_s);
+        if (warp == 0) givens_warp(lane == 0 ? x_s.re : lane == 1 ? x_s.im : lane == 2 ? y_s.re : lane == 3 ? y_s.im : 0.0, rs_s[l & 1]);
         __syncthreads();
-        for (int kk = l; kk <= hi - 1; ++kk) {
-            const cplx a = mkc(rs_s[0], rs_s[1]), b = mkc(rs_s[2], rs_s[3]);
-            // phase 1: rows kk, kk+1 over columns c0..m-1 (H <- G H); Schur vector rows [0, zs)
-            const int c0 = kk > l ? kk - 1 : l;
-            const int ncol = m - c0;
-            const int zs = min(m, max(0, nt - ncol));
-            for (int t = tid; t < ncol + zs; t += nt) {
-                if (t < ncol) {
-                    const int c = c0 + t;
-                    const cplx h1 = H[kk + (size_t)c * m], h2 = H[kk + 1 + (size_t)c * m];
-                    H[kk + (size_t)c * m] = conj(a) * h1 + conj(b) * h2;
-                    // the entry the rotation annihilates (the bulge) is stored as an exact zero
-                    H[kk + 1 + (size_t)c * m] = (kk > l && c == kk - 1) ? mkc(0.0, 0.0) : a * h2 - b * h1;
-                } else {
-                    cplx *zr = Z + (t - ncol);
-                    const cplx h1 = zr[(size_t)kk * m], h2 = zr[(size_t)(kk + 1) * m];
-                    zr[(size_t)kk * m] = h1 * a + h2 * b;
-                    zr[(size_t)(kk + 1) * m] = h2 * conj(a) - h1 * conj(b);
-                }
-            }
-            __syncthreads();
-            // phase 2: columns kk, kk+1 (M <- M G^H) of rows 0..rmax and Schur vector rows [zs, m)
-            const int rmax = (kk + 2 < hi) ? kk + 2 : hi;
+        const int far = far_index();
+        for (int k = l; k <= hi - 1; ++k) {
+            const double *rb = rs_s[k & 1];
+            const cplx a = mkc(rb[0], rb[1]), b = mkc(rb[2], rb[3]);
+            const int part = lane & 1;                 // real or imaginary part of a lane's value
+            // (u p + v q) part, four operations
+            auto part_of = [&](cplx u, cplx p, cplx v, cplx q) {
+                return fma(part ? v.re : -v.im, q.im,
+                           fma(part ? v.im : v.re, q.re, fma(part ? u.re : -u.im, p.im, (part ? u.im : u.re) * p.re)));
+            };
             if (warp == 0) {
-                // rows kk+1..rmax: lane q < 8 computes one real part: column kk + (q >> 2),
-                // row kk + 1 + ((q >> 1) & 1), real (q even) or imaginary part; then the next
-                // rotation from column kk of rows kk+1, kk+2 (lanes 0..3)
-                const int q = lane & 7;
-                const int r = kk + 1 + ((q >> 1) & 1);
-                const int col = kk + (q >> 2);
-                const bool live = lane < 8 && r <= rmax;
-                double val = 0.0;
-                if (live) {
-                    const cplx h1 = H[r + (size_t)kk * m], h2 = H[r + (size_t)(kk + 1) * m];
-                    const cplx o = (q >> 2) == 0 ? h1 * a + h2 * b : h2 * conj(a) - h1 * conj(b);
-                    val = (q & 1) ? o.im : o.re;
+                // lanes 0..3: row k + 1, columns k and k + 1 after the row part; then column k of
+                // rows k + 1 (lanes 0, 1) and k + 2 (lanes 2, 3) after the column part
+                const cplx *col = H + (size_t)(k + ((lane >> 1) & 1)) * m + k;
+                const cplx hu = col[0], hl = col[1];
+                const cplx below = k + 2 <= hi ? H[k + 2 + (size_t)(k + 1) * m] : mkc(0.0, 0.0);
+                bar_two_warps();
+                const double w = part_of(hl, a, hu, -b);
+                const cplx r0 = mkc(__shfl_sync(kFull, w, 0), __shfl_sync(kFull, w, 1)),
+                           r1 = mkc(__shfl_sync(kFull, w, 2), __shfl_sync(kFull, w, 3));
+                const bool second = lane & 2;
+                const double xv = part_of(second ? mkc(0.0, 0.0) : r0, a, second ? below : r1, b);
+                cplx *ck = H + (size_t)k * m;
+                if (k < hi - 1) {
+                    const double r = givens_warp(xv, rs_s[(k + 1) & 1]);
+                    if (lane == 0) {
+                        ck[k + 1] = mkc(r, 0.0);
+                        ck[k + 2] = mkc(0.0, 0.0);
+                    }
+                } else if (lane < 2) {
+                    reinterpret_cast<double *>(ck + hi)[lane] = xv;
                 }
+            } else if (warp == 1) {
+                // rows k, k+1 of columns k..k+2, then columns k, k+1 of rows k..k+2 (column k below
+                // the diagonal is the chain's): lane 4 c + 2 o + part
+                const int c = lane >> 2, o = (lane >> 1) & 1;
+                const bool oc = c < 3 && k + c < m;
+                const cplx *col = H + (size_t)(oc ? k + c : k) * m + k;
+                const cplx hu = col[0], hl = col[1];
+                const cplx below = k + 2 <= hi ? H[k + 2 + (size_t)(k + 1) * m] : mkc(0.0, 0.0);
+                bar_two_warps();
+                const double v = o == 0 ? part_of(hu, conj(a), hl, conj(b)) : part_of(hl, a, hu, -b);
+                if (oc && c < 2) reinterpret_cast<double *>(win_s + 2 * o + c)[part] = v;
+                else if (oc) reinterpret_cast<double *>(H + (size_t)(k + c) * m + k + o)[part] = v;
                 __syncwarp();
-                if (live) reinterpret_cast<double *>(H + r + (size_t)col * m)[q & 1] = val;
-                __syncwarp();
-                if (kk < hi - 1) givens_warp(val, rs_s);
-            } else {
-                const int nh = kk + 1;            // rows 0..kk
-                const int nz = m - zs;
-                for (int t = tid - 32; t < nh + nz; t += nt - 32) {
-                    cplx *hr = t < nh ? H + t : Z + zs + (t - nh);
-                    const cplx h1 = hr[(size_t)kk * m], h2 = hr[(size_t)(kk + 1) * m];
-                    hr[(size_t)kk * m] = h1 * a + h2 * b;
-                    hr[(size_t)(kk + 1) * m] = h2 * conj(a) - h1 * conj(b);
+                const int r = c;                       // row k + r, output column k + o
+                if (r < 3 && k + r <= hi && !(r > 0 && o == 0)) {
+                    const cplx m0 = r < 2 ? win_s[2 * r] : mkc(0.0, 0.0), m1 = r < 2 ? win_s[2 * r + 1] : below;
+                    const double u = o == 0 ? part_of(m0, a, m1, b) : part_of(m1, conj(a), m0, -conj(b));
+                    reinterpret_cast<double *>(H + (size_t)(k + o) * m + k + r)[part] = u;
+                }
+            } else if (far >= 0) {
+                const int na = max(0, m - k - 3), total = na + k + m;
+                for (int t = far; t < total; t += kFarLanes) {
+                    if (t < na) {                      // row part (H <- G H), columns k+3..
+                        cplx *col = H + (size_t)(k + 3 + t) * m + k;
+                        const cplx h1 = col[0], h2 = col[1];
+                        col[0] = conj(a) * h1 + conj(b) * h2;
+                        col[1] = a * h2 - b * h1;
+                    } else {                           // column part (M <- M G^H), rows 0..k-1 and Schur vectors
+                        cplx *row = (t < na + k ? H + (t - na) : Z + (t - na - k)) + (size_t)k * m;
+                        const cplx h1 = row[0], h2 = row[m];
+                        row[0] = h1 * a + h2 * b;
+                        row[m] = h2 * conj(a) - h1 * conj(b);
+                    }
                 }
             }
             __syncthreads();

@@ -6,7 +6,7 @@
 namespace tg {
 
 constexpr int kSmallThreads = 256;
-constexpr int kGdrThreads = 128;                 // GMRES-DR restart kernel block
+constexpr int kGdrThreads = 256;                 // GMRES-DR restart kernel block (eight warps)
 constexpr size_t kGdrSmemMax = 210 * 1024;       // shared memory for W and Z when they fit
 
 struct GdrInfo {
