@@ -2803,12 +2803,14 @@ struct BatchCoarse {
 // reduction slices, the instance table, and the captured iteration graph.
 namespace tg {
 struct BatchAll {
-    DBuf rh, p, v, s, t, r32, e32, r64, rsave, part, st, ctl, ticket, small, seg, colb, colx;
+    DBuf rh, p, v, s, t, r32, e32, r64, rsave, part, st, ctl, ticket, small, seg, colb, colx, map, map_res;
     PinBuf pin;
     cudaStream_t stream = nullptr;
     cudaGraphExec_t graph = nullptr;
     int graph_gx = 0;
-    int gx = 0;                    // tuned blocks per instance (0: not tuned yet)
+    int gx = 0;                    // tuned blocks per instance, on average (0: not tuned yet)
+    int blocks = 0;                // blocks of the iteration graph (the table in map)
+    int blocks_res = 0;            // blocks of the refinement kernels (map_res)
     double tune_us[8] = {0};       // us per iteration of each candidate
     int tune_gx[8] = {0};
     int ntune = 0;
@@ -2890,6 +2892,27 @@ namespace tg {
 // per handle by timing the iteration graph for each candidate (the autotuner).
 constexpr int kMrPartW = 4 * kBatchR > 32 * kBatchR ? 4 * kBatchR : 32 * kBatchR;
 
+// Blocks of a batched launch at most: the partial sums' room (2 KB a block).
+static int batch_max_blocks(const tg_batch *b) { return std::max(16384, b->count + 4096); }
+
+// Gives the instances about `total` blocks in proportion to their points (one at least, and no
+// more than there are groups of 256 points) and copies the blocks' table to buf.
+static int batch_map(tg_batch *b, int64_t total, DBuf &buf, int *blocks) {
+    double points = 0.0;
+    for (const tg_op *op : b->ops) points += op->n;
+    std::vector<int4> map;
+    for (int i = 0; i < b->count; ++i) {
+        const int64_t n = b->ops[i]->n, want = (int64_t)(total * (n / points) + 0.5);
+        const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(want, (n + kThreads - 1) / kThreads)), first = (int)map.size();
+        for (int k = 0; k < nb; ++k) map.push_back(make_int4(i, k, nb, first));
+    }
+    *blocks = (int)map.size();
+    TG_CHECK(buf.ensure(map.size() * sizeof(int4)));
+    TG_CHECK_CUDA(cudaMemcpyAsync(buf.p, map.data(), map.size() * sizeof(int4), cudaMemcpyHostToDevice, b->all.stream));
+    TG_CHECK_CUDA(cudaStreamSynchronize(b->all.stream));
+    return TG_OK;
+}
+
 static int batch_all_ready(tg_batch *b) {
     constexpr int R = kBatchR;
     BatchAll &A = b->all;
@@ -2903,7 +2926,8 @@ static int batch_all_ready(tg_batch *b) {
     TG_CHECK(A.e32.ensure(tot * 4));
     TG_CHECK(A.rsave.ensure(tot * 4));
     TG_CHECK(A.r64.ensure(tot * 8));
-    TG_CHECK(A.part.ensure((size_t)b->count * 128 * kMrPartW * 8));   // up to 128 blocks per instance
+    TG_CHECK(A.part.ensure((size_t)batch_max_blocks(b) * kMrPartW * 8));
+    TG_CHECK(A.map.ensure((size_t)batch_max_blocks(b) * sizeof(int4)));
     TG_CHECK(A.st.ensure((size_t)b->count * R * sizeof(BiState<double>)));
     TG_CHECK(A.ctl.ensure((size_t)b->count * sizeof(MrCtl)));
     // target2, inv, scale (R each), norms (2 R), cvec, dvec (32 R each), capv (R) per instance
@@ -2915,6 +2939,8 @@ static int batch_all_ready(tg_batch *b) {
         TG_CHECK(A.ticket.ensure((size_t)b->count * sizeof(unsigned)));
         TG_CHECK_CUDA(cudaMemsetAsync(A.ticket.p, 0, (size_t)b->count * sizeof(unsigned), A.stream));
     }
+    // refinement kernels: 8 blocks per SM in all
+    if (!A.blocks_res) TG_CHECK(batch_map(b, (int64_t)num_sms() * 8, A.map_res, &A.blocks_res));
     return TG_OK;
 }
 
@@ -2928,6 +2954,7 @@ static MrBatchPtrs batch_ptrs(tg_batch *b, int cap) {
     P.st = A.st.as<BiState<double>>();
     P.ctl = A.ctl.as<MrCtl>();
     P.ticket = A.ticket.as<unsigned>();
+    P.place = A.map.as<int4>();
     P.part = A.part.as<double>();
     P.partw = kMrPartW;
     P.target2 = sm;
@@ -2941,10 +2968,10 @@ static MrBatchPtrs batch_ptrs(tg_batch *b, int cap) {
     return P;
 }
 
-static void batch_iters_all(tg_batch *b, const MrBatchPtrs &P, int gx, int iters, cudaStream_t s) {
+static void batch_iters_all(tg_batch *b, const MrBatchPtrs &P, int iters, cudaStream_t s) {
     constexpr int R = kBatchR;
     BatchAll &A = b->all;
-    const dim3 grid(gx, b->count);
+    const dim3 grid(A.blocks);
     float *rh = A.rh.as<float>(), *p = A.p.as<float>(), *v = A.v.as<float>(), *sv = A.s.as<float>(),
           *t = A.t.as<float>(), *r = A.r32.as<float>(), *x = A.e32.as<float>();
     for (int it = 0; it < iters; ++it) {
@@ -2963,10 +2990,11 @@ static int batch_graph(tg_batch *b, int gx) {
         cudaGraphExecDestroy(A.graph);
         A.graph = nullptr;
     }
+    TG_CHECK(batch_map(b, (int64_t)gx * b->count, A.map, &A.blocks));
     const MrBatchPtrs P = batch_ptrs(b, 0);
     cudaGraph_t graph;
     TG_CHECK_CUDA(cudaStreamBeginCapture(A.stream, cudaStreamCaptureModeThreadLocal));
-    batch_iters_all(b, P, gx, kGraphIters, A.stream);
+    batch_iters_all(b, P, kGraphIters, A.stream);
     TG_CHECK_CUDA(cudaStreamEndCapture(A.stream, &graph));
     const cudaError_t e = cudaGraphInstantiate(&A.graph, graph, 0);
     cudaGraphDestroy(graph);
@@ -2990,7 +3018,7 @@ static int batch_tune(tg_batch *b) {
     const size_t tot = (size_t)b->total;
     cudaStream_t s = A.stream;
     TG_CHECK_CUDA(cudaMemcpyAsync(A.rsave.p, A.r32.p, tot * 4, cudaMemcpyDeviceToDevice, s));
-    const int cands[] = {8, 16, 32, 64, 128};
+    const int cands[] = {8, 16, 32, 64, 128, 256, 512};
     std::vector<double> zeros((size_t)b->count * R, 0.0);
     MrBatchPtrs P0 = batch_ptrs(b, INT_MAX / 2);
     P0.capv = nullptr;
@@ -3001,12 +3029,13 @@ static int batch_tune(tg_batch *b) {
     int best_gx = 16;
     A.ntune = 0;
     for (int gx : cands) {
+        if (gx > 8 && (int64_t)gx * b->count > batch_max_blocks(b) - b->count) break;
         TG_CHECK_CUDA(cudaMemcpyAsync(P0.target2, zeros.data(), zeros.size() * 8, cudaMemcpyHostToDevice, s));
         TG_CHECK_CUDA(cudaMemcpyAsync(A.r32.p, A.rsave.p, tot * 4, cudaMemcpyDeviceToDevice, s));
         TG_CHECK_CUDA(cudaMemsetAsync(A.e32.p, 0, tot * 4, s));
-        launch(k_mrb_bi_init<R>, dim3(gx, b->count), kThreads, 0, s, A.r32.as<float>(), A.rh.as<float>(), A.p.as<float>(), P0);
-        TG_LAUNCH_CHECK();
         TG_CHECK(batch_graph(b, gx));
+        launch(k_mrb_bi_init<R>, A.blocks, kThreads, 0, s, A.r32.as<float>(), A.rh.as<float>(), A.p.as<float>(), P0);
+        TG_LAUNCH_CHECK();
         TG_CHECK_CUDA(cudaGraphLaunch(A.graph, s));          // warm
         TG_CHECK_CUDA(cudaEventRecord(e0, s));
         TG_CHECK_CUDA(cudaGraphLaunch(A.graph, s));
@@ -3058,8 +3087,9 @@ static int batch_solve_all(tg_batch *b, const double *Bv, double *X, const Solve
     TG_CHECK_CUDA(cudaMemcpyAsync(A.seg.p, seg.data(), seg.size() * sizeof(MrSeg), cudaMemcpyHostToDevice, s));
     bool any_defl = false;
     for (const MrSeg &g : seg) any_defl |= g.kk > 0;
-    const int gres = 16;                                          // blocks per instance, refinement kernels
+    const int gres = A.blocks_res;                                // blocks of the refinement kernels
     MrBatchPtrs P = batch_ptrs(b, 0);
+    P.place = A.map_res.as<int4>();
     double *hp = reinterpret_cast<double *>(A.pin.p);
     const size_t BR = (size_t)count * R;
     std::vector<double> nr(BR), nb(BR), nrel(BR), hv(BR), nr_before(BR), hcap(BR);
@@ -3072,7 +3102,7 @@ static int batch_solve_all(tg_batch *b, const double *Bv, double *X, const Solve
     std::vector<int> status(BR);
     auto residual = [&]() -> int {
         TG_PROF(P_RESIDUAL, (3.0 * 8) * b->total, 12.0 * b->total,
-                launch(k_mrb_residual<R>, dim3(gres, count), kThreads, 0, s, Bv, X, A.r64.as<double>(), P));
+                launch(k_mrb_residual<R>, gres, kThreads, 0, s, Bv, X, A.r64.as<double>(), P));
         TG_LAUNCH_CHECK();
         TG_CHECK(batch_readback(b, P.norms, (size_t)count * 2 * R * 8));
         for (int i = 0; i < count; ++i)
@@ -3101,16 +3131,16 @@ static int batch_solve_all(tg_batch *b, const double *Bv, double *X, const Solve
         for (size_t c = 0; c < BR; ++c) hv[c] = status[c] == TG_NOT_CONVERGED ? 1.0 / nr[c] : 0.0;
         TG_CHECK_CUDA(cudaMemcpyAsync(P.inv, hv.data(), BR * 8, cudaMemcpyHostToDevice, s));
         TG_PROF(P_CONVERT, 16.0 * b->total, b->total,
-                launch(k_mrb_scale<R>, dim3(gres, count), kThreads, 0, s, A.r64.as<double>(), A.r32.as<float>(),
+                launch(k_mrb_scale<R>, gres, kThreads, 0, s, A.r64.as<double>(), A.r32.as<float>(),
                                                                          A.e32.as<float>(), P));
         TG_LAUNCH_CHECK();
         for (size_t c = 0; c < BR; ++c) nrel[c] = 1.0;
         if (any_defl) {
             const size_t smem = ((size_t)32 * 128 + 128 * R) * sizeof(float);
             TG_CHECK(set_smem<float>((const void *)k_mrb_proj_dots<R>, smem));
-            TG_PROF(P_GEMV_T, 0, 0, launch(k_mrb_proj_dots<R>, dim3(gres, count), kThreads, smem, s, A.r32.as<float>(), P));
+            TG_PROF(P_GEMV_T, 0, 0, launch(k_mrb_proj_dots<R>, gres, kThreads, smem, s, A.r32.as<float>(), P));
             TG_PROF(P_SMALL, 0, 0, launch(k_mrb_small<R>, count, 256, 0, s, P));
-            TG_PROF(P_PROJ, 0, 0, launch(k_mrb_proj_update<R>, dim3(gres, count), kThreads, 0, s, A.e32.as<float>(),
+            TG_PROF(P_PROJ, 0, 0, launch(k_mrb_proj_update<R>, gres, kThreads, 0, s, A.e32.as<float>(),
                                                                                             A.r32.as<float>(), P));
             TG_LAUNCH_CHECK();
             TG_CHECK(batch_readback(b, P.norms, (size_t)count * 2 * R * 8));
@@ -3143,14 +3173,13 @@ static int batch_solve_all(tg_batch *b, const double *Bv, double *X, const Solve
         TG_CHECK_CUDA(cudaMemcpyAsync(const_cast<double *>(P.capv), hcap.data(), BR * 8, cudaMemcpyHostToDevice, s));
         cap64 = capmax;
         if (A.gx == 0) TG_CHECK(batch_tune(b));           // once per handle, on the first cycle's r32
-        const int gx = A.gx;
+        TG_CHECK(batch_graph(b, A.gx));                   // with the blocks' table of its launches
         TG_CHECK_CUDA(cudaMemcpyAsync(P.target2, hv.data(), BR * 8, cudaMemcpyHostToDevice, s));
         const MrBatchPtrs Pc = batch_ptrs(b, (int)cap64);
         TG_PROF(P_BI_INIT, 12.0 * b->total, 2.0 * b->total,
-                launch(k_mrb_bi_init<R>, dim3(gx, count), kThreads, 0, s, A.r32.as<float>(), A.rh.as<float>(),
+                launch(k_mrb_bi_init<R>, A.blocks, kThreads, 0, s, A.r32.as<float>(), A.rh.as<float>(),
                                                                         A.p.as<float>(), Pc));
         TG_LAUNCH_CHECK();
-        TG_CHECK(batch_graph(b, gx));
         int graphs = 0;
         while (true) {
             TG_CHECK_CUDA(cudaGraphLaunch(A.graph, s));
@@ -3177,7 +3206,7 @@ static int batch_solve_all(tg_batch *b, const double *Bv, double *X, const Solve
         }
         TG_CHECK_CUDA(cudaMemcpyAsync(P.scale, hv.data(), BR * 8, cudaMemcpyHostToDevice, s));
         TG_PROF(P_CONVERT, 12.0 * b->total, 2.0 * b->total,
-                launch(k_mrb_add<R>, dim3(gres, count), kThreads, 0, s, X, A.e32.as<float>(), P));
+                launch(k_mrb_add<R>, gres, kThreads, 0, s, X, A.e32.as<float>(), P));
         TG_LAUNCH_CHECK();
         TG_CHECK(residual());
         // a correction that raised the float64 residual kIrGrowth-fold is undone (x -= ||r|| e)
@@ -3193,7 +3222,7 @@ static int batch_solve_all(tg_batch *b, const double *Bv, double *X, const Solve
         if (undo) {
             TG_CHECK_CUDA(cudaMemcpyAsync(P.scale, hv.data(), BR * 8, cudaMemcpyHostToDevice, s));
             TG_PROF(P_CONVERT, 12.0 * b->total, 2.0 * b->total,
-                    launch(k_mrb_add<R>, dim3(gres, count), kThreads, 0, s, X, A.e32.as<float>(), P));
+                    launch(k_mrb_add<R>, gres, kThreads, 0, s, X, A.e32.as<float>(), P));
             TG_LAUNCH_CHECK();
             TG_CHECK(residual());
         }

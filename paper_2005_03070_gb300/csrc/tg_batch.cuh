@@ -1,10 +1,11 @@
 // Batched multi-instance kernels: many independent instances (each its own operator,
 // deflation basis and R = 8 right-hand sides stored point-major) advanced together, one
-// launch per phase for all of them.  Launch grid (gx, B): blockIdx.y selects the instance,
-// its gx blocks stride over the instance's points, so instances of very different sizes
-// share one launch and the hardware block scheduler balances them.  Reductions are per
-// instance: block partials in a per-instance slice of `part`, the last of the instance's gx
-// blocks (per-instance ticket) adds them in block order (deterministic) and updates that
+// launch per phase for all of them.  A table gives every block its instance and its place among
+// that instance's blocks, which stride over the instance's points.  An instance gets blocks in
+// proportion to its points: with the same number each, the blocks of the largest of a few
+// instances (127^2 .. 511^2: 16 times the points) ran on alone (153 us an iteration for six).
+// Reductions are per instance: block partials in a per-instance slice of `part`, the last of the
+// instance's blocks (per-instance ticket) adds them in block order (deterministic) and updates that
 // instance's R column states.  An instance whose columns have all finished their cycle
 // returns at once (MrCtl::active == 0), so the lock-step host loop wastes no bandwidth on
 // it.  Per point: float32 BiCGStab with the R columns' scalars in device memory (a column
@@ -33,7 +34,8 @@ struct MrBatchPtrs {
     BiState<double> *st;        // [B][R]
     MrCtl *ctl;                 // [B]
     unsigned *ticket;           // [B]
-    double *part;               // [B][gx][partw]
+    const int4 *place;          // per block: instance, block in it, its blocks, its first block
+    double *part;               // [block][partw]
     int partw;                  // doubles per block slot (>= 4 R, >= kk R)
     double *target2;            // [B][R] (negative: the column sits out this cycle)
     double *inv;                // [B][R]
@@ -44,42 +46,70 @@ struct MrBatchPtrs {
     const double *capv = nullptr;   // [B][R] per-column product caps (nullptr: cap for all)
 };
 
-template <int R>
-__device__ __forceinline__ double *seg_part(const MrBatchPtrs &P) {
-    return P.part + (size_t)blockIdx.y * gridDim.x * P.partw;
+struct MrPlace {
+    int b, blk, nblk;
+    double *slice;              // the instance's partial sums
+};
+__device__ __forceinline__ MrPlace mr_place(const MrBatchPtrs &P) {
+    const int4 v = P.place[blockIdx.x];
+    return {v.x, v.y, v.z, P.part + (size_t)v.w * P.partw};
+}
+// Returns true in the last of nblk blocks to arrive (as last_block, for a part of the grid).
+__device__ __forceinline__ bool last_of(unsigned *ticket, int nblk) {
+    __shared__ bool am_last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) am_last = atomicAdd(ticket, 1u) == (unsigned)nblk - 1;
+    __syncthreads();
+    return am_last;
 }
 
 // Block reduction of ND x R per-thread float partials into the instance's slice:
 // slice[block * partw + d * R + r] (double), fixed order: warp shuffle tree, then warps in order.
 template <int ND, int R>
-__device__ __forceinline__ void mrb_block_store(float (&acc)[ND][R], double *slice, int partw, double *red) {
+__device__ __forceinline__ void mrb_block_store(float (&acc)[ND][R], const MrPlace &L, int partw, double *red) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float v[ND * R];
 #pragma unroll
     for (int d = 0; d < ND; ++d)
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-            float s = warp_sum(acc[d][r]);
-            if (lane == 0) red[(warp * ND + d) * R + r] = (double)s;
-        }
+        for (int r = 0; r < R; ++r) v[d * R + r] = acc[d][r];
+    const float s = warp_sums<ND * R>(v);             // lane l: value l
+    if (lane < ND * R) red[warp * ND * R + lane] = (double)s;
     __syncthreads();
     for (int q = threadIdx.x; q < ND * R; q += blockDim.x) {
         double s = red[q];
         for (int w = 1; w < (int)(blockDim.x >> 5); ++w) s += red[w * ND * R + q];
-        slice[(size_t)blockIdx.x * partw + q] = s;
+        L.slice[(size_t)L.blk * partw + q] = s;
     }
 }
 
+// Totals of the instance's NQ values: each warp takes NQ / 8 of them, their loads in flight
+// together, and reduces them in one exchange.
 template <int NQ>
-__device__ __forceinline__ void mrb_final(const double *slice, int partw, double *tot, unsigned *ticket) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int q = warp; q < NQ; q += nw) {
-        double s = 0.0;
-        for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(slice + (size_t)b * partw + q);
-        s = warp_sum(s);
-        if (lane == 0) tot[q] = s;
-    }
+__device__ __forceinline__ void mrb_final(const MrPlace &L, int partw, double *tot, unsigned *ticket) {
+    constexpr int PW = NQ / (kThreads / 32);
+    static_assert(NQ % (kThreads / 32) == 0 && (PW & (PW - 1)) == 0, "a power of two of values per warp");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double s[PW];
+#pragma unroll
+    for (int u = 0; u < PW; ++u) s[u] = 0.0;
+#pragma unroll 2
+    for (int b = lane; b < L.nblk; b += 32)
+#pragma unroll
+        for (int u = 0; u < PW; ++u) s[u] += __ldcg(L.slice + (size_t)b * partw + warp * PW + u);
+    const double r = warp_sums<PW>(s);
+    if (lane < PW) tot[warp * PW + lane] = r;
     __syncthreads();
     if (threadIdx.x == 0) *ticket = 0u;
+}
+
+// the number of running columns, from the R threads that hold one each
+template <int R>
+__device__ __forceinline__ void mrb_active(bool running, MrCtl *ctl) {
+    static_assert(R <= 32, "the columns' threads are in one warp");
+    const unsigned m = __ballot_sync((R == 32 ? 0u : (1u << (R & 31))) - 1u, running);
+    if (threadIdx.x == 0) ctl->active = __popc(m);
 }
 
 // ----------------------------------------------------------------------------- BiCGStab phases
@@ -87,7 +117,8 @@ template <int R>
 __global__ void __launch_bounds__(kThreads) k_mrb_bi_init(const float *__restrict__ r, float *__restrict__ rh,
                                                            float *__restrict__ p, MrBatchPtrs P) {
     pdl_wait();
-    const int b = blockIdx.y;
+    const MrPlace L = mr_place(P);
+    const int b = L.b;
     const MrSeg &S = P.seg[b];
     const int n = S.op.n;
     r += S.off; rh += S.off; p += S.off;
@@ -97,21 +128,22 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_init(const float *__restric
     float acc[1][R];
 #pragma unroll
     for (int q = 0; q < R; ++q) acc[0][q] = 0.f;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+    for (int j = L.blk * blockDim.x + threadIdx.x; j < n; j += L.nblk * blockDim.x) {
         VecR<R> a = ldR<R>(r, j);
         stR<R>(rh, j, a);
         stR<R>(p, j, a);
 #pragma unroll
         for (int q = 0; q < R; ++q) acc[0][q] = fmaf(a.v[q], a.v[q], acc[0][q]);
     }
-    double *slice = seg_part<R>(P);
-    mrb_block_store<1, R>(acc, slice, P.partw, red);
-    if (last_block(P.ticket + b)) {
-        mrb_final<R>(slice, P.partw, tot, P.ticket + b);
-        if (threadIdx.x == 0) {
-            int active = 0;
+    mrb_block_store<1, R>(acc, L, P.partw, red);
+    if (last_of(P.ticket + b, L.nblk)) {
+        mrb_final<R>(L, P.partw, tot, P.ticket + b);
+        // a thread per column here and in the kernels below: one thread for all R took 15 us an
+        // iteration (divisions and float64 compares are chains of 64-clock instructions)
+        if (threadIdx.x < R) {
+            const int q = threadIdx.x;
             const double *t2 = P.target2 + (size_t)b * R;
-            for (int q = 0; q < R; ++q) {
+            {
                 BiState<double> &s = st[q];
                 const double rho = tot[q];
                 s.rho = rho; s.rr = rho; s.ss = 0.0; s.target2 = t2[q]; s.div2 = 1e16 * rho;   // 1e8-fold growth
@@ -123,9 +155,8 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_init(const float *__restric
                 else if (rho <= t2[q]) s.status = 1;
                 else if (fabs(rho) < kTiny) s.status = 2;
                 else s.status = 0;
-                active += s.status == 0;
+                mrb_active<R>(s.status == 0, P.ctl + b);
             }
-            P.ctl[b].active = active;
         }
     }
 }
@@ -134,7 +165,8 @@ template <int R>
 __global__ void __launch_bounds__(kThreads) k_mrb_bi_v(const float *__restrict__ p, const float *__restrict__ rh,
                                                         float *__restrict__ v, MrBatchPtrs P) {
     pdl_wait();
-    const int b = blockIdx.y;
+    const MrPlace L = mr_place(P);
+    const int b = L.b;
     if (P.ctl[b].active == 0) return;
     const MrSeg &S = P.seg[b];
     const DevOp op = S.op;
@@ -150,7 +182,7 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_v(const float *__restrict__
 #pragma unroll
     for (int q = 0; q < R; ++q) acc[0][q] = 0.f;
     const int n = op.n;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+    for (int j = L.blk * blockDim.x + threadIdx.x; j < n; j += L.nblk * blockDim.x) {
         // every column's A p is stored: a column that has left the cycle never reads its v, s
         // or t again (its x and r are frozen; the next cycle starts from p = r), so its
         // values need not be preserved, and the old values are not read
@@ -161,14 +193,13 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_v(const float *__restrict__
             if (on[q]) acc[0][q] = fmaf(h.v[q], y.v[q], acc[0][q]);
         stR<R>(v, j, y);
     }
-    double *slice = seg_part<R>(P);
-    mrb_block_store<1, R>(acc, slice, P.partw, red);
-    if (last_block(P.ticket + b)) {
-        mrb_final<R>(slice, P.partw, tot, P.ticket + b);
-        if (threadIdx.x == 0) {
-            for (int q = 0; q < R; ++q) {
-                BiState<double> &s = st[q];
-                if (s.status != 0) continue;
+    mrb_block_store<1, R>(acc, L, P.partw, red);
+    if (last_of(P.ticket + b, L.nblk)) {
+        mrb_final<R>(L, P.partw, tot, P.ticket + b);
+        if (threadIdx.x < R) {
+            const int q = threadIdx.x;
+            BiState<double> &s = st[q];
+            if (s.status == 0) {
                 const double sigma = tot[q];
                 s.mvps += 1;
                 if (!isfinite(sigma)) s.status = 4;
@@ -183,7 +214,8 @@ template <int R>
 __global__ void __launch_bounds__(kThreads) k_mrb_bi_s(const float *__restrict__ r, const float *__restrict__ v,
                                                         float *__restrict__ s, MrBatchPtrs P) {
     pdl_wait();
-    const int b = blockIdx.y;
+    const MrPlace L = mr_place(P);
+    const int b = L.b;
     if (P.ctl[b].active == 0) return;
     const MrSeg &S = P.seg[b];
     const int n = S.op.n;
@@ -201,7 +233,7 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_s(const float *__restrict__
     float acc[1][R];
 #pragma unroll
     for (int q = 0; q < R; ++q) acc[0][q] = 0.f;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+    for (int j = L.blk * blockDim.x + threadIdx.x; j < n; j += L.nblk * blockDim.x) {
         VecR<R> a = ldR<R>(r, j), bb = ldR<R>(v, j), o;
 #pragma unroll
         for (int q = 0; q < R; ++q) {
@@ -210,14 +242,13 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_s(const float *__restrict__
         }
         stR<R>(s, j, o);
     }
-    double *slice = seg_part<R>(P);
-    mrb_block_store<1, R>(acc, slice, P.partw, red);
-    if (last_block(P.ticket + b)) {
-        mrb_final<R>(slice, P.partw, tot, P.ticket + b);
-        if (threadIdx.x == 0) {
-            for (int q = 0; q < R; ++q) {
-                BiState<double> &c = st[q];
-                if (c.status != 0) continue;
+    mrb_block_store<1, R>(acc, L, P.partw, red);
+    if (last_of(P.ticket + b, L.nblk)) {
+        mrb_final<R>(L, P.partw, tot, P.ticket + b);
+        if (threadIdx.x < R) {
+            const int q = threadIdx.x;
+            BiState<double> &c = st[q];
+            if (c.status == 0) {
                 const double ss = tot[q];
                 c.ss = ss;
                 if (!isfinite(ss)) c.status = 4;
@@ -233,7 +264,8 @@ template <int R>
 __global__ void __launch_bounds__(kThreads) k_mrb_bi_t(const float *__restrict__ s, const float *__restrict__ rh,
                                                         float *__restrict__ t, MrBatchPtrs P) {
     pdl_wait();
-    const int b = blockIdx.y;
+    const MrPlace L = mr_place(P);
+    const int b = L.b;
     if (P.ctl[b].active == 0) return;
     const MrSeg &S = P.seg[b];
     const DevOp op = S.op;
@@ -251,7 +283,7 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_t(const float *__restrict__
 #pragma unroll
         for (int q = 0; q < R; ++q) acc[d][q] = 0.f;
     const int n = op.n;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+    for (int j = L.blk * blockDim.x + threadIdx.x; j < n; j += L.nblk * blockDim.x) {
         VecR<R> y = applyR<R>(op, o32, j, s);
         VecR<R> sv = ldR<R>(s, j), h = ldR<R>(rh, j);     // t stored for every column, as in k_mrb_bi_v
 #pragma unroll
@@ -264,14 +296,13 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_t(const float *__restrict__
         }
         stR<R>(t, j, y);
     }
-    double *slice = seg_part<R>(P);
-    mrb_block_store<4, R>(acc, slice, P.partw, red);
-    if (last_block(P.ticket + b)) {
-        mrb_final<4 * R>(slice, P.partw, tot, P.ticket + b);
-        if (threadIdx.x == 0) {
-            for (int q = 0; q < R; ++q) {
-                BiState<double> &c = st[q];
-                if (c.status != 0 || c.half) continue;
+    mrb_block_store<4, R>(acc, L, P.partw, red);
+    if (last_of(P.ticket + b, L.nblk)) {
+        mrb_final<4 * R>(L, P.partw, tot, P.ticket + b);
+        if (threadIdx.x < R) {
+            const int q = threadIdx.x;
+            BiState<double> &c = st[q];
+            if (c.status == 0 && !c.half) {
                 c.mvps += 1;
                 const double ts = tot[q], tt = tot[R + q], rs = tot[2 * R + q], rt = tot[3 * R + q];
                 if (!isfinite(tt) || !isfinite(ts)) c.status = 4;
@@ -294,7 +325,8 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_x(float *__restrict__ x, fl
                                                         const float *__restrict__ t, const float *__restrict__ v,
                                                         MrBatchPtrs P) {
     pdl_wait();
-    const int b = blockIdx.y;
+    const MrPlace L = mr_place(P);
+    const int b = L.b;
     if (P.ctl[b].active == 0) return;
     const MrSeg &S = P.seg[b];
     const int n = S.op.n;
@@ -320,7 +352,7 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_x(float *__restrict__ x, fl
     float acc[1][R];
 #pragma unroll
     for (int q = 0; q < R; ++q) acc[0][q] = 0.f;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+    for (int j = L.blk * blockDim.x + threadIdx.x; j < n; j += L.nblk * blockDim.x) {
         VecR<R> xv = ldR<R>(x, j), pv = ldR<R>(p, j), sv = ldR<R>(s, j), tv = ldR<R>(t, j), vv = ldR<R>(v, j);
         VecR<R> rv;
         if (full) {
@@ -346,13 +378,12 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_x(float *__restrict__ x, fl
         stR<R>(r, j, rv);
         stR<R>(p, j, pv);
     }
-    double *slice = seg_part<R>(P);
-    mrb_block_store<1, R>(acc, slice, P.partw, red);
-    if (last_block(P.ticket + b)) {
-        mrb_final<R>(slice, P.partw, tot, P.ticket + b);
-        if (threadIdx.x == 0) {
-            int active = 0;
-            for (int q = 0; q < R; ++q) {
+    mrb_block_store<1, R>(acc, L, P.partw, red);
+    if (last_of(P.ticket + b, L.nblk)) {
+        mrb_final<R>(L, P.partw, tot, P.ticket + b);
+        if (threadIdx.x < R) {
+            const int q = threadIdx.x;
+            {
                 BiState<double> &c = st[q];
                 if (c.status == 0 && c.half) {
                     c.rr = c.ss;
@@ -370,9 +401,8 @@ __global__ void __launch_bounds__(kThreads) k_mrb_bi_x(float *__restrict__ x, fl
                     else if (fabs(c.rho_next) < kTiny) c.status = 2;
                     else if (c.mvps >= c.cap) c.status = 3;
                 }
-                active += c.status == 0;
+                mrb_active<R>(c.status == 0, P.ctl + b);
             }
-            P.ctl[b].active = active;
         }
     }
 }
@@ -383,7 +413,8 @@ template <int R>
 __global__ void __launch_bounds__(kThreads) k_mrb_residual(const double *__restrict__ B, const double *__restrict__ X,
                                                             double *__restrict__ r64, MrBatchPtrs P) {
     pdl_wait();
-    const int b = blockIdx.y;
+    const MrPlace L = mr_place(P);
+    const int b = L.b;
     const MrSeg &S = P.seg[b];
     const DevOp op = S.op;
     B += S.off; X += S.off; r64 += S.off;
@@ -394,7 +425,7 @@ __global__ void __launch_bounds__(kThreads) k_mrb_residual(const double *__restr
 #pragma unroll
     for (int q = 0; q < R; ++q) acc[0][q] = acc[1][q] = 0.0;
     const int n = op.n;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+    for (int j = L.blk * blockDim.x + threadIdx.x; j < n; j += L.nblk * blockDim.x) {
 #pragma unroll
         for (int q = 0; q < R; ++q) {
             const double ax = apply_real_d(op, j, [&](int jj) { return X[(size_t)jj * R + q]; });
@@ -413,14 +444,13 @@ __global__ void __launch_bounds__(kThreads) k_mrb_residual(const double *__restr
             if (lane == 0) red[(warp * 2 + d) * R + q] = s2;
         }
     __syncthreads();
-    double *slice = seg_part<R>(P);
     for (int q = threadIdx.x; q < 2 * R; q += blockDim.x) {
         double s2 = red[q];
         for (int w = 1; w < (int)(blockDim.x >> 5); ++w) s2 += red[w * 2 * R + q];
-        slice[(size_t)blockIdx.x * P.partw + q] = s2;
+        L.slice[(size_t)L.blk * P.partw + q] = s2;
     }
-    if (last_block(P.ticket + b)) {
-        mrb_final<2 * R>(slice, P.partw, tot, P.ticket + b);
+    if (last_of(P.ticket + b, L.nblk)) {
+        mrb_final<2 * R>(L, P.partw, tot, P.ticket + b);
         for (int q = threadIdx.x; q < 2 * R; q += blockDim.x) P.norms[(size_t)b * 2 * R + q] = tot[q];
     }
 }
@@ -430,12 +460,13 @@ template <int R>
 __global__ void k_mrb_scale(const double *__restrict__ r64, float *__restrict__ r32, float *__restrict__ e32,
                             MrBatchPtrs P) {
     pdl_wait();
-    const int b = blockIdx.y;
+    const MrPlace L = mr_place(P);
+    const int b = L.b;
     const MrSeg &S = P.seg[b];
     const size_t tot = (size_t)S.op.n * R;
     r64 += S.off; r32 += S.off; e32 += S.off;
     const double *inv = P.inv + (size_t)b * R;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < tot; e += (size_t)gridDim.x * blockDim.x) {
+    for (size_t e = L.blk * (size_t)blockDim.x + threadIdx.x; e < tot; e += (size_t)L.nblk * blockDim.x) {
         r32[e] = (float)(r64[e] * inv[e % R]);
         e32[e] = 0.f;
     }
@@ -445,12 +476,13 @@ __global__ void k_mrb_scale(const double *__restrict__ r64, float *__restrict__ 
 template <int R>
 __global__ void k_mrb_add(double *__restrict__ X, const float *__restrict__ e32, MrBatchPtrs P) {
     pdl_wait();
-    const int b = blockIdx.y;
+    const MrPlace L = mr_place(P);
+    const int b = L.b;
     const MrSeg &S = P.seg[b];
     const size_t tot = (size_t)S.op.n * R;
     X += S.off; e32 += S.off;
     const double *scale = P.scale + (size_t)b * R;
-    for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < tot; e += (size_t)gridDim.x * blockDim.x) {
+    for (size_t e = L.blk * (size_t)blockDim.x + threadIdx.x; e < tot; e += (size_t)L.nblk * blockDim.x) {
         const double sc = scale[e % R];
         if (sc != 0.0) X[e] = fma(sc, (double)e32[e], X[e]);
     }
@@ -463,7 +495,8 @@ template <int R>
 __global__ void __launch_bounds__(kThreads) k_mrb_proj_dots(const float *__restrict__ r, MrBatchPtrs P) {
     pdl_wait();
     constexpr int kChunk = 128;
-    const int b = blockIdx.y;
+    const MrPlace L = mr_place(P);
+    const int b = L.b;
     const MrSeg &S = P.seg[b];
     const int k = S.kk, n = S.op.n;
     if (k == 0) return;
@@ -476,7 +509,7 @@ __global__ void __launch_bounds__(kThreads) k_mrb_proj_dots(const float *__restr
     const int nent = k * R;
     float acc = 0.f;                                       // entry threadIdx.x (< nent)
     const int c = threadIdx.x / R, q = threadIdx.x % R;
-    for (int j0 = blockIdx.x * kChunk; j0 < n; j0 += gridDim.x * kChunk) {
+    for (int j0 = L.blk * kChunk; j0 < n; j0 += L.nblk * kChunk) {
         __syncthreads();
         for (int e = threadIdx.x; e < k * kChunk; e += blockDim.x) {
             const int cc = e / kChunk, jj = e % kChunk;
@@ -490,13 +523,12 @@ __global__ void __launch_bounds__(kThreads) k_mrb_proj_dots(const float *__restr
             for (int jj = 0; jj < kChunk; ++jj) acc = fmaf(wc[jj], rs[jj * R + q], acc);
         }
     }
-    double *slice = seg_part<R>(P);
-    if (threadIdx.x < nent) slice[(size_t)blockIdx.x * P.partw + threadIdx.x] = (double)acc;
-    if (last_block(P.ticket + b)) {
+    if (threadIdx.x < nent) L.slice[(size_t)L.blk * P.partw + threadIdx.x] = (double)acc;
+    if (last_of(P.ticket + b, L.nblk)) {
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
         for (int e = warp; e < nent; e += nw) {
             double s = 0.0;
-            for (int bb = lane; bb < (int)gridDim.x; bb += 32) s += __ldcg(slice + (size_t)bb * P.partw + e);
+            for (int bb = lane; bb < L.nblk; bb += 32) s += __ldcg(L.slice + (size_t)bb * P.partw + e);
             s = warp_sum(s);
             if (lane == 0) tot1[e] = s;
         }
@@ -529,7 +561,8 @@ template <int R>
 __global__ void __launch_bounds__(kThreads) k_mrb_proj_update(float *__restrict__ e, float *__restrict__ r,
                                                                MrBatchPtrs P) {
     pdl_wait();
-    const int b = blockIdx.y;
+    const MrPlace L = mr_place(P);
+    const int b = L.b;
     const MrSeg &S = P.seg[b];
     const int k = S.kk, n = S.op.n;
     if (k == 0) return;
@@ -547,7 +580,7 @@ __global__ void __launch_bounds__(kThreads) k_mrb_proj_update(float *__restrict_
     float acc[1][R];
 #pragma unroll
     for (int q = 0; q < R; ++q) acc[0][q] = 0.f;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
+    for (int j = L.blk * blockDim.x + threadIdx.x; j < n; j += L.nblk * blockDim.x) {
         VecR<R> ev = ldR<R>(e, j), rv = ldR<R>(r, j);
         for (int c = 0; c < k; ++c) {
             const float b1 = S.B1[(size_t)c * n + j], b2 = S.B2[(size_t)c * n + j];
@@ -562,10 +595,9 @@ __global__ void __launch_bounds__(kThreads) k_mrb_proj_update(float *__restrict_
 #pragma unroll
         for (int q = 0; q < R; ++q) acc[0][q] = fmaf(rv.v[q], rv.v[q], acc[0][q]);
     }
-    double *slice = seg_part<R>(P);
-    mrb_block_store<1, R>(acc, slice, P.partw, red);
-    if (last_block(P.ticket + b)) {
-        mrb_final<R>(slice, P.partw, tot, P.ticket + b);
+    mrb_block_store<1, R>(acc, L, P.partw, red);
+    if (last_of(P.ticket + b, L.nblk)) {
+        mrb_final<R>(L, P.partw, tot, P.ticket + b);
         for (int q = threadIdx.x; q < R; q += blockDim.x) P.norms[(size_t)b * 2 * R + q] = tot[q];
     }
 }

@@ -3,7 +3,7 @@
 // with float4 loads; the batched kernels of tg_batch.cuh are built on them.
 #pragma once
 
-#include "tg_kernels.cuh"
+#include "tg_arnoldi.cuh"
 
 namespace tg {
 
