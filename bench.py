@@ -94,12 +94,11 @@ PAPER_RUNS["ex1_511_cubic"] = dict(PAPER_RUNS["ex1_511"], interp="cubic", coarse
 L2_BYTES = 129 * 1024 * 1024
 FP64_PEAK_TFLOPS = 152 * 4 * 2070e6 / 1e12     # 152 SMs x 2 FP64 FMA/clk x 2 flops per FMA x 2070 MHz
 NOMINAL_HBM_GBS = 8000.0                         # the ~8 TB/s nominal HBM3e figure the 70% target refers to
-# DRAM bytes (read + write) per launch over algorithmic bytes per launch, per kernel class,
-# from an ncu capture of a smaller case of the same kernel (profiles/gemv_t_pipe_cd3d191.md:
-# k_gemv_t_pipe<double>, (150.95 + 3.6) MB over 150.9 MB);
-# the traffic of a full-size launch is this ratio times its algorithmic bytes (the traffic
-# grows in proportion to rows x columns).  Remove an entry when its kernel changes.
-NCU_TRAFFIC_RATIO = {"gemv_t": 1.024}
+# DRAM bytes (read + write) per launch over algorithmic bytes per launch, per kernel class, from
+# an ncu capture of a smaller case of the same kernel: the traffic of a full-size launch is this
+# ratio times its algorithmic bytes (it grows in proportion to rows x columns).  An entry goes
+# when its kernel changes.
+NCU_TRAFFIC_RATIO = {}
 
 
 def dgemm_tflops(dev, n=4096, reps=5):

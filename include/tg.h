@@ -295,8 +295,9 @@ int tg_kappa_gradient(const tg_op *op, const void *x, const void *lambda, void *
  *   larger m falls back to one instance per host thread), then prolongs and factors each
  *   basis on `threads` host threads; tg_batch_solve replays the 8-iteration BiCGStab
  *   sequence of all instances as one CUDA graph until every column of the cycle has
- *   finished.  The graph's blocks per instance are chosen on the first solve of a handle
- *   by timing the candidates 8, 16, 32, 64, 128 on the first cycle (tg_batch_tuning).
+ *   finished.  Blocks go to the instances in proportion to their points; the number of blocks
+ *   is chosen on the first solve of a handle by timing the candidates 8, 16, .. 512 blocks per
+ *   instance on average on the first cycle (tg_batch_tuning).
  *   A float32 correction that raises a column's float64 residual more than 4-fold is undone
  *   and that column's cycle cap halved; a column that no float32 cycle can advance finishes
  *   with float64 BiCGStab(-Proj) cycles on its instance's operator and basis
@@ -312,7 +313,7 @@ int tg_batch_setup(tg_batch *b, const void *rhs, int m, int k, int nev, double r
 int tg_batch_solve(tg_batch *b, const void *rhs, void *x, double rtol, int ncyc, int restart_mvps,
                    int64_t max_mvps, int threads, tg_stats *stats, void *stream);
 int tg_destroy_batch(tg_batch *b);
-/* The autotuner's choice for the batched iteration graph: blocks per instance and its
+/* The autotuner's choice for the batched iteration graph: blocks per instance (average) and its
  * time per iteration (microseconds, all instances and columns), and every candidate's
  * (ncand entries of cand_blocks / cand_us, at most 8; any pointer may be NULL).  Zero
  * blocks before the first tg_batch_solve of the handle.                               */
