@@ -2251,7 +2251,7 @@ static int gmresdr_impl(tg_op *op, int transpose, const void *b_fine, int m, int
     TG_CHECK(wsx(op, S_GWI, (size_t)m * 8));
     TG_CHECK(wsx(op, S_GORD, (size_t)m * 4));
     TG_CHECK(wsx(op, S_GERES, (size_t)m * 8));
-    TG_CHECK(wsx(op, S_GWORK, ((size_t)(m + 1) * m + 2 * (size_t)m * m + 3 * (size_t)m + 4) * hs));
+    TG_CHECK(wsx(op, S_GWORK, ((size_t)(m + 1) * m + (size_t)m * m + 3 * (size_t)m + 4) * hs));
     TG_CHECK(wsx(op, S_GY, (size_t)m * m * 16));
     TG_CHECK(wsx(op, S_GG, (size_t)m * m * 16));
     TG_CHECK(wsx(op, S_GINFO, sizeof(GdrInfo)));
@@ -2495,7 +2495,7 @@ static int rayleigh_ritz(tg_op *op, const T *S, const T *W, size_t ld, int n, in
     TG_CHECK(wsx(op, S_AE_WI, (size_t)m * 8));
     TG_CHECK(wsx(op, S_AE_ORD, (size_t)m * 4));
     TG_CHECK(wsx(op, S_AE_ERES, (size_t)m * 8));
-    TG_CHECK(wsx(op, S_AE_WORK, ((size_t)(m + 1) * m + 2 * (size_t)m * m + 3 * (size_t)m + 4) * sizeof(T)));
+    TG_CHECK(wsx(op, S_AE_WORK, ((size_t)(m + 1) * m + (size_t)m * m + 3 * (size_t)m + 4) * sizeof(T)));
     TG_CHECK(wsx(op, S_AE_YW, (size_t)m * m * 16));
     TG_CHECK(wsx(op, S_AE_GW, (size_t)m * m * 16));
     TG_CHECK(wsx(op, S_AE_INFO, sizeof(GdrInfo)));
@@ -2678,7 +2678,7 @@ extern "C" int tg_harmonic_ritz(const void *Hbar, int m, int k, int complex_, vo
         (rc = z.ensure((m + 1) * es)) || (rc = P.ensure((size_t)(m + 1) * (m + 2) * es)) ||
         (rc = Hn.ensure((size_t)(m + 1) * m * es)) || (rc = cn.ensure((m + 2) * es)) || (rc = th.ensure(2 * m * 8)) ||
         (rc = wr.ensure(m * 8)) || (rc = wi.ensure(m * 8)) || (rc = ord.ensure(m * 4)) || (rc = er.ensure(m * 8)) ||
-        (rc = work.ensure(((size_t)(m + 1) * m + 2 * (size_t)m * m + 3 * m + 4) * es)) ||
+        (rc = work.ensure(((size_t)(m + 1) * m + (size_t)m * m + 3 * m + 4) * es)) ||
         (rc = yw.ensure((size_t)m * m * 16)) || (rc = gw.ensure((size_t)m * m * 16)) || (rc = inf.ensure(sizeof(GdrInfo))))
         return rc;
     TG_CHECK_CUDA(cudaMemsetAsync(c.p, 0, (m + 1) * es, s));
@@ -3354,7 +3354,7 @@ static int batch_setup_all(tg_batch *b, const double *R0, int m, int k, int nev,
         TG_CHECK(I.ceres.ensure((size_t)m * 8));
         TG_CHECK(I.cP.ensure((size_t)(m + 1) * (m + 2) * 8));
         TG_CHECK(I.ccn.ensure((size_t)(m + 2) * 8));
-        TG_CHECK(I.cwork.ensure(((size_t)(m + 1) * m + 2 * (size_t)m * m + 3 * (size_t)m + 4) * 8));
+        TG_CHECK(I.cwork.ensure(((size_t)(m + 1) * m + (size_t)m * m + 3 * (size_t)m + 4) * 8));
         TG_CHECK(I.cyw.ensure((size_t)m * m * 16));
         TG_CHECK(I.cgw.ensure((size_t)m * m * 16));
         TG_CHECK(I.cYc.ensure((size_t)nc * (k + 2) * 8));

@@ -40,6 +40,9 @@ template <> struct Cx<double> {
     __device__ static double zero() { return 0.0; }
     __device__ static double one() { return 1.0; }
     __device__ static double sc(double s, double a) { return s * a; }
+    __device__ static double mac(double s, double a, double b) { return fma(a, b, s); }        // s + a b
+    __device__ static double macc(double s, double a, double b) { return fma(a, b, s); }       // s + conj(a) b
+    __device__ static double nmac(double s, double a, double b) { return fma(-a, b, s); }      // s - a b
 };
 template <> struct Cx<cplx> {
     __device__ static cplx cj(cplx a) { return conj(a); }
@@ -50,252 +53,22 @@ template <> struct Cx<cplx> {
     __device__ static cplx zero() { return {0.0, 0.0}; }
     __device__ static cplx one() { return {1.0, 0.0}; }
     __device__ static cplx sc(double s, cplx a) { return s * a; }
+    // four fused operations; s + a * b takes six (the sum of two products, then s)
+    __device__ static cplx mac(cplx s, cplx a, cplx b) {
+        return {fma(a.re, b.re, fma(-a.im, b.im, s.re)), fma(a.re, b.im, fma(a.im, b.re, s.im))};
+    }
+    __device__ static cplx macc(cplx s, cplx a, cplx b) {
+        return {fma(a.re, b.re, fma(a.im, b.im, s.re)), fma(a.re, b.im, fma(-a.im, b.re, s.im))};
+    }
+    __device__ static cplx nmac(cplx s, cplx a, cplx b) {
+        return {fma(-a.re, b.re, fma(a.im, b.im, s.re)), fma(-a.re, b.im, fma(-a.im, b.re, s.im))};
+    }
 };
 
 __device__ __forceinline__ double add(double a, double b) { return a + b; }
 __device__ __forceinline__ cplx add(cplx a, cplx b) { return a + b; }
 __device__ __forceinline__ double subt(double a, double b) { return a - b; }
 __device__ __forceinline__ cplx subt(cplx a, cplx b) { return a - b; }
-
-// Householder vector for x[0..len-1] (strided): v with v[0] = 1 and tau such that
-// (I - tau v v^H) x = beta e_1.  Written to v[], returns tau (0 if x is already beta e_1).
-template <class T>
-__device__ T house(const T *x, int stride, int len, T *v, T *beta_out) {
-    double nrm2 = 0.0;
-    for (int i = 1; i < len; ++i) nrm2 += Cx<T>::ab2(x[i * stride]);
-    T x0 = x[0];
-    if (nrm2 == 0.0) {
-        v[0] = Cx<T>::one();
-        for (int i = 1; i < len; ++i) v[i] = Cx<T>::zero();
-        *beta_out = x0;
-        return Cx<T>::zero();
-    }
-    double a0 = sqrt(Cx<T>::ab2(x0));
-    double alpha = sqrt(Cx<T>::ab2(x0) + nrm2);
-    // beta = -phase(x0) * alpha
-    T ph = a0 > 0 ? Cx<T>::sc(1.0 / a0, x0) : Cx<T>::one();
-    T beta = Cx<T>::sc(-alpha, ph);
-    T v0 = subt(x0, beta);                       // x0 + phase * alpha
-    for (int i = 1; i < len; ++i) v[i] = Cx<T>::div(x[i * stride], v0);
-    v[0] = Cx<T>::one();
-    *beta_out = beta;
-    // tau = (beta - x0) / beta
-    return Cx<T>::div(subt(beta, x0), beta);
-}
-
-// Block-parallel Householder vector: the same reflector as house(), with the norm summed
-// by all threads (fixed order: per-thread strided partials, then warp shuffles, then
-// warps in order) and one reciprocal instead of a division per element.  x and v may
-// not overlap.  Every thread of the block must call it; returns tau, *beta_out.
-template <class T>
-__device__ T house_par(const T *x, int len, T *v, T *beta_out) {
-    __shared__ double red_s[32];
-    __shared__ T tau_sh, beta_sh, inv_sh;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    double p = 0.0;
-    for (int i = 1 + threadIdx.x; i < len; i += blockDim.x) p += Cx<T>::ab2(x[i]);
-    p = warp_sum(p);
-    if (lane == 0) red_s[warp] = p;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double nrm2 = 0.0;
-        for (int w = 0; w < nw; ++w) nrm2 += red_s[w];
-        T x0 = x[0];
-        if (nrm2 == 0.0) {
-            tau_sh = Cx<T>::zero();
-            beta_sh = x0;
-            inv_sh = Cx<T>::zero();
-        } else {
-            // beta = -phase(x0) alpha, alpha = ||x||; v0 = x0 - beta = phase(x0) (|x0| + alpha);
-            // tau = -v0 / beta = (|x0| + alpha) / alpha; 1 / v0 = conj(phase) / (|x0| + alpha).
-            // One rsqrt per square root and one reciprocal (long float64 sequences on this GPU).
-            const double ax2 = Cx<T>::ab2(x0);
-            const double n2 = ax2 + nrm2;
-            const double ia = rsqrt(n2);                      // 1 / alpha
-            const double alpha = n2 * ia;
-            double a0 = 0.0;
-            T ph = Cx<T>::one();
-            if (ax2 > 0.0) {
-                const double ia0 = rsqrt(ax2);
-                a0 = ax2 * ia0;
-                ph = Cx<T>::sc(ia0, x0);
-            }
-            const double s = a0 + alpha;
-            beta_sh = Cx<T>::sc(-alpha, ph);
-            inv_sh = Cx<T>::sc(1.0 / s, Cx<T>::cj(ph));
-            tau_sh = Cx<T>::sc(s * ia, Cx<T>::one());
-        }
-    }
-    __syncthreads();
-    const T inv = inv_sh;
-    const bool zero = Cx<T>::ab2(tau_sh) == 0.0;
-    for (int i = threadIdx.x; i < len; i += blockDim.x)
-        v[i] = i == 0 ? Cx<T>::one() : (zero ? Cx<T>::zero() : Cx<T>::mul(x[i], inv));
-    *beta_out = beta_sh;
-    const T tau = tau_sh;
-    __syncthreads();
-    return tau;
-}
-
-// ----------------------------------------------------------------------------- least squares
-// Householder QR of the (rows x m) matrix W (copy of Hbar) and of the right-hand side;
-// d = R^{-1} (Q^H c)[0..m-1].  All threads participate.
-template <class T>
-__device__ void lsq_solve(T *W, int ldw, int rows, int m, T *rhs, T *d, T *v) {
-    // last row that can be nonzero in column j once columns 0..j-1 are reduced: the running
-    // maximum of each column's last nonzero row (a Hessenberg column j ends at j + 1; the
-    // full leading block left by a GMRES-DR restart ends at k); the reflector of column j
-    // only needs rows j..end_j, which keeps the factorisation exact.
-    __shared__ int end_s[kMaxM + 1];
-    for (int c = threadIdx.x; c < m; c += blockDim.x) {
-        int e = 0;
-        for (int i = rows - 1; i > 0; --i) {
-            const T w = W[i + (size_t)c * ldw];
-            const unsigned long long *b = reinterpret_cast<const unsigned long long *>(&w);
-            bool nz = (b[0] << 1) != 0ull;                    // nonzero, sign bit ignored
-            if (sizeof(T) == 16) nz = nz || (b[1] << 1) != 0ull;
-            if (nz) { e = i; break; }
-        }
-        end_s[c] = e;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0)
-        for (int c = 1; c < m; ++c) end_s[c] = max(end_s[c], end_s[c - 1]);
-    __syncthreads();
-    for (int j = 0; j < m; ++j) {
-        const int len = max(end_s[j], j) - j + 1;
-        T beta;
-        const T tau = house_par<T>(W + j + (size_t)j * ldw, len, v, &beta);
-        // apply H = I - tau v v^H to columns j+1..m-1 and to rhs (column index m)
-        for (int c = j + 1 + threadIdx.x; c <= m; c += blockDim.x) {
-            T *col = (c < m) ? (W + (size_t)c * ldw) : rhs;
-            T s = Cx<T>::zero();
-            for (int i = 0; i < len; ++i) s = add(s, Cx<T>::mul(Cx<T>::cj(v[i]), col[j + i]));
-            s = Cx<T>::mul(tau, s);
-            for (int i = 0; i < len; ++i) col[j + i] = subt(col[j + i], Cx<T>::mul(v[i], s));
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < len; i += blockDim.x) W[j + i + (size_t)j * ldw] = i == 0 ? beta : Cx<T>::zero();
-        __syncthreads();
-    }
-    // back substitution R d = rhs, column oriented: d_i, then all rows above updated at once
-    __shared__ T di_s;
-    for (int i = m - 1; i >= 0; --i) {
-        if (threadIdx.x == 0) {
-            T rii = W[i + (size_t)i * ldw];
-            di_s = Cx<T>::ab2(rii) > 0 ? Cx<T>::div(rhs[i], rii) : Cx<T>::zero();
-            d[i] = di_s;
-        }
-        __syncthreads();
-        const T di = di_s;
-        for (int r = threadIdx.x; r < i; r += blockDim.x) rhs[r] = subt(rhs[r], Cx<T>::mul(W[r + (size_t)i * ldw], di));
-        __syncthreads();
-    }
-}
-
-// Solve A^H f = e_last for the m x m matrix A (column-major, ld lda) by Gaussian
-// elimination with partial pivoting on a copy B = A^H.
-template <class T>
-__device__ void solve_adjoint_last(const T *A, int lda, int m, T *B, T *f, int *piv) {
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-        int i = e % m, j = e / m;
-        B[i + (size_t)j * m] = Cx<T>::cj(A[j + (size_t)i * lda]);
-    }
-    for (int i = threadIdx.x; i < m; i += blockDim.x) f[i] = (i == m - 1) ? Cx<T>::one() : Cx<T>::zero();
-    __syncthreads();
-    __shared__ int p_s;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int j = 0; j < m; ++j) {
-        if (warp == 0) {
-            // partial pivoting: the largest |B[i, j]|, ties to the smallest i
-            double best = -1.0;
-            int p = j;
-            for (int i = j + lane; i < m; i += 32) {
-                double a = Cx<T>::ab2(B[i + (size_t)j * m]);
-                if (a > best) { best = a; p = i; }
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                double ob = __shfl_down_sync(0xffffffffu, best, o);
-                int op = __shfl_down_sync(0xffffffffu, p, o);
-                if (ob > best || (ob == best && op < p)) { best = ob; p = op; }
-            }
-            if (lane == 0) { p_s = p; piv[j] = p; }
-        }
-        __syncthreads();
-        const int p = p_s;
-        if (p != j) {
-            for (int c = threadIdx.x; c < m; c += blockDim.x) {
-                T t = B[j + (size_t)c * m];
-                B[j + (size_t)c * m] = B[p + (size_t)c * m];
-                B[p + (size_t)c * m] = t;
-            }
-            if (threadIdx.x == 0) { T t = f[j]; f[j] = f[p]; f[p] = t; }
-        }
-        __syncthreads();
-        const T pivv = B[j + (size_t)j * m];
-        const bool ok = Cx<T>::ab2(pivv) > 0;
-        const T ipiv = ok ? Cx<T>::div(Cx<T>::one(), pivv) : Cx<T>::zero();
-        for (int i = j + 1 + threadIdx.x; i < m; i += blockDim.x) {
-            if (!ok) break;
-            T l = Cx<T>::mul(B[i + (size_t)j * m], ipiv);
-            for (int c = j + 1; c < m; ++c) B[i + (size_t)c * m] = subt(B[i + (size_t)c * m], Cx<T>::mul(l, B[j + (size_t)c * m]));
-            f[i] = subt(f[i], Cx<T>::mul(l, f[j]));
-            B[i + (size_t)j * m] = Cx<T>::zero();
-        }
-        __syncthreads();
-    }
-    // back substitution U f = f, column oriented
-    __shared__ T fi_s;
-    for (int i = m - 1; i >= 0; --i) {
-        if (threadIdx.x == 0) {
-            T bii = B[i + (size_t)i * m];
-            fi_s = Cx<T>::ab2(bii) > 0 ? Cx<T>::div(f[i], bii) : Cx<T>::zero();
-            f[i] = fi_s;
-        }
-        __syncthreads();
-        const T fi = fi_s;
-        for (int r = threadIdx.x; r < i; r += blockDim.x) f[r] = subt(f[r], Cx<T>::mul(B[r + (size_t)i * m], fi));
-        __syncthreads();
-    }
-}
-
-// ----------------------------------------------------------------------------- Hessenberg form
-// A (m x m, ld m) <- Q^H A Q upper Hessenberg; Z <- Q (Z must hold I on entry).
-template <class T>
-__device__ void hessenberg(T *A, int m, T *Z, T *v) {
-    for (int j = 0; j + 2 < m; ++j) {
-        const int len = m - j - 1;
-        T beta;
-        const T tau = house_par<T>(A + (j + 1) + (size_t)j * m, len, v, &beta);
-        if (Cx<T>::ab2(tau) == 0.0) continue;
-        // left: rows j+1..m-1, columns j..m-1: A <- H A = A - tau v (v^H A)
-        for (int c = j + threadIdx.x; c < m; c += blockDim.x) {
-            T *col = A + (size_t)c * m + j + 1;
-            T s = Cx<T>::zero();
-            for (int i = 0; i < len; ++i) s = add(s, Cx<T>::mul(Cx<T>::cj(v[i]), col[i]));
-            s = Cx<T>::mul(tau, s);
-            for (int i = 0; i < len; ++i) col[i] = subt(col[i], Cx<T>::mul(v[i], s));
-        }
-        __syncthreads();
-        // right: all rows, columns j+1..m-1: A <- A H^H = A - conj(tau) (A v) v^H; Z <- Z H^H
-        for (int rr = threadIdx.x; rr < 2 * m; rr += blockDim.x) {
-            T *M = rr < m ? A : Z;
-            const int r = rr < m ? rr : rr - m;
-            T s = Cx<T>::zero();
-            for (int i = 0; i < len; ++i) s = add(s, Cx<T>::mul(M[r + (size_t)(j + 1 + i) * m], v[i]));
-            s = Cx<T>::mul(s, Cx<T>::cj(tau));
-            for (int i = 0; i < len; ++i)
-                M[r + (size_t)(j + 1 + i) * m] = subt(M[r + (size_t)(j + 1 + i) * m], Cx<T>::mul(s, Cx<T>::cj(v[i])));
-        }
-        __syncthreads();
-    }
-    // clean below the subdiagonal
-    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-        int i = e % m, j = e / m;
-        if (i > j + 1) A[e] = Cx<T>::zero();
-    }
-    __syncthreads();
-}
 
 // ----------------------------------------------------------------------------- Schur form: shared pieces
 // Cost model of the QR sweeps on this GPU: every float64 warp instruction occupies its SM
@@ -334,6 +107,8 @@ __device__ __forceinline__ double rcp_fast(double x) {
 __device__ __forceinline__ bool mid_range(double x) {
     return (unsigned)((__double2hiint(x) >> 20) - 123) < 1800u;
 }
+__device__ __forceinline__ double shfl_all(double v, int l) { return __shfl_sync(kFull, v, l); }
+__device__ __forceinline__ cplx shfl_all(cplx v, int l) { return {shfl_all(v.re, l), shfl_all(v.im, l)}; }
 __device__ __forceinline__ void bar_two_warps() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
 
 // lane's place among the far warps' lanes (2, 3, 5, 6, 7), and their number
@@ -406,6 +181,267 @@ __device__ __forceinline__ double reflect_warp(double x, double y, double z, dou
     const double v = c == 0 ? w0 : c == 1 ? w1 : w2, gv = v * g;
     if (lane < 6) hs[lane] = lane < 3 ? v : gv;
     return beta;
+}
+
+// ----------------------------------------------------------------------------- reflectors
+// One warp: the reflector I - g w w^H (g real) that maps x[0..len-1] to (beta, 0, .., 0): w = x but
+// for w_0 = x_0 - beta, beta = -phase(x_0) ||x||, g = 1 / (||x||^2 + ||x|| |x_0|).  w may be x
+// itself.  A zero tail gives the identity.  Every lane computes the scalars: no shuffle after the
+// norm's, no division of the elements.
+template <class T>
+__device__ __forceinline__ void reflector_warp(const T *x, int len, T *w, double *gs, T *beta) {
+    const int lane = threadIdx.x & 31;
+    bool scaled = false;                // tests on bits and flags: a float64 compare is a link of the chain too
+    double sc = 1.0, mx = 1.0;
+    auto tail = [&]() {
+        double s = 0.0;
+        for (int i = 1 + lane; i < len; i += 32) s += Cx<T>::ab2(scaled ? Cx<T>::sc(sc, x[i]) : x[i]);
+        if (len <= 2) return __shfl_sync(kFull, s, 0);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(kFull, s, o);
+        return s;
+    };
+    double sn = tail();
+    T x0 = x[0];
+    double ax2 = Cx<T>::ab2(x0), n2 = ax2 + sn;
+    if (!mid_range(n2)) {               // rescale (the reflector does not depend on the scale)
+        mx = 0.0;
+        for (int i = lane; i < len; i += 32) {
+            const double *c = reinterpret_cast<const double *>(x + i);
+            mx = fmax(mx, fabs(c[0]));
+            if (sizeof(T) == 16) mx = fmax(mx, fabs(c[sizeof(T) / 8 - 1]));
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(kFull, mx, o));
+        if (mx > 1e-300 && mx < 1e300) {
+            sc = 1.0 / mx;
+            scaled = true;
+            sn = tail();
+            x0 = Cx<T>::sc(sc, x0);
+            ax2 = Cx<T>::ab2(x0);
+            n2 = ax2 + sn;
+        }
+    }
+    T w0 = Cx<T>::zero(), bt = x0;
+    double g = 0.0;
+    if (__double_as_longlong(sn) != 0) {
+        double alpha;
+        if (mid_range(n2)) {
+            const double r0 = rsqrt_seed(n2), h = n2 * r0, e = fma(-h, r0, 1.0);
+            alpha = fma(h * e, fma(0.375, e, 0.5), h);
+        } else {
+            alpha = sqrt(n2);
+        }
+        double a0 = 0.0;
+        T ph = Cx<T>::one();
+        if constexpr (sizeof(T) == sizeof(double)) {
+            a0 = fabs(x0);
+            ph = copysign(1.0, x0);
+        } else if (__double_as_longlong(ax2) != 0) {
+            double ia = rsqrt_seed(ax2);
+            const double e = fma(-(ax2 * ia), ia, 1.0);
+            ia = mid_range(ax2) ? fma(ia, e * fma(0.375, e, 0.5), ia) : rsqrt(ax2);
+            a0 = ax2 * ia;
+            ph = Cx<T>::sc(ia, x0);
+        }
+        const double d = fma(alpha, a0, n2);
+        g = mid_range(d) ? rcp_fast(d) : 1.0 / d;
+        bt = Cx<T>::sc(-alpha, ph);
+        w0 = subt(x0, bt);
+        if (scaled) bt = Cx<T>::sc(mx, bt);
+    } else if (scaled) {
+        bt = Cx<T>::sc(mx, x0);
+    }
+    __syncwarp();
+    if (scaled || w != x)
+        for (int i = 1 + lane; i < len; i += 32) w[i] = scaled ? Cx<T>::sc(sc, x[i]) : x[i];
+    if (lane == 0) { w[0] = w0; *gs = g; *beta = bt; }
+    __syncwarp();
+}
+
+// One warp: x <- (I - g w w^H) x.
+template <class T>
+__device__ __forceinline__ void reflect_vector(T *x, const T *w, int len, double g) {
+    const int lane = threadIdx.x & 31;
+    T s = Cx<T>::zero();
+    if (len <= 2) {                     // every lane the same sum
+        for (int i = 0; i < len; ++i) s = Cx<T>::macc(s, w[i], x[i]);
+        __syncwarp();
+    } else {
+        for (int i = lane; i < len; i += 32) s = Cx<T>::macc(s, w[i], x[i]);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s = add(s, shfl_xor(s, o));
+    }
+    s = Cx<T>::sc(g, s);
+    for (int i = lane; i < len; i += 32) x[i] = Cx<T>::nmac(x[i], s, w[i]);
+    __syncwarp();
+}
+
+// Warps 0 .. nw-1 of a set: the reflector on `items` vectors of stride `stride` starting at
+// base(item): columns x <- (I - g w w^H) x, or rows x <- x (I - g w w^H) (ROWS).  G lanes share an
+// item, so that 60 items occupy all four sub-partitions' float64 units and not those of two warps.
+template <int G, bool ROWS, class T, class Base>
+__device__ __forceinline__ void reflect_items(int items, Base base, size_t stride, const T *w, int len, double g,
+                                              int warp, int nw) {
+    constexpr int per = 32 / G;
+    const int lane = threadIdx.x & 31, part = lane / per, it = lane % per;
+    for (int b = warp * per; b < items; b += nw * per) {
+        const bool on = b + it < items;
+        T *x = base(on ? b + it : b);
+        T s = Cx<T>::zero();
+        for (int i = part; i < len; i += G) s = ROWS ? Cx<T>::mac(s, x[i * stride], w[i]) : Cx<T>::macc(s, w[i], x[i * stride]);
+#pragma unroll
+        for (int o = per; o < 32; o <<= 1) s = add(s, shfl_xor(s, o));
+        s = Cx<T>::sc(g, s);
+        __syncwarp();
+        if (on)
+            for (int i = part; i < len; i += G)
+                x[i * stride] = ROWS ? subt(x[i * stride], Cx<T>::mul(s, Cx<T>::cj(w[i]))) : Cx<T>::nmac(x[i * stride], s, w[i]);
+    }
+}
+
+// ----------------------------------------------------------------------------- least squares
+// Householder QR of the (rows x m) matrix W (copy of Hbar) and of the right-hand side, rows = m + 1;
+// d = R^{-1} (Q^H c)[0..m-1], and f = H_m^{-H} e_m, H_m the first m rows of Hbar.  All threads.
+// After a restart the reflectors past column k have two rows, so the chain from one to the next
+// bounds the factorisation: warp 0 applies reflector j to column j + 1 and computes reflector j + 1
+// while the far warps apply j to the other columns (norm, reflector and update in turn by the block,
+// four barriers a column, took 212 us at m = 60, k = 20; now 117).
+// f comes from the same factorisation.  With Q = [Q_1 q; p^H s] (rows x rows), H_m = Q_1 R, and from
+// Q^H Q = I: f = (Q_1 e_m - q (p^H e_m) / s) / conj(r_mm), which needs the last two columns of Q:
+// the reflectors applied in reverse to two unit vectors by a warp each, beside the back substitution
+// (elimination with pivoting of H_m^H took another 252 us, complex m = 80 1.6 ms).
+template <class T>
+__device__ void lsq_solve(T *W, int ldw, int rows, int m, T *rhs, T *d, T *f, T *diag, T *q1, T *q2, double *gs) {
+    // last row that can be nonzero in column j once columns 0..j-1 are reduced: the running
+    // maximum of each column's last nonzero row (a Hessenberg column j ends at j + 1; the
+    // full leading block left by a GMRES-DR restart ends at k); the reflector of column j
+    // only needs rows j..end_j, which keeps the factorisation exact.
+    __shared__ int end_s[kMaxM + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int c = threadIdx.x; c < m; c += blockDim.x) {
+        int e = 0;
+        for (int i = rows - 1; i > 0; --i) {
+            const T w = W[i + (size_t)c * ldw];
+            const unsigned long long *b = reinterpret_cast<const unsigned long long *>(&w);
+            bool nz = (b[0] << 1) != 0ull;                    // nonzero, sign bit ignored
+            if (sizeof(T) == 16) nz = nz || (b[sizeof(T) / 8 - 1] << 1) != 0ull;
+            if (nz) { e = i; break; }
+        }
+        end_s[c] = e;
+    }
+    for (int i = threadIdx.x; i < rows; i += blockDim.x) {
+        q1[i] = i == m - 1 ? Cx<T>::one() : Cx<T>::zero();
+        q2[i] = i == m ? Cx<T>::one() : Cx<T>::zero();
+    }
+    __syncthreads();
+    if (warp == 0)
+        for (int c = lane, top = 0; c - lane < m; c += 32) {
+            int e = c < m ? max(end_s[c], c) : 0;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int below = __shfl_up_sync(kFull, e, o);
+                if (lane >= o) e = max(e, below);
+            }
+            e = max(e, top);
+            if (c < m) end_s[c] = e;
+            top = __shfl_sync(kFull, e, 31);
+        }
+    __syncthreads();
+    auto col = [&](int j) { return W + j + (size_t)j * ldw; };      // reflector j's rows of column j
+    const int fw = far_index() >> 5;
+    if (warp == 0) reflector_warp<T>(col(0), end_s[0] + 1, col(0), gs, diag);
+    __syncthreads();
+    for (int j = 0; j < m; ++j) {
+        const int len = end_s[j] - j + 1;
+        if (warp == 0) {
+            if (j + 1 < m) {
+                reflect_vector<T>(col(j) + ldw, col(j), len, gs[j]);
+                reflector_warp<T>(col(j + 1), end_s[j + 1] - j, col(j + 1), gs + j + 1, diag + j + 1);
+            }
+        } else if (fw >= 0) {
+            const int nc = max(0, m - j - 2);       // columns j + 2 .. m - 1, then the right-hand side
+            auto base = [&](int it) { return it < nc ? col(j) + (size_t)(it + 2) * ldw : rhs + j; };
+            if (len <= 4) reflect_items<1, false, T>(nc + 1, base, 1, col(j), len, gs[j], fw, kFarLanes / 32);
+            else reflect_items<4, false, T>(nc + 1, base, 1, col(j), len, gs[j], fw, kFarLanes / 32);
+        }
+        __syncthreads();
+    }
+    if (warp == 0) {
+        // back substitution, a lane per row and 32 rows on: d_i, then all rows above at once
+        constexpr int U = kMaxM / 32;
+        T r[U], di[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int i = lane + 32 * u;
+            r[u] = di[u] = Cx<T>::zero();
+            if (i < m) {
+                r[u] = rhs[i];
+                if (Cx<T>::ab2(diag[i]) > 0) di[u] = Cx<T>::div(Cx<T>::one(), diag[i]);
+            }
+        }
+#pragma unroll
+        for (int u = U - 1; u >= 0; --u) {
+            for (int i = min(m - 1, 32 * u + 31); i >= 32 * u; --i) {
+                const T v = shfl_all(Cx<T>::mul(r[u], di[u]), i & 31);
+                if (lane == 0) d[i] = v;
+#pragma unroll
+                for (int t = 0; t <= u; ++t)
+                    if (lane + 32 * t < i) r[t] = Cx<T>::nmac(r[t], W[lane + 32 * t + (size_t)i * ldw], v);
+            }
+        }
+    } else if (warp <= 2) {
+        T *q = warp == 1 ? q1 : q2;
+        for (int j = m - 1; j >= 0; --j) reflect_vector<T>(q + j, col(j), end_s[j] - j + 1, gs[j]);
+    }
+    __syncthreads();
+    const T rmm = diag[m - 1], s = q2[m];
+    const T a = Cx<T>::ab2(s) > 0 ? Cx<T>::div(q1[m], s) : Cx<T>::zero();
+    const T ir = Cx<T>::ab2(rmm) > 0 ? Cx<T>::div(Cx<T>::one(), Cx<T>::cj(rmm)) : Cx<T>::zero();
+    for (int i = threadIdx.x; i < m; i += blockDim.x) f[i] = Cx<T>::mul(Cx<T>::nmac(q1[i], q2[i], a), ir);
+    __syncthreads();
+}
+
+// ----------------------------------------------------------------------------- Hessenberg form
+// A (m x m, ld m) <- Q^H A Q upper Hessenberg; Z <- Q (Z must hold I on entry).  w: 2 (m + 1)
+// elements.  The float64 units bound it: 8/3 m^3 multiply-adds at 2 a clock.  Warp 0 computes
+// a reflector while the other warps apply the one before to Z, which nothing waits for; 4 lanes
+// share a row or column (one thread each left half the sub-partitions idle in the column pass):
+// 420 -> 278 us at m = 60, 2308 -> 1732 us at complex m = 80.
+template <class T>
+__device__ void hessenberg(T *A, int m, T *Z, T *w2) {
+    __shared__ double g_s[2];
+    __shared__ T beta_s;
+    const int warp = threadIdx.x >> 5, fw = far_index() >> 5;
+    constexpr int nw = kGdrThreads / 32;
+    for (int j = 0; j + 1 < m; ++j) {
+        const bool last = j + 2 == m;               // no reflector left: only Z
+        const int len = m - j - 1, slot = j & 1;
+        T *w = w2 + slot * m;
+        if (warp == 0 && !last) reflector_warp<T>(A + (j + 1) + (size_t)j * m, len, w, g_s + slot, &beta_s);
+        // with long rows of Z all warps take part, else those that leave warp 0's unit alone
+        const bool all = last || len * (int)(sizeof(T) / 8) * (int)(sizeof(T) / 8) >= 64;
+        if (j > 0 && (all || fw >= 0) && g_s[slot ^ 1] != 0.0)
+            reflect_items<4, true, T>(m, [&](int r) { return Z + r + (size_t)j * m; }, m, w2 + (slot ^ 1) * m, len + 1,
+                                      g_s[slot ^ 1], all ? warp : fw, all ? nw : kFarLanes / 32);
+        __syncthreads();
+        if (last) break;
+        const double g = g_s[slot];
+        if (g == 0.0) continue;
+        if (threadIdx.x == 0) A[(j + 1) + (size_t)j * m] = beta_s;
+        // left: rows j+1..m-1, columns j+1..m-1
+        reflect_items<4, false, T>(len, [&](int c) { return A + (j + 1) + (size_t)(j + 1 + c) * m; }, 1, w, len, g, warp, nw);
+        __syncthreads();
+        // right: all rows, columns j+1..m-1
+        reflect_items<4, true, T>(m, [&](int r) { return A + r + (size_t)(j + 1) * m; }, m, w, len, g, warp, nw);
+        __syncthreads();
+    }
+    // clean below the subdiagonal
+    for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
+        int i = e % m, j = e / m;
+        if (i > j + 1) A[e] = Cx<T>::zero();
+    }
+    __syncthreads();
 }
 
 // ----------------------------------------------------------------------------- real Schur form
@@ -805,16 +841,40 @@ __device__ void real_schur_eigs(const double *T, int m, double *wr, double *wi) 
     __syncthreads();
 }
 
+// a / b by one reciprocal in the middle of the range
+__device__ __forceinline__ cplx cdiv_fast(cplx a, cplx b) {
+    const double d = abs2(b);
+    if (!mid_range(d)) return cdiv(a, b);
+    const cplx n = a * conj(b);
+    return rcp_fast(d) * n;
+}
+// |z| < small
+__device__ __forceinline__ bool below(cplx z, double small) {
+    const double a = abs2(z), b = small * small;
+    return mid_range(a) && mid_range(b) ? a < b : cabs_(z) < small;
+}
+constexpr int kVecLanes = 8;       // lanes that share an eigenvector's back substitution
+__device__ __forceinline__ cplx group_sum(cplx s, unsigned gm) {
+#pragma unroll
+    for (int o = 1; o < kVecLanes; o <<= 1)
+        s = {s.re + __shfl_xor_sync(gm, s.re, o), s.im + __shfl_xor_sync(gm, s.im, o)};
+    return s;
+}
+
 // Back substitution for the eigenvector of eigenvalue (lr, li) at Schur position j of the
-// real quasi-triangular T (one thread).  Output y (complex, length m, zero below j).
+// real quasi-triangular T.  Output y (complex, length m, zero below j).
+// Eight lanes (mask gm, `part` the lane among them) share a vector: a row's sum is the long serial
+// part, the vectors of a warp take different branches, and a thread per vector kept to one warp
+// (with the products and residuals 319 us at m = 60, k = 20; now 141).
 __device__ void real_schur_vector(const double *T, int m, int j, double lr, double li, cplx *y,
-                                  double tnorm) {
+                                  double tnorm, int part, unsigned gm) {
     const double small = fmax(kEps * tnorm, 1e-300);
     const cplx lam = mkc(lr, li);
-    for (int i = 0; i < m; ++i) y[i] = {0.0, 0.0};
+    for (int i = part; i < m; i += kVecLanes) y[i] = {0.0, 0.0};
+    __syncwarp(gm);
     int top;
     if (li == 0.0) {
-        y[j] = {1.0, 0.0};
+        if (part == 0) y[j] = {1.0, 0.0};
         top = j - 1;
     } else {
         // 2x2 block at (t, t+1) containing j
@@ -822,56 +882,66 @@ __device__ void real_schur_vector(const double *T, int m, int j, double lr, doub
         const int t = jtop ? j : j - 1;
         double a = T[t + (size_t)t * m], b = T[t + (size_t)(t + 1) * m];
         double c = T[(t + 1) + (size_t)t * m], d = T[(t + 1) + (size_t)(t + 1) * m];
-        if (fabs(b) >= fabs(c)) {
-            y[t] = {1.0, 0.0};
-            y[t + 1] = cdiv(lam - mkc(a, 0.0), mkc(b, 0.0));      // (a - lam) y0 + b y1 = 0
-        } else {
-            y[t + 1] = {1.0, 0.0};
-            y[t] = cdiv(lam - mkc(d, 0.0), mkc(c, 0.0));          // c y0 + (d - lam) y1 = 0
-        }
+        cplx yt = {1.0, 0.0}, yb = {1.0, 0.0};
+        if (fabs(b) >= fabs(c)) yb = cdiv(lam - mkc(a, 0.0), mkc(b, 0.0));      // (a - lam) y0 + b y1 = 0
+        else yt = cdiv(lam - mkc(d, 0.0), mkc(c, 0.0));                         // c y0 + (d - lam) y1 = 0
+        if (part == 0) { y[t] = yt; y[t + 1] = yb; }
         top = t - 1;
         j = t + 1;
     }
+    __syncwarp(gm);
     int i = top;
     while (i >= 0) {
         const bool blk = (i > 0) && T[i + (size_t)(i - 1) * m] != 0.0;   // rows (i-1, i) form a block
         if (!blk) {
             cplx s = {0.0, 0.0};
-            for (int l = i + 1; l <= j; ++l) s = s + T[i + (size_t)l * m] * y[l];
+            for (int l = i + 1 + part; l <= j; l += kVecLanes) {
+                const double t = T[i + (size_t)l * m];
+                s = {fma(t, y[l].re, s.re), fma(t, y[l].im, s.im)};
+            }
+            s = group_sum(s, gm);
             cplx den = mkc(T[i + (size_t)i * m], 0.0) - lam;
-            if (cabs_(den) < small) den = mkc(small, 0.0);
-            y[i] = cdiv(-s, den);
+            if (below(den, small)) den = mkc(small, 0.0);
+            const cplx v = cdiv_fast(-s, den);
+            if (part == 0) y[i] = v;
             i -= 1;
         } else {
             const int t = i - 1;
             cplx s0 = {0.0, 0.0}, s1 = {0.0, 0.0};
-            for (int l = i + 1; l <= j; ++l) {
-                s0 = s0 + T[t + (size_t)l * m] * y[l];
-                s1 = s1 + T[i + (size_t)l * m] * y[l];
+            for (int l = i + 1 + part; l <= j; l += kVecLanes) {
+                const double t0 = T[t + (size_t)l * m], t1 = T[i + (size_t)l * m];
+                s0 = {fma(t0, y[l].re, s0.re), fma(t0, y[l].im, s0.im)};
+                s1 = {fma(t1, y[l].re, s1.re), fma(t1, y[l].im, s1.im)};
             }
+            s0 = group_sum(s0, gm);
+            s1 = group_sum(s1, gm);
             // [a-lam b; c d-lam] [y_t; y_i] = -[s0; s1]
             cplx a = mkc(T[t + (size_t)t * m], 0.0) - lam, b = mkc(T[t + (size_t)i * m], 0.0);
             cplx c = mkc(T[i + (size_t)t * m], 0.0), d = mkc(T[i + (size_t)i * m], 0.0) - lam;
             cplx det = a * d - b * c;
             if (cabs_(det) < small * small) det = mkc(small * small, 0.0);
-            y[t] = cdiv(-(d * s0) + b * s1, det);
-            y[i] = cdiv(c * s0 - a * s1, det);
+            const cplx yt = cdiv_fast(-(d * s0) + b * s1, det), yi = cdiv_fast(c * s0 - a * s1, det);
+            if (part == 0) { y[t] = yt; y[i] = yi; }
             i -= 2;
         }
+        __syncwarp(gm);
     }
 }
 
-__device__ void complex_schur_vector(const cplx *T, int m, int j, cplx *y, double tnorm) {
+__device__ void complex_schur_vector(const cplx *T, int m, int j, cplx *y, double tnorm, int part, unsigned gm) {
     const double small = fmax(kEps * tnorm, 1e-300);
     const cplx lam = T[j + (size_t)j * m];
-    for (int i = 0; i < m; ++i) y[i] = {0.0, 0.0};
-    y[j] = {1.0, 0.0};
+    for (int i = part; i < m; i += kVecLanes) y[i] = {i == j ? 1.0 : 0.0, 0.0};
+    __syncwarp(gm);
     for (int i = j - 1; i >= 0; --i) {
         cplx s = {0.0, 0.0};
-        for (int l = i + 1; l <= j; ++l) s = s + T[i + (size_t)l * m] * y[l];
+        for (int l = i + 1 + part; l <= j; l += kVecLanes) s = Cx<cplx>::mac(s, T[i + (size_t)l * m], y[l]);
+        s = group_sum(s, gm);
         cplx den = T[i + (size_t)i * m] - lam;
-        if (cabs_(den) < small) den = mkc(small, 0.0);
-        y[i] = cdiv(-s, den);
+        if (below(den, small)) den = mkc(small, 0.0);
+        const cplx v = cdiv_fast(-s, den);
+        if (part == 0) y[i] = v;
+        __syncwarp(gm);
     }
 }
 
@@ -996,25 +1066,33 @@ __global__ void k_small_gemv(const D *M, int k, const D *c, D *out) {
 
 // ----------------------------------------------------------------------------- GMRES-DR restart
 // See tg_small.cuh for the argument layout.
+// elements of T before the eigenvector work in shared memory: W and Z, rounded up to an even count
+// (the work is complex, 16-byte aligned, and m^2 is odd for odd m)
+__host__ __device__ constexpr size_t gdr_y_offset(int m) {
+    return ((size_t)(m + 1) * m + (size_t)m * m + 1) & ~(size_t)1;
+}
+
 template <class T>
 __device__ __forceinline__ void gmresdr_restart_body(const GdrArgs<T> &a) {
     const int m = a.m;
     const int rows = m + 1;
     const int ldh = a.ldh;
     // W: (m+1) x m (least-squares copy), later the m x m eigen matrix / Schur form;
-    // Z: m x m Schur vectors.  Both live in shared memory when the launch provided it
+    // Z: m x m Schur vectors, later the basis P.  Both live in shared memory when the launch provided it
     // (the QR sweeps are a long chain of dependent small steps, so their latency rules).
     extern __shared__ __align__(16) unsigned char gdr_smem[];
     T *sm = reinterpret_cast<T *>(gdr_smem);
     T *W = a.smem >= 1 ? sm : a.work;
     T *Z = a.smem >= 2 ? sm + (size_t)rows * m : a.work + (size_t)rows * m;
-    T *B = a.smem >= 3 ? sm + (size_t)rows * m + (size_t)m * m : a.work + (size_t)rows * m + (size_t)m * m;  // m x m (LU)
-    T *vtmp = a.work + (size_t)rows * m + 2 * (size_t)m * m;   // 2 (m+1) vectors
+    T *vtmp = a.work + (size_t)rows * m + (size_t)m * m;       // 2 (m+1) vectors
     T *f = vtmp + 2 * (m + 1);
-    cplx *Ysm = a.smem >= 4 ? reinterpret_cast<cplx *>(sm + (size_t)rows * m + 2 * (size_t)m * m) : a.ywork;
+    cplx *Ysm = a.smem >= 3 ? reinterpret_cast<cplx *>(sm + gdr_y_offset(m)) : a.ywork;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     T *res = a.res;
-    __shared__ int piv_s[kMaxM + 1];
+    // vectors of the least-squares solve, the Hessenberg reduction, the ordering and Gram-Schmidt in
+    // turn: with kGdrSmemMax the static shared memory must stay below 17 KB
+    __shared__ T vec_s[3 * (kMaxM + 1)];
+    __shared__ double gs_s[kMaxM];
 
     long long t_mark = clock64();
     const bool rr_mode = a.mode == 1;
@@ -1035,23 +1113,23 @@ __device__ __forceinline__ void gmresdr_restart_body(const GdrArgs<T> &a) {
     }
     for (int i = threadIdx.x; i < rows; i += blockDim.x) vtmp[m + 1 + i] = a.c[i];
     __syncthreads();
-    lsq_solve<T>(W, rows, rows, m, vtmp + (m + 1), a.d, vtmp);
+    lsq_solve<T>(W, rows, rows, m, vtmp + (m + 1), a.d, f, vec_s, vec_s + (kMaxM + 1), vec_s + 2 * (kMaxM + 1), gs_s);
     for (int i = threadIdx.x; i < rows; i += blockDim.x) {
         T s = a.c[i];
-        for (int j = 0; j < m; ++j) s = subt(s, Cx<T>::mul(a.H[i + (size_t)j * ldh], a.d[j]));
+        for (int j = 0; j < m; ++j) s = Cx<T>::nmac(s, a.H[i + (size_t)j * ldh], a.d[j]);
         res[i] = s;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (warp == 0) {
         double s = 0.0;
-        for (int i = 0; i < rows; ++i) s += Cx<T>::ab2(res[i]);
-        a.info->rnorm = sqrt(s);
+        for (int i = lane; i < rows; i += 32) s += Cx<T>::ab2(res[i]);
+        s = warp_sum(s);
+        if (lane == 0) a.info->rnorm = sqrt(s);
     }
 
     __syncthreads();
     if (threadIdx.x == 0) { long long _t = clock64(); a.info->phase[0] = _t - t_mark; t_mark = _t; }
-    // ---- 2. f = H_m^{-H} e_m and the harmonic matrix M = H_m + |h|^2 f e_m^T (in W, ld m)
-    solve_adjoint_last<T>(a.H, ldh, m, B, f, piv_s);
+    // ---- 2. the harmonic matrix M = H_m + |h|^2 f e_m^T (in W, ld m), f = H_m^{-H} e_m
     const T hm = a.H[m + (size_t)(m - 1) * ldh];
     const double hm2 = Cx<T>::ab2(hm);
     for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
@@ -1069,7 +1147,7 @@ __device__ __forceinline__ void gmresdr_restart_body(const GdrArgs<T> &a) {
     if (threadIdx.x == 0) { long long _t = clock64(); a.info->phase[1] = _t - t_mark; t_mark = _t; }
     }   // steps 1-2: GMRES-DR restart only
     // ---- 3. eigen-decomposition of M: Hessenberg, Schur, eigenvalues
-    hessenberg<T>(W, m, Z, vtmp);
+    hessenberg<T>(W, m, Z, vec_s);
     __syncthreads();
     if (threadIdx.x == 0) { long long _t = clock64(); a.info->phase[2] = _t - t_mark; t_mark = _t; }
     int st;
@@ -1108,8 +1186,7 @@ __device__ __forceinline__ void gmresdr_restart_body(const GdrArgs<T> &a) {
     // ---- 4. order and select
     __shared__ int kk_s;
     int *ord = a.order;
-    __shared__ double mod_s[kMaxM];
-    __shared__ double wr_s[kMaxM], wi_s[kMaxM];
+    double *mod_s = reinterpret_cast<double *>(vec_s), *wr_s = mod_s + kMaxM, *wi_s = wr_s + kMaxM;
     for (int i = threadIdx.x; i < m; i += blockDim.x) {
         mod_s[i] = hypot(wr[i], wi[i]);
         wr_s[i] = wr[i];
@@ -1151,13 +1228,14 @@ __device__ __forceinline__ void gmresdr_restart_body(const GdrArgs<T> &a) {
     // a.gwork holds the kept eigenvectors as complex columns (m x kk)
     cplx *G = a.gwork;
     cplx *Y = Ysm;
-    for (int q = threadIdx.x; q < kk; q += blockDim.x) {
-        const int j = ord[q];
+    for (int q = threadIdx.x / kVecLanes; q < kk; q += blockDim.x / kVecLanes) {
+        const int j = ord[q], part = lane % kVecLanes;
+        const unsigned gm = ((1u << kVecLanes) - 1u) << (lane - part);
         cplx *y = Y + (size_t)q * m;
         if constexpr (sizeof(T) == sizeof(double))
-            real_schur_vector(reinterpret_cast<const double *>(W), m, j, wr[j], wi[j], y, tnorm);
+            real_schur_vector(reinterpret_cast<const double *>(W), m, j, wr[j], wi[j], y, tnorm, part, gm);
         else
-            complex_schur_vector(reinterpret_cast<const cplx *>(W), m, j, y, tnorm);
+            complex_schur_vector(reinterpret_cast<const cplx *>(W), m, j, y, tnorm, part, gm);
     }
     __syncthreads();
     for (int e = threadIdx.x; e < m * kk; e += blockDim.x) {
@@ -1173,7 +1251,7 @@ __device__ __forceinline__ void gmresdr_restart_body(const GdrArgs<T> &a) {
                 s.im = fma(zl, y[l].im, s.im);
             }
         } else {
-            for (int l = 0; l < m; ++l) s = s + *reinterpret_cast<const cplx *>(&Z[i + (size_t)l * m]) * y[l];
+            for (int l = 0; l < m; ++l) s = Cx<cplx>::mac(s, *reinterpret_cast<const cplx *>(&Z[i + (size_t)l * m]), y[l]);
         }
         G[i + (size_t)q * m] = s;
     }
@@ -1257,9 +1335,8 @@ __device__ __forceinline__ void gmresdr_restart_body(const GdrArgs<T> &a) {
     if (threadIdx.x == 0) { long long _t = clock64(); a.info->phase[5] = _t - t_mark; t_mark = _t; }
     // ---- 6. P_k: orthonormal basis of the kept span (real: Re/Im of pairs), m x kk
     //          then P_{k+1} = orth([[P_k; 0], z]), stored (m+1) x (kk+1) with ld m+1.
-    T *P = a.P;
     __shared__ int ncol_s;
-    __shared__ int colof_s[kMaxM + 1];
+    int *colof_s = reinterpret_cast<int *>(gs_s);
     if (threadIdx.x == 0) {
         int col = 0;
         for (int q = 0; q < kk; ++q) {
@@ -1275,6 +1352,8 @@ __device__ __forceinline__ void gmresdr_restart_body(const GdrArgs<T> &a) {
         ncol_s = col;
     }
     __syncthreads();
+    // built in the Schur vectors' place (they are not read any more) where it fits
+    T *P = rows * (ncol_s + 1) <= m * m ? Z : a.P;
     for (int q = warp; q < kk; q += nwarps) {
         const int c0 = colof_s[q];
         if (c0 < 0) continue;
@@ -1321,25 +1400,35 @@ __device__ __forceinline__ void gmresdr_restart_body(const GdrArgs<T> &a) {
     if (!rr_mode)
         for (int i = threadIdx.x; i < rows; i += blockDim.x) P[i + (size_t)nc * rows] = a.z[i];
     __syncthreads();
-    // classical Gram-Schmidt applied twice over the nc + 1 columns (length m+1): per column,
-    // the projections on the previous columns in parallel, then the update in parallel
-    __shared__ T proj_s[kMaxM + 2];
-    __shared__ double nrm_s;
+    // classical Gram-Schmidt applied twice over the nc + 1 columns (length m+1): per column, the
+    // projections on the previous columns, then the update, G lanes to a sum (a thread to a sum in
+    // global memory took 160 us at m = 60, k = 20, now 90; complex m = 80 1.85 -> 0.57 ms)
+    T *proj_s = vec_s;
+    __shared__ double inv_s;
     const int clast = rr_mode ? nc - 1 : nc;
     for (int c = 0; c <= clast; ++c) {
         T *pc = P + (size_t)c * rows;
-        for (int pass = 0; pass < 2; ++pass) {
-            for (int q = threadIdx.x; q < c; q += blockDim.x) {
-                const T *pq = P + (size_t)q * rows;
-                T sacc = Cx<T>::zero();
-                for (int i = 0; i < rows; ++i) sacc = add(sacc, Cx<T>::mul(Cx<T>::cj(pq[i]), pc[i]));
-                proj_s[q] = sacc;
+        for (int pass = 0; pass < 2 && c > 0; ++pass) {
+            constexpr int G = 8, per = 32 / G;
+            const int part = lane / per, it = lane % per;
+            for (int b = warp * per; b < c; b += nwarps * per) {
+                const T *pq = P + (size_t)min(b + it, c - 1) * rows;
+                T s = Cx<T>::zero();
+                for (int i = part; i < rows; i += G) s = Cx<T>::macc(s, pq[i], pc[i]);
+#pragma unroll
+                for (int o = per; o < 32; o <<= 1) s = add(s, shfl_xor(s, o));
+                if (part == 0 && b + it < c) proj_s[b + it] = s;
             }
             __syncthreads();
-            for (int i = threadIdx.x; i < rows; i += blockDim.x) {
-                T acc = pc[i];
-                for (int q = 0; q < c; ++q) acc = subt(acc, Cx<T>::mul(proj_s[q], P[i + (size_t)q * rows]));
-                pc[i] = acc;
+            constexpr int G2 = 4, per2 = 32 / G2;
+            const int part2 = lane / per2, it2 = lane % per2;
+            for (int b = warp * per2; b < rows; b += nwarps * per2) {
+                const int i = min(b + it2, rows - 1);
+                T s = Cx<T>::zero();
+                for (int q = part2; q < c; q += G2) s = Cx<T>::mac(s, proj_s[q], P[i + (size_t)q * rows]);
+#pragma unroll
+                for (int o = per2; o < 32; o <<= 1) s = add(s, shfl_xor(s, o));
+                if (part2 == 0 && b + it2 < rows) pc[i] = subt(pc[i], s);
             }
             __syncthreads();
         }
@@ -1347,13 +1436,15 @@ __device__ __forceinline__ void gmresdr_restart_body(const GdrArgs<T> &a) {
             double sq2 = 0.0;
             for (int i = lane; i < rows; i += 32) sq2 += Cx<T>::ab2(pc[i]);
             sq2 = warp_sum(sq2);
-            if (lane == 0) nrm_s = sqrt(sq2);
+            if (lane == 0) inv_s = sq2 > 0.0 ? rsqrt(sq2) : 0.0;
         }
         __syncthreads();
-        const double inv = nrm_s > 0 ? 1.0 / nrm_s : 0.0;
+        const double inv = inv_s;
         for (int i = threadIdx.x; i < rows; i += blockDim.x) pc[i] = Cx<T>::sc(inv, pc[i]);
         __syncthreads();
     }
+    if (P != a.P)
+        for (int e = threadIdx.x; e < rows * (clast + 1); e += blockDim.x) a.P[e] = P[e];
 
     __syncthreads();
     if (threadIdx.x == 0) { long long _t = clock64(); a.info->phase[6] = _t - t_mark; t_mark = _t; }
@@ -1363,19 +1454,19 @@ __device__ __forceinline__ void gmresdr_restart_body(const GdrArgs<T> &a) {
     for (int e = threadIdx.x; e < rows * nc; e += blockDim.x) {
         const int i = e % rows, q = e / rows;
         T s = Cx<T>::zero();
-        for (int j = 0; j < m; ++j) s = add(s, Cx<T>::mul(a.H[i + (size_t)j * ldh], P[j + (size_t)q * rows]));
+        for (int j = 0; j < m; ++j) s = Cx<T>::mac(s, a.H[i + (size_t)j * ldh], P[j + (size_t)q * rows]);
         W[i + (size_t)q * rows] = s;
     }
     __syncthreads();
     for (int e = threadIdx.x; e < (nc + 1) * nc; e += blockDim.x) {
         const int i = e % (nc + 1), q = e / (nc + 1);
         T s = Cx<T>::zero();
-        for (int l = 0; l < rows; ++l) s = add(s, Cx<T>::mul(Cx<T>::cj(P[l + (size_t)i * rows]), W[l + (size_t)q * rows]));
+        for (int l = 0; l < rows; ++l) s = Cx<T>::macc(s, P[l + (size_t)i * rows], W[l + (size_t)q * rows]);
         a.Hnew[i + (size_t)q * ldh] = s;
     }
     for (int i = threadIdx.x; i <= nc; i += blockDim.x) {
         T s = Cx<T>::zero();
-        for (int l = 0; l < rows; ++l) s = add(s, Cx<T>::mul(Cx<T>::cj(P[l + (size_t)i * rows]), res[l]));
+        for (int l = 0; l < rows; ++l) s = Cx<T>::macc(s, P[l + (size_t)i * rows], res[l]);
         a.cnew[i] = s;
     }
     __syncthreads();
@@ -1383,7 +1474,7 @@ __device__ __forceinline__ void gmresdr_restart_body(const GdrArgs<T> &a) {
 }
 
 template <class T>
-__global__ void __launch_bounds__(kGdrThreads) k_gmresdr_restart(GdrArgs<T> a) {
+__global__ void __launch_bounds__(kGdrThreads, 1) k_gmresdr_restart(GdrArgs<T> a) {
     pdl_wait();
     gmresdr_restart_body<T>(a);
 }
@@ -1391,7 +1482,7 @@ __global__ void __launch_bounds__(kGdrThreads) k_gmresdr_restart(GdrArgs<T> a) {
 // many independent restart steps, one block each (the batched coarse phase): block b runs
 // args[b] when active[b] is set
 template <class T>
-__global__ void __launch_bounds__(kGdrThreads) k_gmresdr_restart_batch(const GdrArgs<T> *args, const int *active) {
+__global__ void __launch_bounds__(kGdrThreads, 1) k_gmresdr_restart_batch(const GdrArgs<T> *args, const int *active) {
     pdl_wait();
     if (!active[blockIdx.x]) return;
     const GdrArgs<T> a = args[blockIdx.x];
@@ -1460,20 +1551,26 @@ template <class D>
 void launch_small_gemv(const D *M, int k, const D *c, D *out, cudaStream_t s) {
     launch(k_small_gemv<D>, 1, kSmallThreads, 0, s, M, k, c, out);
 }
+// W, Z (T) and the eigenvector work Y (complex, m x m) go to shared memory in that order while
+// they fit
+template <class T>
+size_t gmresdr_restart_smem(int m, int *parts) {
+    const size_t mm = m;
+    const size_t w = (mm + 1) * mm;
+    const size_t sizes[3] = {w * sizeof(T), (gdr_y_offset(m) - w) * sizeof(T), mm * mm * sizeof(cplx)};
+    size_t smem = 0;
+    *parts = 0;
+    for (int q = 0; q < 3 && smem + sizes[q] <= kGdrSmemMax; ++q) {
+        smem += sizes[q];
+        *parts = q + 1;
+    }
+    return smem;
+}
 template <class T>
 cudaError_t launch_gmresdr_restart(const GdrArgs<T> &a_in, cudaStream_t s) {
     GdrArgs<T> a = a_in;
-    // W, Z, B (T) and the eigenvector work Y (complex, m x m) go to shared memory in that
-    // order while they fit
-    const size_t m = a.m;
-    const size_t parts[4] = {(m + 1) * m * sizeof(T), m * m * sizeof(T), m * m * sizeof(T), m * m * sizeof(cplx)};
-    size_t smem = 0;
-    a.smem = 0;
-    for (int q = 0; q < 4 && smem + parts[q] <= kGdrSmemMax; ++q) {
-        smem += parts[q];
-        a.smem = q + 1;
-    }
-    if (smem > 48 * 1024) {
+    const size_t smem = gmresdr_restart_smem<T>(a.m, &a.smem);
+    if (smem > 30 * 1024) {         // 48 KB with the static part
         // without the raised limit the launch would fail; report the attribute call instead
         const cudaError_t e = smem_attr_once((const void *)k_gmresdr_restart<T>, (int)kGdrSmemMax);
         if (e != cudaSuccess) return e;
@@ -1482,22 +1579,10 @@ cudaError_t launch_gmresdr_restart(const GdrArgs<T> &a_in, cudaStream_t s) {
     return cudaGetLastError();
 }
 template <class T>
-size_t gmresdr_restart_smem(int m, int *parts) {
-    const size_t mm = m;
-    const size_t sizes[4] = {(mm + 1) * mm * sizeof(T), mm * mm * sizeof(T), mm * mm * sizeof(T), mm * mm * sizeof(cplx)};
-    size_t smem = 0;
-    *parts = 0;
-    for (int q = 0; q < 4 && smem + sizes[q] <= kGdrSmemMax; ++q) {
-        smem += sizes[q];
-        *parts = q + 1;
-    }
-    return smem;
-}
-template <class T>
 cudaError_t launch_gmresdr_restart_batch(const GdrArgs<T> *args, const int *active, int count, int m, cudaStream_t s) {
     int parts = 0;
     const size_t smem = gmresdr_restart_smem<T>(m, &parts);
-    if (smem > 48 * 1024) {
+    if (smem > 30 * 1024) {         // 48 KB with the static part
         const cudaError_t e = smem_attr_once((const void *)k_gmresdr_restart_batch<T>, (int)kGdrSmemMax);
         if (e != cudaSuccess) return e;
     }

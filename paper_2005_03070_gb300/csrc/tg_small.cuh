@@ -36,7 +36,7 @@ struct GdrArgs {
     T *P;            // out: P_{k+1}, (m+1) x (kk+1), ld m+1; its first kk columns (m rows) are P_k
     T *Hnew;         // out: P_{k+1}^H Hbar P_k, (kk+1) x kk, leading dimension ldh
     T *cnew;         // out: P_{k+1}^H res, kk+1
-    T *work;         // scratch: (m+1) m + 2 m^2 + 3 m + 2 elements of T
+    T *work;         // scratch: (m+1) m + m^2 + 3 m + 2 elements of T
     cplx *ywork;     // scratch: m * m complex
     cplx *gwork;     // scratch: m * m complex
     GdrInfo *info;
