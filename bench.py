@@ -97,8 +97,8 @@ NOMINAL_HBM_GBS = 8000.0                         # the ~8 TB/s nominal HBM3e fig
 # DRAM bytes (read + write) per launch over algorithmic bytes per launch, per kernel class, from
 # an ncu capture of a smaller case of the same kernel: the traffic of a full-size launch is this
 # ratio times its algorithmic bytes (it grows in proportion to rows x columns).  An entry goes
-# when its kernel changes.
-NCU_TRAFFIC_RATIO = {}
+# when its kernel changes.  gemv_t: k_arn_dots_pipe<double> at 127^3 x 45, (737.5 + 3.0) MB over 737.4 MB.
+NCU_TRAFFIC_RATIO = {"gemv_t": 1.004}
 
 
 def dgemm_tflops(dev, n=4096, reps=5):
