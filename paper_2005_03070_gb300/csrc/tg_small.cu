@@ -448,14 +448,18 @@ __device__ void hessenberg(T *A, int m, T *Z, T *w2) {
 // Francis double-shift QR on the real upper Hessenberg H (m x m, ld m), accumulating Z.
 // Returns 0 on success, 1 if an eigenvalue failed to converge in 40 m sweeps.
 __device__ int real_schur(double *H, int m, double *Z) {
-    __shared__ int hi_s, l_s, status_s, act_s;
+    __shared__ int hi_s, l_s, status_s;
+    // what to do next, by turns in two places: after a deflation warp 0 goes on to the next decision
+    // at once, and a slower warp may not have read this one yet (every warp has read the one before
+    // last: a block barrier lies between)
+    __shared__ int act_s[2];
     __shared__ double hs_s[2][6];      // w and g w of the current and the next reflector
     __shared__ double win_s[9];
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
     if (tid == 0) { hi_s = m - 1; status_s = 0; }
     __syncthreads();
     int its = 0, total = 0;
-    while (true) {
+    for (int turn = 0;; turn ^= 1) {
         if (tid < 32) {
             // the active block: the largest l <= hi with a negligible H[l, l-1] (0 if none),
             // found by warp 0 with a ballot over the candidates
@@ -477,18 +481,19 @@ __device__ int real_schur(double *H, int m, double *Z) {
             }
             if (lane == 0) {
                 if (l > 0) H[l + (size_t)(l - 1) * m] = 0.0;
-                act_s = 0;
-                if (hi < 0) act_s = -1;
+                int act = 0;
+                if (hi < 0) act = -1;
                 else {
                     l_s = l;
-                    if (l == hi) { hi_s = hi - 1; act_s = 1; }
-                    else if (l == hi - 1) { act_s = 2; }   // 2x2 block: standardise below
-                    else act_s = 3;                         // QR sweep on l..hi
+                    if (l == hi) { hi_s = hi - 1; act = 1; }
+                    else if (l == hi - 1) { act = 2; }   // 2x2 block: standardise below
+                    else act = 3;                         // QR sweep on l..hi
                 }
+                act_s[turn] = act;
             }
         }
         __syncthreads();
-        const int act = act_s;
+        const int act = act_s[turn];
         if (act < 0) break;
         if (act == 1) { its = 0; continue; }
         const int hi = hi_s, l = l_s;
@@ -671,7 +676,8 @@ __device__ int real_schur(double *H, int m, double *Z) {
 __device__ __forceinline__ double cabs1(cplx a) { return fabs(a.re) + fabs(a.im); }
 
 __device__ int complex_schur(cplx *H, int m, cplx *Z) {
-    __shared__ int hi_s, l_s, act_s, status_s;
+    __shared__ int hi_s, l_s, status_s;
+    __shared__ int act_s[2];        // by turns, as in real_schur
     __shared__ double rs_s[2][4];   // a.re, a.im, b.re, b.im of the current and the next rotation
     __shared__ cplx win_s[6];
     __shared__ cplx x_s, y_s;
@@ -679,7 +685,7 @@ __device__ int complex_schur(cplx *H, int m, cplx *Z) {
     if (tid == 0) { hi_s = m - 1; status_s = 0; }
     __syncthreads();
     int its = 0, total = 0;
-    while (true) {
+    for (int turn = 0;; turn ^= 1) {
         if (tid < 32) {
             const int hi = hi_s;
             __syncwarp();          // every lane has read hi_s before lane 0 may update it
@@ -699,17 +705,18 @@ __device__ int complex_schur(cplx *H, int m, cplx *Z) {
             }
             if (lane == 0) {
                 if (l > 0) H[l + (size_t)(l - 1) * m] = {0.0, 0.0};
-                act_s = 0;
-                if (hi <= 0) act_s = -1;
+                int act = 0;
+                if (hi <= 0) act = -1;
                 else {
                     l_s = l;
-                    if (l == hi) { hi_s = hi - 1; act_s = 1; }
-                    else act_s = 2;
+                    if (l == hi) { hi_s = hi - 1; act = 1; }
+                    else act = 2;
                 }
+                act_s[turn] = act;
             }
         }
         __syncthreads();
-        const int act = act_s;
+        const int act = act_s[turn];
         if (act < 0) break;
         if (act == 1) { its = 0; continue; }
         ++its;
