@@ -2885,29 +2885,23 @@ namespace tg {
 
 // Batched float32-inner / float64-refinement BiCGStab(ncyc)-Proj(k) over every instance at
 // once: all instances advance their cycles in lock-step, one launch per phase for all of
-// them (grid (gx, count)), the 8-iteration sequence of the four BiCGStab phases is one CUDA
-// graph replayed until every column of the cycle has finished.  Per column: the schedule,
-// safeguards and statistics of the single-instance float32 refinement.  gx (blocks per
-// instance) is chosen once
-// per handle by timing the iteration graph for each candidate (the autotuner).
+// them (blocks by the table of batch_blocks), the 8-iteration sequence of the four BiCGStab phases is
+// one CUDA graph replayed until every column of the cycle has finished.  Per column: the schedule,
+// safeguards and statistics of the single-instance float32 refinement.  gx (blocks per instance on
+// average) is chosen once per handle by timing the iteration graph for each candidate (the
+// autotuner).
 constexpr int kMrPartW = 4 * kBatchR > 32 * kBatchR ? 4 * kBatchR : 32 * kBatchR;
 
-// Blocks of a batched launch at most: the partial sums' room (2 KB a block).
-static int batch_max_blocks(const tg_batch *b) { return std::max(16384, b->count + 4096); }
-
-// Gives the instances about `total` blocks in proportion to their points (one at least, and no
-// more than there are groups of 256 points) and copies the blocks' table to buf.
+// Copies the table of about `total` blocks (batch_blocks) to buf.
 static int batch_map(tg_batch *b, int64_t total, DBuf &buf, int *blocks) {
-    double points = 0.0;
-    for (const tg_op *op : b->ops) points += op->n;
-    std::vector<int4> map;
-    for (int i = 0; i < b->count; ++i) {
-        const int64_t n = b->ops[i]->n, want = (int64_t)(total * (n / points) + 0.5);
-        const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(want, (n + kThreads - 1) / kThreads)), first = (int)map.size();
-        for (int k = 0; k < nb; ++k) map.push_back(make_int4(i, k, nb, first));
+    std::vector<int64_t> n;
+    for (const tg_op *op : b->ops) n.push_back(op->n);
+    const std::vector<int4> map = batch_blocks(n, total);
+    if ((int64_t)map.size() > batch_room(b->count)) {
+        set_error("a batched launch of %zu blocks does not fit the room for its partial sums", map.size());
+        return TG_BAD_ARG;
     }
     *blocks = (int)map.size();
-    TG_CHECK(buf.ensure(map.size() * sizeof(int4)));
     TG_CHECK_CUDA(cudaMemcpyAsync(buf.p, map.data(), map.size() * sizeof(int4), cudaMemcpyHostToDevice, b->all.stream));
     TG_CHECK_CUDA(cudaStreamSynchronize(b->all.stream));
     return TG_OK;
@@ -2926,8 +2920,10 @@ static int batch_all_ready(tg_batch *b) {
     TG_CHECK(A.e32.ensure(tot * 4));
     TG_CHECK(A.rsave.ensure(tot * 4));
     TG_CHECK(A.r64.ensure(tot * 8));
-    TG_CHECK(A.part.ensure((size_t)batch_max_blocks(b) * kMrPartW * 8));
-    TG_CHECK(A.map.ensure((size_t)batch_max_blocks(b) * sizeof(int4)));
+    const size_t room = (size_t)batch_room(b->count);
+    TG_CHECK(A.part.ensure(room * kMrPartW * 8));
+    TG_CHECK(A.map.ensure(room * sizeof(int4)));
+    TG_CHECK(A.map_res.ensure(room * sizeof(int4)));
     TG_CHECK(A.st.ensure((size_t)b->count * R * sizeof(BiState<double>)));
     TG_CHECK(A.ctl.ensure((size_t)b->count * sizeof(MrCtl)));
     // target2, inv, scale (R each), norms (2 R), cvec, dvec (32 R each), capv (R) per instance
@@ -3029,7 +3025,7 @@ static int batch_tune(tg_batch *b) {
     int best_gx = 16;
     A.ntune = 0;
     for (int gx : cands) {
-        if (gx > 8 && (int64_t)gx * b->count > batch_max_blocks(b) - b->count) break;
+        if (!batch_fits(gx, b->count)) break;
         TG_CHECK_CUDA(cudaMemcpyAsync(P0.target2, zeros.data(), zeros.size() * 8, cudaMemcpyHostToDevice, s));
         TG_CHECK_CUDA(cudaMemcpyAsync(A.r32.p, A.rsave.p, tot * 4, cudaMemcpyDeviceToDevice, s));
         TG_CHECK_CUDA(cudaMemsetAsync(A.e32.p, 0, tot * 4, s));

@@ -13,9 +13,35 @@
 // float64 coefficients.
 #pragma once
 
+#include <algorithm>
+#include <cstdint>
+#include <vector>
+
 #include "tg_mrhs.cuh"
 
 namespace tg {
+
+// Blocks that a batch's tables may hold, the room of the partial sums (2 KB a block).  A table for
+// gx blocks per instance on average has at most gx + 1 times `count` (every instance's share is
+// rounded, and at least one), so the smallest candidate, 8, always fits.
+inline int64_t batch_room(int64_t count) { return std::max<int64_t>(16384, 9 * count); }
+inline bool batch_fits(int64_t gx, int64_t count) { return (gx + 1) * count <= batch_room(count); }
+
+// The table of a launch of about `total` blocks: instance, block in it, its blocks and its first
+// block, in proportion to the instances' points n (one block at least, and no more than there are
+// groups of kThreads points).
+inline std::vector<int4> batch_blocks(const std::vector<int64_t> &n, int64_t total) {
+    double points = 0.0;
+    for (const int64_t v : n) points += (double)v;
+    std::vector<int4> map;
+    for (size_t i = 0; i < n.size(); ++i) {
+        const int64_t want = (int64_t)(total * (n[i] / points) + 0.5);
+        const int64_t nb = std::max<int64_t>(1, std::min<int64_t>(want, (n[i] + kThreads - 1) / kThreads));
+        const int first = (int)map.size();
+        for (int k = 0; k < nb; ++k) map.push_back(make_int4((int)i, k, (int)nb, first));
+    }
+    return map;
+}
 
 // One instance of a batch (device copy, read by every block of the instance).
 struct MrSeg {
