@@ -142,6 +142,12 @@ int tg_restrict(const tg_op *op, const void *fine, void *coarse, int ncols, void
 #define TG_INTERP_CUBIC  1
 int tg_op_set_interp(tg_op *op, int interp);
 
+/* Limits of the waits in this operator's one-launch cycles (small real grids: the blocks of a
+ * launch meet at barriers), in polls of about half a microsecond: `start` for the first barrier
+ * of a launch, `step` for the later ones (default 2^20 each).  A launch whose wait runs out
+ * ends by itself and its solve returns TG_SYNC_TIMEOUT.                               */
+int tg_op_sync_limits(tg_op *op, int start, int step);
+
 /* ------------------------------------------------------------------ phase 1: coarse solve
  * GMRES-DR(m,k) (Section 2.1) on the coarse operator (transpose = 1: on A_c^T, giving
  * left eigenvectors for the adjoint solve), right-hand side b_c = restrict(b_fine)

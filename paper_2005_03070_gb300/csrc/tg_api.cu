@@ -208,7 +208,7 @@ enum Slot {
     S_IG, S_IU, S_IP, S_IPR, S_IPRI, S_IT, S_IINFO,
     S_AE_S, S_AE_W, S_AE_H, S_AE_WW, S_AE_HA, S_AE_Y, S_AE_U, S_AE_P, S_AE_Z, S_AE_TH, S_AE_WR, S_AE_WI,
     S_AE_ORD, S_AE_ERES, S_AE_WORK, S_AE_YW, S_AE_GW, S_AE_INFO, S_AE_DUM, S_PADX, S_PADR, S_AE_HR, S_AE_WWR, S_IP32,
-    S_P2, S_V2, S_BAR,
+    S_P2, S_V2,
     S_COUNT
 };
 
@@ -250,6 +250,7 @@ struct tg_op {
     PinBuf pin;
     unsigned ws_gen = 0;                 // bumped whenever a workspace buffer is (re)allocated
     std::vector<tg::GdrGraph> graphs;    // captured coarse GMRES-DR cycles
+    tg::SyncLimits sync;                 // limits of the one-launch cycles' waits
     cudaStream_t cap_stream = nullptr;   // private stream for captures (the caller's may be
                                          // the legacy stream, which cannot be captured)
     tg_op() = default;
@@ -299,6 +300,7 @@ struct SmallArea {
     static constexpr size_t arn_nrm = 40960;    // ||w||^2, 1 / ||w|| (+ 32); Arnoldi: beta, 1 / beta, t (+ 64)
     static constexpr size_t gmres_inv = 41984;  // 1 / ||r|| of a GMRES cycle
     static constexpr size_t arn_c = 49152;      // Arnoldi: first-pass coefficients h1
+    static constexpr size_t sync = 57344;       // SyncWords of a one-launch cycle
     static constexpr size_t bytes = 1 << 16;
 };
 static_assert(kMaxCols * 16 <= 8192, "coefficient vectors must fit their slots");
@@ -875,6 +877,13 @@ extern "C" int tg_op_set_interp(tg_op *op, int interp) {
     return TG_OK;
 }
 
+extern "C" int tg_op_sync_limits(tg_op *op, int start, int step) {
+    TG_ARG(op && start >= 0 && step >= 0, "bad argument");
+    op->sync.start = start;
+    op->sync.step = step;
+    return TG_OK;
+}
+
 extern "C" int tg_restrict(const tg_op *op, const void *fine, void *coarse, int ncols, void *stream) {
     TG_ARG(op && coarse && fine && ncols >= 0, "bad argument");
     return restrict_impl(op, fine, coarse, ncols, (cudaStream_t)stream);
@@ -1089,10 +1098,10 @@ template <class T> constexpr int pers_max_rows(bool idr) {
 }
 
 // Queues one cooperative launch of a cycle kernel over the whole GPU (fewer blocks than SMs for
-// fewer than 32 points each) and its zeroed barrier word.
+// fewer than 32 points each) and its zeroed barrier words.
 template <class K, class Args>
 static int persist_launch(K kernel, const DevOp &A, const DevOp32 &A32, const Args &a, cudaStream_t s) {
-    TG_CHECK_CUDA(cudaMemsetAsync(a.bar, 0, sizeof(unsigned), s));
+    TG_CHECK_CUDA(cudaMemsetAsync(a.words, 0, sizeof(SyncWords), s));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(std::max(1, std::min(num_sms(), (A.n + 31) / 32)));
     cfg.blockDim = dim3(kPersThreads);
@@ -1107,8 +1116,24 @@ static int persist_launch(K kernel, const DevOp &A, const DevOp32 &A32, const Ar
 }
 static int persist_ready(tg_op *op, cudaStream_t s) {
     // two reduction buffers and the projection's partial sums
-    TG_CHECK(red_ready(op, (size_t)(2 * kPersPart + kPersCols) * num_sms() * sizeof(double), s));
-    return wsx(op, S_BAR, 64);
+    return red_ready(op, (size_t)(2 * kPersPart + kPersCols) * num_sms() * sizeof(double), s);
+}
+static SyncWords *persist_words(tg_op *op) {
+    return reinterpret_cast<SyncWords *>(wsp<char>(op, S_SMALL) + SmallArea::sync);
+}
+// Reads a launch's report (bytes at dev) and its barrier words; a wait that gave up is an error
+// whatever the report says.
+static int persist_look(tg_op *op, const void *dev, void *host, size_t bytes, const char *what, cudaStream_t s) {
+    char *pin = reinterpret_cast<char *>(op->pin.p);
+    SyncWords *w = reinterpret_cast<SyncWords *>(pin + (1 << 15));
+    TG_CHECK_CUDA(cudaMemcpyAsync(w, persist_words(op), sizeof(SyncWords), cudaMemcpyDeviceToHost, s));
+    TG_CHECK(readback(op, dev, bytes, s));
+    memcpy(host, pin, bytes);
+    if (w->failed) {
+        set_error("a grid barrier of the %s cycle timed out", what);
+        return TG_SYNC_TIMEOUT;
+    }
+    return TG_OK;
 }
 
 // Runs the cycle that `a` describes (first launch and continuations); res: the launch's report.
@@ -1123,18 +1148,15 @@ static int bicg_persist_run(tg_op *op, const DevOp &A, const DevOp32 &A32, BiPer
     a.rh = w.rh; a.p[0] = w.p; a.p[1] = wsp<T>(op, S_P2); a.v[0] = w.v; a.v[1] = wsp<T>(op, S_V2);
     a.s = w.s; a.t = w.t;
     a.part = wsp<double>(op, S_PART);
-    a.bar = wsp<unsigned>(op, S_BAR);
+    a.words = persist_words(op);
+    a.limits = op->sync;
     a.out = reinterpret_cast<BiPersOut *>(wsp<char>(op, S_SMALL) + SmallArea::bistate);
     a.max_iters = 1024;              // bounds one launch to some tens of milliseconds
     static_assert(sizeof(BiPersOut) <= SmallArea::dot_out - SmallArea::bistate, "the report fits its slot");
     *res = BiPersOut{};
     double xb, fl;
     op_cost(A, &xb, &fl);
-    auto look = [&]() -> int {
-        TG_CHECK(readback(op, a.out, sizeof(BiPersOut), s));
-        memcpy(res, op->pin.p, sizeof(BiPersOut));
-        return TG_OK;
-    };
+    auto look = [&]() { return persist_look(op, a.out, res, sizeof(BiPersOut), "BiCGStab", s); };
     for (a.first = 1;; a.first = 0) {
         const int it0 = res->st.iters, ev = prof_begin(s);
         TG_CHECK(persist_launch(k_bi_persist<T>, A, A32, a, s));
@@ -1147,10 +1169,6 @@ static int bicg_persist_run(tg_op *op, const DevOp &A, const DevOp32 &A32, BiPer
             set_error("BiCGStab cycle exceeded its product cap");
             return TG_SYNC_TIMEOUT;
         }
-    }
-    if (res->st.status == kStatusSync) {
-        set_error("a grid barrier of the BiCGStab cycle timed out");
-        return TG_SYNC_TIMEOUT;
     }
     return TG_OK;
 }
@@ -1587,23 +1605,19 @@ static int idr_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r, 
             IdrPersArgs<T> a;
             a.P = P; a.x = x; a.r = r; a.G = G; a.U = U; a.t = t; a.ld = ld;
             a.part = wsp<double>(op, S_PART);
-            a.bar = wsp<unsigned>(op, S_BAR);
+            a.words = persist_words(op);
+            a.limits = op->sync;
             a.st = st; a.target2 = target2; a.kappa = kappa; a.s = sd; a.cap = cap;
             a.max_rounds = 64;           // bounds one launch to a few milliseconds
             IdrState<double> h{};
             for (a.first = 1;; a.first = 0) {
                 TG_PROF(P_IDR_CYCLE, 0, 0, TG_CHECK(persist_launch(k_idr_persist<T>, A, A32, a, s)));
-                TG_CHECK(readback(op, st, sizeof(h), s));
-                memcpy(&h, op->pin.p, sizeof(h));
+                TG_CHECK(persist_look(op, st, &h, sizeof(h), "IDR", s));
                 if (h.status != 0) break;
                 if ((int64_t)h.rounds * (sd + 1) > (int64_t)cap + 2 * (sd + 1)) {
                     set_error("IDR cycle exceeded its product cap");
                     return TG_SYNC_TIMEOUT;
                 }
-            }
-            if (h.status == kStatusSync) {
-                set_error("a grid barrier of the IDR cycle timed out");
-                return TG_SYNC_TIMEOUT;
             }
             out->mvps = h.mvps;
             out->iters = h.rounds;

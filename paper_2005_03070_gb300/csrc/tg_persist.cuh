@@ -12,8 +12,9 @@
 // the owner's values), so x / r / p are updated in the pass that forms v = A p, and s in the pass
 // that forms t = A s.  p and v alternate between two buffers, because neighbours still read the
 // old ones.
-// Data of other blocks is read past the L1 cache (__ldcg).  Every wait ends after kSyncPolls
-// polls with an error status that the host turns into TG_SYNC_TIMEOUT.
+// Data of other blocks is read past the L1 cache (__ldcg).  Every wait ends after a limited number
+// of polls; the block that gives up says so in a word of its own, every block then leaves at its next
+// barrier, and the host turns the word into TG_SYNC_TIMEOUT.
 #pragma once
 
 #include "tg_arnoldi.cuh"
@@ -22,32 +23,56 @@
 namespace tg {
 
 constexpr int kPersThreads = 256;
-constexpr unsigned kSyncPolls = 1u << 20;     // about half a second
-constexpr int kStatusSync = 9;                // cycle status of a barrier that gave up
 constexpr int kPersPart = 16;                 // reduced values per pass at most
 
-// The blocks' meeting point: bar is zero at launch and counts arrivals; part holds two buffers
-// of kPersPart x blocks partial sums (a block can write the next but one reduction only after
-// all have read this one).
+// Polls of a wait (half a microsecond each): the first barrier of a launch, and the later ones.
+struct SyncLimits {
+    unsigned start = 1u << 20, step = 1u << 20;
+};
+
+// The barrier's words, zero at launch.  count: arrivals, and kSyncGaveUp once a block has given up;
+// failed: written only by that block, never cleared within a launch.
+struct SyncWords {
+    unsigned count, failed;
+};
+constexpr unsigned kSyncGaveUp = 0x80000000u;
+constexpr unsigned kFailedStart = 1, kFailedStep = 2;
+
+// The blocks' meeting point: part holds two buffers of kPersPart x blocks partial sums (a block can
+// write the next but one reduction only after all have read this one).  Once ok is false (for all
+// threads of a block alike) it stays false, and nothing waits or counts any more: sums are
+// meaningless then, and their callers leave.
 struct GridSync {
-    unsigned *bar;
+    SyncWords *w;
     double *part;
+    SyncLimits limits;
     unsigned round;
     int parity;
     bool ok;
-    __device__ GridSync(unsigned *b, double *p) : bar(b), part(p), round(0), parity(0), ok(true) {}
+    __device__ GridSync(SyncWords *words, double *p, SyncLimits l)
+        : w(words), part(p), limits(l), round(0), parity(0), ok(true) {}
     __device__ void wait() {
         __shared__ bool ok_s;          // rewritten after the next barrier's first __syncthreads only
+        if (!ok) return;
         ++round;
         __syncthreads();
         if (threadIdx.x == 0) {        // the release covers the block's writes (ordered by the barrier above)
-            const unsigned target = round * gridDim.x;
+            const unsigned target = round * gridDim.x, limit = round == 1 ? limits.start : limits.step;
             unsigned seen = 0, polls = 0;
-            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-            do {
-                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(bar) : "memory");
-            } while (seen < target && ++polls < kSyncPolls);
-            ok_s = seen >= target;
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&w->count) : "memory");
+            while (true) {
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&w->count) : "memory");
+                if (seen >= target) break;               // complete, or kSyncGaveUp is set
+                if (polls++ < limit) continue;
+                // give up, unless the barrier is completed or given up first: both are the same word
+                const unsigned old = atomicCAS(&w->count, seen, seen | kSyncGaveUp);
+                if (old == seen) {
+                    w->failed = round == 1 ? kFailedStart : kFailedStep;
+                    seen = kSyncGaveUp;
+                    break;
+                }
+            }
+            ok_s = seen < kSyncGaveUp;
         }
         __syncthreads();
         ok = ok_s;
@@ -118,7 +143,8 @@ template <class T>
 struct BiPersArgs {
     T *x, *r, *rh, *p[2], *v[2], *s, *t;      // x, r: T = float and whole: the correction and its residual
     double *part;
-    unsigned *bar;
+    SyncWords *words;
+    SyncLimits limits;
     BiPersOut *out;
     double target2;                           // whole = 0
     int cap, first, max_iters;                // first: the cycle starts here (r_hat = p = r)
@@ -187,7 +213,7 @@ template <class T>
 __global__ void __launch_bounds__(kPersThreads, 1) k_bi_persist(DevOp op, DevOp32 o32, BiPersArgs<T> a) {
     __shared__ BiState<double> S;
     __shared__ double tot[kPersPart];
-    GridSync gs(a.bar, a.part);
+    GridSync gs(a.words, a.part, a.limits);
     const int n = op.n, per = (n + gridDim.x - 1) / gridDim.x;
     const int lo = min(n, (int)blockIdx.x * per), hi = min(n, lo + per);
     T *p = a.p[0], *p2 = a.p[1], *v = a.v[0], *v2 = a.v[1];      // the current p and v, and the other buffers
@@ -381,15 +407,12 @@ __global__ void __launch_bounds__(kPersThreads, 1) k_bi_persist(DevOp op, DevOp3
         gs.sum<2>(acc, tot);
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        if (!gs.ok) S.status = kStatusSync;
-        if (blockIdx.x == 0 || !gs.ok) {
-            a.out->st = S;
-            a.out->nr = nr_s;
-            a.out->rt = rt_s;
-            a.out->rr = tot[0];
-            a.out->bb = tot[1];
-        }
+    if (threadIdx.x == 0 && blockIdx.x == 0) {
+        a.out->st = S;
+        a.out->nr = nr_s;
+        a.out->rt = rt_s;
+        a.out->rr = tot[0];
+        a.out->bb = tot[1];
     }
 }
 
@@ -399,7 +422,8 @@ struct IdrPersArgs {
     T *x, *r, *G, *U, *t;
     size_t ld;
     double *part;
-    unsigned *bar;
+    SyncWords *words;
+    SyncLimits limits;
     IdrState<double> *st;
     double target2, kappa;
     int s, cap, first, max_rounds;
@@ -415,7 +439,7 @@ __global__ void __launch_bounds__(kPersThreads, 1) k_idr_persist(DevOp op, DevOp
     __shared__ double tot[kPersPart];
     __shared__ T cs[M], al[M];
     __shared__ double inv[M];                      // 1 / M_kk
-    GridSync gs(a.bar, a.part);
+    GridSync gs(a.words, a.part, a.limits);
     const int n = op.n, s = a.s, per = (n + gridDim.x - 1) / gridDim.x;
     const int lo = min(n, (int)blockIdx.x * per), hi = min(n, lo + per);
     const size_t ld = a.ld;
@@ -603,10 +627,7 @@ __global__ void __launch_bounds__(kPersThreads, 1) k_idr_persist(DevOp op, DevOp
             __syncthreads();
         }
     }
-    if (threadIdx.x == 0) {
-        if (!gs.ok) S.status = kStatusSync;
-        if (blockIdx.x == 0 || !gs.ok) *a.st = S;
-    }
+    if (threadIdx.x == 0 && blockIdx.x == 0) *a.st = S;
 }
 
 }  // namespace tg

@@ -33,8 +33,8 @@ INTERP = {"linear": 0, "cubic": 1}
 
 EXPORTS = [
     "tg_status_string", "tg_last_error", "tg_setup_operator", "tg_destroy_op", "tg_op_size", "tg_apply",
-    "tg_prolong", "tg_restrict", "tg_op_set_interp", "tg_coarse_gmresdr", "tg_defl_from_basis", "tg_destroy_defl",
-    "tg_defl_copy", "tg_project", "tg_solve_proj", "tg_solve_idr", "tg_improve_defl", "tg_adjoint_solve",
+    "tg_prolong", "tg_restrict", "tg_op_set_interp", "tg_op_sync_limits", "tg_coarse_gmresdr", "tg_defl_from_basis",
+    "tg_destroy_defl", "tg_defl_copy", "tg_project", "tg_solve_proj", "tg_solve_idr", "tg_improve_defl", "tg_adjoint_solve",
     "tg_kappa_gradient",
     "tg_harmonic_ritz", "tg_harmonic_ritz_noalloc", "tg_profile_enable", "tg_profile_read", "tg_launch_count",
     "tg_batch_create", "tg_batch_layout", "tg_batch_setup", "tg_batch_solve", "tg_destroy_batch",
@@ -84,6 +84,7 @@ def load() -> C.CDLL:
         "tg_prolong": (i32, [vp, vp, vp, i32, vp]),
         "tg_restrict": (i32, [vp, vp, vp, i32, vp]),
         "tg_op_set_interp": (i32, [vp, i32]),
+        "tg_op_sync_limits": (i32, [vp, i32, i32]),
         "tg_coarse_gmresdr": (i32, [vp, i32, vp, i32, i32, i32, dbl, dbl, i32, vp, C.POINTER(vp), i32, i32,
                                     C.POINTER(TgStats), vp]),
         "tg_defl_from_basis": (i32, [vp, i32, vp, i32, i32, i32, C.POINTER(vp), vp]),
@@ -182,6 +183,10 @@ class Operator:
         _check(_lib.tg_apply(self._h, level, int(transpose), precision, _ptr(x), _ptr(y), _stream(stream)),
                "tg_apply")
         return y
+
+    def sync_limits(self, start, step):
+        """tg_op_sync_limits: polls of the first and of the later waits of a one-launch cycle."""
+        _check(_lib.tg_op_sync_limits(self._h, int(start), int(step)), "tg_op_sync_limits")
 
     def prolong(self, coarse, fine=None, stream=None):
         ncols = coarse.numel() // self.nc
