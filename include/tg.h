@@ -144,8 +144,9 @@ int tg_op_set_interp(tg_op *op, int interp);
 
 /* Limits of the waits in this operator's one-launch cycles (small real grids: the blocks of a
  * launch meet at barriers), in polls of about half a microsecond: `start` for the first barrier
- * of a launch, `step` for the later ones (default 2^20 each).  A launch whose wait runs out
- * ends by itself and its solve returns TG_SYNC_TIMEOUT.                               */
+ * of a launch (default 2^16), `step` for the later ones (default 2^20).  A launch whose wait
+ * runs out ends by itself.  At the first barrier nothing is lost: the solve goes on as a chain
+ * of launches.  At a later one it returns TG_SYNC_TIMEOUT.                             */
 int tg_op_sync_limits(tg_op *op, int start, int step);
 
 /* ------------------------------------------------------------------ phase 1: coarse solve

@@ -251,6 +251,7 @@ struct tg_op {
     unsigned ws_gen = 0;                 // bumped whenever a workspace buffer is (re)allocated
     std::vector<tg::GdrGraph> graphs;    // captured coarse GMRES-DR cycles
     tg::SyncLimits sync;                 // limits of the one-launch cycles' waits
+    bool one_launch = true;              // false once a cycle's launch could not start (per solve)
     cudaStream_t cap_stream = nullptr;   // private stream for captures (the caller's may be
                                          // the legacy stream, which cannot be captured)
     tg_op() = default;
@@ -1097,6 +1098,10 @@ template <class T> constexpr int pers_max_rows(bool idr) {
     return sizeof(T) == 4 ? 6 << 16 : idr ? 13 << 16 : 9 << 16;
 }
 
+// A launch that did not start: refused (more blocks than the stream's SMs take, or no cooperative
+// launches), or given up at its first barrier.  Nothing was written.
+constexpr int kNotStarted = -1;
+
 // Queues one cooperative launch of a cycle kernel over the whole GPU (fewer blocks than SMs for
 // fewer than 32 points each) and its zeroed barrier words.
 template <class K, class Args>
@@ -1111,7 +1116,12 @@ static int persist_launch(K kernel, const DevOp &A, const DevOp32 &A32, const Ar
     at.val.cooperative = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    TG_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kernel, A, A32, a));
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, A, A32, a);
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported || e == cudaErrorLaunchOutOfResources) {
+        (void)cudaGetLastError();
+        return kNotStarted;
+    }
+    TG_CHECK_CUDA(e);
     return TG_OK;
 }
 static int persist_ready(tg_op *op, cudaStream_t s) {
@@ -1122,12 +1132,13 @@ static SyncWords *persist_words(tg_op *op) {
     return reinterpret_cast<SyncWords *>(wsp<char>(op, S_SMALL) + SmallArea::sync);
 }
 // Reads a launch's report (bytes at dev) and its barrier words; a wait that gave up is an error
-// whatever the report says.
+// whatever the report says (at the first barrier there is none, and host keeps the last one).
 static int persist_look(tg_op *op, const void *dev, void *host, size_t bytes, const char *what, cudaStream_t s) {
     char *pin = reinterpret_cast<char *>(op->pin.p);
     SyncWords *w = reinterpret_cast<SyncWords *>(pin + (1 << 15));
     TG_CHECK_CUDA(cudaMemcpyAsync(w, persist_words(op), sizeof(SyncWords), cudaMemcpyDeviceToHost, s));
     TG_CHECK(readback(op, dev, bytes, s));
+    if (w->failed == kFailedStart) return kNotStarted;
     memcpy(host, pin, bytes);
     if (w->failed) {
         set_error("a grid barrier of the %s cycle timed out", what);
@@ -1137,6 +1148,8 @@ static int persist_look(tg_op *op, const void *dev, void *host, size_t bytes, co
 }
 
 // Runs the cycle that `a` describes (first launch and continuations); res: the launch's report.
+// kNotStarted: a launch did not start, and from here on the solve's cycles are chains of launches.  If
+// that was a continuation (a.first = 0), x, r, r_hat and p[0] are current and res->st holds the cycle's state.
 template <class T>
 static int bicg_persist_run(tg_op *op, const DevOp &A, const DevOp32 &A32, BiPersArgs<T> &a, int n, BiPersOut *res,
                             cudaStream_t s) {
@@ -1159,11 +1172,13 @@ static int bicg_persist_run(tg_op *op, const DevOp &A, const DevOp32 &A32, BiPer
     auto look = [&]() { return persist_look(op, a.out, res, sizeof(BiPersOut), "BiCGStab", s); };
     for (a.first = 1;; a.first = 0) {
         const int it0 = res->st.iters, ev = prof_begin(s);
-        TG_CHECK(persist_launch(k_bi_persist<T>, A, A32, a, s));
-        if (ev >= 0) TG_CHECK(look());           // the work of a profiled launch is counted by its iterations
+        int rc = persist_launch(k_bi_persist<T>, A, A32, a, s);
+        if (rc == TG_OK && ev >= 0) rc = look();           // the work of a profiled launch is counted by its iterations
         const double its = res->st.iters - it0;
         prof_end(ev, P_BI_CYCLE, its * n * (17.0 + 2 * xb / 8) * sizeof(T), its * n * (2 * fl + 26), s);
-        if (ev < 0) TG_CHECK(look());
+        if (rc == TG_OK && ev < 0) rc = look();
+        if (rc == kNotStarted) op->one_launch = false;
+        if (rc != TG_OK) return rc;
         if (res->st.status != 0) break;
         if (res->st.iters > a.cap) {
             set_error("BiCGStab cycle exceeded its product cap");
@@ -1173,13 +1188,17 @@ static int bicg_persist_run(tg_op *op, const DevOp &A, const DevOp32 &A32, BiPer
     return TG_OK;
 }
 
+// *begun: after kNotStarted, whether a part of the cycle ran (its state is then in *left)
 template <class T>
 static int bicg_persist(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r, int n, double target2, int cap,
-                        CycleOut *out, cudaStream_t s) {
+                        CycleOut *out, BiState<double> *left, bool *begun, cudaStream_t s) {
     BiPersArgs<T> a{};
     a.x = x; a.r = r; a.target2 = target2; a.cap = cap;
     BiPersOut o;
-    TG_CHECK(bicg_persist_run<T>(op, A, A32, a, n, &o, s));
+    const int rc = bicg_persist_run<T>(op, A, A32, a, n, &o, s);
+    *begun = !a.first;
+    *left = o.st;
+    if (rc != TG_OK) return rc;
     out->mvps = o.st.mvps;
     out->iters = o.st.iters;
     out->status = o.st.status;
@@ -1192,15 +1211,22 @@ static int bicg_persist(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *
 // k_bi_pad (rows of pitch P, a multiple of 4 above N, zero padding): x and r are copied in
 // at the start and back at the end, and every vector of the cycle has length P N^2.
 // padded > 0: x and r are already in that layout (the cycle proper).
+// resume: the state of a cycle whose first part ran in one launch (bicg_persist_run; unpadded).
 template <class T>
 static int bicg_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r, int n, double target2, int cap,
-                      CycleOut *out, cudaStream_t s, int padded = 0) {
+                      CycleOut *out, cudaStream_t s, int padded = 0, const BiState<double> *resume = nullptr) {
     using D = typename ST<T>::D;
+    BiState<double> left;
     if constexpr (sizeof(T) != 16) {
-        if (n <= pers_max_rows<T>(false) && !padded) return bicg_persist<T>(op, A, A32, x, r, n, target2, cap, out, s);
+        if (n <= pers_max_rows<T>(false) && !padded && op->one_launch) {
+            bool begun;
+            const int rc = bicg_persist<T>(op, A, A32, x, r, n, target2, cap, out, &left, &begun, s);
+            if (rc != kNotStarted) return rc;
+            if (begun) resume = &left;
+        }
     }
     if constexpr (std::is_same<T, float>::value) {
-        if (A.kind == DK_CD3D && !padded) {
+        if (A.kind == DK_CD3D && !padded && !resume) {
             const size_t np = (size_t)pad_pitch(A.N) * A.N * A.N;
             TG_CHECK(wsx(op, S_PADX, np * 4));
             TG_CHECK(wsx(op, S_PADR, np * 4));
@@ -1239,7 +1265,10 @@ static int bicg_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r,
     D *part = wsp<D>(op, S_PART);
     unsigned *tk = wsp<unsigned>(op, S_TICKET);
     BiState<D> *st = reinterpret_cast<BiState<D> *>(wsp<char>(op, S_SMALL) + SmallArea::bistate);
-    TG_PROF(P_BI_INIT, 3.0 * nb * sizeof(T), 2.0 * nb, launch(k_bi_init<T>, g, kThreads, 0, s, r, w.rh, w.p, n, target2, cap, part, tk, st));
+    if (resume)
+        TG_CHECK_CUDA(cudaMemcpyAsync(st, resume, sizeof(BiState<double>), cudaMemcpyHostToDevice, s));
+    else
+        TG_PROF(P_BI_INIT, 3.0 * nb * sizeof(T), 2.0 * nb, launch(k_bi_init<T>, g, kThreads, 0, s, r, w.rh, w.p, n, target2, cap, part, tk, st));
     TG_LAUNCH_CHECK();
     // float32 streaming updates with 16-byte aligned vectors: 4 points per thread
     bool use_v4 = false;
@@ -1287,7 +1316,7 @@ static int bicg_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r,
         TG_CHECK(readback(op, st, sizeof(BiState<D>), s));
         memcpy(&h, op->pin.p, sizeof(h));
         if (h.status != 0) break;
-        if (launched > cap + 8) {   // the cap test ends a cycle after `cap` products; this cannot trigger
+        if (launched > h.cap + 8) {   // the cap test ends a cycle after `cap` products; this cannot trigger
             set_error("BiCGStab cycle exceeded its product cap");
             return TG_SYNC_TIMEOUT;
         }
@@ -1309,7 +1338,7 @@ static int bicg_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r,
     // launches queued after the cycle ended returned at once: relabel them so the
     // per-class totals hold only the iterations that ran
     if (g_prof.on) {
-        const int ran = h.iters;       // full or half iterations executed
+        const int ran = h.iters - (resume ? resume->iters : 0);       // full or half iterations executed
         int it = 0;
         for (size_t q = rec0; q < g_prof.recs.size(); ++q) {
             ProfRec &pr = g_prof.recs[q];
@@ -1356,16 +1385,18 @@ static void hist_push(tg_stats *st, double relres, double rt, int64_t mvps) {
 // launch's own projection takes.
 template <class T>
 static bool whole_cycles(const tg_op *op, const tg_defl *df) {
-    return !op->cplx_ && op->n <= pers_max_rows<T>(false) && (!df || df->kk <= kPersCols);
+    return !op->cplx_ && op->one_launch && op->n <= pers_max_rows<T>(false) && (!df || df->kk <= kPersCols);
 }
 
 // One whole cycle (tg_persist.cuh): projection, tolerance, BiCGStab, and the float64 residual of
 // the updated x.  nr: in ||r||, out the norm after the projection; *nr_new, *nb: the residual's.
+// kNotStarted: as bicg_persist_run; with *begun the projection and a part of the cycle ran (*nr, *rt
+// and the state *left are theirs), else nothing.
 template <class T>
 static int bicg_whole(tg_op *op, const DevOp &A, const DevOp32 &A32, const tg_defl *df, const double *b, double *x,
                       double *r, T *xc, T *rc, double *xbak, const T *W, const T *B1, const T *B2, const SolveCfg &cfg,
                       int cyc, double floor, int cap, double *nr, double *nb, double *rt, double *nr_new,
-                      CycleOut *co, cudaStream_t s) {
+                      CycleOut *co, BiState<double> *left, bool *begun, cudaStream_t s) {
     BiPersArgs<T> a{};
     a.whole = 1;
     a.x = xc; a.r = rc; a.b = b; a.x64 = x; a.r64 = r; a.xbak = xbak;
@@ -1380,10 +1411,14 @@ static int bicg_whole(tg_op *op, const DevOp &A, const DevOp32 &A32, const tg_de
         a.pw = pow(cfg.rtol, (double)cyc / cfg.ncyc);
     }
     BiPersOut o;
-    TG_CHECK(bicg_persist_run<T>(op, A, A32, a, op->n, &o, s));
-    *co = CycleOut{o.st.mvps, o.st.iters, o.st.status, o.st.rr};
+    const int ret = bicg_persist_run<T>(op, A, A32, a, op->n, &o, s);
+    *begun = !a.first;
+    *left = o.st;
+    if (ret != TG_OK && !(ret == kNotStarted && *begun)) return ret;
     *nr = o.nr;
     *rt = o.rt;
+    if (ret != TG_OK) return ret;
+    *co = CycleOut{o.st.mvps, o.st.iters, o.st.status, o.st.rr};
     *nr_new = sqrt(o.rr);
     *nb = sqrt(o.bb);
     return TG_OK;
@@ -1424,9 +1459,12 @@ static int solve_bicg64(tg_op *op, int transpose, const tg_defl *df, const T *b,
     int status = TG_NOT_CONVERGED;
     if (!std::isfinite(nr)) status = TG_NAN;
     else if (nb == 0.0 || nr <= cfg.rtol * nb) status = TG_OK;
-    const bool whole = whole_cycles<double>(op, df);
+    op->one_launch = true;
     while (status == TG_NOT_CONVERGED) {
         ++cyc;
+        bool whole = whole_cycles<double>(op, df), begun = false;
+        double rt;
+        BiState<double> left;
         const bool sched = cfg.ncyc && cyc <= cfg.ncyc;   // beyond ncyc: finish with rtol ||b|| / ||r||
         int64_t cap64 = cfg.max_mvps - mvps;
         if (cfg.restart_mvps > 0 && cap64 > cfg.restart_mvps) cap64 = cfg.restart_mvps;
@@ -1434,27 +1472,35 @@ static int solve_bicg64(tg_op *op, int transpose, const tg_defl *df, const T *b,
         CycleOut co;
         if constexpr (std::is_same<T, double>::value) {
             if (whole) {
-                double rt, nr_new, nb_old = nb;
+                double nr_new, nb_old = nb;
                 const double *W, *B1, *B2;
                 proj_data64<double>(df, &W, &B1, &B2);
-                TG_CHECK(bicg_whole<double>(op, A, A32, df, b, x, r, x, r, nullptr, W, B1, B2, cfg, cyc, 0.0,
-                                            (int)cap64, &nr, &nb, &rt, &nr_new, &co, s));
-                hist_push(st, nr / nb_old, rt, mvps);
-                mvps += co.mvps;
-                if (co.status == 4) { nb = nb_old; status = TG_NAN; break; }
-                nr = nr_new;
+                const int rc = bicg_whole<double>(op, A, A32, df, b, x, r, x, r, nullptr, W, B1, B2, cfg, cyc, 0.0,
+                                                  (int)cap64, &nr, &nb, &rt, &nr_new, &co, &left, &begun, s);
+                if (rc == kNotStarted) {
+                    whole = false;
+                } else {
+                    TG_CHECK(rc);
+                    hist_push(st, nr / nb_old, rt, mvps);
+                    mvps += co.mvps;
+                    if (co.status == 4) { nb = nb_old; status = TG_NAN; break; }
+                    nr = nr_new;
+                }
             }
         }
         if (!whole) {
-            if (df && df->kk > 0) {                                    // step a
-                TG_CHECK(project64<T>(op, df, x, r, s));
-                double rr;
-                TG_CHECK(dot_host<T>(op, r, nullptr, n, &rr, nullptr, s));
-                nr = sqrt(rr);
+            if (!begun) {
+                if (df && df->kk > 0) {                                // step a
+                    TG_CHECK(project64<T>(op, df, x, r, s));
+                    double rr;
+                    TG_CHECK(dot_host<T>(op, r, nullptr, n, &rr, nullptr, s));
+                    nr = sqrt(rr);
+                }
+                rt = sched ? cycle_tol(cfg.rtol, nb, nr, cyc, cfg.ncyc) : cfg.rtol * nb / nr;   // step b
             }
-            double rt = sched ? cycle_tol(cfg.rtol, nb, nr, cyc, cfg.ncyc) : cfg.rtol * nb / nr;   // step b
             hist_push(st, nr / nb, rt, mvps);
-            TG_CHECK(bicg_cycle<T>(op, A, A32, x, r, n, (rt * nr) * (rt * nr), (int)cap64, &co, s));   // step c
+            TG_CHECK(bicg_cycle<T>(op, A, A32, x, r, n, (rt * nr) * (rt * nr), (int)cap64, &co, s, 0,
+                                   begun ? &left : nullptr));   // step c
             mvps += co.mvps;
             if (co.status == 4) { status = TG_NAN; break; }
             TG_CHECK(true_residual<T>(op, A, b, x, r, &nr, &nb, s));
@@ -1498,9 +1544,12 @@ static int solve_bicg_ir(tg_op *op, int transpose, const tg_defl *df, const doub
     if (!std::isfinite(nr)) status = TG_NAN;
     else if (nb == 0.0 || nr <= cfg.rtol * nb) status = TG_OK;
     const int g = grid_for(n, 8);
-    const bool whole = whole_cycles<float>(op, df);
+    op->one_launch = true;
     while (status == TG_NOT_CONVERGED) {
         ++cyc;
+        bool whole = whole_cycles<float>(op, df), begun = false;
+        double rt, nrp = nr;                // nrp: residual norm after the projection
+        BiState<double> left;
         const bool sched = cfg.ncyc && cyc <= cfg.ncyc;   // beyond ncyc: finish with rtol ||b|| / ||r||
         int64_t cap64 = cfg.max_mvps - mvps;
         // a float32 cycle that stagnates above its target ends after kIrCycleCap products
@@ -1510,32 +1559,41 @@ static int solve_bicg_ir(tg_op *op, int transpose, const tg_defl *df, const doub
         CycleOut co;
         const double nr_before = nr;
         if (whole) {
-            double rt, nr_new;
+            double nr_new;
             const double nb_old = nb;
-            TG_CHECK(bicg_whole<float>(op, A, A32, df, b, x, r, e32, r32, xbak, df ? df->W32.as<float>() : nullptr,
-                                       df ? df->B1_32.as<float>() : nullptr, df ? df->B2_32.as<float>() : nullptr, cfg,
-                                       cyc, 1e-6, (int)cap64, &nr, &nb, &rt, &nr_new, &co, s));
-            hist_push(st, nr / nb_old, rt, mvps);
-            mvps += co.mvps;
-            nr = nr_new;
-        } else {
-            // correction equation A e = r, scaled so that ||r32|| = 1
-            TG_PROF(P_CONVERT, 12.0 * n, n, launch_d2f_scaled(g, s, r, r32, n, 1.0 / nr));
-            TG_CHECK_CUDA(cudaMemsetAsync(e32, 0, (size_t)n * 4, s));
-            double scale = nr;
-            double nrel = 1.0;
-            if (df && df->kk > 0) {
-                TG_CHECK(project_impl<float>(op, df, df->W32.as<float>(), df->B1_32.as<float>(), df->B2_32.as<float>(),
-                                             e32, r32, n, s));
-                double rr;
-                TG_CHECK(dot_host<float>(op, r32, nullptr, n, &rr, nullptr, s));
-                nrel = sqrt(rr);
+            const int rc = bicg_whole<float>(op, A, A32, df, b, x, r, e32, r32, xbak, df ? df->W32.as<float>() : nullptr,
+                                             df ? df->B1_32.as<float>() : nullptr, df ? df->B2_32.as<float>() : nullptr,
+                                             cfg, cyc, 1e-6, (int)cap64, &nrp, &nb, &rt, &nr_new, &co, &left, &begun, s);
+            if (rc == kNotStarted) {
+                whole = false;
+            } else {
+                TG_CHECK(rc);
+                hist_push(st, nrp / nb_old, rt, mvps);
+                mvps += co.mvps;
+                nr = nr_new;
             }
-            const double nrp = nrel * scale;    // residual norm after the projection
-            double rt = sched ? cycle_tol(cfg.rtol, nb, nrp, cyc, cfg.ncyc) : cfg.rtol * nb / nrp;
-            if (rt < 1e-6) rt = 1e-6;   // a float32 cycle cannot resolve more; refinement continues
+        }
+        if (!whole) {
+            const double scale = nr;
+            double nrel = 1.0;
+            if (!begun) {
+                // correction equation A e = r, scaled so that ||r32|| = 1
+                TG_PROF(P_CONVERT, 12.0 * n, n, launch_d2f_scaled(g, s, r, r32, n, 1.0 / nr));
+                TG_CHECK_CUDA(cudaMemsetAsync(e32, 0, (size_t)n * 4, s));
+                if (df && df->kk > 0) {
+                    TG_CHECK(project_impl<float>(op, df, df->W32.as<float>(), df->B1_32.as<float>(),
+                                                 df->B2_32.as<float>(), e32, r32, n, s));
+                    double rr;
+                    TG_CHECK(dot_host<float>(op, r32, nullptr, n, &rr, nullptr, s));
+                    nrel = sqrt(rr);
+                }
+                nrp = nrel * scale;
+                rt = sched ? cycle_tol(cfg.rtol, nb, nrp, cyc, cfg.ncyc) : cfg.rtol * nb / nrp;
+                if (rt < 1e-6) rt = 1e-6;   // a float32 cycle cannot resolve more; refinement continues
+            }
             hist_push(st, nrp / nb, rt, mvps);
-            TG_CHECK(bicg_cycle<float>(op, A, A32, e32, r32, n, (rt * nrel) * (rt * nrel), (int)cap64, &co, s));
+            TG_CHECK(bicg_cycle<float>(op, A, A32, e32, r32, n, (rt * nrel) * (rt * nrel), (int)cap64, &co, s, 0,
+                                       begun ? &left : nullptr));
             mvps += co.mvps;
             // keep x: a float32 correction that does not lower the float64 residual is undone
             TG_CHECK_CUDA(cudaMemcpyAsync(xbak, x, (size_t)n * 8, cudaMemcpyDeviceToDevice, s));
@@ -1599,8 +1657,9 @@ static int idr_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r, 
     D *part = wsp<D>(op, S_PART);
     unsigned *tk = wsp<unsigned>(op, S_TICKET);
     IdrState<D> *st = reinterpret_cast<IdrState<D> *>(wsp<char>(op, S_SMALL) + SmallArea::idr);
+    bool begun = false;            // a part of the cycle ran in one launch; its state is in st
     if constexpr (sizeof(T) != 16) {
-        if (n <= pers_max_rows<T>(true)) {
+        if (n <= pers_max_rows<T>(true) && op->one_launch) {
             TG_CHECK(persist_ready(op, s));
             IdrPersArgs<T> a;
             a.P = P; a.x = x; a.r = r; a.G = G; a.U = U; a.t = t; a.ld = ld;
@@ -1610,34 +1669,42 @@ static int idr_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r, 
             a.st = st; a.target2 = target2; a.kappa = kappa; a.s = sd; a.cap = cap;
             a.max_rounds = 64;           // bounds one launch to a few milliseconds
             IdrState<double> h{};
+            int rc = TG_OK;
             for (a.first = 1;; a.first = 0) {
-                TG_PROF(P_IDR_CYCLE, 0, 0, TG_CHECK(persist_launch(k_idr_persist<T>, A, A32, a, s)));
-                TG_CHECK(persist_look(op, st, &h, sizeof(h), "IDR", s));
+                TG_PROF(P_IDR_CYCLE, 0, 0, rc = persist_launch(k_idr_persist<T>, A, A32, a, s));
+                if (rc == TG_OK) rc = persist_look(op, st, &h, sizeof(h), "IDR", s);
+                if (rc == kNotStarted) break;
+                TG_CHECK(rc);
                 if (h.status != 0) break;
                 if ((int64_t)h.rounds * (sd + 1) > (int64_t)cap + 2 * (sd + 1)) {
                     set_error("IDR cycle exceeded its product cap");
                     return TG_SYNC_TIMEOUT;
                 }
             }
-            out->mvps = h.mvps;
-            out->iters = h.rounds;
-            out->status = h.status;
-            out->rr = h.rr;
-            return TG_OK;
+            if (rc == TG_OK) {
+                out->mvps = h.mvps;
+                out->iters = h.rounds;
+                out->status = h.status;
+                out->rr = h.rr;
+                return TG_OK;
+            }
+            op->one_launch = false;
+            begun = !a.first;
         }
     }
     const double es = sizeof(T);
     double xb, fl;
     op_cost(A, &xb, &fl);
     const double cf = sizeof(T) == 16 ? 4.0 : 1.0;
-    TG_PROF(P_IDR_UPD, (1.0 + sd) * n * es, 2.0 * (sd + 1) * n * cf,
-            launch(k_idr_init<T>, g, kThreads, 0, s, r, P, ld, n, sd, target2, cap, kappa, part, tk, st));
+    if (!begun)
+        TG_PROF(P_IDR_UPD, (1.0 + sd) * n * es, 2.0 * (sd + 1) * n * cf,
+                launch(k_idr_init<T>, g, kThreads, 0, s, r, P, ld, n, sd, target2, cap, kappa, part, tk, st));
     TG_LAUNCH_CHECK();
     int batch = 1, launched = 0;
     IdrState<D> h{};
     while (true) {
         for (int b = 0; b < batch; ++b) {
-            const int first = launched + b == 0;
+            const int first = launched + b == 0 && !begun;
             for (int k = 0; k < sd; ++k) {
                 TG_PROF(P_IDR_UPD, (2.0 + (first ? 0.0 : 2.0 * (sd - k))) * n * es, 4.0 * (sd - k) * n * cf,
                         launch(k_idr_u<T>, g, kThreads, 0, s, r, G, U, ld, n, k, first, st));
@@ -1701,6 +1768,7 @@ static int solve_idr64(tg_op *op, const tg_defl *df, const T *b, T *x, const Sol
     TG_CHECK(true_residual<T>(op, A, b, x, r, &nr, &nb, s));
     int64_t mvps = 0;
     int cyc = 0;
+    op->one_launch = true;
     int status = TG_NOT_CONVERGED;
     if (!std::isfinite(nr)) status = TG_NAN;
     else if (nb == 0.0 || nr <= cfg.rtol * nb) status = TG_OK;
@@ -1781,6 +1849,7 @@ static int solve_idr_ir(tg_op *op, const tg_defl *df, const double *b, double *x
     TG_CHECK(true_residual<double>(op, A, b, x, r, &nr, &nb, s));
     int64_t mvps = 0;
     int cyc = 0, fp64_cycles = 0;
+    op->one_launch = true;
     int status = TG_NOT_CONVERGED;
     if (!std::isfinite(nr)) status = TG_NAN;
     else if (nb == 0.0 || nr <= cfg.rtol * nb) status = TG_OK;

@@ -13,8 +13,11 @@
 // that forms t = A s.  p and v alternate between two buffers, because neighbours still read the
 // old ones.
 // Data of other blocks is read past the L1 cache (__ldcg).  Every wait ends after a limited number
-// of polls; the block that gives up says so in a word of its own, every block then leaves at its next
-// barrier, and the host turns the word into TG_SYNC_TIMEOUT.
+// of polls; the block that gives up says so in a word of its own, and every block then leaves at its
+// next barrier.  The first barrier of a launch comes before anything is written: if it is given up
+// (blocks of other streams hold SMs that the launch needs), or the launch is refused (the stream owns
+// fewer SMs), the host runs the cycle, or what is left of it, as a chain of launches.  Past it all blocks are
+// resident, and a wait that runs out is TG_SYNC_TIMEOUT.
 #pragma once
 
 #include "tg_arnoldi.cuh"
@@ -27,7 +30,7 @@ constexpr int kPersPart = 16;                 // reduced values per pass at most
 
 // Polls of a wait (half a microsecond each): the first barrier of a launch, and the later ones.
 struct SyncLimits {
-    unsigned start = 1u << 20, step = 1u << 20;
+    unsigned start = 1u << 16, step = 1u << 20;
 };
 
 // The barrier's words, zero at launch.  count: arrivals, and kSyncGaveUp once a block has given up;
@@ -218,6 +221,8 @@ __global__ void __launch_bounds__(kPersThreads, 1) k_bi_persist(DevOp op, DevOp3
     const int lo = min(n, (int)blockIdx.x * per), hi = min(n, lo + per);
     T *p = a.p[0], *p2 = a.p[1], *v = a.v[0], *v2 = a.v[1];      // the current p and v, and the other buffers
     __shared__ double nr_s, rt_s;
+    gs.wait();
+    if (!gs.ok) return;                            // nothing is written yet
     if (a.first) {
         if constexpr (std::is_same<T, float>::value) {
             if (a.whole) {
@@ -443,6 +448,8 @@ __global__ void __launch_bounds__(kPersThreads, 1) k_idr_persist(DevOp op, DevOp
     const int n = op.n, s = a.s, per = (n + gridDim.x - 1) / gridDim.x;
     const int lo = min(n, (int)blockIdx.x * per), hi = min(n, lo + per);
     const size_t ld = a.ld;
+    gs.wait();
+    if (!gs.ok) return;                            // nothing is written yet
     auto shadow = [&](T ri, int i, T (&acc)[M + 1]) {      // f = P^H r, ||r||^2
 #pragma unroll
         for (int q = 0; q < M; ++q)
