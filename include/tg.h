@@ -143,11 +143,12 @@ int tg_restrict(const tg_op *op, const void *fine, void *coarse, int ncols, void
 int tg_op_set_interp(tg_op *op, int interp);
 
 /* Limits of the waits in this operator's one-launch cycles (small real grids: the blocks of a
- * launch meet at barriers), in polls of about half a microsecond: `start` for the first barrier
- * of a launch (default 2^16), `step` for the later ones (default 2^20).  A launch whose wait
- * runs out ends by itself.  At the first barrier nothing is lost: the solve goes on as a chain
- * of launches.  At a later one it returns TG_SYNC_TIMEOUT.                             */
-int tg_op_sync_limits(tg_op *op, int start, int step);
+ * launch meet at barriers), in polls of about half a microsecond (0: give up at once): `start`
+ * and `again` for the first barrier of a cycle's first launch and of its later launches (default
+ * 2^16), `step` for every other barrier (default 2^20).  A launch whose wait runs out ends by
+ * itself.  At its first barrier nothing is lost: the solve goes on as a chain of launches.  At
+ * another one the solve returns TG_SYNC_TIMEOUT.                                       */
+int tg_op_sync_limits(tg_op *op, int start, int again, int step);
 
 /* ------------------------------------------------------------------ phase 1: coarse solve
  * GMRES-DR(m,k) (Section 2.1) on the coarse operator (transpose = 1: on A_c^T, giving

@@ -878,9 +878,10 @@ extern "C" int tg_op_set_interp(tg_op *op, int interp) {
     return TG_OK;
 }
 
-extern "C" int tg_op_sync_limits(tg_op *op, int start, int step) {
-    TG_ARG(op && start >= 0 && step >= 0, "bad argument");
+extern "C" int tg_op_sync_limits(tg_op *op, int start, int again, int step) {
+    TG_ARG(op && start >= 0 && again >= 0 && step >= 0, "bad argument");
     op->sync.start = start;
+    op->sync.again = again;
     op->sync.step = step;
     return TG_OK;
 }

@@ -28,9 +28,10 @@ namespace tg {
 constexpr int kPersThreads = 256;
 constexpr int kPersPart = 16;                 // reduced values per pass at most
 
-// Polls of a wait (half a microsecond each): the first barrier of a launch, and the later ones.
+// Polls of a wait (half a microsecond each; none: the wait is given up at once): the first barrier
+// of a cycle's first launch and of its later launches, and every other barrier.
 struct SyncLimits {
-    unsigned start = 1u << 16, step = 1u << 20;
+    unsigned start = 1u << 16, again = 1u << 16, step = 1u << 20;
 };
 
 // The barrier's words, zero at launch.  count: arrivals, and kSyncGaveUp once a block has given up;
@@ -48,22 +49,26 @@ constexpr unsigned kFailedStart = 1, kFailedStep = 2;
 struct GridSync {
     SyncWords *w;
     double *part;
-    SyncLimits limits;
+    unsigned first, step;          // limits of the launch's first barrier and of the others
     unsigned round;
     int parity;
     bool ok;
-    __device__ GridSync(SyncWords *words, double *p, SyncLimits l)
-        : w(words), part(p), limits(l), round(0), parity(0), ok(true) {}
+    __device__ GridSync(SyncWords *words, double *p, const SyncLimits &l, bool cycle_start)
+        : w(words), part(p), first(cycle_start ? l.start : l.again), step(l.step), round(0), parity(0), ok(true) {}
     __device__ void wait() {
         __shared__ bool ok_s;          // rewritten after the next barrier's first __syncthreads only
         if (!ok) return;
         ++round;
         __syncthreads();
         if (threadIdx.x == 0) {        // the release covers the block's writes (ordered by the barrier above)
-            const unsigned target = round * gridDim.x, limit = round == 1 ? limits.start : limits.step;
+            const unsigned target = round * gridDim.x, limit = round == 1 ? first : step;
             unsigned seen = 0, polls = 0;
             asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&w->count) : "memory");
-            while (true) {
+            if (limit == 0) {
+                seen = kSyncGaveUp;
+                if (!(atomicOr(&w->count, kSyncGaveUp) & kSyncGaveUp)) w->failed = round == 1 ? kFailedStart : kFailedStep;
+            }
+            while (limit != 0) {
                 asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&w->count) : "memory");
                 if (seen >= target) break;               // complete, or kSyncGaveUp is set
                 if (polls++ < limit) continue;
@@ -216,7 +221,7 @@ template <class T>
 __global__ void __launch_bounds__(kPersThreads, 1) k_bi_persist(DevOp op, DevOp32 o32, BiPersArgs<T> a) {
     __shared__ BiState<double> S;
     __shared__ double tot[kPersPart];
-    GridSync gs(a.words, a.part, a.limits);
+    GridSync gs(a.words, a.part, a.limits, a.first);
     const int n = op.n, per = (n + gridDim.x - 1) / gridDim.x;
     const int lo = min(n, (int)blockIdx.x * per), hi = min(n, lo + per);
     T *p = a.p[0], *p2 = a.p[1], *v = a.v[0], *v2 = a.v[1];      // the current p and v, and the other buffers
@@ -444,7 +449,7 @@ __global__ void __launch_bounds__(kPersThreads, 1) k_idr_persist(DevOp op, DevOp
     __shared__ double tot[kPersPart];
     __shared__ T cs[M], al[M];
     __shared__ double inv[M];                      // 1 / M_kk
-    GridSync gs(a.words, a.part, a.limits);
+    GridSync gs(a.words, a.part, a.limits, a.first);
     const int n = op.n, s = a.s, per = (n + gridDim.x - 1) / gridDim.x;
     const int lo = min(n, (int)blockIdx.x * per), hi = min(n, lo + per);
     const size_t ld = a.ld;

@@ -84,7 +84,7 @@ def load() -> C.CDLL:
         "tg_prolong": (i32, [vp, vp, vp, i32, vp]),
         "tg_restrict": (i32, [vp, vp, vp, i32, vp]),
         "tg_op_set_interp": (i32, [vp, i32]),
-        "tg_op_sync_limits": (i32, [vp, i32, i32]),
+        "tg_op_sync_limits": (i32, [vp, i32, i32, i32]),
         "tg_coarse_gmresdr": (i32, [vp, i32, vp, i32, i32, i32, dbl, dbl, i32, vp, C.POINTER(vp), i32, i32,
                                     C.POINTER(TgStats), vp]),
         "tg_defl_from_basis": (i32, [vp, i32, vp, i32, i32, i32, C.POINTER(vp), vp]),
@@ -184,9 +184,10 @@ class Operator:
                "tg_apply")
         return y
 
-    def sync_limits(self, start, step):
-        """tg_op_sync_limits: polls of the first and of the later waits of a one-launch cycle."""
-        _check(_lib.tg_op_sync_limits(self._h, int(start), int(step)), "tg_op_sync_limits")
+    def sync_limits(self, start=1 << 16, again=1 << 16, step=1 << 20):
+        """tg_op_sync_limits: polls of the waits of a one-launch cycle: the first of the cycle's first
+        launch, the first of its later launches, every other one."""
+        _check(_lib.tg_op_sync_limits(self._h, int(start), int(again), int(step)), "tg_op_sync_limits")
 
     def prolong(self, coarse, fine=None, stream=None):
         ncols = coarse.numel() // self.nc

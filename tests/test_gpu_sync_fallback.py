@@ -13,7 +13,6 @@ import pytest
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-WAITS = 1 << 20
 HOW = ["f64", "f32_ir", "idr", "idr_f32"]
 
 
@@ -53,33 +52,77 @@ def test_first_wait_runs_out(kind, N, how, k):
         g = torch.Generator(device="cuda").manual_seed(3)
         defl = A.defl_from_basis(torch.randn(k, A.n, dtype=torch.float64, device="cuda", generator=g), k,
                                  precision="f32_ir" if "f32" in how else "f64")
-    A.sync_limits(0, WAITS)
+    A.sync_limits(start=0)
     _solved(A, b, *_solve(A, b, how, defl)[:2])
-    A.sync_limits(WAITS, WAITS)
+    A.sync_limits()
     _solved(A, b, *_solve(A, b, how, defl)[:2])
 
 
-@pytest.mark.parametrize("method", ["bicgstab", "idr"])
-def test_a_later_launch_cannot_start(method):
-    """The indefinite Helmholtz problem whose cycle takes several launches.  With a limit of a few
-    polls some launches start and some do not, so that the chain takes the cycle over at its start or
-    in the middle.  Its residual is the solution's in every case, and the cap on products holds."""
+def _classes(f):
+    """Launches per class of the profile that f() adds."""
+    from paper_2005_03070_gb300 import tg
+    def read():
+        return {k: v["launches"] for k, v in tg.tg_profile_read().items() if isinstance(v, dict)}
+    tg.tg_profile_enable(True)
+    try:
+        before = read()
+        f()
+        after = read()
+    finally:
+        tg.tg_profile_enable(False)
+    return {k: v - before.get(k, 0) for k, v in after.items()}
+
+
+@pytest.mark.parametrize("method,precision", [("bicgstab", "f64"), ("bicgstab", "f32_ir"), ("idr", "f64"), ("idr", "f32_ir")])
+@pytest.mark.parametrize("profiled", [False, True])
+@pytest.mark.parametrize("k", [0, 8])
+def test_a_later_launch_cannot_start(method, precision, profiled, k):
+    """The indefinite Helmholtz problem whose cycle takes several launches: the chain takes it over
+    after the first.  The residual is the solution's, and the cap on products holds."""
     from paper_2005_03070_gb300 import tg
     A = tg.Operator("cd2d", 63, (0.0,), mass=-2500.0)
     g = torch.Generator(device="cuda").manual_seed(4)
     b = torch.randn(A.n, dtype=torch.float64, device="cuda", generator=g)
     P = torch.randn(2, A.n, dtype=torch.float64, device="cuda", generator=g)
-    for start in list(range(12)) * 2:
-        A.sync_limits(start, WAITS)
-        x = torch.zeros_like(b)
+    defl = A.defl_from_basis(torch.randn(k, A.n, dtype=torch.float64, device="cuda", generator=g), k,
+                             precision=precision) if k else None
+    x = torch.zeros_like(b)
+    cap = 5999
+    A.sync_limits(again=0)
+    out = []
+
+    def run():
         if method == "idr":
-            status, st = A.solve_idr(b, x, P, None, rtol=1e-15, ncyc=0, restart_mvps=2999, max_mvps=2999)
+            out.append(A.solve_idr(b, x, P, defl, rtol=1e-15, ncyc=0, restart_mvps=cap, max_mvps=cap, precision=precision))
         else:
-            status, st = A.solve(b, x, None, rtol=1e-15, ncyc=0, restart_mvps=5999, max_mvps=5999)
-        assert status in (tg.TG_OK, tg.TG_NOT_CONVERGED, tg.TG_BREAKDOWN)
-        rel = ((b - A.apply(x)).norm() / b.norm()).item()
-        assert st[0]["mvps"] <= (2999 if method == "idr" else 5999) + 3
-        assert abs(rel - st[0]["relres"]) <= 1e-12 * max(1.0, rel)
+            out.append(A.solve(b, x, defl, precision=precision, rtol=1e-15, ncyc=0, restart_mvps=cap, max_mvps=cap))
+    if profiled:
+        n = _classes(run)
+        if precision == "f64":
+            # the first launch and the one that gave up; the cycle went on and did not start again
+            assert n["idr_cycle" if method == "idr" else "bicg_cycle"] == 2
+            assert n.get("bicg_init", 0) == 0
+            assert n["idr_apply" if method == "idr" else "bicg_x"] > 0
+    else:
+        run()
+    status, st = out[0]
+    assert status in (tg.TG_OK, tg.TG_NOT_CONVERGED, tg.TG_BREAKDOWN)
+    rel = ((b - A.apply(x)).norm() / b.norm()).item()
+    assert st[0]["mvps"] <= cap + 3
+    assert abs(rel - st[0]["relres"]) <= 1e-12 * max(1.0, rel)
+
+
+@pytest.mark.parametrize("kind,N", [("cd2d", 127), ("cd3d", 31)])
+@pytest.mark.parametrize("precision", ["f64", "f32_ir"])
+def test_idr_taken_over_converges(kind, N, precision):
+    """A cycle of more than 64 rounds with one shadow column, taken over after its first launch."""
+    A, b = _problem(N, kind)
+    P = torch.randn(1, A.n, dtype=torch.float64, device="cuda", generator=torch.Generator(device="cuda").manual_seed(5))
+    A.sync_limits(again=0)
+    x = torch.zeros_like(b)
+    status, st = A.solve_idr(b, x, P, None, rtol=1e-10, ncyc=1, precision=precision)
+    assert st[0]["mvps"] > 2 * 64
+    _solved(A, b, status, x)
 
 
 @pytest.mark.parametrize("how", HOW)

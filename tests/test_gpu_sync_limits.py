@@ -1,12 +1,9 @@
-"""A one-launch cycle whose barrier wait runs out: the launch ends by itself, the solve reports it,
-and the operator solves as before afterwards.  With a limit of no polls at the later barriers every
-block that is not among the last of its barrier gives up, so a solve of many barriers cannot pass."""
+"""A one-launch cycle whose barrier wait is given up: the launch ends by itself, the solve reports it,
+and the operator solves as before afterwards."""
 import pytest
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
-
-WAITS = 1 << 20
 
 
 def _solve(A, b, how):
@@ -28,14 +25,14 @@ def test_a_wait_that_runs_out_is_reported(how):
     b = torch.randn(A.n, dtype=torch.float64, device="cuda", generator=torch.Generator(device="cuda").manual_seed(1))
     status, x0, st0 = _solve(A, b, how)
     assert status == tg.TG_OK
-    A.sync_limits(WAITS, 0)
+    A.sync_limits(step=0)
     for _ in range(3):
         try:
             status = _solve(A, b, how)[0]
         except tg.TgError as e:
             status = e.status
         assert status == tg.TG_SYNC_TIMEOUT
-    A.sync_limits(WAITS, WAITS)
+    A.sync_limits()
     status, x, st = _solve(A, b, how)
     assert status == tg.TG_OK and st["mvps"] == st0["mvps"]
     assert torch.equal(x, x0)
@@ -44,7 +41,7 @@ def test_a_wait_that_runs_out_is_reported(how):
 def test_limits_are_checked():
     from paper_2005_03070_gb300 import tg
     A = tg.Operator("cd2d", 15, (1.0,))
-    for bad in ((-1, 1), (1, -1)):
+    for bad in ((-1, 1, 1), (1, -1, 1), (1, 1, -1)):
         with pytest.raises(tg.TgError) as e:
             A.sync_limits(*bad)
         assert e.value.status == tg.TG_BAD_ARG
