@@ -26,6 +26,13 @@
 namespace tg {
 
 constexpr int kPersThreads = 256;
+// Blocks of a cycle kernel that fit an SM, so that solves on other streams run beside it: launches
+// that each take the SMs' registers run in turn (202 registers a thread where nothing bounds them).
+// ms a solve with eight threads that each have an operator and a stream, chain of launches / one block an
+// SM / these: IDR(4) 127^2 7.2 / 11.4 / 5.5, float32 + refinement 63^3 2.7 / 3.3 / 2.4, float64 511^2
+// 49 / 58 / 41; one thread alone is 0 to 2% slower than with one block.
+template <class T> constexpr int kBiPersBlocks = sizeof(T) == 4 ? 3 : 2;
+constexpr int kIdrPersBlocks = 3;
 constexpr int kPersPart = 16;                 // reduced values per pass at most
 
 // Polls of a wait (half a microsecond each; none: the wait is given up at once): the first barrier
@@ -218,7 +225,7 @@ __device__ __forceinline__ void pers_project(const BiPersArgs<T> &a, GridSync &g
 // A BiCGStab cycle, or the next max_iters iterations of one.  Scalar steps and exits are those of
 // k_bi_init, k_bi_v, k_bi_s, k_bi_t and k_bi_x.  On return x, r and (status 0) p[0] are current.
 template <class T>
-__global__ void __launch_bounds__(kPersThreads, 1) k_bi_persist(DevOp op, DevOp32 o32, BiPersArgs<T> a) {
+__global__ void __launch_bounds__(kPersThreads, kBiPersBlocks<T>) k_bi_persist(DevOp op, DevOp32 o32, BiPersArgs<T> a) {
     __shared__ BiState<double> S;
     __shared__ double tot[kPersPart];
     GridSync gs(a.words, a.part, a.limits, a.first);
@@ -443,7 +450,7 @@ struct IdrPersArgs {
 // Per k two barriers: the update of step k - 1 and U_k touch a block's own points only and share
 // a pass, then G_k = A U_k; the dimension reduction takes three.
 template <class T>
-__global__ void __launch_bounds__(kPersThreads, 1) k_idr_persist(DevOp op, DevOp32 o32, IdrPersArgs<T> a) {
+__global__ void __launch_bounds__(kPersThreads, kIdrPersBlocks) k_idr_persist(DevOp op, DevOp32 o32, IdrPersArgs<T> a) {
     constexpr int M = kIdrMaxS;
     __shared__ IdrState<double> S;
     __shared__ double tot[kPersPart];
