@@ -416,28 +416,35 @@ static TsmSplitCfg tsm_split_cfg(int p, int q, bool in_place) {
     return best;
 }
 
-template <class T, int WR>
+template <class T, int WR, bool SC>
 static int tsm_split(const TsmSplitCfg &c, const T *In, size_t ldi, int p, const T *S, int lds, int q, T *Out,
-                     size_t ldo, int n, cudaStream_t s) {
-    TG_CHECK(set_smem<T>((const void *)k_tsm_split<T, WR>, c.smem, -2048));
+                     size_t ldo, int n, cudaStream_t s, const T *norm2, int nstride) {
+    TG_CHECK(set_smem<T>((const void *)k_tsm_split<T, WR, SC>, c.smem, -2048));
     const int f = sizeof(T) == 16 ? 2 : 1, CT = (f * q + 7) / 8;
     const int gy = (CT + c.ctb - 1) / c.ctb, tiles = (n + 16 * WR - 1) / (16 * WR);
     const int gx = std::max(1, std::min(tiles, std::max(1, num_sms() / gy)));
-    launch(k_tsm_split<T, WR>, dim3(gx, gy), kTsmThreads, c.smem, s, In, ldi, p, S, lds, q, Out, ldo, n, c.ctb, c.nbuf);
+    launch(k_tsm_split<T, WR, SC>, dim3(gx, gy), kTsmThreads, c.smem, s, In, ldi, p, S, lds, q, Out, ldo, n, c.ctb, c.nbuf,
+           norm2, nstride);
     return TG_OK;
 }
 
-// Out (n x q) = In (n x p) S (p x q)
+// Out (n x q) = In (n x p) S (p x q).  The columns of In have unit norm, or norm2[i nstride] (device) is
+// the square of column i's.
 template <class T>
-static int tsm(const T *In, size_t ldi, int p, const T *S, int lds, int q, T *Out, size_t ldo, int n, cudaStream_t s) {
-    if (n >= kSplitMinRows && q >= 4) {
+static int tsm(const T *In, size_t ldi, int p, const T *S, int lds, int q, T *Out, size_t ldo, int n, cudaStream_t s,
+               const T *norm2 = nullptr, int nstride = 0) {
+    if (n >= kSplitMinRows && q >= 4 && p <= kMaxCols) {
         const TsmSplitCfg c = tsm_split_cfg<T>(p, q, In == Out);
         if (c.wr) {
+            auto go = [&](auto sc) {
+                constexpr bool SC = decltype(sc)::value;
+                return c.wr == 8   ? tsm_split<T, 8, SC>(c, In, ldi, p, S, lds, q, Out, ldo, n, s, norm2, nstride)
+                       : c.wr == 4 ? tsm_split<T, 4, SC>(c, In, ldi, p, S, lds, q, Out, ldo, n, s, norm2, nstride)
+                                   : tsm_split<T, 2, SC>(c, In, ldi, p, S, lds, q, Out, ldo, n, s, norm2, nstride);
+            };
             int rc = TG_OK;
             TG_PROF(P_TSM, (double)(p + q) * n * sizeof(T), 2.0 * p * q * n * (sizeof(T) == 16 ? 4 : 1),
-                    rc = c.wr == 8   ? tsm_split<T, 8>(c, In, ldi, p, S, lds, q, Out, ldo, n, s)
-                         : c.wr == 4 ? tsm_split<T, 4>(c, In, ldi, p, S, lds, q, Out, ldo, n, s)
-                                     : tsm_split<T, 2>(c, In, ldi, p, S, lds, q, Out, ldo, n, s));
+                    rc = norm2 ? go(std::true_type{}) : go(std::false_type{}));
             TG_CHECK(rc);
             TG_LAUNCH_CHECK();
             return TG_OK;
@@ -619,7 +626,7 @@ static int cholqr2(tg_op *op, const T *A, int k, int n, T *Q, T *R, T *Rinv, int
     TG_CHECK(gram<T>(op, A, A, n, k, n, 1, G.as<T>(), s));
     TG_PROF(P_SMALL, 0, 1.0 * k * k * k, launch_chol_inv<T>(G.as<T>(), k, R1.as<T>(), R1i.as<T>(), info_dev, s));
     TG_LAUNCH_CHECK();
-    TG_CHECK(tsm<T>(A, n, k, R1i.as<T>(), k, k, Q, n, n, s));
+    TG_CHECK(tsm<T>(A, n, k, R1i.as<T>(), k, k, Q, n, n, s, G.as<T>(), k + 1));
     TG_CHECK(gram<T>(op, Q, Q, n, k, n, 1, G.as<T>(), s));
     TG_PROF(P_SMALL, 0, 1.0 * k * k * k, launch_chol_inv<T>(G.as<T>(), k, R2.as<T>(), R2i.as<T>(), info_dev + 1, s));
     TG_LAUNCH_CHECK();
@@ -921,7 +928,12 @@ static int build_defl(tg_op *op, int transpose, tg_defl *d, cudaStream_t s) {
         DBuf &Ry = op->ws[S_GAL_RY], &Ryi = op->ws[S_GAL_RYI], &W = op->ws[S_GAL_W];
         TG_CHECK(d->AV.ensure(nb));
         TG_CHECK(cholqr2<T>(op, Y, kk, n, d->Q.as<T>(), Ry.as<T>(), Ryi.as<T>(), info, s));
-        TG_CHECK(tsm<T>(AY, n, kk, Ryi.as<T>(), kk, kk, d->AV.as<T>(), n, n, s));
+        if (n >= kSplitMinRows) {            // the norms of A Y for the product's scales
+            TG_CHECK(gram<T>(op, AY, AY, n, kk, n, 1, W.as<T>(), s));
+            TG_CHECK(tsm<T>(AY, n, kk, Ryi.as<T>(), kk, kk, d->AV.as<T>(), n, n, s, W.as<T>(), kk + 1));
+        } else {
+            TG_CHECK(tsm<T>(AY, n, kk, Ryi.as<T>(), kk, kk, d->AV.as<T>(), n, n, s));
+        }
         TG_CHECK(gram<T>(op, d->Q.as<T>(), d->AV.as<T>(), n, kk, n, 0, d->R.as<T>(), s));
         TG_PROF(P_SMALL, 0, 2.0 * kk * kk * kk, launch_inverse<T>(d->R.as<T>(), kk, d->M.as<T>(), W.as<T>(), info + 2, s));
         TG_LAUNCH_CHECK();

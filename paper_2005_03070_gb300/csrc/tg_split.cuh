@@ -4,7 +4,7 @@
 // The float64 unit of this GPU issues 2 multiply-adds per clock and SM; both products need p
 // (or k) of them per value read and sat at 0.84-0.93 of that rate, 7 to 30 times above the time
 // their bytes take.  The split moves the multiply-adds to mma.sync (1007 f16 multiply-adds per
-// clock and SM measured) without losing accuracy:
+// clock and SM measured):
 //   - a vector along the contraction (a row of In, a column of S, a 128-row piece of a Gram
 //     column) is scaled by its largest exponent and each value becomes a 62-bit integer; a
 //     value within 2^9 of the largest keeps all its 53 bits, smaller ones are cut at 2^-61 of it;
@@ -15,8 +15,16 @@
 //     over 128 terms (2^24) exactly; pairs of digits i, j with i + j <= 7 are kept (36 of 64),
 //     which leaves an error of about 2^-58 of the largest products;
 //   - the eight diagonals i + j are added as integers and rounded to float64 once.
-// So a result is rounded once at 2^-53 instead of once per term.  Rows (or pieces) that hold an
-// infinity, a NaN or magnitudes outside 2^-823..2^823 are computed in plain float64.
+// So a sum of p terms is off by at most p 2^-58 times the product of the two vectors' largest values,
+// and is then rounded once.  Where one vector's largest value meets a small one of the other, that is more
+// than float64 sums lose.  In the Gram product both vectors are columns, and the bound is below the
+// rounding of the columns' norms, however they are scaled.  In Out = In S a row of In may hold a
+// large and a small column: Q = A R^-1 multiplies the small one by a large entry of R^-1.  There column
+// i of In and row i of S are scaled by opposite powers of two, so that In's columns have norms between 1 and
+// 2 (the callers have them from a Gram matrix, or know the columns to be unit vectors): column c of Out is
+// then off by no more than p^1.5 2^-56 max_i ||In_i|| |S_ic|, whatever the scales, where float64 sums have
+// p 2^-53 sum_i ||In_i|| |S_ic|.  Rows (or pieces) that hold an infinity, a NaN or magnitudes outside
+// 2^-823..2^823, and products whose norms are not positive and finite, are computed in plain float64.
 #pragma once
 
 #include <cuda_fp16.h>
@@ -127,6 +135,8 @@ __device__ __forceinline__ double split_rescale(double r, int E1, int E2) { retu
 // n = 191^3, p = q = 30: 3.0 ms (the float64 unit: 11.2); complex128, n = 32^4, p = q = 40: 2.0 ms
 // (10.9).  The mma take 0.9 ms of the 3.0 and the bytes 0.5; issuing the conversions and joins
 // (27 thousand warp instructions a 128-row tile, 2 a clock) bounds it.
+// SC: norm2[i nstride] is the square of the norm of In's column i (device), and the scales above are
+// taken from it; else the columns are taken to be of unit norm.  Scaling is integer work on the exponents.
 constexpr int kTsmThreads = 512, kTsmWarps = 16, kTsmCt = 2;
 struct TsmSplitCfg {
     int wr, nbuf, ctb;      // row warps, buffers, n-tiles (8 columns) per block
@@ -137,10 +147,21 @@ template <class T> __host__ __device__ __forceinline__ int split_pc(int p) {
     return sizeof(T) == 16 ? 8 * split_kt(2 * p) : 16 * split_kt(p);
 }
 
-template <class T, int WR>
+// exponent of the norm whose square is n2 (0 and *ok = false when that is not positive and finite)
+__device__ __forceinline__ int split_norm_exp(double n2, bool *ok) {
+    *ok = n2 > 0.0 && isfinite(n2);
+    return *ok ? ilogb(n2) >> 1 : 0;
+}
+// x 2^-e by the exponent field; zero when that leaves no normal number
+__device__ __forceinline__ double split_scale(double x, int e) {
+    const int hi = __double2hiint(x), mag = hi & 0x7fffffff, m = mag < 0x100000 ? 0 : max(mag - (e << 20), 0);
+    return __hiloint2double((hi & 0x80000000) | m, __double2loint(x));
+}
+
+template <class T, int WR, bool SC>
 __global__ void __launch_bounds__(kTsmThreads, 1) k_tsm_split(const T *In, size_t ldi, int p, const T *__restrict__ S,
                                                            int lds, int q, T *Out, size_t ldo, int n, int ctb,
-                                                           int nbuf) {
+                                                           int nbuf, const T *__restrict__ norm2, int nstride) {
     pdl_wait();
     constexpr bool kC = sizeof(T) == 16;
     constexpr int R = 16 * WR, RS = R + 2, WC = kTsmWarps / WR;
@@ -151,20 +172,24 @@ __global__ void __launch_bounds__(kTsmThreads, 1) k_tsm_split(const T *In, size_
     uint2 *sf = reinterpret_cast<uint2 *>(smem_raw);                           // [KT][nct][8][32]
     T *tiles = reinterpret_cast<T *>(smem_raw + (size_t)KT * ctb * kSplitDigits * 256);
     __shared__ int ecol[8 * 32];
+    __shared__ short ein[SC ? kMaxCols + 16 : 1];              // exponents of In's columns, 0 past the last
     __shared__ int bad_s;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int g = lane >> 2, tq = lane & 3;
     const double *Sd = reinterpret_cast<const double *>(S);
-    // real entry (k, c) of S
+    // real entry (k, c) of S, its row scaled
     auto s_at = [&](int k, int c) -> double {
         if (k >= pr || c >= qr) return 0.0;
+        double v;
         if constexpr (kC) {
             const double *e = Sd + 2 * ((size_t)(k >> 1) + (size_t)(c >> 1) * lds);
             const int a = k & 1, b = c & 1;
-            return a == b ? e[0] : (a ? -e[1] : e[1]);
+            v = a == b ? e[0] : (a ? -e[1] : e[1]);
         } else {
-            return Sd[(size_t)k + (size_t)c * lds];
+            v = Sd[(size_t)k + (size_t)c * lds];
         }
+        if constexpr (SC) v = scalbn(v, ein[kC ? k >> 1 : k]);
+        return v;
     };
     const int ntiles = (n + R - 1) / R;
     const bool vec = kC || !(((uintptr_t)In | (ldi * sizeof(T))) & 15);      // 16-byte aligned columns
@@ -199,6 +224,14 @@ __global__ void __launch_bounds__(kTsmThreads, 1) k_tsm_split(const T *In, size_
     // digits of S: column exponents first, a warp per column
     if (tid == 0) bad_s = 0;
     __syncthreads();
+    if constexpr (SC) {
+        for (int i = tid; i < pc; i += kTsmThreads) {
+            bool ok = true;
+            ein[i] = (short)(i < p ? split_norm_exp(*reinterpret_cast<const double *>(norm2 + (size_t)i * nstride), &ok) : 0);
+            if (!ok) bad_s = 1;
+        }
+        __syncthreads();
+    }
     for (int c = warp; c < 8 * nct; c += kTsmWarps) {
         int mg = 0;
         for (int k = lane; k < pr; k += 32) mg = max(mg, split_mag(s_at(k, 8 * ct0 + c)));
@@ -239,6 +272,10 @@ __global__ void __launch_bounds__(kTsmThreads, 1) k_tsm_split(const T *In, size_
                 const double *td = reinterpret_cast<const double *>(tl);
                 x0 = td[k * RS + 8 * h];
                 x1 = td[(k + 1) * RS + 8 * h];
+            }
+            if constexpr (SC) {
+                x0 = split_scale(x0, ein[kC ? k >> 1 : k]);
+                x1 = split_scale(x1, ein[kC ? k >> 1 : k + 1]);
             }
         };
         int mg[2] = {0, 0};
