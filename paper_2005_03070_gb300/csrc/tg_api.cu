@@ -355,10 +355,11 @@ static const DevOp32 &pick32(const tg_op *op, int level, int transpose) {
 }
 
 template <class T>
-static int launch_apply(const DevOp &A, const DevOp32 &A32, const T *x, T *y, cudaStream_t s) {
+static int launch_apply(const DevOp &A, const DevOp32 &A32, const T *x, T *y, cudaStream_t s,
+                        const int *skip = nullptr) {
     double xb, fl;
     op_cost(A, &xb, &fl);
-    TG_PROF(P_APPLY, (2.0 * sizeof(T) + xb * (sizeof(T) == 4 ? 0.5 : 1.0)) * A.n, fl * A.n, launch(k_apply<T>, grid_for(A.n, 8), kThreads, 0, s, A, A32, x, y));
+    TG_PROF(P_APPLY, (2.0 * sizeof(T) + xb * (sizeof(T) == 4 ? 0.5 : 1.0)) * A.n, fl * A.n, launch(k_apply<T>, grid_for(A.n, 8), kThreads, 0, s, A, A32, x, y, skip));
     TG_LAUNCH_CHECK();
     return TG_OK;
 }
@@ -2093,11 +2094,11 @@ static int solve_gmres64(tg_op *op, int transpose, const tg_defl *df, const T *b
         TG_LAUNCH_CHECK();
         const int mm = (int)((cfg.max_mvps - mvps) < m ? (cfg.max_mvps - mvps) : m);
         // the sweeps of step j finish Hbar column j - 1; once a column meets the target (done) the
-        // launches after it return at once, so the host looks only every kGmresLook steps
+        // launches after it, products too, return at once, so the host looks only every kGmresLook steps
         constexpr int kGmresLook = 16;
         GivensState hg{};
         for (int j = 0; j <= mm && !hg.done; ++j) {
-            if (j < mm) TG_CHECK(launch_apply<T>(A, A32, V + (size_t)j * ldv, V + (size_t)(j + 1) * ldv, s));
+            if (j < mm) TG_CHECK(launch_apply<T>(A, A32, V + (size_t)j * ldv, V + (size_t)(j + 1) * ldv, s, &gs->done));
             TG_CHECK(arnoldi_sweeps<T>(op, V, ldv, n, j, j == mm, 0, reinterpret_cast<T *>(Hb), ldh, s, &gs->done));
             if (j > 0) {
                 TG_PROF(P_GIVENS, 0, 6.0 * j, launch_givens_step<D>(Hb, H, ldh, j - 1, wsp<D>(op, S_FCS), wsp<D>(op, S_FSN), wsp<D>(op, S_FG), gs, s));

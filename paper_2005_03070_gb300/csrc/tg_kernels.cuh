@@ -48,10 +48,12 @@ template <class T> struct Part { using P = T; };          // per-thread partial 
 template <> struct Part<float> { using P = float; };
 
 // ----------------------------------------------------------------------------- y = A x
+// skip: when set and nonzero on the device, nothing is done (nullptr: never)
 template <class T>
 __global__ void __launch_bounds__(kThreads) k_apply(DevOp op, DevOp32 o32, const T *__restrict__ x,
-                                                     T *__restrict__ y) {
+                                                     T *__restrict__ y, const int *skip) {
     pdl_wait();
+    if (skip && *skip) return;
     const int n = op.n;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
         y[i] = Apply<T>::at(op, o32, i, [&](int j) { return x[j]; });
