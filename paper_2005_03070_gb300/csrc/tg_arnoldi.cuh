@@ -25,17 +25,13 @@ namespace tg {
 template <class D>
 struct ArnState {
     D *s, *z, *h1;        // kMaxCols each
-    double *beta;         // beta, 1 / beta (0 when u vanished), 1 when s is small (else 0)
+    double *beta;         // beta, 1 / beta (0 when u vanished)
     D *t;
     D *part;              // block partials [gridDim.x][2 (j + 1)], then the groups'
     unsigned *ticket;     // ticket 0 and one per group of blocks, zero between launches
     const int *skip;      // when set and nonzero, the sweeps return at once (nullptr: never)
 };
 
-// V s is a correction of rounding size: with ||s|| <= 2^-34 ||u||, its float32 sums (errors below
-// 2^-22 of each term) change v_j by less than 2^-56 of its size, and the float64 unit, which bounds
-// the float64 update, has only V z left: one multiply-add per value of V instead of two.
-constexpr double kArnSmall2 = 0x1p-68;
 constexpr int kArnGroup = 16;       // blocks per group of the two-level reduction
 constexpr int kArnTickets = 256;    // ticket words: 1 + gridDim.x / kArnGroup at most
 constexpr int kArnCols = 64;        // columns per grid y of the plain dots kernel
@@ -142,7 +138,6 @@ __device__ __forceinline__ void arn_scalars(const D *tot, int j, int nv, const A
             const double beta = b2 > 0.0 ? sqrt(b2) : (b2 == b2 ? 0.0 : b2), inv = beta > 0.0 ? 1.0 / beta : (beta == beta ? 0.0 : beta);
             a.beta[0] = beta;
             a.beta[1] = inv;
-            a.beta[2] = ss <= kArnSmall2 * dreal(tot[nv * j]) ? 1.0 : 0.0;
             if (nv == 2) a.t[0] = rscale(inv, dsub(tot[2 * j + 1], sz));
         }
     }
@@ -320,28 +315,6 @@ __device__ __forceinline__ float4 scal(double s, const float4 &a) {
     return make_float4(f * a.x, f * a.y, f * a.z, f * a.w);
 }
 
-// The correction V s in float32 (see kArnSmall2): the top 24 bits of a float64 by integer
-// operations (a conversion instruction runs at the float64 rate); magnitudes below 2^-126 give
-// (nearly) zero, and the columns of V are unit vectors.
-__device__ __forceinline__ float trunc_f(double v) {
-    const int hi = __double2hiint(v);
-    const int e = max((hi & 0x7fffffff) - 0x38000000, 0);
-    return __int_as_float((int)__funnelshift_l((unsigned)__double2loint(v), (unsigned)e, 3) | (hi & 0x80000000));
-}
-struct cplxf { float re, im; };
-template <class T> struct ArnLow { using type = T; };
-template <> struct ArnLow<double> { using type = float; };
-template <> struct ArnLow<cplx> { using type = cplxf; };
-__device__ __forceinline__ float axpy_low(float s, double v, float x) { return fmaf(s, trunc_f(v), x); }
-__device__ __forceinline__ cplxf axpy_low(cplxf s, cplx v, cplxf x) {
-    const float a = trunc_f(v.re), b = trunc_f(v.im);
-    return {fmaf(s.re, a, fmaf(-s.im, b, x.re)), fmaf(s.re, b, fmaf(s.im, a, x.im))};
-}
-__device__ __forceinline__ float to_low(double s) { return (float)s; }
-__device__ __forceinline__ cplxf to_low(cplx s) { return {(float)s.re, (float)s.im}; }
-__device__ __forceinline__ double from_low(float x) { return (double)x; }
-__device__ __forceinline__ cplx from_low(cplxf x) { return {(double)x.re, (double)x.im}; }
-
 // The update sweep; the grid's last block does the Hessenberg column instead of rows.  F4: 4
 // rows per thread as float4 (float32, 16-byte aligned columns, rows padded to the leading
 // dimension).  CS threads share a row and take every CS-th column: with one thread a row, a grid
@@ -358,14 +331,9 @@ __global__ void __launch_bounds__(kThreads) k_arn_update(T *__restrict__ V, size
         arn_hessenberg<HT>(H, ldh, j, j0, last, a);
         return;
     }
-    using L = typename ArnLow<T>::type;
-    constexpr bool kLow = !std::is_same<L, T>::value;
     __shared__ T ss[MC], zs[MC];         // in the vector type, converted once per block
-    __shared__ L sl[kLow ? MC : 1];
     __shared__ X red[CS > 1 ? 2 * kThreads : 1];
-    const bool low = kLow && a.beta[2] != 0.0;
     for (int c = threadIdx.x; c < j; c += blockDim.x) {
-        if constexpr (kLow) sl[c] = to_low(a.s[c]);
         ss[c] = KS<T>::of(a.s[c]);
         zs[c] = last ? ST<T>::zero() : KS<T>::of(a.z[c]);
     }
@@ -378,20 +346,7 @@ __global__ void __launch_bounds__(kThreads) k_arn_update(T *__restrict__ V, size
     for (int64_t base = (int64_t)blockIdx.x * RB; base < rows; base += (int64_t)nb * RB) {
         const int64_t row = base + r;
         X x{}, y{};
-        if (kLow && low) {
-            if constexpr (kLow) {
-                L xl{};
-                if (row < rows) {
-#pragma unroll 8
-                    for (int c = q; c < j; c += CS) {
-                        const T v = VX[(size_t)c * ld + row];
-                        xl = axpy_low(sl[c], v, xl);
-                        if (!last) y = axpy(zs[c], v, y);
-                    }
-                }
-                x = from_low(xl);
-            }
-        } else if (row < rows) {
+        if (row < rows) {
 #pragma unroll 8
             for (int c = q; c < j; c += CS) {
                 const X v = VX[(size_t)c * ld + row];
