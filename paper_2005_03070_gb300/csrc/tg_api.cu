@@ -298,7 +298,7 @@ struct SmallArea {
     static constexpr size_t proj_d = 16384;     // projection coefficients d
     static constexpr size_t arn_h1 = 24576;     // V^H w, first pass; Arnoldi: s
     static constexpr size_t arn_h2 = 32768;     // second pass; Arnoldi: z
-    static constexpr size_t arn_nrm = 40960;    // ||w||^2, 1 / ||w|| (+ 32); Arnoldi: beta, 1 / beta, t (+ 64)
+    static constexpr size_t arn_nrm = 40960;    // ||w||^2, 1 / ||w|| (+ 32); Arnoldi: beta (4 values), t (+ 64)
     static constexpr size_t gmres_inv = 41984;  // 1 / ||r|| of a GMRES cycle
     static constexpr size_t arn_c = 49152;      // Arnoldi: first-pass coefficients h1
     static constexpr size_t sync = 57344;       // SyncWords of a one-launch cycle
@@ -1984,6 +1984,7 @@ static int arnoldi_sweeps(tg_op *op, T *V, size_t ldv, int n, int j, int last, i
     a.part = wsp<D>(op, S_PART);
     a.ticket = wsp<unsigned>(op, S_TICKET);
     a.skip = skip;
+    a.j0 = j0;
     const int ev = prof_begin(s);
     if (piped) {
         if constexpr (kReal) {

@@ -10,6 +10,9 @@
 //   update  v_j = (u - V s) / beta and the next u = (w - V z - t v_j) / beta in one sweep;
 //   Hbar    column j-1 is h1 + s over beta; the next h1 = ([z; t] - Hbar s) / beta, because
 //           A v_j = (w - A V s) / beta and A V s = V_{0..j} Hbar s.
+// u is kept times a power of two g that brings its norm near 1 (s, beta and w, z, t carry it too and
+// lose it in the quotients): without it w = A u grows as ||A||^2 and u^H w as its cube, which left the
+// range of a float32 basis at ||A|| = 7e12.
 // A last pair of sweeps without w (last = 1) finishes column m.  Against two complete passes per
 // step (four sweeps and nine launches) this reads the basis half as often, in three launches;
 // the operations on it are the same.  Against that form: the float32 basis of 127^3 rows, bound by
@@ -25,7 +28,8 @@ namespace tg {
 template <class D>
 struct ArnState {
     D *s, *z, *h1;        // kMaxCols each
-    double *beta;         // beta, 1 / beta (0 when u vanished)
+    double *beta;         // beta / g, 1 / beta (0 when u vanished), 1 / g, and the next g
+    int j0;               // the run's first column: g = 1 there
     D *t;
     D *part;              // block partials [gridDim.x][2 (j + 1)], then the groups'
     unsigned *ticket;     // ticket 0 and one per group of blocks, zero between launches
@@ -111,6 +115,9 @@ __device__ __forceinline__ P warp_sums(P (&v)[NV]) {
     return r;
 }
 
+// high word of the largest part's magnitude
+__device__ __forceinline__ int dmag(double a) { return __double2hiint(a) & 0x7fffffff; }
+__device__ __forceinline__ int dmag(cplx a) { return max(dmag(a.re), dmag(a.im)); }
 __device__ __forceinline__ double cmulc(double a, double b) { return a * b; }
 __device__ __forceinline__ cplx cmulc(cplx a, cplx b) { return ST<cplx>::conj_mul(a, b); }
 __device__ __forceinline__ double rscale(double s, double a) { return s * a; }
@@ -126,19 +133,34 @@ __device__ __forceinline__ void arn_scalars(const D *tot, int j, int nv, const A
     if (threadIdx.x < 32) {
         double ss = 0.0;
         D sz = dzero<D>();
+        int mag = 0;                     // high word of the largest part of z, then of t
         for (int c = threadIdx.x; c < j; c += 32) {
             const D s = tot[nv * c];
             ss += dreal(cmulc(s, s));
-            if (nv == 2) sz = dadd(sz, cmulc(s, tot[2 * c + 1]));
+            if (nv == 2) {
+                sz = dadd(sz, cmulc(s, tot[2 * c + 1]));
+                mag = max(mag, dmag(tot[2 * c + 1]));
+            }
         }
         ss = warp_sum(ss);
         if (nv == 2) sz = warp_sum(sz);
+        mag = __reduce_max_sync(0xffffffffu, mag);
         if (threadIdx.x == 0) {
             const double b2 = dreal(tot[nv * j]) - ss;
             const double beta = b2 > 0.0 ? sqrt(b2) : (b2 == b2 ? 0.0 : b2), inv = beta > 0.0 ? 1.0 / beta : (beta == beta ? 0.0 : beta);
-            a.beta[0] = beta;
+            const double ginv = j > a.j0 ? __hiloint2double((2046 << 20) - __double2hiint(a.beta[3]), 0) : 1.0;
+            a.beta[0] = beta * ginv;
             a.beta[1] = inv;
-            if (nv == 2) a.t[0] = rscale(inv, dsub(tot[2 * j + 1], sz));
+            a.beta[2] = ginv;
+            if (nv == 2) {
+                a.t[0] = rscale(inv, dsub(tot[2 * j + 1], sz));
+                // the next u is of the size of A v_j: of its parts in V, z and t over beta, or of the last one
+                mag = max(mag, dmag(a.t[0]));
+                const int eb = dmag(beta) >> 20;
+                int e = mag >= 0x100000 && eb > 0 ? (mag >> 20) - eb : -500;
+                if (j > a.j0 && eb > 0) e = max(e, (dmag(a.beta[0]) >> 20) - 1023);
+                a.beta[3] = e > -500 && e < 500 ? __hiloint2double((1023 - e) << 20, 0) : 1.0;
+            }
         }
     }
 }
@@ -279,7 +301,8 @@ __device__ __forceinline__ void arn_hessenberg(HT *H, int ldh, int j, int j0, in
     const double inv = a.beta[1];
     if (j > j0) {
         HT *col = H + (size_t)(j - 1) * ldh;
-        for (int i = threadIdx.x; i < j; i += blockDim.x) col[i] = dadd(a.h1[i], a.s[i]);
+        const double ginv = a.beta[2];
+        for (int i = threadIdx.x; i < j; i += blockDim.x) col[i] = dadd(a.h1[i], rscale(ginv, a.s[i]));
         if (threadIdx.x == 0) {
             HT b = ST<HT>::zero();
             *reinterpret_cast<double *>(&b) = a.beta[0];
@@ -338,7 +361,7 @@ __global__ void __launch_bounds__(kThreads) k_arn_update(T *__restrict__ V, size
         zs[c] = last ? ST<T>::zero() : KS<T>::of(a.z[c]);
     }
     __syncthreads();
-    const double inv = a.beta[1];
+    const double inv = a.beta[1], ginv = last ? 0.0 : inv * a.beta[3];
     const T mt = last ? ST<T>::zero() : neg(KS<T>::of(a.t[0]));
     const int rows = (n + W - 1) / W, r = threadIdx.x % RB, q = threadIdx.x / RB;
     const size_t ld = ldv / W;
@@ -369,7 +392,7 @@ __global__ void __launch_bounds__(kThreads) k_arn_update(T *__restrict__ V, size
         if (row < rows) {
             const X v = scal(inv, sub(u[row], x));
             u[row] = v;
-            if (!last) w[row] = scal(inv, axpy(mt, v, sub(w[row], y)));
+            if (!last) w[row] = scal(ginv, axpy(mt, v, sub(w[row], y)));
         }
     }
 }

@@ -15,9 +15,9 @@ def _op(N, e):
     return A, torch.randn(A.n, dtype=torch.float64, device="cuda", generator=g)
 
 
-def _coarse(N, e, m, k, precision):
+def _coarse(N, e, m, k, precision, cycles=4):
     A, b = _op(N, e)
-    xc, d, st, _ = A.coarse_gmresdr(b, m, k, rtolev=1e-8, rtol=1e-12, max_cycles=4, precision=precision)
+    xc, d, st, _ = A.coarse_gmresdr(b, m, k, rtolev=1e-8, rtol=1e-12, max_cycles=cycles, precision=precision)
     return xc * 2.0 ** e, d.copy(0), st["coarse_mvps"], st["cycles"]
 
 
@@ -30,6 +30,24 @@ def _same(got, want):
 @pytest.mark.parametrize("e", [-200, -60, 60, 200])
 def test_coarse_f64(N, m, k, e):
     _same(_coarse(N, e, m, k, "f64"), _coarse(N, 0, m, k, "f64"))
+
+
+@pytest.mark.parametrize("N,m,k", [(31, 24, 8), (33, 20, 7), (127, 30, 15), (255, 40, 12)])
+@pytest.mark.parametrize("e", [-60, -30, 30, 60])
+def test_coarse_f32(N, m, k, e):
+    """The float32 basis: values of A, about 2^17 at most, stay within 2^-80 .. 2^80."""
+    _same(_coarse(N, e, m, k, "f32_ir"), _coarse(N, 0, m, k, "f32_ir"))
+
+
+@pytest.mark.parametrize("N,m", [(31, 24), (127, 30)])
+@pytest.mark.parametrize("e", [-340, 340])
+def test_coarse_far(N, m, e):
+    """Norms whose cube leaves the float64 range.  Squares of squares do too, so that the small problems
+    rescale by other numbers than powers of two: one cycle, whose solution is compared to 1e-9 as in
+    the other one-cycle tests."""
+    got, want = _coarse(N, e, m, 8, "f64", 1), _coarse(N, 0, m, 8, "f64", 1)
+    assert got[2:] == want[2:]
+    assert ((got[0] - want[0]).norm() / want[0].norm()).item() <= 1e-9
 
 
 @pytest.mark.parametrize("N", [33, 127])
