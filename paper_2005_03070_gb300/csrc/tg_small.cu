@@ -739,7 +739,7 @@ __device__ int complex_schur(cplx *H, int m, cplx *Z) {
                 cplx disc = p * p + b * c;
                 // principal square root
                 double r = cabs_(disc);
-                double sr = sqrt(0.5 * (r + disc.re));
+                double sr = sqrt(fmax(0.0, 0.5 * (r + disc.re)));     // hypot may fall short of |disc.re|
                 double si = sqrt(fmax(0.0, 0.5 * (r - disc.re)));
                 if (disc.im < 0) si = -si;
                 cplx sq_ = mkc(sr, si);
