@@ -20,6 +20,7 @@
 // few float64 instructions on the critical path (see the Schur form section).
 #include <cfloat>
 #include <cmath>
+#include "tg_fastmath.cuh"
 #include "tg_small.cuh"
 
 namespace tg {
@@ -89,24 +90,6 @@ __device__ __forceinline__ cplx subt(cplx a, cplx b) { return a - b; }
 // took 3600 (Schur form of a restart 4.6 -> 3.5 ms).
 constexpr unsigned kFull = 0xffffffffu;
 
-// Seeds good to about 2^-20 (rsqrt.approx.ftz.f64, rcp.approx.ftz.f64) and one cubic step each:
-// r (1 + e (1/2 + 3/8 e)) with e = 1 - x r^2 (Halley), r (1 + e + e^2) with e = 1 - x r.  The
-// remaining error is below 2^-58 for x in the normal range.
-__device__ __forceinline__ double rsqrt_seed(double x) {
-    double r;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    return r;
-}
-__device__ __forceinline__ double rcp_fast(double x) {
-    double r;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    const double e = fma(-x, r, 1.0);
-    return fma(r, fma(e, e, e), r);
-}
-// 2^-900 < x < 2^900, on the exponent bits
-__device__ __forceinline__ bool mid_range(double x) {
-    return (unsigned)((__double2hiint(x) >> 20) - 123) < 1800u;
-}
 __device__ __forceinline__ double shfl_all(double v, int l) { return __shfl_sync(kFull, v, l); }
 __device__ __forceinline__ cplx shfl_all(cplx v, int l) { return {shfl_all(v.re, l), shfl_all(v.im, l)}; }
 __device__ __forceinline__ void bar_two_warps() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
@@ -143,8 +126,7 @@ __device__ __forceinline__ double givens_warp(double v, double *rs) {
             u = v * (1.0 / mx);
             s2 = norm2(u);
         }
-        const double r0 = rsqrt_seed(s2), e = fma(-(s2 * r0), r0, 1.0);
-        const double inv = fma(r0, e * fma(0.375, e, 0.5), r0);
+        const double inv = rsqrt_fast(s2);
         out = u * inv;
         r = s2 * inv * mx;
     }
@@ -168,8 +150,7 @@ __device__ __forceinline__ double reflect_warp(double x, double y, double z, dou
         n2 = fma(x, x, sn);
     }
     if (__double_as_longlong(sn) != 0) {       // tests on the bits: a float64 compare is a link of the chain too
-        const double r0 = rsqrt_seed(n2), h = n2 * r0, e = fma(-h, r0, 1.0);
-        const double alpha = fma(h * e, fma(0.375, e, 0.5), h);
+        const double alpha = sqrt_fast(n2);
         g = rcp_fast(fma(alpha, fabs(x), n2));
         const double bs = -copysign(alpha, x);
         w0 = x - bs;
@@ -225,22 +206,14 @@ __device__ __forceinline__ void reflector_warp(const T *x, int len, T *w, double
     T w0 = Cx<T>::zero(), bt = x0;
     double g = 0.0;
     if (__double_as_longlong(sn) != 0) {
-        double alpha;
-        if (mid_range(n2)) {
-            const double r0 = rsqrt_seed(n2), h = n2 * r0, e = fma(-h, r0, 1.0);
-            alpha = fma(h * e, fma(0.375, e, 0.5), h);
-        } else {
-            alpha = sqrt(n2);
-        }
+        const double alpha = mid_range(n2) ? sqrt_fast(n2) : sqrt(n2);
         double a0 = 0.0;
         T ph = Cx<T>::one();
         if constexpr (sizeof(T) == sizeof(double)) {
             a0 = fabs(x0);
             ph = copysign(1.0, x0);
         } else if (__double_as_longlong(ax2) != 0) {
-            double ia = rsqrt_seed(ax2);
-            const double e = fma(-(ax2 * ia), ia, 1.0);
-            ia = mid_range(ax2) ? fma(ia, e * fma(0.375, e, 0.5), ia) : rsqrt(ax2);
+            const double ia = mid_range(ax2) ? rsqrt_fast(ax2) : rsqrt(ax2);
             a0 = ax2 * ia;
             ph = Cx<T>::sc(ia, x0);
         }
