@@ -301,7 +301,6 @@ struct SmallArea {
     static constexpr size_t arn_nrm = 40960;    // ||w||^2, 1 / ||w|| (+ 32); Arnoldi: beta (4 values), t (+ 64)
     static constexpr size_t gmres_inv = 41984;  // 1 / ||r|| of a GMRES cycle
     static constexpr size_t arn_c = 49152;      // Arnoldi: first-pass coefficients h1
-    static constexpr size_t sync = 57344;       // SyncWords of a one-launch cycle
     static constexpr size_t bytes = 1 << 16;
 };
 static_assert(kMaxCols * 16 <= 8192, "coefficient vectors must fit their slots");
@@ -1142,19 +1141,22 @@ static int persist_ready(tg_op *op, cudaStream_t s) {
     // two reduction buffers and the projection's partial sums
     return red_ready(op, (size_t)(2 * kPersPart + kPersCols) * num_sms() * sizeof(double), s);
 }
-static SyncWords *persist_words(tg_op *op) {
-    return reinterpret_cast<SyncWords *>(wsp<char>(op, S_SMALL) + SmallArea::sync);
-}
-// Reads a launch's report (bytes at dev) and its barrier words; a wait that gave up is an error
-// whatever the report says (at the first barrier there is none, and host keeps the last one).
-static int persist_look(tg_op *op, const void *dev, void *host, size_t bytes, const char *what, cudaStream_t s) {
-    char *pin = reinterpret_cast<char *>(op->pin.p);
-    SyncWords *w = reinterpret_cast<SyncWords *>(pin + (1 << 15));
-    TG_CHECK_CUDA(cudaMemcpyAsync(w, persist_words(op), sizeof(SyncWords), cudaMemcpyDeviceToHost, s));
-    TG_CHECK(readback(op, dev, bytes, s));
-    if (w->failed == kFailedStart) return kNotStarted;
-    memcpy(host, pin, bytes);
-    if (w->failed) {
+// A cycle's report and, behind it, the barrier words of its launch.
+template <class R> struct PersReport {
+    R r;
+    SyncWords words;
+};
+static_assert(sizeof(PersReport<BiPersOut>) <= SmallArea::dot_out - SmallArea::bistate &&
+              sizeof(PersReport<IdrState<double>>) <= SmallArea::proj_c - SmallArea::idr, "the reports fit their slots");
+// Reads a launch's report; a wait that gave up is an error whatever the report says (at the first barrier
+// there is none, and *host keeps the last one).
+template <class R>
+static int persist_look(tg_op *op, const PersReport<R> *dev, R *host, const char *what, cudaStream_t s) {
+    TG_CHECK(readback(op, dev, sizeof(*dev), s));
+    const PersReport<R> *got = reinterpret_cast<const PersReport<R> *>(op->pin.p);
+    if (got->words.failed == kFailedStart) return kNotStarted;
+    memcpy(host, &got->r, sizeof(R));
+    if (got->words.failed) {
         set_error("a grid barrier of the %s cycle timed out", what);
         return TG_SYNC_TIMEOUT;
     }
@@ -1175,15 +1177,15 @@ static int bicg_persist_run(tg_op *op, const DevOp &A, const DevOp32 &A32, BiPer
     a.rh = w.rh; a.p[0] = w.p; a.p[1] = wsp<T>(op, S_P2); a.v[0] = w.v; a.v[1] = wsp<T>(op, S_V2);
     a.s = w.s; a.t = w.t;
     a.part = wsp<double>(op, S_PART);
-    a.words = persist_words(op);
+    PersReport<BiPersOut> *rep = reinterpret_cast<PersReport<BiPersOut> *>(wsp<char>(op, S_SMALL) + SmallArea::bistate);
+    a.words = &rep->words;
     a.limits = op->sync;
-    a.out = reinterpret_cast<BiPersOut *>(wsp<char>(op, S_SMALL) + SmallArea::bistate);
+    a.out = &rep->r;
     a.max_iters = 1024;              // bounds one launch to some tens of milliseconds
-    static_assert(sizeof(BiPersOut) <= SmallArea::dot_out - SmallArea::bistate, "the report fits its slot");
     *res = BiPersOut{};
     double xb, fl;
     op_cost(A, &xb, &fl);
-    auto look = [&]() { return persist_look(op, a.out, res, sizeof(BiPersOut), "BiCGStab", s); };
+    auto look = [&]() { return persist_look(op, rep, res, "BiCGStab", s); };
     for (a.first = 1;; a.first = 0) {
         const int it0 = res->st.iters, ev = prof_begin(s);
         int rc = persist_launch(k_bi_persist<T>, A, A32, a, s);
@@ -1678,15 +1680,17 @@ static int idr_cycle(tg_op *op, const DevOp &A, const DevOp32 &A32, T *x, T *r, 
             IdrPersArgs<T> a;
             a.P = P; a.x = x; a.r = r; a.G = G; a.U = U; a.t = t; a.ld = ld;
             a.part = wsp<double>(op, S_PART);
-            a.words = persist_words(op);
+            PersReport<IdrState<double>> *rep =
+                reinterpret_cast<PersReport<IdrState<double>> *>(wsp<char>(op, S_SMALL) + SmallArea::idr);
+            a.words = &rep->words;
             a.limits = op->sync;
-            a.st = st; a.target2 = target2; a.kappa = kappa; a.s = sd; a.cap = cap;
+            a.st = &rep->r; a.target2 = target2; a.kappa = kappa; a.s = sd; a.cap = cap;
             a.max_rounds = 64;           // bounds one launch to a few milliseconds
             IdrState<double> h{};
             int rc = TG_OK;
             for (a.first = 1;; a.first = 0) {
                 TG_PROF(P_IDR_CYCLE, 0, 0, rc = persist_launch(k_idr_persist<T>, A, A32, a, s));
-                if (rc == TG_OK) rc = persist_look(op, st, &h, sizeof(h), "IDR", s);
+                if (rc == TG_OK) rc = persist_look(op, rep, &h, "IDR", s);
                 if (rc == kNotStarted) break;
                 TG_CHECK(rc);
                 if (h.status != 0) break;
