@@ -1103,10 +1103,12 @@ struct CycleOut {
 
 // Cycles on real grids of up to this many points run in one cooperative launch (tg_persist.cuh);
 // beyond, the neighbours' recomputed updates and one block per SM cost more than the launches.
-// us per product, one launch / chain of launches: BiCGStab float64 127^2 7.1 / 21 (plain launches),
-// 511^2 18.5 / 34, 767^2 36 / 40, 79^3 42 / 50, 95^3 67 / 58; float32 + refinement 127^2 6.0 / 20,
-// 639^2 15.9 / 17.8, 71^3 23.6 / 24.8, 79^3 29 / 27; IDR(4) 511^2 28 / 70, 767^2 55 / 79, 95^3 100 / 107,
-// 1023^2 126 / 103.
+// us per product, one launch / chain of launches: BiCGStab float64 127^2 5.3 / 10.7, 511^2 17.7 / 30.6,
+// 767^2 35.4 / 38.5, 83^3 38.2 / 40.4, past the limit 895^2 44.8 / 43.2, 93^3 48.0 / 45.7; float32 +
+// refinement 127^2 4.4 / 10.0, 623^2 13.9 / 16.6, 71^3 16.0 / 16.0, past it 767^2 19.6 / 18.7, 79^3 20.0 /
+// 17.4; IDR(4) 127^2 11.2 / 18.6, 511^2 28.9 / 60.4, 895^2 77.7 / 88.0, 93^3 77.0 / 91.4, past it 1023^2
+// 129 / 103, 101^3 127 / 106.  One limit serves 2D and 3D: it lies near the earlier crossing, the 3D one; a 2D
+// float32 grid between it and 700^2 would gain up to 10%.
 template <class T> constexpr int pers_max_rows(bool idr) {
     return sizeof(T) == 4 ? 6 << 16 : idr ? 13 << 16 : 9 << 16;
 }

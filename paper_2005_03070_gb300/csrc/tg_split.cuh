@@ -132,7 +132,7 @@ __device__ __forceinline__ double split_rescale(double r, int E1, int E2) { retu
 // registers left two warps per scheduler, whose conversion, mma and join phases did not overlap
 // (n = 191^3, p = q = 30: 3.0 ms).  gridDim.y splits the columns when the digits of all of S do not fit
 // (in place, Out = In, only with gridDim.y = 1: each tile is staged before it is written).
-// n = 191^3, p = q = 30: 3.0 ms (the float64 unit: 11.2); complex128, n = 32^4, p = q = 40: 2.0 ms
+// n = 191^3, p = q = 30: 3.0 ms, with scales 3.4 (the float64 unit: 11.2); complex128, n = 32^4, p = q = 40: 2.0 ms
 // (10.9).  The mma take 0.9 ms of the 3.0 and the bytes 0.5; issuing the conversions and joins
 // (27 thousand warp instructions a 128-row tile, 2 a clock) bounds it.
 // SC: norm2[i nstride] is the square of the norm of In's column i (device), and the scales above are
